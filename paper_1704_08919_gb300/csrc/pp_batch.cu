@@ -232,12 +232,12 @@ BatchTable make_batch_table(bool all, int default_cfg)
 const BatchTable &batch_table(int precision, int scheme)
 {
     static const BatchTable t[3][3] = {
-        {make_batch_table<ScalarPolicy<double, false>>(false, 0),
+        {make_batch_table<Rk4Policy<double, false>>(false, 0),
          make_batch_table<MagnusPolicy<double, false>>(false, 0),
          make_batch_table<SplitPolicy<double, false>>(false, 0)},
-        {make_batch_table<PackedPolicy<true>>(true, 0), make_batch_table<MagnusPolicy<float, true>>(true, 2),
+        {make_batch_table<Rk4Policy<float, true>>(true, 0), make_batch_table<MagnusPolicy<float, true>>(true, 2),
          make_batch_table<SplitPolicy<float, true>>(true, 0)},
-        {make_batch_table<PackedPolicy<false>>(true, 0),
+        {make_batch_table<Rk4Policy<float, false>>(true, 0),
          make_batch_table<MagnusPolicy<float, false>>(true, 0),
          make_batch_table<SplitPolicy<float, false>>(true, 3)},
     };

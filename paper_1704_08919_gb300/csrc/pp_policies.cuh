@@ -10,6 +10,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "pp_internal.cuh"
 
 namespace {
@@ -22,17 +24,6 @@ constexpr int kGroup = 128;
 struct alignas(32) dbl4 {
     double x, y, z, w;
 };
-template <typename T>
-struct Vec4;
-template <>
-struct Vec4<float> {
-    using type = float4;
-};
-template <>
-struct Vec4<double> {
-    using type = dbl4;
-};
-
 // e = -i (h . sigma) z for a 2-vector z = (z0r, z0i, z1r, z1i).
 template <typename T>
 __device__ __forceinline__ void rot(T hx, T hy, T hz, const T z[4], T e[4])
@@ -41,16 +32,6 @@ __device__ __forceinline__ void rot(T hx, T hy, T hz, const T z[4], T e[4])
     e[1] = fma(hy, -z[3], fma(hx, -z[2], -hz * z[0]));
     e[2] = fma(hz, -z[3], fma(hy, z[0], hx * z[1]));
     e[3] = fma(hz, z[2], fma(hy, z[1], -hx * z[0]));
-}
-
-// acc += -i (h . sigma) z
-template <typename T>
-__device__ __forceinline__ void rot_acc(T hx, T hy, T hz, const T z[4], T acc[4])
-{
-    acc[0] = fma(hy, -z[2], fma(hx, z[3], fma(hz, z[1], acc[0])));
-    acc[1] = fma(hy, -z[3], fma(hx, -z[2], fma(-hz, z[0], acc[1])));
-    acc[2] = fma(hz, -z[3], fma(hy, z[0], fma(hx, z[1], acc[2])));
-    acc[3] = fma(hz, z[2], fma(hy, z[1], fma(-hx, z[0], acc[3])));
 }
 
 // Node i of linspace(a, b, n), rounded exactly as a + ((b - a) * i) / (n - 1).
@@ -93,32 +74,78 @@ __device__ __forceinline__ double proj_pos2(double hx, double hy, double hz, con
 }
 
 // ---------------------------------------------------------------- stepping policies
-// A policy supplies the per-step table entry (Entry), the tile length, the
-// per-thread state and the RK4 step.  Table entry n holds the potential of
-// step n scaled for the stages: (dt/3) A(t_{n+1/2}) and (dt/6) A(t_{n+1}).
+// A policy supplies the per-step table entry (Entry), the per-thread state and the step.
 
-// Scalar policy: T = double (parity path) or float (COMP: compensated state).
+// Low part of dt x p against its rounding hi to T.
+template <typename T>
+__device__ __forceinline__ T low_part(double dt, double p, T hi)
+{
+    if constexpr (sizeof(T) == 8)
+        return fma(dt, p, -hi);
+    else
+        return (T)(dt * p - (double)hi);
+}
+
+// Classical RK4 with the step matrix in closed form.  A product of h's Pauli matrices is
+// (a.sigma)(b.sigma) = a.b + i (a x b).sigma, so the step
+//     1 - i dt/6 (H_0 + 4 H_m + H_1) - dt^2/6 (H_m H_0 + H_m^2 + H_1 H_m)
+//       + i dt^3/12 (H_m^2 H_0 + H_1 H_m^2) + dt^4/24 H_1 H_m^2 H_0,   H = h.sigma,
+// (the four stages multiplied out) is alpha - i g.sigma with real alpha and g.  With u = dt h_m,
+// c = dt (h_0 + h_1 - 2 h_m) and d = dt (h_1 - h_0), which do not depend on the mode and have no z part,
+// M = |u|^2, Y = u.c and q = (|c|^2 - |d|^2) / 4:
+//     alpha - 1 = -M/2 - Y/6 + M (M + Y + q) / 24
+//     g = (1 - M/6) u + (1/6 - M/12) c + (1/6 - M/24) d x u - (M/48) (d x c)_z z.
+// The first two terms of g keep their form under the reflection y -> -y that takes spin channel s = +1 to
+// s = -1 and the last two change sign, so everything but g's last additions is formed once for both channels.
+// 30 multiply-adds to form the step and 16 per channel to apply it, 62 in all, where the four stages applied to
+// the state took 148 (FP64) and 184 (compensated FP32).  The path is bound by the FP64 / FP32 lanes, so the time
+// follows: 2 pulses on 64 x 64 x 32 modes, 8192 steps in FP64 576.6 -> 241.1 ms; 32 x 32 x 16 modes, 4000 steps
+// 40.3 -> 16.9 ms; in compensated FP32, 8 pulses on 600 modes, 800 steps 208 -> 132 us (whole calls).
+// The rounding of dt p to T is the same at every step and would add up as a phase, so its low part joins
+// g at no cost (the sum's first product becomes a multiply-add).  COMP: the state is a two-float (hi, lo) pair
+// and the increment is formed apart and added by Fast2Sum.
+// In FP64 the table keeps dt (A_m, A_1) alone (32 bytes a step) and each CTA expands a span of it in shared
+// memory; in FP32 the table holds the expanded entry (32 bytes).
 template <typename T, bool COMP>
-struct ScalarPolicy {
-    using Entry = typename Vec4<T>::type;
+struct Rk4Policy {
+    struct alignas(sizeof(T) * 8) Coef {
+        T ax, ay, cx, cy, dx, dy, q, p;  // p = (d x c)_z / 48
+    };
+    static constexpr bool kExpands = sizeof(T) == 8;
+    using Entry = typename std::conditional<kExpands, dbl4, Coef>::type;
 
-    __device__ static Entry make_entry(double ax3, double ay3, double ax6, double ay6)
+    __device__ static __forceinline__ Coef coef(double a0x, double a0y, double amx, double amy, double a1x,
+                                                double a1y)
     {
-        Entry e;
-        e.x = (T)ax3;
-        e.y = (T)ay3;
-        e.z = (T)ax6;
-        e.w = (T)ay6;
+        Coef e;
+        const double cx = fma(2.0, amx, -(a0x + a1x)), cy = fma(2.0, amy, -(a0y + a1y));
+        const double dx = a0x - a1x, dy = a0y - a1y;
+        e.ax = (T)amx;
+        e.ay = (T)amy;
+        e.cx = (T)cx;
+        e.cy = (T)cy;
+        e.dx = (T)dx;
+        e.dy = (T)dy;
+        e.q = (T)(0.25 * (fma(cx, cx, cy * cy) - fma(dx, dx, dy * dy)));
+        e.p = (T)((dx * cy - dy * cx) / 48.0);
         return e;
+    }
+
+    __device__ static Entry make_entry(double dt, double a0x, double a0y, double amx, double amy, double a1x,
+                                       double a1y)
+    {
+        if constexpr (kExpands)
+            return dbl4{dt * amx, dt * amy, dt * a1x, dt * a1y};
+        else
+            return coef(dt * a0x, dt * a0y, dt * amx, dt * amy, dt * a1x, dt * a1y);
     }
 
     struct State {
         T hi[2][4], lo[2][4];
-        T px3, py3, px6, py6, ez3, ez6, q6x, q6y;
+        T px, py, uz, uz2, lx, ly, lz;  // dt p_x, dt p_y, dt eps, its square, and the first three's low parts
     };
 
-    __device__ static void init(State &st, const double v[2][4], double px, double py, double eperp,
-                                double d3, double d6, double ax0, double ay0)
+    __device__ static void init(State &st, const double v[2][4], double px, double py, double eperp, double dt)
     {
 #pragma unroll
         for (int s = 0; s < 2; ++s)
@@ -127,58 +154,61 @@ struct ScalarPolicy {
                 st.hi[s][q] = (T)v[s][q];
                 st.lo[s][q] = (T)(v[s][q] - (double)st.hi[s][q]);
             }
-        st.px3 = (T)(d3 * px);
-        st.py3 = (T)(d3 * py);
-        st.px6 = (T)(d6 * px);
-        st.py6 = (T)(d6 * py);
-        st.ez3 = (T)(d3 * eperp);
-        st.ez6 = (T)(d6 * eperp);
-        st.q6x = st.px6 - (T)(d6 * ax0);
-        st.q6y = st.py6 - (T)(d6 * ay0);
+        st.px = (T)(dt * px);
+        st.py = (T)(dt * py);
+        st.uz = (T)(dt * eperp);
+        st.uz2 = (T)((dt * eperp) * (dt * eperp));
+        st.lx = low_part(dt, px, st.px);
+        st.ly = low_part(dt, py, st.py);
+        st.lz = low_part(dt, eperp, st.uz);
     }
 
-    __device__ static __forceinline__ void step(State &st, const Entry &e)
+    __device__ static __forceinline__ void step(State &st, const Coef &e)
     {
-        const T q3x = st.px3 - e.x, q3y = st.py3 - e.y;
-        const T n6x = st.px6 - e.z, n6y = st.py6 - e.w;
+        const T ux = st.px - e.ax, uy = st.py - e.ay;
+        const T M = fma(ux, ux, fma(uy, uy, st.uz2));
+        const T Y = fma(ux, e.cx, uy * e.cy);
+        const T e1 = fma(M, (T)(-1.0 / 6.0), (T)1);
+        const T e2 = fma(M, (T)(-1.0 / 12.0), (T)(1.0 / 6.0));
+        const T k = fma(M, (T)(-1.0 / 24.0), (T)(1.0 / 6.0));
+        const T Ex = fma(ux, e1, fma(e.cx, e2, st.lx));
+        const T Ey = fma(uy, e1, fma(e.cy, e2, st.ly));
+        const T Ez = fma(st.uz, e1, st.lz);
+        const T kz = k * st.uz;
+        const T Oz = fma(k, fma(e.dx, uy, -e.dy * ux), -M * e.p);
+        const T am1 = fma(M, fma((M + Y) + e.q, (T)(1.0 / 24.0), (T)-0.5), Y * (T)(-1.0 / 6.0));
+        const T al = (T)1 + am1;
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-            const T a6 = s ? -st.q6y : st.q6y;
-            const T a3 = s ? -q3y : q3y;
-            const T b6 = s ? -n6y : n6y;
-            T e1[4], e2[4], y[4], S[4];
-            rot(st.q6x, a6, st.ez6, st.hi[s], e1);
+            const T gx = s ? fma(-e.dy, kz, Ex) : fma(e.dy, kz, Ex);
+            const T gy = s ? fma(-e.dx, kz, -Ey) : fma(-e.dx, kz, Ey);
+            const T gz = s ? Ez - Oz : Ez + Oz;
+            const T *z = st.hi[s];
+            if (COMP) {
+                T D[4];
+                D[0] = fma(gz, z[1], fma(gx, z[3], fma(-gy, z[2], am1 * z[0])));
+                D[1] = fma(-gz, z[0], fma(-gx, z[2], fma(-gy, z[3], am1 * z[1])));
+                D[2] = fma(gx, z[1], fma(gy, z[0], fma(-gz, z[3], am1 * z[2])));
+                D[3] = fma(-gx, z[0], fma(gy, z[1], fma(gz, z[2], am1 * z[3])));
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                y[q] = fma((T)3, e1[q], st.hi[s][q]);
-            rot(q3x, a3, st.ez3, y, e2);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                y[q] = fma((T)1.5, e2[q], st.hi[s][q]);
-                S[q] = e1[q] + e2[q];
-            }
-            rot(q3x, a3, st.ez3, y, e2);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                y[q] = fma((T)3, e2[q], st.hi[s][q]);
-                S[q] = S[q] + e2[q];
-                if (COMP)
-                    S[q] = S[q] + st.lo[s][q];
-            }
-            rot_acc(n6x, b6, st.ez6, y, S);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (COMP) {
-                    const T h = st.hi[s][q] + S[q];
-                    st.lo[s][q] = S[q] - (h - st.hi[s][q]);
+                for (int q = 0; q < 4; ++q) {
+                    const T Dl = D[q] + st.lo[s][q];
+                    const T h = st.hi[s][q] + Dl;
+                    st.lo[s][q] = Dl - (h - st.hi[s][q]);
                     st.hi[s][q] = h;
-                } else {
-                    st.hi[s][q] = st.hi[s][q] + S[q];
                 }
+            } else {
+                // the small products first: the state's own term is added last, in one rounding
+                T nz[4];
+                nz[0] = fma(al, z[0], fma(gz, z[1], fma(gx, z[3], -gy * z[2])));
+                nz[1] = fma(al, z[1], fma(-gz, z[0], fma(-gx, z[2], -gy * z[3])));
+                nz[2] = fma(al, z[2], fma(gx, z[1], fma(gy, z[0], -gz * z[3])));
+                nz[3] = fma(al, z[3], fma(-gx, z[0], fma(gy, z[1], gz * z[2])));
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    st.hi[s][q] = nz[q];
             }
         }
-        st.q6x = n6x;
-        st.q6y = n6y;
     }
 
     __device__ static void psi(const State &st, int s, double out[4], double, double, double,
@@ -187,180 +217,6 @@ struct ScalarPolicy {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             out[q] = COMP ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
-    }
-};
-
-// Packed FP32 policy: both spin channels in one 64-bit register pair per state
-// component (low half: s = +1, high half: s = -1), advanced together by the
-// sm_100+ packed instructions fma/add/sub/mul.rn.f32x2.  Channel s = -1 sees
-// h_y -> -h_y, so the table carries (A_x, A_x) and (A_y, -A_y) pairs; every
-// coefficient is also formed with the opposite sign, because the real form of
-// -i h.sigma has both signs of each coefficient.  Compensated (two-float) state.
-typedef unsigned long long f2;
-
-__device__ __forceinline__ f2 pk2(float a, float b)
-{
-    f2 d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
-    return d;
-}
-__device__ __forceinline__ void unpk2(f2 v, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f2 ffma2(f2 a, f2 b, f2 c)
-{
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f2 fadd2(f2 a, f2 b)
-{
-    f2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 fsub2(f2 a, f2 b)
-{
-    f2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 fmul2(f2 a, f2 b)
-{
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-// Scaled h at one time point, with both signs: (hx, -hx, hy, -hy) as channel pairs.
-struct H2 {
-    f2 x, nx, y, ny;
-};
-
-// e = -i (h . sigma) z for both channels (see rot()).
-__device__ __forceinline__ void rot2(const H2 &h, f2 hz, f2 nhz, const f2 z[4], f2 e[4])
-{
-    e[0] = ffma2(h.ny, z[2], ffma2(h.x, z[3], fmul2(hz, z[1])));
-    e[1] = ffma2(h.ny, z[3], ffma2(h.nx, z[2], fmul2(nhz, z[0])));
-    e[2] = ffma2(nhz, z[3], ffma2(h.y, z[0], fmul2(h.x, z[1])));
-    e[3] = ffma2(hz, z[2], ffma2(h.y, z[1], fmul2(h.nx, z[0])));
-}
-
-__device__ __forceinline__ void rot2_acc(const H2 &h, f2 hz, f2 nhz, const f2 z[4], f2 acc[4])
-{
-    acc[0] = ffma2(h.ny, z[2], ffma2(h.x, z[3], ffma2(hz, z[1], acc[0])));
-    acc[1] = ffma2(h.ny, z[3], ffma2(h.nx, z[2], ffma2(nhz, z[0], acc[1])));
-    acc[2] = ffma2(nhz, z[3], ffma2(h.y, z[0], ffma2(h.x, z[1], acc[2])));
-    acc[3] = ffma2(hz, z[2], ffma2(h.y, z[1], ffma2(h.nx, z[0], acc[3])));
-}
-
-struct alignas(32) PackedEntry {
-    f2 ax3, ay3, ax6, ay6;  // (dt/3)(A_x, A_x), (dt/3)(A_y, -A_y), (dt/6)(...), (dt/6)(...)
-};
-
-template <bool COMP>
-struct PackedPolicy {
-    using Entry = PackedEntry;
-
-    __device__ static Entry make_entry(double ax3, double ay3, double ax6, double ay6)
-    {
-        Entry e;
-        const float a = (float)ax3, b = (float)ay3, c = (float)ax6, d = (float)ay6;
-        e.ax3 = pk2(a, a);
-        e.ay3 = pk2(b, -b);
-        e.ax6 = pk2(c, c);
-        e.ay6 = pk2(d, -d);
-        return e;
-    }
-
-    struct State {
-        f2 hi[4], lo[4];
-        f2 px3, py3, px6, py6, ez3, nez3, ez6, nez6;
-        H2 h6;  // (dt/6) h at the current time t_n
-    };
-
-    __device__ static __forceinline__ H2 make_h(f2 px, f2 py, f2 ax, f2 ay)
-    {
-        H2 h;
-        h.x = fsub2(px, ax);
-        h.nx = fsub2(ax, px);
-        h.y = fsub2(py, ay);
-        h.ny = fsub2(ay, py);
-        return h;
-    }
-
-    __device__ static void init(State &st, const double v[2][4], double px, double py, double eperp,
-                                double d3, double d6, double ax0, double ay0)
-    {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float h0 = (float)v[0][q], h1 = (float)v[1][q];
-            st.hi[q] = pk2(h0, h1);
-            st.lo[q] = pk2((float)(v[0][q] - (double)h0), (float)(v[1][q] - (double)h1));
-        }
-        const float x3 = (float)(d3 * px), y3 = (float)(d3 * py);
-        const float x6 = (float)(d6 * px), y6 = (float)(d6 * py);
-        const float z3 = (float)(d3 * eperp), z6 = (float)(d6 * eperp);
-        st.px3 = pk2(x3, x3);
-        st.py3 = pk2(y3, -y3);
-        st.px6 = pk2(x6, x6);
-        st.py6 = pk2(y6, -y6);
-        st.ez3 = pk2(z3, z3);
-        st.nez3 = pk2(-z3, -z3);
-        st.ez6 = pk2(z6, z6);
-        st.nez6 = pk2(-z6, -z6);
-        const float a = (float)(d6 * ax0), b = (float)(d6 * ay0);
-        st.h6 = make_h(st.px6, st.py6, pk2(a, a), pk2(b, -b));
-    }
-
-    __device__ static __forceinline__ void step(State &st, const Entry &e)
-    {
-        const f2 three = pk2(3.0f, 3.0f), half3 = pk2(1.5f, 1.5f);
-        const H2 h3 = make_h(st.px3, st.py3, e.ax3, e.ay3);
-        const H2 hn = make_h(st.px6, st.py6, e.ax6, e.ay6);
-        f2 e1[4], e2[4], y[4], S[4];
-        rot2(st.h6, st.ez6, st.nez6, st.hi, e1);
-        #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            y[q] = ffma2(three, e1[q], st.hi[q]);
-        rot2(h3, st.ez3, st.nez3, y, e2);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            y[q] = ffma2(half3, e2[q], st.hi[q]);
-            S[q] = fadd2(e1[q], e2[q]);
-        }
-        rot2(h3, st.ez3, st.nez3, y, e2);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            y[q] = ffma2(three, e2[q], st.hi[q]);
-            S[q] = fadd2(S[q], e2[q]);
-            if (COMP)
-                S[q] = fadd2(S[q], st.lo[q]);
-        }
-        rot2_acc(hn, st.ez6, st.nez6, y, S);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const f2 h = fadd2(st.hi[q], S[q]);
-            if (COMP)
-                st.lo[q] = fsub2(S[q], fsub2(h, st.hi[q]));
-            st.hi[q] = h;
-        }
-        st.h6 = hn;
-    }
-
-    __device__ static void psi(const State &st, int s, double out[4], double, double, double,
-                               double)
-    {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float h0, h1, l0, l1;
-            unpk2(st.hi[q], h0, h1);
-            unpk2(st.lo[q], l0, l1);
-            if (!COMP)
-                l0 = l1 = 0.0f;
-            out[q] = s ? (double)h1 + (double)l1 : (double)h0 + (double)l0;
-        }
     }
 };
 
@@ -778,17 +634,14 @@ struct SplitPolicy {
     }
 };
 
-// Table builders: RK4 policies take (dt/3) A_{n+1/2} and (dt/6) A_{n+1};
-// the Magnus policy the Simpson mean and the commutator coefficients; the
-// split policy dt A_{n+1/2}.
-template <class P>
-__device__ __forceinline__ typename P::Entry table_entry(const P *, const double *Ax,
-                                                         const double *Ay, int n, double dt,
-                                                         const pp_grid &)
+// Table builders: RK4 takes dt A at the step's start, middle and end; the Magnus policy the Simpson mean
+// and the commutator coefficients; the split policy dt A_{n+1/2}.
+template <typename T, bool C>
+__device__ __forceinline__ typename Rk4Policy<T, C>::Entry
+table_entry(const Rk4Policy<T, C> *, const double *Ax, const double *Ay, int n, double dt, const pp_grid &)
 {
-    const double d3 = dt / 3.0, d6 = dt / 6.0;
-    return P::make_entry(d3 * Ax[2 * n + 1], d3 * Ay[2 * n + 1], d6 * Ax[2 * n + 2],
-                         d6 * Ay[2 * n + 2]);
+    return Rk4Policy<T, C>::make_entry(dt, Ax[2 * n], Ay[2 * n], Ax[2 * n + 1], Ay[2 * n + 1], Ax[2 * n + 2],
+                                       Ay[2 * n + 2]);
 }
 template <typename T, bool C>
 __device__ __forceinline__ typename MagnusPolicy<T, C>::Entry
@@ -806,26 +659,17 @@ table_entry(const SplitPolicy<T, C> *, const double *Ax, const double *Ay, int n
     return SplitPolicy<T, C>::make_entry2(dt, Ax[2 * n + 1], Ay[2 * n + 1]);
 }
 
-// State initialisation: the RK4 policies take the stage scales dt/3 and dt/6.
+// Policies whose table entries are expanded in shared memory, kExpandSpan steps at a time.
+constexpr int kExpandSpan = 128;
 template <class P>
-__device__ __forceinline__ void policy_init(typename P::State &st, const double v[2][4], double px,
-                                            double py, double eperp, double dt, double ax0,
-                                            double ay0, int)
-{
-    P::init(st, v, px, py, eperp, dt / 3.0, dt / 6.0, ax0, ay0);
-}
-
-template <class P>
-struct UsesDtInit {
+struct Expands {
     static constexpr bool value = false;
+    using Coef = char;
 };
-template <typename T, bool C>
-struct UsesDtInit<MagnusPolicy<T, C>> {
+template <bool C>
+struct Expands<Rk4Policy<double, C>> {
     static constexpr bool value = true;
-};
-template <typename T, bool C>
-struct UsesDtInit<SplitPolicy<T, C>> {
-    static constexpr bool value = true;
+    using Coef = typename Rk4Policy<double, C>::Coef;
 };
 
 // Policies whose series steps let the state's norm grow (rescale between tiles).
@@ -902,6 +746,7 @@ struct ItemSmem {
     __align__(128) V buf[2][TILE];
     __align__(8) uint64_t bar[2];
     double red[THREADS / 32];
+    typename Expands<P>::Coef coef[Expands<P>::value ? kExpandSpan : 1];
 };
 
 template <class P, int THREADS, int TILE_BYTES, bool WIDE>
@@ -953,10 +798,7 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
         double v[2][4];
         eig_neg(Pinx, Piny, eperp, v[0]);
         eig_neg(Pinx, -Piny, eperp, v[1]);
-        if constexpr (UsesDtInit<P>::value)
-            P::init(st, v, px, py, eperp, dt);
-        else
-            policy_init<P>(st, v, px, py, eperp, dt, Ax[0], Ay[0], 0);
+        P::init(st, v, px, py, eperp, dt);
     }
 
     bool timed_out = false;
@@ -973,7 +815,27 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
             break;
         }
         const int nst = min(TILE, ns - t * TILE);
-        if (active) {
+        if constexpr (Expands<P>::value) {
+            const V *tb = sm.buf[b];
+            for (int k0 = 0; k0 < nst; k0 += kExpandSpan) {
+                const int m1 = min(kExpandSpan, nst - k0);
+                if (tid < m1) {
+                    // the step's start is the end of the step before it
+                    const int n = t * TILE + k0 + tid;
+                    const double a0x = n ? (k0 + tid ? tb[k0 + tid - 1].z : trow[n - 1].z) : dt * Ax[0];
+                    const double a0y = n ? (k0 + tid ? tb[k0 + tid - 1].w : trow[n - 1].w) : dt * Ay[0];
+                    const V e = tb[k0 + tid];
+                    sm.coef[tid] = P::coef(a0x, a0y, e.x, e.y, e.z, e.w);
+                }
+                __syncthreads();
+                if (active) {
+#pragma unroll 2
+                    for (int kk = 0; kk < m1; ++kk)
+                        P::step(st, sm.coef[kk]);
+                }
+                __syncthreads();  // every thread is done with coef
+            }
+        } else if (active) {
             const V *tb = sm.buf[b];
             if constexpr (WIDE) {
                 for (int kk = 0; kk < nst; ++kk)

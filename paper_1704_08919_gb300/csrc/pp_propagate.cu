@@ -18,15 +18,10 @@
 // (pair_prod_homo) is
 //     f(p) = sum_s |<+, h_s(t_end) | U_s |-, h_s(t_0)>|^2.
 //
-// RK4 in increment form (one step, M_t = -i h(t).sigma, z = dt/6):
-//     e1 = z M_n psi,             y1 = psi + 3 e1
-//     e2 = 2z M_{n+1/2} y1,       y2 = psi + 1.5 e2
-//     e3 = 2z M_{n+1/2} y2,       y3 = psi + 3 e3
-//     psi <- psi + (e1 + e2 + e3 + z M_{n+1} y3)
-// which is the classical psi + dt/6 (k1 + 2 k2 + 2 k3 + k4).  In the FP32 path
-// the state is a two-float (hi, lo) pair and the increment is added with
-// Fast2Sum, so the O(1) state does not lose the small increments' low bits;
-// the initial state, the projection and the momentum sum are FP64.
+// The step of each scheme acts on a 2-level state as alpha - i g.sigma with real alpha and g
+// (pp_policies.cuh).  In the compensated FP32 path the state is a two-float (hi, lo) pair and the increment is
+// added with Fast2Sum, so the O(1) state does not lose the small increments' low bits; the initial state,
+// the projection and the momentum sum are FP64 in every path.
 #include <map>
 #include <mutex>
 
@@ -299,13 +294,13 @@ struct PolicySlot {
 
 const PolicySlot &policy_slot(int precision, int scheme)
 {
-    static const ConfigTable<ScalarPolicy<double, false>, true> d_rk4;  // tunable: small FP64 grids
+    static const ConfigTable<Rk4Policy<double, false>, true> d_rk4;  // tunable: small FP64 grids
     static const ConfigTable<MagnusPolicy<double, false>, false> d_mag;
     static const ConfigTable<SplitPolicy<double, false>, false> d_spl;
-    static const ConfigTable<PackedPolicy<true>, true> f_rk4;
+    static const ConfigTable<Rk4Policy<float, true>, true> f_rk4;
     static const ConfigTable<MagnusPolicy<float, true>, true> f_mag;
     static const ConfigTable<SplitPolicy<float, true>, true> f_spl;
-    static const ConfigTable<PackedPolicy<false>, true> x_rk4;
+    static const ConfigTable<Rk4Policy<float, false>, true> x_rk4;
     static const ConfigTable<MagnusPolicy<float, false>, true> x_mag;
     static const ConfigTable<SplitPolicy<float, false>, true> x_spl;
     // defaults from timing the 64-candidate workload on GB300 (see the tuner)
