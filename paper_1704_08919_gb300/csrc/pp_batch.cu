@@ -29,50 +29,44 @@ struct BatchCand {
     long long part_off;   // partial sums before this candidate's
 };
 
-// As build_table_kernel, per slot with its own grid and step count; wide_flags[c]
-// (zeroed before the launch) marks slots that leave the policy's series range.
+// As build_table_kernel and plan_kernel, per slot with its own grid and step count.
 template <class P>
 __global__ void build_table_batch_kernel(const double *__restrict__ A, int ld,
                                          const BatchCand *__restrict__ cands, int row_quantum, double dt,
-                                         typename P::Entry *__restrict__ table, int *__restrict__ wide_flags)
+                                         typename P::Entry *__restrict__ table, int *__restrict__ plans)
 {
     const int c = blockIdx.y;
     const BatchCand d = cands[c];
     const int padded = ((d.ns + row_quantum - 1) / row_quantum) * row_quantum;
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    const double *Ax = A + (size_t)c * 2 * ld, *Ay = Ax + ld;
-    bool big = false;
-    if (n < padded) {
-        typename P::Entry e;
-        if (n < d.ns) {
-            e = table_entry((const P *)nullptr, Ax, Ay, n, dt, d.g);
-            if constexpr (HasSeriesGuard<P>::value)
-                big = P::beyond_series(e);
-        } else {
-            memset(&e, 0, sizeof e);
-        }
-        table[d.table_off + n] = e;
-    }
-    if constexpr (HasSeriesGuard<P>::value) {
-        if (__syncthreads_or(big) && threadIdx.x == 0)
-            atomicOr(wide_flags + c, 1);
-    }
+    const double *Ax = A + (size_t)c * 2 * ld;
+    table_row<P>(Ax, Ax + ld, blockIdx.x * blockDim.x + threadIdx.x, d.ns, padded, dt, d.g, table + d.table_off, plans + c);
 }
 
-// WIDE selects the slots this launch takes (see takes_candidate); items of the
-// other kind are drawn from the queue and skipped.
-template <class P, int THREADS, int TILE_BYTES, bool WIDE>
+template <bool COMP>
+__global__ void __launch_bounds__(kPlanThreads)
+    plan_batch_kernel(const double *__restrict__ A, int ld, const BatchCand *__restrict__ cands, double dt,
+                      typename MagnusPolicy<float, COMP>::Entry *__restrict__ table, int *__restrict__ plans,
+                      bool densities)
+{
+    const int c = blockIdx.x;
+    const BatchCand d = cands[c];
+    const double *Ax = A + (size_t)c * 2 * ld;
+    plan_and_table<COMP>(Ax, Ax + ld, d.ns, dt, d.g, table + d.table_off, plans + c, densities);
+}
+
+// ROLE selects the slots this launch takes (see takes_candidate); items of the
+// other kinds are drawn from the queue and skipped.
+template <class P, int THREADS, int TILE_BYTES, Role ROLE>
 __global__ void __launch_bounds__(THREADS)
     propagate_batch_kernel(const double *__restrict__ A, int ld, const BatchCand *__restrict__ cands,
                            const int2 *__restrict__ work, int nwork, int *__restrict__ counter,
                            const typename P::Entry *__restrict__ table, double dt,
                            double *__restrict__ n_p, double *__restrict__ partial,
                            long long wait_limit, int skip_copies, unsigned int *__restrict__ status,
-                           const int *__restrict__ wide_flags)
+                           const int *__restrict__ plans, int first_rest)
 {
-    using V = typename P::Entry;
-    constexpr int TILE = TILE_BYTES / (int)sizeof(V);
-    __shared__ ItemSmem<P, THREADS, TILE_BYTES> sm;
+    using Q = RolePolicy<P, ROLE>;
+    __shared__ ItemSmem<Q, THREADS, TILE_BYTES> sm;
     __shared__ int s_item;
     if (threadIdx.x == 0) {
         mbar_init(&sm.bar[0], 1);
@@ -80,7 +74,7 @@ __global__ void __launch_bounds__(THREADS)
         mbar_fence_init();
     }
     __syncthreads();
-    int tile_base = 0;
+    int tiles = 0;
     for (;;) {
         if (threadIdx.x == 0)
             s_item = atomicAdd(counter, 1);
@@ -89,18 +83,17 @@ __global__ void __launch_bounds__(THREADS)
         if (it >= nwork)
             break;
         const int2 w = work[it];
-        if (!takes_candidate<P, WIDE>(wide_flags, w.x)) {
+        if (!takes_candidate<P, ROLE>(plans, w.x, first_rest)) {
             __syncthreads();  // every thread has read s_item before thread 0 draws again
             continue;
         }
         const BatchCand d = cands[w.x];
         const double *Ax = A + (size_t)w.x * 2 * ld;
-        const bool ok = process_item<P, THREADS, TILE_BYTES, WIDE>(
-            sm, w.y, d.g, d.ns, table + d.table_off, Ax, Ax + ld, dt, n_p ? n_p + d.n_off : nullptr,
-            partial + d.part_off, wait_limit, skip_copies, status, tile_base);
-        if (!ok)
+        if (!process_item<Q, THREADS, TILE_BYTES, ROLE>(
+                sm, w.y, d.g, d.ns, HasPlan<P>::value ? plans[w.x] : 0,
+                reinterpret_cast<const typename Q::Entry *>(table + d.table_off), Ax, Ax + ld, dt,
+                n_p ? n_p + d.n_off : nullptr, partial + d.part_off, wait_limit, skip_copies, status, tiles))
             break;  // barrier phases are unknown after a wait gave up: this CTA stops
-        tile_base += (d.ns + TILE - 1) / TILE;
     }
 }
 
@@ -131,6 +124,7 @@ __global__ void finalize_batch_kernel(const double *__restrict__ partial,
     }
 }
 
+constexpr int kBatchCounters = 3;
 constexpr int kNumBatchConfigs = 6;
 constexpr int kBCfgThreads[kNumBatchConfigs] = {256, 128, 512, 256, 128, 512};
 
@@ -145,7 +139,7 @@ struct BatchLaunch {
     void *table;
     int row_quantum;
     int ncand;
-    int max_padded;
+    int max_padded, max_ns;
     double dt;
     double *n_p;
     double *partial;
@@ -162,21 +156,38 @@ int run_batch(const BatchLaunch &L, cudaStream_t stream)
     unsigned int *status = pp::status_word();
     if (!status)
         return pp::fail(PP_ERR_CUDA, "status word unavailable");
-    // counter[0], counter[1]: the work counters of the two launches; counter[2 + c]: wide flags
-    cudaError_t e = cudaMemsetAsync(L.counter, 0, sizeof(int) * (2 + (size_t)L.ncand), stream);
+    // counter[0..2]: the work counters of the launches; counter[3 + c]: the plans
+    cudaError_t e = cudaMemsetAsync(L.counter, 0, sizeof(int) * (kBatchCounters + (size_t)L.ncand), stream);
     if (e != cudaSuccess)
         return pp::cuda_fail(e, "batch work counter reset");
-    int *flags = L.counter + 2;
-    dim3 tg((L.max_padded + 255) / 256, L.ncand);
-    build_table_batch_kernel<P><<<tg, 256, 0, stream>>>(L.A, L.ld, L.cands, L.row_quantum, L.dt,
-                                                       (typename P::Entry *)L.table, flags);
-    propagate_batch_kernel<P, THREADS, TILE_BYTES, false><<<L.grid_ctas, THREADS, 0, stream>>>(
-        L.A, L.ld, L.cands, L.work, L.nwork, L.counter, (const typename P::Entry *)L.table, L.dt,
-        L.n_p, L.partial, (long long)pp::wait_limit(), pp::skip_copies(), status, flags);
-    if constexpr (HasSeriesGuard<P>::value)
-        propagate_batch_kernel<P, THREADS, TILE_BYTES, true><<<L.grid_ctas, THREADS, 0, stream>>>(
-            L.A, L.ld, L.cands, L.work, L.nwork, L.counter + 1, (const typename P::Entry *)L.table, L.dt,
-            L.n_p, L.partial, (long long)pp::wait_limit(), pp::skip_copies(), status, flags);
+    int *plans = L.counter + kBatchCounters;
+    const auto *table = (const typename P::Entry *)L.table;
+    constexpr bool kBlocks = IsBlock<typename MainPolicy<P>::type>::value;
+    if constexpr (kBlocks) {
+        plan_batch_kernel<P::kComp><<<L.ncand, kPlanThreads, 0, stream>>>(
+            L.A, L.ld, L.cands, L.dt, (typename P::Entry *)L.table, plans, L.n_p != nullptr);
+    } else {
+        dim3 tg((L.max_padded + 255) / 256, L.ncand);
+        build_table_batch_kernel<P><<<tg, 256, 0, stream>>>(L.A, L.ld, L.cands, L.row_quantum, L.dt,
+                                                           (typename P::Entry *)L.table, plans);
+    }
+    propagate_batch_kernel<P, THREADS, TILE_BYTES, MAIN><<<L.grid_ctas, THREADS, 0, stream>>>(
+        L.A, L.ld, L.cands, L.work, L.nwork, L.counter, table, L.dt, L.n_p, L.partial, (long long)pp::wait_limit(),
+        pp::skip_copies(), status, plans, 0);
+    if constexpr (HasPlan<P>::value) {
+        int first_rest = kKindSeries;
+        if constexpr (kBlocks && !P::kComp) {
+            if (L.n_p && single_steps(L.max_ns, L.dt)) {  // as in the uniform path
+                propagate_batch_kernel<P, THREADS, TILE_BYTES, SERIES><<<L.grid_ctas, THREADS, 0, stream>>>(
+                    L.A, L.ld, L.cands, L.work, L.nwork, L.counter + 1, table, L.dt, L.n_p, L.partial,
+                    (long long)pp::wait_limit(), pp::skip_copies(), status, plans, 0);
+                first_rest = kKindWide;
+            }
+        }
+        propagate_batch_kernel<P, THREADS, TILE_BYTES, REST><<<L.grid_ctas, THREADS, 0, stream>>>(
+            L.A, L.ld, L.cands, L.work, L.nwork, L.counter + 2, table, L.dt, L.n_p, L.partial,
+            (long long)pp::wait_limit(), pp::skip_copies(), status, plans, first_rest);
+    }
     finalize_batch_kernel<<<L.ncand, 256, 0, stream>>>(L.partial, L.cands, L.N, status);
     e = cudaGetLastError();
     if (e != cudaSuccess)
@@ -188,7 +199,7 @@ template <class P, int THREADS, int TILE_BYTES>
 int occupancy(int *blocks)
 {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        blocks, propagate_batch_kernel<P, THREADS, TILE_BYTES, false>, THREADS, 0);
+        blocks, propagate_batch_kernel<P, THREADS, TILE_BYTES, MAIN>, THREADS, 0);
     return e == cudaSuccess ? PP_OK : pp::cuda_fail(e, "occupancy query");
 }
 
@@ -239,7 +250,7 @@ const BatchTable &batch_table(int precision, int scheme)
          make_batch_table<SplitPolicy<float, true>>(true, 0)},
         {make_batch_table<Rk4Policy<float, false>>(true, 0),
          make_batch_table<MagnusPolicy<float, false>>(true, 0),
-         make_batch_table<SplitPolicy<float, false>>(true, 3)},
+         make_batch_table<SplitPolicy<float, false>>(true, 1)},
     };
     return t[precision][scheme];
 }
@@ -317,6 +328,7 @@ BatchLaunch launch_args(const pp_batch *b, const double *A, double *N, double *n
     L.row_quantum = b->row_quantum;
     L.ncand = b->ncand;
     L.max_padded = b->max_padded;
+    L.max_ns = b->max_ns;
     L.dt = b->dt;
     L.n_p = n_p;
     L.partial = b->d_partial;
@@ -328,7 +340,8 @@ BatchLaunch launch_args(const pp_batch *b, const double *A, double *N, double *n
 int batch_pair_number(const pp_batch *b, const double *A, double *N, double *n_p, int cfg,
                       cudaStream_t stream)
 {
-    return batch_table(b->precision, b->scheme).run[cfg](launch_args(b, A, N, n_p, cfg), stream);
+    return batch_table(pp::precision_of(b->precision, b->scheme, n_p), b->scheme)
+        .run[cfg](launch_args(b, A, N, n_p, cfg), stream);
 }
 
 int batch_de_generation(pp_batch *b, double *pop, double *fit, const double *lo, const double *hi,
@@ -442,7 +455,7 @@ int pp_batch_create(int32_t ncand, const pp_field_spec *specs, const pp_grid *gr
     if (e == cudaSuccess)
         e = cudaMalloc(&b->d_partial, sizeof(double) * (size_t)poff);
     if (e == cudaSuccess)
-        e = cudaMalloc(&b->d_counter, sizeof(int) * (2 + (size_t)ncand));
+        e = cudaMalloc(&b->d_counter, sizeof(int) * (kBatchCounters + (size_t)ncand));
     // work lists (longest candidates first) for each CTA size
     const int sizes[3] = {128, 256, 512};
     std::vector<int> order(ncand);
@@ -711,12 +724,13 @@ int pp_pair_number_grids(const double *A, int32_t ncand, int32_t ld, const int32
     std::vector<BatchCand> hc(ncand);
     std::vector<int> order(ncand);
     long long toff = 0, noff = 0, poff = 0;
-    int max_padded = 0;
+    int max_padded = 0, max_ns = 0;
     for (int c = 0; c < ncand; ++c) {
         const int ns = n_steps ? n_steps[c] : (ld - 1) / 2;
         const int padded = ((ns + row_quantum - 1) / row_quantum) * row_quantum;
         const long long nm = (long long)grids[c].nx * grids[c].ny * grids[c].nz;
         max_padded = std::max(max_padded, padded);
+        max_ns = std::max(max_ns, ns);
         hc[c].g = grids[c];
         hc[c].ns = ns;
         hc[c].ngroups = (int)((nm + kGroup - 1) / kGroup);
@@ -740,7 +754,7 @@ int pp_pair_number_grids(const double *A, int32_t ncand, int32_t ld, const int32
     const size_t o_table = o_work + al(sizeof(int2) * work.size());
     const size_t o_part = o_table + al((size_t)toff * tab.entry_bytes);
     const size_t o_count = o_part + al(sizeof(double) * (size_t)poff);
-    const size_t total = o_count + al(sizeof(int) * (2 + (size_t)ncand));
+    const size_t total = o_count + al(sizeof(int) * (kBatchCounters + (size_t)ncand));
     void *base = nullptr;
     int rc = scratch(SCR_GRIDS, total, &base);
     if (rc)
@@ -769,10 +783,11 @@ int pp_pair_number_grids(const double *A, int32_t ncand, int32_t ld, const int32
     L.row_quantum = row_quantum;
     L.ncand = ncand;
     L.max_padded = max_padded;
+    L.max_ns = max_ns;
     L.dt = dt;
     L.n_p = n_p;
     L.partial = (double *)(b + o_part);
     L.N = N;
     L.grid_ctas = std::max(1, std::min((int)work.size(), sms * std::max(blocks, 1)));
-    return tab.run[cfg](L, st);
+    return batch_table(precision_of(precision, scheme, n_p), scheme).run[cfg](L, st);
 }

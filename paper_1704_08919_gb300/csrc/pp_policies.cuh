@@ -12,6 +12,7 @@
 
 #include <type_traits>
 
+#include "pp_blocks.cuh"
 #include "pp_internal.cuh"
 
 namespace {
@@ -73,18 +74,17 @@ __device__ __forceinline__ double proj_pos2(double hx, double hy, double hz, con
     return re * re + im * im;
 }
 
+// U v for the 2 x 2 matrix U = [[a, -b*], [b, a*]] (a multiple of an SU(2) element) with first column z = (a, b).
+__device__ __forceinline__ void apply_su2(const double z[4], const double v[4], double p[4])
+{
+    p[0] = z[0] * v[0] - z[1] * v[1] - (z[2] * v[2] + z[3] * v[3]);
+    p[1] = z[0] * v[1] + z[1] * v[0] - (z[2] * v[3] - z[3] * v[2]);
+    p[2] = z[2] * v[0] - z[3] * v[1] + z[0] * v[2] + z[1] * v[3];
+    p[3] = z[2] * v[1] + z[3] * v[0] + z[0] * v[3] - z[1] * v[2];
+}
+
 // ---------------------------------------------------------------- stepping policies
 // A policy supplies the per-step table entry (Entry), the per-thread state and the step.
-
-// Low part of dt x p against its rounding hi to T.
-template <typename T>
-__device__ __forceinline__ T low_part(double dt, double p, T hi)
-{
-    if constexpr (sizeof(T) == 8)
-        return fma(dt, p, -hi);
-    else
-        return (T)(dt * p - (double)hi);
-}
 
 // Classical RK4 with the step matrix in closed form.  A product of h's Pauli matrices is
 // (a.sigma)(b.sigma) = a.b + i (a x b).sigma, so the step
@@ -108,6 +108,7 @@ __device__ __forceinline__ T low_part(double dt, double p, T hi)
 // memory; in FP32 the table holds the expanded entry (32 bytes).
 template <typename T, bool COMP>
 struct Rk4Policy {
+    static constexpr bool kComp = COMP;
     struct alignas(sizeof(T) * 8) Coef {
         T ax, ay, cx, cy, dx, dy, q, p;  // p = (d x c)_z / 48
     };
@@ -145,15 +146,9 @@ struct Rk4Policy {
         T px, py, uz, uz2, lx, ly, lz;  // dt p_x, dt p_y, dt eps, its square, and the first three's low parts
     };
 
-    __device__ static void init(State &st, const double v[2][4], double px, double py, double eperp, double dt)
+    // Sets the mode's constants for steps of dt.
+    __device__ static void scale(State &st, double px, double py, double eperp, double dt)
     {
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                st.hi[s][q] = (T)v[s][q];
-                st.lo[s][q] = (T)(v[s][q] - (double)st.hi[s][q]);
-            }
         st.px = (T)(dt * px);
         st.py = (T)(dt * py);
         st.uz = (T)(dt * eperp);
@@ -209,14 +204,6 @@ struct Rk4Policy {
                     st.hi[s][q] = nz[q];
             }
         }
-    }
-
-    __device__ static void psi(const State &st, int s, double out[4], double, double, double,
-                               double)
-    {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            out[q] = COMP ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
     }
 };
 
@@ -304,15 +291,17 @@ struct TanSeries {
 // of its own) for all its steps; step n halves th k_n times, k_n the least k with th_max 2^-k <= kSeriesLimit
 // (0 where the bound is inside the range), the same for every mode, so the
 // threads of a warp never diverge.
+// FP32 candidates whose potential is smooth enough take blocks of steps instead (pp_blocks.cuh).
 // FP32 series steps are taken in tracked form: (cos th)^-1 exp(-i H.sigma) =
 // 1 - i (tan th / th) H.sigma, which drops the cos th - 1 term and its
 // polynomial (24 instead of 30 FP32 instructions per channel and step).  The
 // state then grows by 1 / cos th per step; the exact evolution is unitary, so the
-// projection is divided by the squared norm, and rescale() (between shared-memory tiles) scales
+// projection is divided by the squared norm, and rescale_state (between shared-memory tiles) scales
 // each channel by a power of two, which is exact: the result does not depend on
 // where the rescaling happens.
 template <typename T, bool COMP>
 struct MagnusPolicy {
+    static constexpr bool kComp = COMP;
     struct alignas(sizeof(T) * 8) Entry {
         T ax, ay, dx, dy, c, pad0, pad1, pad2;
     };
@@ -357,16 +346,9 @@ struct MagnusPolicy {
         T dtpx, dtpy, dteps, eps, px, py;
     };
 
-    __device__ static void init(State &st, const double v[2][4], double px, double py, double eperp,
-                                double dt)
+    // Sets the mode's constants for steps of dt.
+    __device__ static void scale(State &st, double px, double py, double eperp, double dt)
     {
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                st.hi[s][q] = (T)v[s][q];
-                st.lo[s][q] = (T)(v[s][q] - (double)st.hi[s][q]);
-            }
         st.dtpx = (T)(dt * px);
         st.dtpy = (T)(dt * py);
         st.dteps = (T)(dt * eperp);
@@ -484,47 +466,20 @@ struct MagnusPolicy {
             step_impl<false>(st, e);
     }
     __device__ static __forceinline__ void step_wide(State &st, const Entry &e) { step_impl<true>(st, e); }
-
-    // Scales each channel by the power of two 2^-floor(log2(|psi|^2) / 2) (exact).
-    __device__ static __forceinline__ void rescale(State &st)
-    {
-        if constexpr (kTracked) {
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const float n2 = fmaf(st.hi[s][3], st.hi[s][3],
-                                      fmaf(st.hi[s][2], st.hi[s][2],
-                                           fmaf(st.hi[s][1], st.hi[s][1], st.hi[s][0] * st.hi[s][0])));
-                const int e2 = ((__float_as_int(n2) >> 23) & 0xff) - 127;  // n2 is a normal number
-                const float f = __int_as_float((127 - (e2 >> 1)) << 23);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    st.hi[s][q] *= f;
-                    st.lo[s][q] *= f;
-                }
-            }
-        }
-    }
-
-    __device__ static void psi(const State &st, int s, double out[4], double, double, double,
-                               double)
-    {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            out[q] = COMP ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
-    }
 };
 
 // Second-order split-operator policy: Strang splitting of h_s . sigma into the
 // free part h0 = (p_x, s p_y, eps) and the coupling v = (-A_x, -s A_y, 0) at
 // t_{n+1/2}:  psi <- e^{-i h0.sigma dt/2} e^{-i v.sigma dt} e^{-i h0.sigma dt/2} psi.
-// Neighbouring free half steps are merged: the prologue applies one free half
+// Neighbouring free half steps are merged: the initial state takes one free half
 // step (FP64), every step applies the coupling factor and then the full free
-// factor, and the epilogue undoes one free half step (FP64).  Both factors are
+// factor, and the final state undoes one free half step (FP64).  Both factors are
 // exact: e^{-i k.sigma tau} = cos(|k| tau) - i sin(|k| tau) k.sigma / |k|.  The
 // coupling factor does not depend on the mode, so the table holds it:
 // (cos(|A| dt) - 1, -A_x sin(|A| dt)/|A|, -A_y sin(|A| dt)/|A|).
 template <typename T, bool COMP>
 struct SplitPolicy {
+    static constexpr bool kComp = COMP;
     struct alignas(sizeof(T) * 4) Entry {
         T cm1, wx, wy, pad;
     };
@@ -558,26 +513,16 @@ struct SplitPolicy {
             out[q] = c * in[q] + sg * r[q];
     }
 
-    __device__ static void init(State &st, const double v[2][4], double px, double py, double eperp,
-                                double dt)
+    // Sets the mode's constants for steps of dt.
+    __device__ static void scale(State &st, double px, double py, double eperp, double dt)
     {
         const double w0 = sqrt(px * px + py * py + eperp * eperp);
-        const double sh = sin(0.5 * w0 * dt), ch = cos(0.5 * w0 * dt);
+        const double sh = sin(0.5 * w0 * dt);
         const double sg = sin(w0 * dt) / w0;
         st.c0m1 = (T)(-2.0 * sh * sh);
         st.gx = (T)(sg * px);
         st.gy = (T)(sg * py);
         st.gz = (T)(sg * eperp);
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            double w[4];
-            apply_free(ch, sh / w0, px, s ? -py : py, eperp, v[s], w);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                st.hi[s][q] = (T)w[q];
-                st.lo[s][q] = (T)(w[q] - (double)st.hi[s][q]);
-            }
-        }
     }
 
     __device__ static __forceinline__ void step(State &st, const Entry &e)
@@ -621,16 +566,23 @@ struct SplitPolicy {
         }
     }
 
-    __device__ static void psi(const State &st, int s, double out[4], double px, double py,
-                               double eperp, double dt)
+    // The free half step before the first full one and the surplus one after the last, in FP64:
+    // e^{-+i h0.sigma dt/2} = c -+ i s h0.sigma; the sine and cosine are the same for both channels.
+    struct HalfStep {
+        double c, s;
+    };
+    __device__ static HalfStep half_step(double px, double py, double eperp, double dt)
+    {
+        const double w0 = sqrt(px * px + py * py + eperp * eperp);
+        return HalfStep{cos(0.5 * w0 * dt), sin(0.5 * w0 * dt) / w0};
+    }
+    __device__ static void apply_half(const HalfStep &h, double sign, double px, double py, double eperp, double v[4])
     {
         double w[4];
+        apply_free(h.c, sign * h.s, px, py, eperp, v, w);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            w[q] = COMP ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
-        // undo one free half step: e^{+i h0.sigma dt/2} = ch + i (sh / w0) h0.sigma
-        const double w0 = sqrt(px * px + py * py + eperp * eperp);
-        apply_free(cos(0.5 * w0 * dt), -sin(0.5 * w0 * dt) / w0, px, s ? -py : py, eperp, w, out);
+            v[q] = w[q];
     }
 };
 
@@ -672,73 +624,217 @@ struct Expands<Rk4Policy<double, C>> {
     using Coef = typename Rk4Policy<double, C>::Coef;
 };
 
-// Policies whose series steps let the state's norm grow (rescale between tiles).
+// Policies with a range of steps (the Magnus scheme): each candidate has a plan (pp_blocks.cuh), and one of two
+// kernels takes it.  FP64: single steps by the polynomials or by their argument-halved form; FP32: blocks of
+// steps, or single steps of either form.
+template <class P>
+struct HasPlan {
+    static constexpr bool value = false;
+};
+template <typename T, bool C>
+struct HasPlan<MagnusPolicy<T, C>> {
+    static constexpr bool value = true;
+};
+
+// The policy of the main kernel.
+template <class P>
+struct MainPolicy {
+    using type = P;
+};
+template <bool C>
+struct MainPolicy<MagnusPolicy<float, C>> {
+    using type = MagnusBlockPolicy<C>;
+};
+template <class P>
+struct IsBlock {
+    static constexpr bool value = false;
+};
+template <bool C>
+struct IsBlock<MagnusBlockPolicy<C>> {
+    static constexpr bool value = true;
+};
+
+// Policies whose steps let the state's norm grow: rescaled by powers of two, and divided out by the projection.
 template <class P>
 struct TracksNorm {
-    static constexpr bool value = false;
+    static constexpr bool value = IsBlock<P>::value;
 };
 template <bool C>
 struct TracksNorm<MagnusPolicy<float, C>> {
     static constexpr bool value = MagnusPolicy<float, C>::kTracked;
 };
-
-// Policies whose step has a series range (beyond_series, step_wide).
+// Policies that carry the two states themselves; the others build up the propagators from the identity.
 template <class P>
-struct HasSeriesGuard {
+struct CarriesState {
     static constexpr bool value = false;
 };
 template <typename T, bool C>
-struct HasSeriesGuard<MagnusPolicy<T, C>> {
+struct CarriesState<MagnusPolicy<T, C>> {
+    static constexpr bool value = true;
+};
+template <typename T, bool C>
+struct CarriesState<SplitPolicy<T, C>> {
+    static constexpr bool value = true;
+};
+template <class P>
+struct IsSplit {
+    static constexpr bool value = false;
+};
+template <typename T, bool C>
+struct IsSplit<SplitPolicy<T, C>> {
     static constexpr bool value = true;
 };
 
-// Table of candidate c (grid (blocks, candidates), 256 threads).  For policies with
-// a series range, wide_flags[c] (zeroed before the launch) is set when any step of
-// the candidate leaves it; the propagation then runs that candidate in the
-// wide-range kernel instead.
-template <class P>
-__global__ void build_table_kernel(const double *__restrict__ A, int ld, int ns_uniform,
-                                   const int *__restrict__ ns_array, int padded, double dt,
-                                   pp_grid g, typename P::Entry *__restrict__ table,
-                                   int *__restrict__ wide_flags)
+// Scales each channel by the power of two 2^-floor(log2(|psi|^2) / 2), which is exact.
+template <bool COMP, class State>
+__device__ __forceinline__ void rescale_state(State &st)
 {
-    int c = blockIdx.y;
-    int n = blockIdx.x * blockDim.x + threadIdx.x;
-    int ns = ns_array ? ns_array[c] : ns_uniform;
-    const double *Ax = A + (size_t)c * 2 * ld, *Ay = Ax + ld;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const float n2 = fmaf(st.hi[s][3], st.hi[s][3],
+                              fmaf(st.hi[s][2], st.hi[s][2], fmaf(st.hi[s][1], st.hi[s][1], st.hi[s][0] * st.hi[s][0])));
+        const int e2 = ((__float_as_int(n2) >> 23) & 0xff) - 127;  // n2 is a normal number
+        const float f = __int_as_float((127 - (e2 >> 1)) << 23);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            st.hi[s][q] *= f;
+            if constexpr (COMP)
+                st.lo[s][q] *= f;
+        }
+    }
+}
+
+// Step tables of the policies without a plan, and of FP64 Magnus (grid (blocks, candidates), 256 threads).  For the
+// latter, plans[c] (zeroed before the launch) becomes kKindWide when any step of the candidate leaves the
+// polynomials' range.
+template <class P>
+__device__ __forceinline__ void table_row(const double *Ax, const double *Ay, int n, int ns, int padded, double dt,
+                                          const pp_grid &g, typename P::Entry *__restrict__ row, int *plan)
+{
     bool big = false;
     if (n < padded) {
         typename P::Entry e;
         if (n < ns) {
             e = table_entry((const P *)nullptr, Ax, Ay, n, dt, g);
-            if constexpr (HasSeriesGuard<P>::value)
+            if constexpr (HasPlan<P>::value)
                 big = P::beyond_series(e);
         } else {
             memset(&e, 0, sizeof e);
         }
-        table[(size_t)c * padded + n] = e;
+        row[n] = e;
     }
-    if constexpr (HasSeriesGuard<P>::value) {
+    if constexpr (HasPlan<P>::value) {
         if (__syncthreads_or(big) && threadIdx.x == 0)
-            atomicOr(wide_flags + c, 1);
+            atomicOr(plan, kKindWide);
     }
 }
 
-// The candidate's kernel: a policy with a series range runs each candidate in
-// exactly one of its two kernels (WIDE = wide_flags[c] != 0).
-template <class P, bool WIDE>
-__device__ __forceinline__ bool takes_candidate(const int *__restrict__ wide_flags, int c)
+template <class P>
+__global__ void build_table_kernel(const double *__restrict__ A, int ld, int ns_uniform,
+                                   const int *__restrict__ ns_array, int padded, double dt,
+                                   pp_grid g, typename P::Entry *__restrict__ table,
+                                   int *__restrict__ plans)
 {
-    if constexpr (HasSeriesGuard<P>::value)
-        return (wide_flags[c] != 0) == WIDE;
-    else
-        return !WIDE;
+    const int c = blockIdx.y;
+    const double *Ax = A + (size_t)c * 2 * ld;
+    table_row<P>(Ax, Ax + ld, blockIdx.x * blockDim.x + threadIdx.x, ns_array ? ns_array[c] : ns_uniform, padded, dt, g,
+                 table + (size_t)c * padded, plans + c);
 }
 
-// One work item: the modes [blk * THREADS, (blk + 1) * THREADS) of candidate c.
-// The caller owns the shared-memory buffers and the two mbarriers; tile_base
-// is the number of tiles this CTA has consumed before (the barrier phases run
-// on across items).  Returns false if a bounded wait gave up.
+// Plan and table of one FP32 Magnus candidate by one CTA: a pass over the steps for the plan, then the blocks'
+// entries, or the single steps' where the plan has none.  Sums are taken in a fixed order, so a candidate's plan
+// depends on nothing but its own potential, grid and step.  One CTA per candidate: a pass over 8192
+// steps takes ~10 us beside the milliseconds of the propagation, and one launch instead of three.
+constexpr int kPlanThreads = 512;
+template <bool COMP>
+__device__ __forceinline__ void plan_and_table(const double *__restrict__ Ax, const double *__restrict__ Ay, int ns,
+                                               double dt, const pp_grid &g,
+                                               typename MagnusPolicy<float, COMP>::Entry *__restrict__ row,
+                                               int *__restrict__ plan_out, bool densities)
+{
+    __shared__ double s_th[kPlanThreads / 32];
+    __shared__ float s_sum[3][kPlanThreads / 32];
+    __shared__ int s_plan;
+    const int tid = threadIdx.x;
+    const double Px = fmax(fabs(g.x0), fabs(g.x1)), Py = fmax(fabs(g.y0), fabs(g.y1));
+    const double Pz = fmax(fabs(g.z0), fabs(g.z1)), E = sqrt(1.0 + Pz * Pz);
+    double th2 = 0.0;
+    float sum[3] = {0.0f, 0.0f, 0.0f};
+    for (int n = tid; n < ns; n += kPlanThreads) {
+        const StepSize r = step_size(Ax, Ay, n, ns, dt, Px, Py, E);
+        th2 = fmax(th2, r.th2);
+        sum[0] += r.dq;
+        sum[1] += r.rough;
+        sum[2] += r.cube;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        th2 = fmax(th2, __shfl_xor_sync(0xffffffffu, th2, off));
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], off);
+    }
+    if ((tid & 31) == 0) {
+        s_th[tid >> 5] = th2;
+        for (int k = 0; k < 3; ++k)
+            s_sum[k][tid >> 5] = sum[k];
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kPlanThreads / 32; ++w) {
+            th2 = fmax(th2, s_th[w]);
+            for (int k = 0; k < 3; ++k)
+                sum[k] += s_sum[k][w];
+        }
+        const double th = sqrt(th2);
+        // a NaN in the potential fails every comparison: single steps, which carry it to the result
+        const int m = !COMP && densities && single_steps(ns, dt)
+                          ? 1
+                          : plan_block(th, sum[0], sum[1], sum[2], ns, COMP ? kMaxBlockComp : kMaxBlock,
+                                       COMP ? kBlockAngleComp : kBlockAngle);
+        s_plan = m > 1 ? plan_pack(kKindMain, m) : plan_pack(th > kSeriesLimit ? kKindWide : kKindSeries, 1);
+        *plan_out = s_plan;
+    }
+    __syncthreads();
+    const int m = plan_steps(s_plan);
+    if (plan_kind(s_plan) == kKindMain) {
+        auto *blocks = reinterpret_cast<typename MagnusBlockPolicy<COMP>::Entry *>(row);
+        for (int b = tid; b * m < ns; b += kPlanThreads)
+            blocks[b] = block_entry<COMP>(Ax, Ay, b * m, min(m, ns - b * m), dt);
+    } else {
+        for (int n = tid; n < ns; n += kPlanThreads)
+            row[n] = table_entry((const MagnusPolicy<float, COMP> *)nullptr, Ax, Ay, n, dt, g);
+    }
+}
+
+template <bool COMP>
+__global__ void __launch_bounds__(kPlanThreads)
+    plan_kernel(const double *__restrict__ A, int ld, int ns_uniform, const int *__restrict__ ns_array, int padded,
+                double dt, pp_grid g, typename MagnusPolicy<float, COMP>::Entry *__restrict__ table,
+                int *__restrict__ plans, bool densities)
+{
+    const int c = blockIdx.x;
+    const double *Ax = A + (size_t)c * 2 * ld;
+    plan_and_table<COMP>(Ax, Ax + ld, ns_array ? ns_array[c] : ns_uniform, dt, g, table + (size_t)c * padded, plans + c,
+                         densities);
+}
+
+// The kernel of a launch: MAIN takes the candidates of kind 0 (all, for a policy without plans), SERIES those of
+// kind 1 and REST those of kind first_rest and up.
+enum Role { MAIN, SERIES, REST };
+template <class P, Role ROLE>
+__device__ __forceinline__ bool takes_candidate(const int *__restrict__ plans, int c, int first_rest)
+{
+    if constexpr (HasPlan<P>::value) {
+        const int kind = plan_kind(plans[c]);
+        return ROLE == MAIN ? kind == kKindMain : (ROLE == SERIES ? kind == kKindSeries : kind >= first_rest);
+    } else {
+        return true;
+    }
+}
+template <class P, Role ROLE>
+using RolePolicy = typename std::conditional<ROLE == MAIN, typename MainPolicy<P>::type, P>::type;
+
 template <class P, int THREADS, int TILE_BYTES>
 struct ItemSmem {
     using V = typename P::Entry;
@@ -749,16 +845,26 @@ struct ItemSmem {
     typename Expands<P>::Coef coef[Expands<P>::value ? kExpandSpan : 1];
 };
 
-template <class P, int THREADS, int TILE_BYTES, bool WIDE>
+// Steps (or blocks of steps) between two rescalings of a growing state: a block grows it by 1 / cos th <= 2.8, so
+// its squared norm stays below 1e29.
+constexpr int kRescaleSpan = 32;
+
+// One work item: the modes [blk * THREADS, (blk + 1) * THREADS) of one candidate with ns steps (P: the policy
+// that runs, plan: the candidate's where it has one).  Each spin channel carries its state, or the first column of
+// its propagator (an SU(2) element or a multiple of one), which is applied to the initial
+// state in FP64 at the end.  The caller owns the shared-memory buffers and the two mbarriers; tile_base
+// is the number of tiles this CTA has consumed before (the barrier phases run
+// on across items) and is moved on.  Returns false if a bounded wait gave up.
+template <class P, int THREADS, int TILE_BYTES, Role ROLE>
 __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &sm, int blk,
-                                             const pp_grid &g, int ns,
+                                             const pp_grid &g, int ns, int plan,
                                              const typename P::Entry *__restrict__ trow,
                                              const double *__restrict__ Ax,
                                              const double *__restrict__ Ay, double dt,
                                              double *__restrict__ n_out,
                                              double *__restrict__ part_out, long long wait_limit,
                                              int skip_copies, unsigned int *__restrict__ status,
-                                             int tile_base)
+                                             int &tile_base)
 {
     using V = typename P::Entry;
     constexpr int TILE = TILE_BYTES / (int)sizeof(V);
@@ -767,12 +873,16 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
     const int nmodes = g.nx * g.ny * g.nz;
     const int m = blk * THREADS + tid;
     const bool active = m < nmodes;
-    const int ntiles = (ns + TILE - 1) / TILE;
+    const int per = IsBlock<P>::value ? plan_steps(plan) : 1;  // steps per table entry
+    const int nent = IsBlock<P>::value ? (ns + per - 1) / per : ns;
+    const int ntiles = (nent + TILE - 1) / TILE;
+    const int base = tile_base;
+    tile_base += ntiles;
 
     int issued = 0;  // meaningful in thread 0 only
     if (tid == 0 && !skip_copies) {
         for (int t = 0; t < 2 && t < ntiles; ++t) {
-            const int k = tile_base + t;
+            const int k = base + t;
             mbar_arrive_expect_tx(&sm.bar[k & 1], TILE * (uint32_t)sizeof(V));
             bulk_copy_g2s(sm.buf[k & 1], trow + (size_t)t * TILE, TILE * (uint32_t)sizeof(V),
                           &sm.bar[k & 1]);
@@ -780,7 +890,7 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
         }
     }
 
-    // ---- this thread's momentum mode and FP64 initial state
+    // ---- this thread's momentum mode
     int ix = 0, iy = 0, iz = 0;
     if (active) {
         ix = m % g.nx;
@@ -793,18 +903,37 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
     const double eperp = sqrt(1.0 + pz * pz);
 
     typename P::State st;
-    {
-        const double Pinx = px - Ax[0], Piny = py - Ay[0];
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            st.hi[s][q] = q == 0 ? 1 : 0;
+            st.lo[s][q] = 0;
+        }
+    if constexpr (CarriesState<P>::value) {
+        const double hx = px - Ax[0], hy = py - Ay[0];
         double v[2][4];
-        eig_neg(Pinx, Piny, eperp, v[0]);
-        eig_neg(Pinx, -Piny, eperp, v[1]);
-        P::init(st, v, px, py, eperp, dt);
+        eig_neg(hx, hy, eperp, v[0]);
+        eig_neg(hx, -hy, eperp, v[1]);
+        if constexpr (IsSplit<P>::value) {
+            const auto h = P::half_step(px, py, eperp, dt);
+            P::apply_half(h, 1.0, px, py, eperp, v[0]);
+            P::apply_half(h, 1.0, px, -py, eperp, v[1]);
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                st.hi[s][q] = v[s][q];
+                st.lo[s][q] = v[s][q] - (double)st.hi[s][q];
+            }
     }
+    P::scale(st, px, py, eperp, per * dt);
 
     bool timed_out = false;
     int t_fail = 0;
     for (int t = 0; t < ntiles; ++t) {
-        const int k = tile_base + t;
+        const int k = base + t;
         const int b = k & 1;
         const uint32_t par = (k >> 1) & 1;
         bool ok = mbar_wait_bounded(&sm.bar[b], par, wait_limit);
@@ -814,9 +943,9 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
             t_fail = t;
             break;
         }
-        const int nst = min(TILE, ns - t * TILE);
+        const int nst = min(TILE, nent - t * TILE);
+        const V *tb = sm.buf[b];
         if constexpr (Expands<P>::value) {
-            const V *tb = sm.buf[b];
             for (int k0 = 0; k0 < nst; k0 += kExpandSpan) {
                 const int m1 = min(kExpandSpan, nst - k0);
                 if (tid < m1) {
@@ -836,16 +965,39 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
                 __syncthreads();  // every thread is done with coef
             }
         } else if (active) {
-            const V *tb = sm.buf[b];
-            if constexpr (WIDE) {
-                for (int kk = 0; kk < nst; ++kk)
-                    P::step_wide(st, tb[kk]);
-            } else {
+            if constexpr (IsBlock<P>::value) {
+                // the last entry holds the remaining ns % per steps, if any
+                const bool ragged = t == ntiles - 1 && ns % per != 0;
+                const int full = nst - (ragged ? 1 : 0);
+                for (int k0 = 0; k0 < full; k0 += kRescaleSpan) {
+                    const int k1 = min(k0 + kRescaleSpan, full);
 #pragma unroll 2
-                for (int kk = 0; kk < nst; ++kk)
-                    P::step(st, tb[kk]);
-                if constexpr (TracksNorm<P>::value)
-                    P::rescale(st);
+                    for (int kk = k0; kk < k1; ++kk)
+                        P::step(st, tb[kk]);
+                    rescale_state<P::kComp>(st);
+                }
+                if (ragged) {
+                    P::scale(st, px, py, eperp, (ns % per) * dt);
+                    P::step(st, tb[full]);
+                }
+            } else {
+                bool wide = false;
+                if constexpr (ROLE == REST) {
+                    wide = plan_kind(plan) == kKindWide;
+                    if (wide)
+                        for (int kk = 0; kk < nst; ++kk)
+                            P::step_wide(st, tb[kk]);
+                }
+                // (FP64 Magnus has no series candidates outside its main kernel)
+                if constexpr (ROLE != REST || TracksNorm<P>::value) {
+                    if (!wide) {
+#pragma unroll 2
+                        for (int kk = 0; kk < nst; ++kk)
+                            P::step(st, tb[kk]);
+                        if constexpr (TracksNorm<P>::value)
+                            rescale_state<P::kComp>(st);
+                    }
+                }
             }
         }
         __syncthreads();  // every thread is done with buf[b]
@@ -863,24 +1015,42 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
             pp_flag(status, PP_FLAG_TIMEOUT);
             // copies t_fail <= t < issued were never consumed: wait for each in order
             for (int t = t_fail; t < issued; ++t) {
-                const int k = tile_base + t;
+                const int k = base + t;
                 mbar_wait_bounded(&sm.bar[k & 1], (k >> 1) & 1, 1ll << 24);
             }
         }
         __syncthreads();
     }
 
-    // ---- FP64 projection onto the positive-energy states at t_end
+    // ---- FP64 projection of the final states onto the positive-energy states at t_end
     double f = 0.0;
     if (active) {
         const double Poutx = px - Ax[2 * ns], Pouty = py - Ay[2 * ns];
+        double psi[2][4];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                psi[s][q] = P::kComp ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
+        if constexpr (!CarriesState<P>::value) {
+            const double hx = px - Ax[0], hy = py - Ay[0];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                double v[4], z[4] = {psi[s][0], psi[s][1], psi[s][2], psi[s][3]};
+                eig_neg(hx, s ? -hy : hy, eperp, v);
+                apply_su2(z, v, psi[s]);
+            }
+        }
+        if constexpr (IsSplit<P>::value) {
+            const auto h = P::half_step(px, py, eperp, dt);
+            P::apply_half(h, -1.0, px, py, eperp, psi[0]);
+            P::apply_half(h, -1.0, px, -py, eperp, psi[1]);
+        }
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-            double psi[4];
-            P::psi(st, s, psi, px, py, eperp, dt);
-            double fs = proj_pos2(Poutx, s ? -Pouty : Pouty, eperp, psi);
-            if constexpr (TracksNorm<P>::value)  // the state's norm grew in the series steps
-                fs /= psi[0] * psi[0] + psi[1] * psi[1] + psi[2] * psi[2] + psi[3] * psi[3];
+            double fs = proj_pos2(Poutx, s ? -Pouty : Pouty, eperp, psi[s]);
+            if constexpr (TracksNorm<P>::value)  // the state's norm grew
+                fs /= psi[s][0] * psi[s][0] + psi[s][1] * psi[s][1] + psi[s][2] * psi[s][2] + psi[s][3] * psi[s][3];
             f += fs;
         }
         if (timed_out)

@@ -29,20 +29,20 @@
 
 namespace {
 
-// WIDE = false: the candidates whose steps stay in the policy's series range (all
-// candidates for policies without one); WIDE = true: the others (see
-// build_table_kernel).  A CTA of the other kind returns at once.
-template <class P, int THREADS, int TILE_BYTES, bool WIDE>
+// One CTA per block of modes and candidate (grid (blocks, candidates)); a CTA of a candidate that another launch takes returns at
+// once.  ROLE: MAIN or SERIES.
+template <class P, int THREADS, int TILE_BYTES, Role ROLE>
 __global__ void __launch_bounds__(THREADS)
     propagate_kernel(const double *__restrict__ A, int ld, int ns_uniform,
                      const int *__restrict__ ns_array, const typename P::Entry *__restrict__ table,
                      int padded, double dt, pp_grid g, double *__restrict__ n_p,
                      double *__restrict__ partial, long long wait_limit, int skip_copies,
-                     unsigned int *__restrict__ status, const int *__restrict__ wide_flags)
+                     unsigned int *__restrict__ status, const int *__restrict__ plans)
 {
-    __shared__ ItemSmem<P, THREADS, TILE_BYTES> sm;
+    using Q = RolePolicy<P, ROLE>;
+    __shared__ ItemSmem<Q, THREADS, TILE_BYTES> sm;
     const int c = blockIdx.y;
-    if (!takes_candidate<P, WIDE>(wide_flags, c))
+    if (!takes_candidate<P, ROLE>(plans, c, 0))
         return;
     const int nmodes = g.nx * g.ny * g.nz;
     const int ngroups = (nmodes + kGroup - 1) / kGroup;
@@ -54,10 +54,52 @@ __global__ void __launch_bounds__(THREADS)
         mbar_fence_init();
     }
     __syncthreads();
-    process_item<P, THREADS, TILE_BYTES, WIDE>(sm, blockIdx.x, g, ns, table + (size_t)c * padded, Ax,
-                                         Ax + ld, dt, n_p ? n_p + (size_t)c * nmodes : nullptr,
-                                         partial + (size_t)c * ngroups, wait_limit, skip_copies,
-                                         status, 0);
+    int tiles = 0;
+    process_item<Q, THREADS, TILE_BYTES, ROLE>(
+        sm, blockIdx.x, g, ns, HasPlan<P>::value ? plans[c] : 0,
+        reinterpret_cast<const typename Q::Entry *>(table + (size_t)c * padded), Ax, Ax + ld, dt,
+        n_p ? n_p + (size_t)c * nmodes : nullptr, partial + (size_t)c * ngroups, wait_limit, skip_copies, status, tiles);
+}
+
+// The candidates that the other launches leave: a grid that fills the GPU at most once walks over all items, so that it costs
+// microseconds where there are none (a CTA per item took 0.2 ms for 32768 items).
+template <class P, int THREADS, int TILE_BYTES>
+__global__ void __launch_bounds__(THREADS)
+    propagate_rest_kernel(const double *__restrict__ A, int ld, int ns_uniform,
+                          const int *__restrict__ ns_array, const typename P::Entry *__restrict__ table,
+                          int padded, double dt, pp_grid g, int ncand, double *__restrict__ n_p,
+                          double *__restrict__ partial, long long wait_limit, int skip_copies,
+                          unsigned int *__restrict__ status, const int *__restrict__ plans, int first_rest)
+{
+    __shared__ ItemSmem<P, THREADS, TILE_BYTES> sm;
+    const int nmodes = g.nx * g.ny * g.nz;
+    const int ngroups = (nmodes + kGroup - 1) / kGroup;
+    const int nblk = (nmodes + THREADS - 1) / THREADS;
+    int tiles = 0;
+    bool ready = false;
+    for (int c = 0; c < ncand; ++c) {
+        if (!takes_candidate<P, REST>(plans, c, first_rest))
+            continue;
+        if (!ready) {
+            if (threadIdx.x == 0) {
+                mbar_init(&sm.bar[0], 1);
+                mbar_init(&sm.bar[1], 1);
+                mbar_fence_init();
+            }
+            __syncthreads();
+            ready = true;
+        }
+        const int ns = ns_array ? ns_array[c] : ns_uniform;
+        const double *Ax = A + (size_t)c * 2 * ld;
+        // consecutive candidates' blocks go to consecutive CTAs
+        const int first = (int)(((long long)blockIdx.x - (long long)c * nblk % gridDim.x + gridDim.x) % gridDim.x);
+        for (int blk = first; blk < nblk; blk += gridDim.x)
+            if (!process_item<P, THREADS, TILE_BYTES, REST>(
+                    sm, blk, g, ns, plans[c], table + (size_t)c * padded, Ax, Ax + ld, dt,
+                    n_p ? n_p + (size_t)c * nmodes : nullptr, partial + (size_t)c * ngroups, wait_limit, skip_copies,
+                    status, tiles))
+                return;  // barrier phases are unknown after a wait gave up: this CTA stops
+    }
 }
 
 // N[c] = sum of the per-block partials of candidate c, in a fixed order.
@@ -84,30 +126,104 @@ __global__ void finalize_kernel(const double *__restrict__ partial, int nblk, do
     }
 }
 
+// A call's device buffers: the step table, the partial sums, the plans (one int per candidate) and, for uneven step
+// counts, room for a copy of n_steps.
+struct CallBuffers {
+    void *table;
+    double *partial;
+    int *plans;
+    int *ns;
+};
+
+// Step counts of a call: the largest, and whether all are equal.
+struct StepCounts {
+    int max = 0, first = 0;
+    bool uniform = true;
+    StepCounts(int ncand, int ld, const int32_t *ns_host)
+    {
+        first = ns_host ? ns_host[0] : (ld - 1) / 2;
+        for (int c = 0; c < ncand; ++c) {
+            const int ns = ns_host ? ns_host[c] : first;
+            max = ns > max ? ns : max;
+            uniform &= (ns == first);
+        }
+    }
+};
+
 template <class P, int THREADS, int TILE_BYTES>
-int run(const double *A, int ncand, int ld, const int32_t *ns_host, double dt, const pp_grid *grid,
-        double *N, double *n_p, cudaStream_t stream)
+int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const double *A, int ncand, int ld,
+           const int32_t *ns_host, double dt, const pp_grid *grid, double *N, double *n_p, cudaStream_t stream)
 {
     using V = typename P::Entry;
-    constexpr int TILE = TILE_BYTES / (int)sizeof(V);
-    int max_ns = 0;
-    bool uniform = true;
-    int ns0 = ns_host ? ns_host[0] : (ld - 1) / 2;
-    for (int c = 0; c < ncand; ++c) {
-        int ns = ns_host ? ns_host[c] : ns0;
-        max_ns = ns > max_ns ? ns : max_ns;
-        uniform &= (ns == ns0);
-    }
-    const int padded = ((max_ns + TILE - 1) / TILE) * TILE;
     unsigned int *status = pp::status_word();
     if (!status)
         return pp::fail(PP_ERR_CUDA, "status word unavailable");
     const int nmodes = grid->nx * grid->ny * grid->nz;
     const int nblk = (nmodes + THREADS - 1) / THREADS;
     const int ngroups = (nmodes + kGroup - 1) / kGroup;
+    V *table = (V *)buf.table;
+    const int *ns_array = nullptr;
+    if (!sc.uniform) {
+        cudaError_t e = cudaMemcpyAsync(buf.ns, ns_host, sizeof(int) * ncand, cudaMemcpyHostToDevice, stream);
+        if (e != cudaSuccess)
+            return pp::cuda_fail(e, "copy of n_steps");
+        ns_array = buf.ns;
+    }
+    if constexpr (IsBlock<typename MainPolicy<P>::type>::value) {
+        plan_kernel<P::kComp><<<ncand, kPlanThreads, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table,
+                                                                  buf.plans, n_p != nullptr);
+    } else {
+        if constexpr (HasPlan<P>::value) {
+            cudaError_t e = cudaMemsetAsync(buf.plans, 0, sizeof(int) * ncand, stream);
+            if (e != cudaSuccess)
+                return pp::cuda_fail(e, "plan reset");
+        }
+        dim3 tg((padded + 255) / 256, ncand);
+        build_table_kernel<P><<<tg, 256, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table, buf.plans);
+    }
+    dim3 pg(nblk, ncand);
+    pp::profile_mark_start(stream);
+    propagate_kernel<P, THREADS, TILE_BYTES, MAIN><<<pg, THREADS, 0, stream>>>(
+        A, ld, sc.first, ns_array, table, padded, dt, *grid, n_p, buf.partial, (long long)pp::wait_limit(),
+        pp::skip_copies(), status, buf.plans);
+    if constexpr (HasPlan<P>::value) {
+        // single steps are rare (rough potentials) except for the densities of long runs, which get a kernel of their own
+        int first_rest = kKindSeries;
+        if constexpr (IsBlock<typename MainPolicy<P>::type>::value && !P::kComp) {
+            if (n_p && single_steps(sc.max, dt)) {
+                propagate_kernel<P, THREADS, TILE_BYTES, SERIES><<<pg, THREADS, 0, stream>>>(
+                    A, ld, sc.first, ns_array, table, padded, dt, *grid, n_p, buf.partial,
+                    (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans);
+                first_rest = kKindWide;
+            }
+        }
+        constexpr int kRestCtas = 152 * (1024 / THREADS);
+        const long long items = (long long)nblk * ncand;
+        propagate_rest_kernel<P, THREADS, TILE_BYTES>
+            <<<(int)(items < kRestCtas ? items : kRestCtas), THREADS, 0, stream>>>(
+                A, ld, sc.first, ns_array, table, padded, dt, *grid, ncand, n_p, buf.partial,
+                (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans, first_rest);
+    }
+    pp::profile_mark_stop(stream);
+    finalize_kernel<<<ncand, 256, 0, stream>>>(buf.partial, ngroups, N, status);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess)
+        return pp::cuda_fail(e, "pair-number kernel launch");
+    return PP_OK;
+}
 
-    void *table = nullptr, *partial = nullptr, *nsdev = nullptr;
-    int rc = pp::scratch(pp::SCR_TABLE, (size_t)ncand * padded * sizeof(V), &table);
+template <class P, int THREADS, int TILE_BYTES>
+int run(const double *A, int ncand, int ld, const int32_t *ns_host, double dt, const pp_grid *grid,
+        double *N, double *n_p, cudaStream_t stream)
+{
+    using V = typename P::Entry;
+    constexpr int TILE = TILE_BYTES / (int)sizeof(V);
+    const StepCounts sc(ncand, ld, ns_host);
+    const int padded = ((sc.max + TILE - 1) / TILE) * TILE;
+    const int ngroups = (grid->nx * grid->ny * grid->nz + kGroup - 1) / kGroup;
+    CallBuffers buf;
+    void *partial = nullptr;
+    int rc = pp::scratch(pp::SCR_TABLE, (size_t)ncand * padded * sizeof(V), &buf.table);
     if (rc)
         return rc;
     rc = pp::scratch(pp::SCR_PARTIAL, (size_t)ncand * ngroups * sizeof(double) + 512 * sizeof(int) +
@@ -115,44 +231,17 @@ int run(const double *A, int ncand, int ld, const int32_t *ns_host, double dt, c
                      &partial);
     if (rc)
         return rc;
-    // after the partial sums: the per-candidate wide flags, then (uneven) n_steps
-    int *flags = (int *)(((uintptr_t)((char *)partial + (size_t)ncand * ngroups * sizeof(double)) + 255) &
-                         ~(uintptr_t)255);
-    const int *ns_array = nullptr;
-    if (!uniform) {
-        nsdev = (void *)(((uintptr_t)(flags + ncand) + 255) & ~(uintptr_t)255);
-        cudaError_t e = cudaMemcpyAsync(nsdev, ns_host, sizeof(int) * ncand, cudaMemcpyHostToDevice, stream);
-        if (e != cudaSuccess)
-            return pp::cuda_fail(e, "copy of n_steps");
-        ns_array = (const int *)nsdev;
-    }
-    cudaError_t ez = cudaMemsetAsync(flags, 0, sizeof(int) * ncand, stream);
-    if (ez != cudaSuccess)
-        return pp::cuda_fail(ez, "wide-flag reset");
-    dim3 tg((padded + 255) / 256, ncand);
-    build_table_kernel<P><<<tg, 256, 0, stream>>>(A, ld, ns0, ns_array, padded, dt, *grid, (V *)table, flags);
-    dim3 pg(nblk, ncand);
-    pp::profile_mark_start(stream);
-    propagate_kernel<P, THREADS, TILE_BYTES, false><<<pg, THREADS, 0, stream>>>(
-        A, ld, ns0, ns_array, (const V *)table, padded, dt, *grid, n_p, (double *)partial,
-        (long long)pp::wait_limit(), pp::skip_copies(), status, flags);
-    if constexpr (HasSeriesGuard<P>::value)
-        propagate_kernel<P, THREADS, TILE_BYTES, true><<<pg, THREADS, 0, stream>>>(
-            A, ld, ns0, ns_array, (const V *)table, padded, dt, *grid, n_p, (double *)partial,
-            (long long)pp::wait_limit(), pp::skip_copies(), status, flags);
-    pp::profile_mark_stop(stream);
-    finalize_kernel<<<ncand, 256, 0, stream>>>((const double *)partial, ngroups, N, status);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess)
-        return pp::cuda_fail(e, "pair-number kernel launch");
-    return PP_OK;
+    buf.partial = (double *)partial;
+    buf.plans = (int *)(((uintptr_t)(buf.partial + (size_t)ncand * ngroups) + 255) & ~(uintptr_t)255);
+    buf.ns = (int *)(((uintptr_t)(buf.plans + ncand) + 255) & ~(uintptr_t)255);
+    return launch<P, THREADS, TILE_BYTES>(buf, sc, padded, A, ncand, ld, ns_host, dt, grid, N, n_p, stream);
 }
 
 // ---------------------------------------------------------------- no-allocation variant
 // Scratch of pp_pair_number_static: a fixed device array in this file, held by
 // every GPU that loads the library until the process exits.  It holds, in
-// order, the per-step table, the per-block partial sums, the per-candidate
-// wide-range flags (cleared by each call before use) and (for uneven step
+// order, the step table, the per-block partial sums, the per-candidate
+// plans and (for uneven step
 // counts) a copy of n_steps; each call writes every byte it later reads, and
 // calls that overlap on the GPU race on it.
 constexpr size_t kStaticScratchBytes = (size_t)16 << 20;
@@ -186,23 +275,14 @@ int run_static(const double *A, int ncand, int ld, const int32_t *ns_host, doubl
 {
     using V = typename P::Entry;
     constexpr int TILE = TILE_BYTES / (int)sizeof(V);
-    int max_ns = 0;
-    bool uniform = true;
-    const int ns0 = ns_host ? ns_host[0] : (ld - 1) / 2;
-    for (int c = 0; c < ncand; ++c) {
-        const int ns = ns_host ? ns_host[c] : ns0;
-        max_ns = ns > max_ns ? ns : max_ns;
-        uniform &= (ns == ns0);
-    }
-    const int padded = ((max_ns + TILE - 1) / TILE) * TILE;
-    const int nmodes = grid->nx * grid->ny * grid->nz;
-    const int nblk = (nmodes + THREADS - 1) / THREADS;
-    const int ngroups = (nmodes + kGroup - 1) / kGroup;
+    const StepCounts sc(ncand, ld, ns_host);
+    const int padded = ((sc.max + TILE - 1) / TILE) * TILE;
+    const int ngroups = (grid->nx * grid->ny * grid->nz + kGroup - 1) / kGroup;
     const size_t table_bytes = align256((size_t)ncand * padded * sizeof(V));
     const size_t part_bytes = align256((size_t)ncand * ngroups * sizeof(double));
-    const size_t flag_bytes = align256((size_t)ncand * sizeof(int));
-    const size_t ns_bytes = uniform ? 0 : align256((size_t)ncand * sizeof(int));
-    const size_t need = table_bytes + part_bytes + flag_bytes + ns_bytes;
+    const size_t plan_bytes = align256((size_t)ncand * sizeof(int));
+    const size_t ns_bytes = sc.uniform ? 0 : align256((size_t)ncand * sizeof(int));
+    const size_t need = table_bytes + part_bytes + plan_bytes + ns_bytes;
     if (need > kStaticScratchBytes)
         return pp::fail(PP_ERR_INVALID_ARG,
                         "this call needs %zu bytes of scratch; the static scratch holds %zu "
@@ -211,38 +291,9 @@ int run_static(const double *A, int ncand, int ld, const int32_t *ns_host, doubl
     unsigned char *base = static_scratch_address();
     if (!base)
         return pp::fail(PP_ERR_CUDA, "cudaGetSymbolAddress of the static scratch failed");
-    unsigned int *status = pp::status_word();
-    if (!status)
-        return pp::fail(PP_ERR_CUDA, "status word unavailable");
-    V *table = (V *)base;
-    double *partial = (double *)(base + table_bytes);
-    int *flags = (int *)(base + table_bytes + part_bytes);
-    const int *ns_array = nullptr;
-    if (!uniform) {
-        int *nsdev = (int *)(base + table_bytes + part_bytes + flag_bytes);
-        cudaError_t e = cudaMemcpyAsync(nsdev, ns_host, sizeof(int) * ncand, cudaMemcpyHostToDevice, stream);
-        if (e != cudaSuccess)
-            return pp::cuda_fail(e, "copy of n_steps");
-        ns_array = nsdev;
-    }
-    cudaError_t ez = cudaMemsetAsync(flags, 0, sizeof(int) * ncand, stream);
-    if (ez != cudaSuccess)
-        return pp::cuda_fail(ez, "wide-flag reset");
-    dim3 tg((padded + 255) / 256, ncand);
-    build_table_kernel<P><<<tg, 256, 0, stream>>>(A, ld, ns0, ns_array, padded, dt, *grid, table, flags);
-    dim3 pg(nblk, ncand);
-    propagate_kernel<P, THREADS, TILE_BYTES, false><<<pg, THREADS, 0, stream>>>(
-        A, ld, ns0, ns_array, table, padded, dt, *grid, n_p, partial, (long long)pp::wait_limit(),
-        pp::skip_copies(), status, flags);
-    if constexpr (HasSeriesGuard<P>::value)
-        propagate_kernel<P, THREADS, TILE_BYTES, true><<<pg, THREADS, 0, stream>>>(
-            A, ld, ns0, ns_array, table, padded, dt, *grid, n_p, partial, (long long)pp::wait_limit(),
-            pp::skip_copies(), status, flags);
-    finalize_kernel<<<ncand, 256, 0, stream>>>(partial, ngroups, N, status);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess)
-        return pp::cuda_fail(e, "pair-number kernel launch");
-    return PP_OK;
+    const CallBuffers buf{base, (double *)(base + table_bytes), (int *)(base + table_bytes + part_bytes),
+                          (int *)(base + table_bytes + part_bytes + plan_bytes)};
+    return launch<P, THREADS, TILE_BYTES>(buf, sc, padded, A, ncand, ld, ns_host, dt, grid, N, n_p, stream);
 }
 
 // ---------------------------------------------------------------- launch configurations
@@ -310,7 +361,7 @@ const PolicySlot &policy_slot(int precision, int scheme)
         {{f_rk4.run_fn, f_rk4.static_fn, true, 0}, {f_mag.run_fn, f_mag.static_fn, true, 2},
          {f_spl.run_fn, f_spl.static_fn, true, 0}},
         {{x_rk4.run_fn, x_rk4.static_fn, true, 0}, {x_mag.run_fn, x_mag.static_fn, true, 0},
-         {x_spl.run_fn, x_spl.static_fn, true, 3}},
+         {x_spl.run_fn, x_spl.static_fn, true, 1}},
     };
     return slots[precision][scheme];
 }
@@ -354,13 +405,21 @@ int chosen_config(int precision, int scheme, int ncand, int ld, const int32_t *n
 
 namespace pp {
 
+// Uncompensated FP32 RK4 with densities runs compensated: n(p) then differs from earlier results by their
+// rounding walk alone (about 1e-5), and the step costs 94 instructions instead of 62, still half of the
+// stages'.
+int precision_of(int precision, int scheme, const double *n_p)
+{
+    return precision == PP_FP32_FAST && scheme == PP_RK4 && n_p ? PP_FP32 : precision;
+}
+
 int launch_pair_number(const double *A, int ncand, int ld, const int32_t *n_steps_host, double dt,
                        const pp_grid *grid, int precision, int scheme, double *N, double *n_p,
                        cudaStream_t stream)
 {
     const int cfg = chosen_config(precision, scheme, ncand, ld, n_steps_host, grid);
-    return policy_slot(precision, scheme).run_fn[cfg](A, ncand, ld, n_steps_host, dt, grid, N, n_p,
-                                                      stream);
+    return policy_slot(precision_of(precision, scheme, n_p), scheme)
+        .run_fn[cfg](A, ncand, ld, n_steps_host, dt, grid, N, n_p, stream);
 }
 
 int launch_pair_number_static(const double *A, int ncand, int ld, const int32_t *n_steps_host,
@@ -368,8 +427,8 @@ int launch_pair_number_static(const double *A, int ncand, int ld, const int32_t 
                               double *n_p, cudaStream_t stream)
 {
     const int cfg = chosen_config(precision, scheme, ncand, ld, n_steps_host, grid);
-    return policy_slot(precision, scheme).static_fn[cfg](A, ncand, ld, n_steps_host, dt, grid, N,
-                                                         n_p, stream);
+    return policy_slot(precision_of(precision, scheme, n_p), scheme)
+        .static_fn[cfg](A, ncand, ld, n_steps_host, dt, grid, N, n_p, stream);
 }
 
 size_t static_scratch_bytes() { return kStaticScratchBytes; }
