@@ -354,13 +354,16 @@ const PolicySlot &policy_slot(int precision, int scheme)
     static const ConfigTable<Rk4Policy<float, false>, true> x_rk4;
     static const ConfigTable<MagnusPolicy<float, false>, true> x_mag;
     static const ConfigTable<SplitPolicy<float, false>, true> x_spl;
-    // defaults from timing the 64-candidate workload on GB300 (see the tuner)
+    // Defaults from timing all configurations (pp_tune_pair_number) on 64 x 64 x 32 modes: CTAs of 128 threads leave less of
+    // the last wave idle and overlap one CTA's FP64 projection with another's steps (FP64 RK4 30.2 ms
+    // instead of 34.5 ms at 256 threads; on 32 x 32 x 16 modes 8.5 instead of 16.9 ms, 128 CTAs instead of 64 for 152
+    // SMs; FP32 Magnus 12.6 instead of 13.0 ms, RK4 12.3 instead of 12.9 ms).
     static const PolicySlot slots[3][3] = {
-        {{d_rk4.run_fn, d_rk4.static_fn, true, 0}, {d_mag.run_fn, d_mag.static_fn, false, 0},
+        {{d_rk4.run_fn, d_rk4.static_fn, true, 1}, {d_mag.run_fn, d_mag.static_fn, false, 0},
          {d_spl.run_fn, d_spl.static_fn, false, 0}},
-        {{f_rk4.run_fn, f_rk4.static_fn, true, 0}, {f_mag.run_fn, f_mag.static_fn, true, 2},
+        {{f_rk4.run_fn, f_rk4.static_fn, true, 4}, {f_mag.run_fn, f_mag.static_fn, true, 1},
          {f_spl.run_fn, f_spl.static_fn, true, 0}},
-        {{x_rk4.run_fn, x_rk4.static_fn, true, 0}, {x_mag.run_fn, x_mag.static_fn, true, 0},
+        {{x_rk4.run_fn, x_rk4.static_fn, true, 1}, {x_mag.run_fn, x_mag.static_fn, true, 1},
          {x_spl.run_fn, x_spl.static_fn, true, 1}},
     };
     return slots[precision][scheme];
