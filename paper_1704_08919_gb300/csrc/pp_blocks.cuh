@@ -5,7 +5,7 @@
 // Why.  The FP32 Magnus paths are bound by the FP32 lanes: 52 instructions per mode and step for
 // forming a step's generator and applying it to both spin channels, with the pipe 80% busy.  A time grid that
 // resolves the pulse makes the generators of neighbouring steps nearly equal, so the product of m of them is
-// exp(-i Omega.sigma) with an Omega that a short expansion gives to far below FP32 rounding: 78
+// exp(-i Omega.sigma) with an Omega that a short expansion gives to far below FP32 rounding: 73
 // instructions per m = 8 steps (compensated state, m = 4: 112 per 4 steps instead of 84 per step).
 // Fewer roundings also make the result more accurate: n(p) 2.6 times nearer to the FP64 step's (relative 2-norm 4.6e-6
 // instead of 1.2e-5 at 8192 steps), N 3 times.  One generation of 64 pulses on 64 x 64 x 32 modes, 8192 steps:
@@ -25,7 +25,7 @@
 //     Y = 1 + 2x/21 + x^2/105,  l = 0.6 (1 - m^-4),
 // C the sum of the steps' own z parts at S = 0 and of the commutators of the delta_j there.  The decimal
 // coefficients were fitted to the exact product in 40-digit arithmetic.  |Omega|^2 = x up to terms of this
-// order that are already in the coefficients, so tan th / th = sin th / (th cos th) is a function of x alone and shared by both
+// order that are already in the coefficients, so tan th / th is a function of x alone and shared by both
 // channels: in tracked form (MagnusPolicy) a channel costs 3 additions for its vector and 12 multiply-adds.
 //
 // When.  The expansion is left off where a next term of it could be seen; m is chosen per candidate from the
@@ -54,25 +54,22 @@ constexpr double kBlockAngleComp = 0.6;  // the tangent's polynomial
 // (about 1e-8 |h| dt per step and component at |h| dt ~ 0.1).
 constexpr float kBlockTol = 1.6e-7f;
 
-// sin(th)/th and cos(th) on th^2 <= kBlockAngle^2, (tan(th)/th - 1)/th^2 on th^2 <= kBlockAngleComp^2: interpolation
-// at the Chebyshev nodes of the range (relative errors 4e-10, 2e-11 and 3e-10 before rounding).
+// tan(th)/th on x = th^2 <= kBlockAngle^2 as a quotient, least squares at the Chebyshev nodes with the coefficients
+// rounded to FP32 one after the other (relative error 3e-10 with the rounded ones; 6 instructions and a reciprocal
+// where a sine and a cosine take 10), and (tan(th)/th - 1)/x on x <= kBlockAngleComp^2 by interpolation there (3e-10 before
+// rounding), for the compensated step, whose small rest must not carry the quotient's rounding.
 struct BlockSeries {
-    __host__ __device__ static __forceinline__ float sinc(float x)
+    __host__ __device__ static __forceinline__ float tanc(float x)
     {
-        float r = 2.66688473844e-6f;
-        r = fmaf(x, r, -0.000198301286838f);
-        r = fmaf(x, r, 0.00833327615921f);
-        r = fmaf(x, r, -0.166666656385f);
-        return fmaf(x, r, 0.999999999704f);
-    }
-    __host__ __device__ static __forceinline__ float cosine(float x)
-    {
-        float r = -2.66687022516e-7f;
-        r = fmaf(x, r, 2.47872608804e-5f);
-        r = fmaf(x, r, -0.00138887821597f);
-        r = fmaf(x, r, 0.0416666630688f);
-        r = fmaf(x, r, -0.499999999556f);
-        return fmaf(x, r, 0.999999999991f);
+        const float n = fmaf(x, fmaf(x, 0.002050169976f, -0.1215235665f), 1.0f);
+        float d = fmaf(x, -9.92794885e-5f, 0.02033581212f);
+        d = fmaf(x, d, -0.4548569024f);
+        d = fmaf(x, d, 1.0f);
+#ifdef __CUDA_ARCH__
+        return __fdividef(n, d);
+#else
+        return n / d;
+#endif
     }
     __host__ __device__ static __forceinline__ float tanm1(float x)
     {
@@ -124,35 +121,30 @@ struct MagnusBlockPolicy {
             tm1 = x * BlockSeries::tanm1(x);
             t = 1.0f + tm1;
         } else {
-            const float sn = BlockSeries::sinc(x), cs = BlockSeries::cosine(x);
-#ifdef __CUDA_ARCH__
-            t = __fdividef(sn, cs);
-#else
-            t = sn / cs;
-#endif
+            t = BlockSeries::tanc(x);
             tm1 = 0.0f;
         }
         const float y = fmaf(t * x, fmaf(x, 1.0f / 105.0f, 2.0f / 21.0f), t);
         const float xy = x * y;
-        const float qy = q * y;
+        const float qy = q * y, yr = y * r;
         // E
         const float f = fmaf(q * 0.144f, q, fmaf(x, e.c1, e.c0));
         float Ex, Ey, Ez;
         if constexpr (COMP) {
             // formed as S plus a small rest, so that the rest's roundings stay below S's
-            const float g = fmaf(y, r, fmaf(f, t, tm1));
+            const float g = fmaf(f, t, yr + tm1);
             Ex = fmaf(g, Sx, fmaf(qy, e.dx, fmaf(-xy, e.qx, st.lx)));
             Ey = fmaf(g, Sy, fmaf(qy, e.dy, fmaf(-xy, e.qy, st.ly)));
             Ez = fmaf(g, st.sz, st.lz);
         } else {
-            const float g = fmaf(y, r, f * t);
+            const float g = fmaf(f, t, yr);
             Ex = fmaf(g, Sx, fmaf(qy, e.dx, fmaf(-xy, e.qx, st.lx)));
             Ey = fmaf(g, Sy, fmaf(qy, e.dy, fmaf(-xy, e.qy, st.ly)));
             Ez = fmaf(g, st.sz, st.lz);
         }
         // O
-        const float a1 = fmaf(t * 3.427f, r, t);
-        const float a3 = (q * -3.318f) * t;
+        const float a1 = fmaf(3.427f, yr, t);
+        const float a3 = -3.318f * qy;
         const float wx = fmaf(a1, e.wx, fmaf(xy, e.vx, a3 * e.qx));
         const float wy = fmaf(a1, e.wy, fmaf(xy, e.vy, a3 * e.qy));
         const float zc = fmaf(Sx, wy, fmaf(-Sy, wx, t * fmaf(x, e.cz1, e.cz)));
