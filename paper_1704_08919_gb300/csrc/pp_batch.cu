@@ -250,7 +250,7 @@ const BatchTable &batch_table(int precision, int scheme)
          make_batch_table<SplitPolicy<float, true>>(true, 0)},
         {make_batch_table<Rk4Policy<float, false>>(true, 0),
          make_batch_table<MagnusPolicy<float, false>>(true, 0),
-         make_batch_table<SplitPolicy<float, false>>(true, 1)},
+         make_batch_table<SplitPolicy<float, false>>(true, 0)},
     };
     return t[precision][scheme];
 }

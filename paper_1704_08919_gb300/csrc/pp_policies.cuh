@@ -4,7 +4,7 @@
 // (RK4, fourth-order Magnus, second-order split operator; FP64, FP32 and FP32
 // with compensated state), the table builder and the work-item body shared by
 // the uniform kernel (pp_propagate.cu) and the persistent batch kernel
-// (pp_batch.cu).  Included by those two files only (internal linkage).
+// (pp_batch.cu).  Internal linkage (pp_qke.cu takes the grid's nodes and weights from here).
 #pragma once
 
 #include <math.h>
@@ -43,44 +43,63 @@ __device__ __forceinline__ double axis_node(int i, int n, double a, double b)
     return __dadd_rn(a, __ddiv_rn(__dmul_rn(__dsub_rn(b, a), (double)i), (double)(n - 1)));
 }
 
-__device__ __forceinline__ double axis_weight(int i, int n, double a, double b, int mirror)
+// Trapezoid weight of an interior node.
+__device__ __forceinline__ double axis_weight(int n, double a, double b, int mirror)
 {
     if (n == 1)
         return 1.0;
-    double d = __ddiv_rn(__dsub_rn(b, a), (double)(n - 1));
-    double w = (i == 0 || i == n - 1) ? __dmul_rn(0.5, d) : d;
-    return mirror ? __dmul_rn(2.0, w) : w;
+    const double d = __ddiv_rn(__dsub_rn(b, a), (double)(n - 1));
+    return mirror ? __dmul_rn(2.0, d) : d;
 }
 
-// Normalised eigenvectors of h . sigma (h_z = eps_perp >= 1 > 0), FP64.
-// negative: (-(hx - i hy), w + hz) / sqrt(2 w (w + hz)); positive: (w + hz, hx + i hy) / same.
-__device__ __forceinline__ void eig_neg(double hx, double hy, double hz, double v[4])
+// ... and of node i: half at the ends (exact).
+__device__ __forceinline__ double node_weight(int i, int n, double w)
 {
-    double w = sqrt(hx * hx + hy * hy + hz * hz);
-    double nr = 1.0 / sqrt(2.0 * w * (w + hz));
-    v[0] = -hx * nr;
-    v[1] = hy * nr;
-    v[2] = (w + hz) * nr;
+    return n > 1 && (i == 0 || i == n - 1) ? 0.5 * w : w;
+}
+
+// Normalised eigenvectors of h . sigma (h_z = eps_perp >= 1 > 0), FP64, with w = |h|:
+// negative: (-(hx - i hy), w + hz) / sqrt(2 w (w + hz)); positive: (w + hz, hx + i hy) / same.
+// Both spin channels (hy -> -hy) share the components' magnitudes, so the roots are taken once per mode: reciprocal square
+// roots, because the FP64 pipe (1/64 of the FP32 rate) is 15% busy with the work before the first and after the last step
+// at 1024 blocks of steps per mode, and more for shorter pulses.
+struct Eigen {
+    double x, y, z;  // hx, hy and w + hz over sqrt(2 w (w + hz))
+};
+__device__ __forceinline__ Eigen eigen(double hx, double hy, double hz)
+{
+    const double h2 = fma(hx, hx, fma(hy, hy, hz * hz));
+    const double w = h2 * rsqrt(h2), a = w + hz;
+    const double nr = rsqrt(2.0 * w * a);
+    return Eigen{hx * nr, hy * nr, a * nr};
+}
+
+__device__ __forceinline__ void eig_neg(const Eigen &e, int s, double v[4])
+{
+    v[0] = -e.x;
+    v[1] = s ? -e.y : e.y;
+    v[2] = e.z;
     v[3] = 0.0;
 }
 
-__device__ __forceinline__ double proj_pos2(double hx, double hy, double hz, const double p[4])
+__device__ __forceinline__ double proj_pos2(const Eigen &e, int s, const double p[4])
 {
-    double w = sqrt(hx * hx + hy * hy + hz * hz);
-    double nr = 1.0 / sqrt(2.0 * w * (w + hz));
-    double u0 = (w + hz) * nr, u2 = hx * nr, u3 = hy * nr;  // u1 = 0
-    double re = u0 * p[0] + u2 * p[2] + u3 * p[3];
-    double im = u0 * p[1] + u2 * p[3] - u3 * p[2];
-    return re * re + im * im;
+    const double y = s ? -e.y : e.y;
+    const double re = fma(e.z, p[0], fma(e.x, p[2], y * p[3]));
+    const double im = fma(e.z, p[1], fma(e.x, p[3], -y * p[2]));
+    return fma(re, re, im * im);
 }
 
-// U v for the 2 x 2 matrix U = [[a, -b*], [b, a*]] (a multiple of an SU(2) element) with first column z = (a, b).
-__device__ __forceinline__ void apply_su2(const double z[4], const double v[4], double p[4])
+// U v for the 2 x 2 matrix U = [[a, -b*], [b, a*]] (a multiple of an SU(2) element) with first column z = (a, b) and the
+// negative state v of channel s.
+__device__ __forceinline__ void apply_su2(const double z[4], const Eigen &e, int s, double p[4])
 {
-    p[0] = z[0] * v[0] - z[1] * v[1] - (z[2] * v[2] + z[3] * v[3]);
-    p[1] = z[0] * v[1] + z[1] * v[0] - (z[2] * v[3] - z[3] * v[2]);
-    p[2] = z[2] * v[0] - z[3] * v[1] + z[0] * v[2] + z[1] * v[3];
-    p[3] = z[2] * v[1] + z[3] * v[0] + z[0] * v[3] - z[1] * v[2];
+    double v[4];
+    eig_neg(e, s, v);
+    p[0] = fma(z[0], v[0], fma(-z[1], v[1], -z[2] * v[2]));
+    p[1] = fma(z[0], v[1], fma(z[1], v[0], z[3] * v[2]));
+    p[2] = fma(z[2], v[0], fma(-z[3], v[1], z[0] * v[2]));
+    p[3] = fma(z[2], v[1], fma(z[3], v[0], -z[1] * v[2]));
 }
 
 // ---------------------------------------------------------------- stepping policies
@@ -842,6 +861,7 @@ struct ItemSmem {
     __align__(128) V buf[2][TILE];
     __align__(8) uint64_t bar[2];
     double red[THREADS / 32];
+    double weight[3];  // of the grid's interior nodes, per axis
     typename Expands<P>::Coef coef[Expands<P>::value ? kExpandSpan : 1];
 };
 
@@ -890,6 +910,11 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
         }
     }
 
+    if (tid < 3)  // read after the barriers of the tile loop
+        sm.weight[tid] = tid == 0   ? axis_weight(g.nx, g.x0, g.x1, 0)
+                         : tid == 1 ? axis_weight(g.ny, g.y0, g.y1, 0)
+                                    : axis_weight(g.nz, g.z0, g.z1, g.mirror_z);
+
     // ---- this thread's momentum mode
     int ix = 0, iy = 0, iz = 0;
     if (active) {
@@ -912,9 +937,10 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
         }
     if constexpr (CarriesState<P>::value) {
         const double hx = px - Ax[0], hy = py - Ay[0];
+        const Eigen e = eigen(hx, hy, eperp);
         double v[2][4];
-        eig_neg(hx, hy, eperp, v[0]);
-        eig_neg(hx, -hy, eperp, v[1]);
+        eig_neg(e, 0, v[0]);
+        eig_neg(e, 1, v[1]);
         if constexpr (IsSplit<P>::value) {
             const auto h = P::half_step(px, py, eperp, dt);
             P::apply_half(h, 1.0, px, py, eperp, v[0]);
@@ -1034,11 +1060,11 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
                 psi[s][q] = P::kComp ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
         if constexpr (!CarriesState<P>::value) {
             const double hx = px - Ax[0], hy = py - Ay[0];
+            const Eigen e = eigen(hx, hy, eperp);
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
-                double v[4], z[4] = {psi[s][0], psi[s][1], psi[s][2], psi[s][3]};
-                eig_neg(hx, s ? -hy : hy, eperp, v);
-                apply_su2(z, v, psi[s]);
+                const double z[4] = {psi[s][0], psi[s][1], psi[s][2], psi[s][3]};
+                apply_su2(z, e, s, psi[s]);
             }
         }
         if constexpr (IsSplit<P>::value) {
@@ -1046,12 +1072,16 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
             P::apply_half(h, -1.0, px, py, eperp, psi[0]);
             P::apply_half(h, -1.0, px, -py, eperp, psi[1]);
         }
+        const Eigen e = eigen(Poutx, Pouty, eperp);
+        const double f0 = proj_pos2(e, 0, psi[0]), f1 = proj_pos2(e, 1, psi[1]);
+        if constexpr (TracksNorm<P>::value) {  // the states' norms grew
+            double n[2];
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            double fs = proj_pos2(Poutx, s ? -Pouty : Pouty, eperp, psi[s]);
-            if constexpr (TracksNorm<P>::value)  // the state's norm grew
-                fs /= psi[s][0] * psi[s][0] + psi[s][1] * psi[s][1] + psi[s][2] * psi[s][2] + psi[s][3] * psi[s][3];
-            f += fs;
+            for (int s = 0; s < 2; ++s)
+                n[s] = fma(psi[s][0], psi[s][0], fma(psi[s][1], psi[s][1], fma(psi[s][2], psi[s][2], psi[s][3] * psi[s][3])));
+            f = fma(f0, n[1], f1 * n[0]) / (n[0] * n[1]);
+        } else {
+            f = f0 + f1;
         }
         if (timed_out)
             f = __longlong_as_double(0x7ff8000000000000ll);
@@ -1060,9 +1090,8 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
     }
     double wf = 0.0;
     if (active) {
-        double w = __dmul_rn(__dmul_rn(axis_weight(ix, g.nx, g.x0, g.x1, 0),
-                                       axis_weight(iy, g.ny, g.y0, g.y1, 0)),
-                             axis_weight(iz, g.nz, g.z0, g.z1, g.mirror_z));
+        const double w = __dmul_rn(__dmul_rn(node_weight(ix, g.nx, sm.weight[0]), node_weight(iy, g.ny, sm.weight[1])),
+                                   node_weight(iz, g.nz, sm.weight[2]));
         wf = w * f;
     }
     // fixed-order reduction over groups of kGroup modes

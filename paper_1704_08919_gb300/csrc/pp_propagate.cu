@@ -364,7 +364,7 @@ const PolicySlot &policy_slot(int precision, int scheme)
         {{f_rk4.run_fn, f_rk4.static_fn, true, 4}, {f_mag.run_fn, f_mag.static_fn, true, 1},
          {f_spl.run_fn, f_spl.static_fn, true, 0}},
         {{x_rk4.run_fn, x_rk4.static_fn, true, 1}, {x_mag.run_fn, x_mag.static_fn, true, 1},
-         {x_spl.run_fn, x_spl.static_fn, true, 1}},
+         {x_spl.run_fn, x_spl.static_fn, true, 0}},
     };
     return slots[precision][scheme];
 }

@@ -337,8 +337,9 @@ __device__ __forceinline__ ModeGeom mode_geom(const pp_grid &g, int m)
     r.px = axis_node(ix, g.nx, g.x0, g.x1);
     r.py = axis_node(iy, g.ny, g.y0, g.y1);
     r.pz = axis_node(iz, g.nz, g.z0, g.z1);
-    r.w = r.active ? __dmul_rn(__dmul_rn(axis_weight(ix, g.nx, g.x0, g.x1, 0), axis_weight(iy, g.ny, g.y0, g.y1, 0)),
-                               axis_weight(iz, g.nz, g.z0, g.z1, g.mirror_z))
+    r.w = r.active ? __dmul_rn(__dmul_rn(node_weight(ix, g.nx, axis_weight(g.nx, g.x0, g.x1, 0)),
+                                         node_weight(iy, g.ny, axis_weight(g.ny, g.y0, g.y1, 0))),
+                               node_weight(iz, g.nz, axis_weight(g.nz, g.z0, g.z1, g.mirror_z)))
                    : 0.0;
     return r;
 }
