@@ -46,13 +46,14 @@ __host__ __device__ __forceinline__ T low_part(double dt, double p, T hi)
         return (T)(dt * p - (double)hi);
 }
 
-constexpr int kMaxBlock = 8;        // steps per block, uncompensated FP32
+constexpr int kMaxBlock = 10;       // steps per block, uncompensated FP32
 constexpr int kMaxBlockComp = 4;    // compensated: a block's own rounding grows with its angle
-constexpr double kBlockAngle = 1.2;      // most |Omega| per block: sine and cosine as polynomials below
+constexpr double kBlockAngle = 1.3;      // most |Omega| per block: the tangent's quotient, and the growth of the state
 constexpr double kBlockAngleComp = 0.6;  // the tangent's polynomial
-// Most estimated error of an amplitude per sqrt(step): a fifth of the rounding walk that FP32 steps take
-// (about 1e-8 |h| dt per step and component at |h| dt ~ 0.1).
-constexpr float kBlockTol = 1.6e-7f;
+// Most estimated error of an amplitude per sqrt(step).  At this line (m = 10 at steps of 0.0244) the expansion is off by
+// 2e-7 in n(p) (2-norm) and 1e-7 in N, FP32 rounding by 2e-6 to 1e-5 and 2e-7; m = 8 (1.6e-7) left 5e-8 and
+// 2e-8, m = 12 (1.5e-6) 7e-7 and 4e-7, more than rounding leaves in N.
+constexpr float kBlockTol = 6e-7f;
 
 // tan(th)/th on x = th^2 <= kBlockAngle^2 as a quotient, least squares at the Chebyshev nodes with the coefficients
 // rounded to FP32 one after the other (relative error 3e-10 with the rounded ones; 6 instructions and a reciprocal
@@ -61,9 +62,9 @@ constexpr float kBlockTol = 1.6e-7f;
 struct BlockSeries {
     __host__ __device__ static __forceinline__ float tanc(float x)
     {
-        const float n = fmaf(x, fmaf(x, 0.002050169976f, -0.1215235665f), 1.0f);
-        float d = fmaf(x, -9.92794885e-5f, 0.02033581212f);
-        d = fmaf(x, d, -0.4548569024f);
+        const float n = fmaf(x, fmaf(x, 0.002055725548f, -0.121581383f), 1.0f);
+        float d = fmaf(x, -9.984654753e-5f, 0.02036063932f);
+        d = fmaf(x, d, -0.4549147189f);
         d = fmaf(x, d, 1.0f);
 #ifdef __CUDA_ARCH__
         return __fdividef(n, d);

@@ -865,8 +865,8 @@ struct ItemSmem {
     typename Expands<P>::Coef coef[Expands<P>::value ? kExpandSpan : 1];
 };
 
-// Steps (or blocks of steps) between two rescalings of a growing state: a block grows it by 1 / cos th <= 2.8, so
-// its squared norm stays below 1e29.
+// Blocks of steps between two rescalings of a growing state: a block grows it by 1 / cos th <= 3.74, so its squared
+// norm stays below 1e38.
 constexpr int kRescaleSpan = 32;
 
 // One work item: the modes [blk * THREADS, (blk + 1) * THREADS) of one candidate with ns steps (P: the policy
