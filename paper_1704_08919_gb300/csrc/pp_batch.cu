@@ -43,12 +43,12 @@ __global__ void build_table_batch_kernel(const double *__restrict__ A, int ld,
 }
 
 template <bool COMP>
-__global__ void __launch_bounds__(kPlanThreads)
+__global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(kPlanThreads)
     plan_batch_kernel(const double *__restrict__ A, int ld, const BatchCand *__restrict__ cands, double dt,
                       typename MagnusPolicy<float, COMP>::Entry *__restrict__ table, int *__restrict__ plans,
                       bool densities)
 {
-    const int c = blockIdx.x;
+    const int c = blockIdx.x / kPlanCtas;
     const BatchCand d = cands[c];
     const double *Ax = A + (size_t)c * 2 * ld;
     plan_and_table<COMP>(Ax, Ax + ld, d.ns, dt, d.g, table + d.table_off, plans + c, densities);
@@ -164,7 +164,7 @@ int run_batch(const BatchLaunch &L, cudaStream_t stream)
     const auto *table = (const typename P::Entry *)L.table;
     constexpr bool kBlocks = IsBlock<typename MainPolicy<P>::type>::value;
     if constexpr (kBlocks) {
-        plan_batch_kernel<P::kComp><<<L.ncand, kPlanThreads, 0, stream>>>(
+        plan_batch_kernel<P::kComp><<<L.ncand * kPlanCtas, kPlanThreads, 0, stream>>>(
             L.A, L.ld, L.cands, L.dt, (typename P::Entry *)L.table, plans, L.n_p != nullptr);
     } else {
         dim3 tg((L.max_padded + 255) / 256, L.ncand);
@@ -530,8 +530,8 @@ int pp_batch_synth(pp_batch *b, const double *params, double *A, void *stream)
     clear_error();
     if (!b || !params || !A)
         return fail(PP_ERR_INVALID_ARG, "batch, params and A must not be NULL");
-    return launch_synth_batch(params, b->ncand, &b->specs[0], b->d_synth_desc, b->d_coef, b->max_M,
-                              2 * b->max_ns + 1, b->ld, A, (cudaStream_t)stream);
+    return launch_synth_batch(params, b->ncand, &b->specs[0], b->d_synth_desc, b->d_coef,
+                              b->max_M, 2 * b->max_ns + 1, b->ld, A, (cudaStream_t)stream);
 }
 
 int pp_batch_pair_number(pp_batch *b, const double *A, double *N, double *n_p, void *stream)

@@ -6,7 +6,7 @@
 // forming a step's generator and applying it to both spin channels, with the pipe 80% busy.  A time grid that
 // resolves the pulse makes the generators of neighbouring steps nearly equal, so the product of m of them is
 // exp(-i Omega.sigma) with an Omega that a short expansion gives to far below FP32 rounding: 73
-// instructions per m = 8 steps (compensated state, m = 4: 112 per 4 steps instead of 84 per step).
+// instructions per m <= 10 steps (compensated state, m = 4: 112 per 4 steps instead of 84 per step).
 // Fewer roundings also make the result more accurate: n(p) 2.6 times nearer to the FP64 step's (relative 2-norm 4.6e-6
 // instead of 1.2e-5 at 8192 steps), N 3 times.  One generation of 64 pulses on 64 x 64 x 32 modes, 8192 steps:
 // 112.8 -> 27.0 ms; 8 uneven pulses on 47 x 45 x 23 modes, up to 9001 steps, compensated: 7.4 -> 2.9 ms.
@@ -48,8 +48,8 @@ __host__ __device__ __forceinline__ T low_part(double dt, double p, T hi)
 
 constexpr int kMaxBlock = 10;       // steps per block, uncompensated FP32
 constexpr int kMaxBlockComp = 4;    // compensated: a block's own rounding grows with its angle
-constexpr double kBlockAngle = 1.3;      // most |Omega| per block: the tangent's quotient, and the growth of the state
-constexpr double kBlockAngleComp = 0.6;  // the tangent's polynomial
+constexpr float kBlockAngle = 1.3f;      // most |Omega| per block: the tangent's quotient, and the growth of the state
+constexpr float kBlockAngleComp = 0.6f;  // the tangent's polynomial
 // Most estimated error of an amplitude per sqrt(step).  At this line (m = 10 at steps of 0.0244) the expansion is off by
 // 2e-7 in n(p) (2-norm) and 1e-7 in N, FP32 rounding by 2e-6 to 1e-5 and 2e-7; m = 8 (1.6e-7) left 5e-8 and
 // 2e-8, m = 12 (1.5e-6) 7e-7 and 4e-7, more than rounding leaves in N.
@@ -208,23 +208,21 @@ __host__ __device__ inline bool single_steps(int n, double dt) { return (double)
 
 // What plan_block reads of one step: the bound on its angle (squared) and the size of the expansion's terms.
 struct StepSize {
-    double th2;
-    float dq, rough, cube;
+    float th2, dq, rough, cube;
 };
 
 // The block size from the largest angle of a step, th, and the sums of StepSize over the n steps.  The first neglected
 // terms are of second order in the pulse's change over the block, S^2 W Q with W = m^2 d / 6 and
 // Q = m^3 q / 180 (d = dt^2 A', q = dt^3 A''), and of third, S W^3; what the moments leave out
-// where the samples are not smooth goes with their own differences (rough).  Against the exact product over random
-// pulses (dt 0.02 to 0.05, fluence 0.3 to 13, momenta to 2.5) a plan within kBlockTol is off by at most
-// 3e-7 in n(p) (2-norm) and 1e-7 in N; FP32 rounding alone leaves 2e-6 to 2e-5 in n(p).
-__host__ __device__ inline int plan_block(double th, float dq, float rough, float cube, int n, int most, double angle)
+// where the samples are not smooth goes with their own differences (rough).  The weights were fitted to the exact product
+// over random pulses (dt 0.02 to 0.05, fluence 0.3 to 13, momenta to 2.5).
+__host__ __device__ inline int plan_block(float th, float dq, float rough, float cube, int n, int most, float angle)
 {
     const float per = 1.0f / sqrtf((float)n);
     for (int m = most; m >= 2; --m) {
         if (m > n || !(m * th <= angle))
             continue;
-        const float s = (float)(m * th), m2 = (float)(m * m);
+        const float s = m * th, m2 = (float)(m * m);
         const float e1 = s * s * m2 * m2 * (1.0f / 320.0f) * dq;  // 3.4 / 1080, m^5 per block, 1/m blocks per step
         const float e2 = s * s * s * (float)m * (0.03f / 180.0f) * rough;
         const float e3 = s * m2 * m2 * (float)m * (0.05f / 216.0f) * cube;
@@ -234,38 +232,36 @@ __host__ __device__ inline int plan_block(double th, float dq, float rough, floa
     return 1;
 }
 
-// Abar, end differences and the angle's bound of step n of the samples (Ax, Ay).
-__host__ __device__ __forceinline__ StepSize step_size(const double *Ax, const double *Ay, int n, int ns, double dt, double Px,
-                                              double Py, double E)
+// Step n of the samples (Ax, Ay): the bound on its angle over the grid (MagnusPolicy, rounded up) and the differences.
+// Everything is taken from the samples less the step's first, in FP32: FP64 work would bound the planning.
+__host__ __device__ __forceinline__ StepSize step_size(const double *Ax, const double *Ay, int n, int ns, float h,
+                                                       float Px, float Py, float E)
 {
     StepSize r;
-    const double a0x = Ax[2 * n], a0y = Ay[2 * n], ahx = Ax[2 * n + 1], ahy = Ay[2 * n + 1], a1x = Ax[2 * n + 2],
-                 a1y = Ay[2 * n + 2];
-    const double d6 = dt * dt / 6.0;
-    const double dx = a1x - a0x, dy = a1y - a0y;
-    const double ax = dt * (a0x + 4.0 * ahx + a1x) / 6.0, ay = dt * (a0y + 4.0 * ahy + a1y) / 6.0;
-    const double c = d6 * (a0x * a1y - a0y * a1x);
-    const double bx = dt * Px + fabs(ax) + E * d6 * fabs(dy);
-    const double by = dt * Py + fabs(ay) + E * d6 * fabs(dx);
-    const double bz = dt * E + d6 * (fabs(dy) * Px + fabs(dx) * Py) + fabs(c);
-    r.th2 = bx * bx + by * by + bz * bz;
-    const float h = (float)dt;
-    const float fdx = (float)dx, fdy = (float)dy;
-    const float d = h * sqrtf(fdx * fdx + fdy * fdy);
+    const double a0x = Ax[2 * n], a0y = Ay[2 * n];
+    auto rx = [&](int k) { return (float)(Ax[2 * n + k] - a0x); };
+    auto ry = [&](int k) { return (float)(Ay[2 * n + k] - a0y); };
+    const float x0 = (float)a0x, y0 = (float)a0y;
+    const float hx = rx(1), hy = ry(1), dx = rx(2), dy = ry(2);
+    const float d6 = h * h * (1.0f / 6.0f);
+    const float ax = h * fabsf(x0 + (4.0f * hx + dx) * (1.0f / 6.0f)), ay = h * fabsf(y0 + (4.0f * hy + dy) * (1.0f / 6.0f));
+    const float ux = d6 * fabsf(dx), uy = d6 * fabsf(dy);
+    const float bx = h * Px + ax + E * uy, by = h * Py + ay + E * ux;
+    const float bz = h * E + uy * Px + ux * Py + d6 * fabsf(x0 * dy - y0 * dx);
+    r.th2 = 1.000002f * (bx * bx + by * by + bz * bz);
+    const float d = h * sqrtf(dx * dx + dy * dy);
     // second differences, inside the step and across its end; third and fourth across the steps
-    const float hx = (float)(a0x + a1x - 2.0 * ahx), hy = (float)(a0y + a1y - 2.0 * ahy);
-    float q = 4.0f * sqrtf(hx * hx + hy * hy);
+    const float ix = dx - 2.0f * hx, iy = dy - 2.0f * hy;
+    float q = 4.0f * sqrtf(ix * ix + iy * iy);
     float v3 = 0.0f, f4 = 0.0f;
     if (n + 2 <= ns) {
-        const double a2x = Ax[2 * n + 4], a2y = Ay[2 * n + 4];
-        const float sx = (float)(a2x + a0x - 2.0 * a1x), sy = (float)(a2y + a0y - 2.0 * a1y);
+        const float sx = rx(4) - 2.0f * dx, sy = ry(4) - 2.0f * dy;
         q = fmaxf(q, sqrtf(sx * sx + sy * sy));
         if (n >= 1) {
-            const float ox = (float)(Ax[2 * n - 2] + a1x - 2.0 * a0x), oy = (float)(Ay[2 * n - 2] + a1y - 2.0 * a0y);
+            const float ox = rx(-2) + dx, oy = ry(-2) + dy;
             v3 = fabsf(sx - ox) + fabsf(sy - oy);
             // the middles' own second difference against the ends' fourth-order one
-            const float mx = (float)(Ax[2 * n + 3] + Ax[2 * n - 1] - 2.0 * ahx),
-                        my = (float)(Ay[2 * n + 3] + Ay[2 * n - 1] - 2.0 * ahy);
+            const float mx = rx(3) + rx(-1) - 2.0f * hx, my = ry(3) + ry(-1) - 2.0f * hy;
             f4 = fabsf(mx - 0.5f * (sx + ox)) + fabsf(my - 0.5f * (sy + oy));
         }
     }
@@ -276,25 +272,36 @@ __host__ __device__ __forceinline__ StepSize step_size(const double *Ax, const d
     return r;
 }
 
-// Entry of the block of m steps that starts at step n0.  The sum of the m potentials in FP64; everything else is a
-// small difference, taken from the samples less the block's mean and kept in FP32.
+// Entry of the block of m steps that starts at step n0.  The potential at its start in FP64; everything else is a small
+// difference, taken from the samples less that and kept in FP32.
 template <bool COMP>
 __host__ __device__ __forceinline__ typename MagnusBlockPolicy<COMP>::Entry block_entry(const double *Ax, const double *Ay,
                                                                                int n0, int m, double dt)
 {
-    double sx = 0.0, sy = 0.0;
-    for (int j = n0; j < n0 + m; ++j) {
-        sx += fma(4.0, Ax[2 * j + 1], Ax[2 * j] + Ax[2 * j + 2]);
-        sy += fma(4.0, Ay[2 * j + 1], Ay[2 * j] + Ay[2 * j + 2]);
+    const double x0 = Ax[2 * n0], y0 = Ay[2 * n0];
+    auto rx = [&](int k) { return (float)(Ax[k] - x0); };
+    auto ry = [&](int k) { return (float)(Ay[k] - y0); };
+    float sx = 0.0f, sy = 0.0f;  // sum of Abar - A(start)
+    {
+        float ex = 0.0f, ey = 0.0f;
+        for (int k = 2 * n0 + 1; k < 2 * (n0 + m); k += 2) {
+            const float fx = rx(k + 1), fy = ry(k + 1);
+            sx += 4.0f * rx(k) + (ex + fx);
+            sy += 4.0f * ry(k) + (ey + fy);
+            ex = fx;
+            ey = fy;
+        }
     }
-    const double bx = sx / (6.0 * m), by = sy / (6.0 * m);  // mean potential
+    sx *= 1.0f / 6.0f;
+    sy *= 1.0f / 6.0f;
+    const float bx = sx / (float)m, by = sy / (float)m;  // mean potential
     const float h = (float)dt, im = 1.0f / (float)m;
     float m1x = 0, m1y = 0, m2x = 0, m2y = 0, m3x = 0, m3y = 0, vx = 0, vy = 0, ux = 0, uy = 0, cz = 0, cx = 0, cy = 0;
-    float a0x = (float)(Ax[2 * n0] - bx), a0y = (float)(Ay[2 * n0] - by);
+    float a0x = -bx, a0y = -by;
     for (int j = 0; j < m; ++j) {
         const int k = 2 * (n0 + j);
-        const float ahx = (float)(Ax[k + 1] - bx), ahy = (float)(Ay[k + 1] - by);
-        const float a1x = (float)(Ax[k + 2] - bx), a1y = (float)(Ay[k + 2] - by);
+        const float ahx = rx(k + 1) - bx, ahy = ry(k + 1) - by;
+        const float a1x = rx(k + 2) - bx, a1y = ry(k + 2) - by;
         const float t = ((float)j + 0.5f) * im - 0.5f;
         // delta_j = -dt (Abar_j - mean)
         const float dx = h * (-1.0f / 6.0f) * (a0x + 4.0f * ahx + a1x), dy = h * (-1.0f / 6.0f) * (a0y + 4.0f * ahy + a1y);
@@ -323,8 +330,8 @@ __host__ __device__ __forceinline__ typename MagnusBlockPolicy<COMP>::Entry bloc
     const float W2 = w0x * w0x + w0y * w0y;
     // third order in the change: -1/840 |D|^2 of the unit-interval slope D = -6 W
     const float third = 1.0f - 0.257f * (1.0f - i4) * W2;
-    e.ax = (float)(dt * (sx / 6.0));
-    e.ay = (float)(dt * (sy / 6.0));
+    e.ax = (float)(dt * (m * x0 + sx));
+    e.ay = (float)(dt * (m * y0 + sy));
     e.c0 = COMP ? -l * W2 : 1.0f - l * W2;
     e.c1 = -0.241f * l * W2;
     e.qx = 2.0f * m2x - 2.0f * ux * im;

@@ -10,6 +10,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "pp_blocks.cuh"
@@ -760,79 +762,92 @@ __global__ void build_table_kernel(const double *__restrict__ A, int ld, int ns_
                  table + (size_t)c * padded, plans + c);
 }
 
-// Plan and table of one FP32 Magnus candidate by one CTA: a pass over the steps for the plan, then the blocks'
-// entries, or the single steps' where the plan has none.  Sums are taken in a fixed order, so a candidate's plan
-// depends on nothing but its own potential, grid and step.  One CTA per candidate: a pass over 8192
-// steps takes ~10 us beside the milliseconds of the propagation, and one launch instead of three.
-constexpr int kPlanThreads = 512;
+// Plan and table of one FP32 Magnus candidate by one cluster of CTAs: a pass over the steps for the plan, whose sums the
+// CTAs exchange through distributed shared memory, then the blocks' entries, or the single steps' where the plan has
+// none.  Sums are taken in a fixed order, so a candidate's plan depends on nothing but its own potential, grid and
+// step.  One launch (a pass over all steps, a choice and a second pass would be three), spread over 8 SMs per candidate
+// because the conversions from FP64 bound it: one CTA per candidate took
+// 250 us for 64 candidates of 8192 steps and 69 us for 16 of 2048 (2 pulses on 64 x 64 x 32 modes: 0.93 -> 0.71 ms a
+// call together with the synthesis' change).
+constexpr int kPlanThreads = 256, kPlanCtas = 8;
 template <bool COMP>
 __device__ __forceinline__ void plan_and_table(const double *__restrict__ Ax, const double *__restrict__ Ay, int ns,
                                                double dt, const pp_grid &g,
                                                typename MagnusPolicy<float, COMP>::Entry *__restrict__ row,
                                                int *__restrict__ plan_out, bool densities)
 {
-    __shared__ double s_th[kPlanThreads / 32];
-    __shared__ float s_sum[3][kPlanThreads / 32];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ float s_warp[4][kPlanThreads / 32], s_cta[4];
     __shared__ int s_plan;
-    const int tid = threadIdx.x;
-    const double Px = fmax(fabs(g.x0), fabs(g.x1)), Py = fmax(fabs(g.y0), fabs(g.y1));
-    const double Pz = fmax(fabs(g.z0), fabs(g.z1)), E = sqrt(1.0 + Pz * Pz);
-    double th2 = 0.0;
-    float sum[3] = {0.0f, 0.0f, 0.0f};
-    for (int n = tid; n < ns; n += kPlanThreads) {
-        const StepSize r = step_size(Ax, Ay, n, ns, dt, Px, Py, E);
-        th2 = fmax(th2, r.th2);
-        sum[0] += r.dq;
-        sum[1] += r.rough;
-        sum[2] += r.cube;
+    const int tid = threadIdx.x, rank = (int)cluster.block_rank();
+    const int at = rank * kPlanThreads + tid;
+    constexpr int kStride = kPlanCtas * kPlanThreads;
+    const float Px = (float)fmax(fabs(g.x0), fabs(g.x1)), Py = (float)fmax(fabs(g.y0), fabs(g.y1));
+    const float Pz = (float)fmax(fabs(g.z0), fabs(g.z1)), E = sqrtf(1.0f + Pz * Pz);
+    float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // th2's maximum, then the sums
+    for (int n = at; n < ns; n += kStride) {
+        const StepSize r = step_size(Ax, Ay, n, ns, (float)dt, Px, Py, E);
+        sum[0] = fmaxf(sum[0], r.th2);
+        sum[1] += r.dq;
+        sum[2] += r.rough;
+        sum[3] += r.cube;
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        th2 = fmax(th2, __shfl_xor_sync(0xffffffffu, th2, off));
+    for (int k = 0; k < 4; ++k) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-            sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], off);
-    }
-    if ((tid & 31) == 0) {
-        s_th[tid >> 5] = th2;
-        for (int k = 0; k < 3; ++k)
-            s_sum[k][tid >> 5] = sum[k];
+        for (int off = 16; off > 0; off >>= 1) {
+            const float o = __shfl_xor_sync(0xffffffffu, sum[k], off);
+            sum[k] = k == 0 ? fmaxf(sum[k], o) : sum[k] + o;
+        }
+        if ((tid & 31) == 0)
+            s_warp[k][tid >> 5] = sum[k];
     }
     __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < kPlanThreads / 32; ++w) {
-            th2 = fmax(th2, s_th[w]);
-            for (int k = 0; k < 3; ++k)
-                sum[k] += s_sum[k][w];
+    if (tid < 4) {
+        float v = s_warp[tid][0];
+        for (int w = 1; w < kPlanThreads / 32; ++w)
+            v = tid == 0 ? fmaxf(v, s_warp[tid][w]) : v + s_warp[tid][w];
+        s_cta[tid] = v;
+    }
+    cluster.sync();
+    if (tid == 0) {  // every CTA forms the same plan
+        float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int r = 0; r < kPlanCtas; ++r) {
+            const float *o = cluster.map_shared_rank(s_cta, r);
+            v[0] = fmaxf(v[0], o[0]);
+            for (int k = 1; k < 4; ++k)
+                v[k] += o[k];
         }
-        const double th = sqrt(th2);
+        const float th = sqrtf(v[0]);
         // a NaN in the potential fails every comparison: single steps, which carry it to the result
         const int m = !COMP && densities && single_steps(ns, dt)
                           ? 1
-                          : plan_block(th, sum[0], sum[1], sum[2], ns, COMP ? kMaxBlockComp : kMaxBlock,
+                          : plan_block(th, v[1], v[2], v[3], ns, COMP ? kMaxBlockComp : kMaxBlock,
                                        COMP ? kBlockAngleComp : kBlockAngle);
-        s_plan = m > 1 ? plan_pack(kKindMain, m) : plan_pack(th > kSeriesLimit ? kKindWide : kKindSeries, 1);
-        *plan_out = s_plan;
+        s_plan = m > 1 ? plan_pack(kKindMain, m) : plan_pack(th > (float)kSeriesLimit ? kKindWide : kKindSeries, 1);
+        if (rank == 0)
+            *plan_out = s_plan;
     }
-    __syncthreads();
+    cluster.sync();  // s_plan is there, and no CTA leaves while another reads its sums
     const int m = plan_steps(s_plan);
     if (plan_kind(s_plan) == kKindMain) {
         auto *blocks = reinterpret_cast<typename MagnusBlockPolicy<COMP>::Entry *>(row);
-        for (int b = tid; b * m < ns; b += kPlanThreads)
+        for (int b = at; b * m < ns; b += kStride)
             blocks[b] = block_entry<COMP>(Ax, Ay, b * m, min(m, ns - b * m), dt);
     } else {
-        for (int n = tid; n < ns; n += kPlanThreads)
+        for (int n = at; n < ns; n += kStride)
             row[n] = table_entry((const MagnusPolicy<float, COMP> *)nullptr, Ax, Ay, n, dt, g);
     }
 }
 
 template <bool COMP>
-__global__ void __launch_bounds__(kPlanThreads)
+__global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(kPlanThreads)
     plan_kernel(const double *__restrict__ A, int ld, int ns_uniform, const int *__restrict__ ns_array, int padded,
                 double dt, pp_grid g, typename MagnusPolicy<float, COMP>::Entry *__restrict__ table,
                 int *__restrict__ plans, bool densities)
 {
-    const int c = blockIdx.x;
+    const int c = blockIdx.x / kPlanCtas;
     const double *Ax = A + (size_t)c * 2 * ld;
     plan_and_table<COMP>(Ax, Ax + ld, ns_array ? ns_array[c] : ns_uniform, dt, g, table + (size_t)c * padded, plans + c,
                          densities);

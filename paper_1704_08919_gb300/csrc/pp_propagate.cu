@@ -170,7 +170,7 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
         ns_array = buf.ns;
     }
     if constexpr (IsBlock<typename MainPolicy<P>::type>::value) {
-        plan_kernel<P::kComp><<<ncand, kPlanThreads, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table,
+        plan_kernel<P::kComp><<<ncand * kPlanCtas, kPlanThreads, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table,
                                                                   buf.plans, n_p != nullptr);
     } else {
         if constexpr (HasPlan<P>::value) {

@@ -80,18 +80,17 @@ static double block_error(const V &X, const V &Y, int n0, int m, double dt, doub
     }
     return worst;
 }
-static int plan(const V &X, const V &Y, int n, double dt, double P, double Z, int most, double angle)
+static int plan(const V &X, const V &Y, int n, double dt, double P, double Z, int most, float angle)
 {
-    double th2 = 0;
-    float s[3] = {0, 0, 0};
+    float th2 = 0, s[3] = {0, 0, 0};
     for (int j = 0; j < n; ++j) {
-        const StepSize r = step_size(X.data(), Y.data(), j, n, dt, P, P, sqrt(1 + Z * Z));
-        th2 = fmax(th2, r.th2);
+        const StepSize r = step_size(X.data(), Y.data(), j, n, (float)dt, (float)P, (float)P, sqrtf(1 + Z * Z));
+        th2 = fmaxf(th2, r.th2);
         s[0] += r.dq;
         s[1] += r.rough;
         s[2] += r.cube;
     }
-    return plan_block(sqrt(th2), s[0], s[1], s[2], n, most, angle);
+    return plan_block(sqrtf(th2), s[0], s[1], s[2], n, most, angle);
 }
 static void pulse(int n, double dt, double noise, unsigned seed, V &X, V &Y)
 {
