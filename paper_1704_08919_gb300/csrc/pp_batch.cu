@@ -278,7 +278,6 @@ struct pp_batch {
     void *d_table = nullptr;
     double *d_partial = nullptr;
     void *d_synth_desc = nullptr, *d_coef = nullptr;
-    int max_M = 0;
     double *d_A = nullptr, *d_trial = nullptr, *d_tfit = nullptr;
     unsigned long long *d_gen = nullptr;
     // captured DE loop
@@ -352,7 +351,7 @@ int batch_de_generation(pp_batch *b, double *pop, double *fit, const double *lo,
                                           b->d_trial, st);
     if (!rc)
         rc = pp::launch_synth_batch(b->d_trial, b->ncand, &b->specs[0], b->d_synth_desc, b->d_coef,
-                                    b->max_M, 2 * b->max_ns + 1, b->ld, b->d_A, st);
+                                    2 * b->max_ns + 1, b->ld, b->d_A, st);
     if (!rc)
         rc = batch_pair_number(b, b->d_A, b->d_tfit, nullptr, b->cfg, st);
     if (!rc)
@@ -490,7 +489,7 @@ int pp_batch_create(int32_t ncand, const pp_field_spec *specs, const pp_grid *gr
         batch_free(b);
         return cuda_fail(e, "batch allocation");
     }
-    int rc = synth_batch_prepare(ncand, specs, &b->d_synth_desc, &b->d_coef, &b->max_M);
+    int rc = synth_batch_prepare(ncand, specs, &b->d_synth_desc, &b->d_coef);
     // persistent grid sizes
     int sms = 0;
     if (!rc && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev) != cudaSuccess)
@@ -531,7 +530,7 @@ int pp_batch_synth(pp_batch *b, const double *params, double *A, void *stream)
     if (!b || !params || !A)
         return fail(PP_ERR_INVALID_ARG, "batch, params and A must not be NULL");
     return launch_synth_batch(params, b->ncand, &b->specs[0], b->d_synth_desc, b->d_coef,
-                              b->max_M, 2 * b->max_ns + 1, b->ld, A, (cudaStream_t)stream);
+                              2 * b->max_ns + 1, b->ld, A, (cudaStream_t)stream);
 }
 
 int pp_batch_pair_number(pp_batch *b, const double *A, double *N, double *n_p, void *stream)

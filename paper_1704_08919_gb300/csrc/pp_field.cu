@@ -9,8 +9,7 @@
 //     E_l(t_k) = Re sum_j C_j z_k^j,         C_j = s E~_j e^{-i Phi_j} (-1)^j
 //     A_l(t_k) = -Im sum_j D_j (z_k^j - 1),  D_j = C_j / Omega_j
 // (A = -int_{-T/2}^t E, so A(-T/2) = 0 and, by periodicity, A(T/2) = 0).
-// Each sum is evaluated by Horner's rule in z_k after factoring z_k^{j_first};
-// z_k comes from sincospi of an exactly reduced argument.  The fluence of the
+// z_k and z_k^{j_first} come from sincospi of exactly reduced arguments, the powers between by multiplication.  The fluence of the
 // unit-scale field over one period is (T/2) sum_{l,j} E~_{l,j}^2, and
 // s = sqrt(U_const / that).
 #include <math.h>
@@ -26,37 +25,42 @@ constexpr int kMaxOrder = 8;
 
 // Cox-de Boor recursion on the clamped knot vector (order copies of w_min,
 // equidistant interior breakpoints, order copies of w_max); order-1 indicators
-// of [t_i, t_{i+1}) with the last non-empty interval closed on the right.
+// of [t_i, t_{i+1}) with the last non-empty interval closed on the right.  Only the `order` functions that are
+// nonzero at w are formed (the others stay 0): the FP64 divisions of the whole triangle were most of the spectrum's
+// time (31 us for 16 candidates of 15 modes).
 __device__ void bspline_basis(int K, int order, double wmin, double wmax, double w, double *B)
 {
-    double t[kMaxK + kMaxOrder];
-    double b[kMaxK + kMaxOrder];
-    const int nk = K + order;
     const int nbrk = K - order + 2;
-    for (int i = 0; i < order; ++i) {
-        t[i] = wmin;
-        t[K + i] = wmax;
-    }
-    for (int i = 1; i < nbrk - 1; ++i)
-        t[order - 1 + i] = wmin + (wmax - wmin) * (double)i / (double)(nbrk - 1);
-    int last = -1;
-    for (int i = 0; i < nk - 1; ++i)
-        if (t[i] < t[i + 1])
-            last = i;
-    for (int i = 0; i < nk - 1; ++i) {
-        bool inside = (t[i] <= w && w < t[i + 1]) || (i == last && w == t[i + 1]);
-        b[i] = inside ? 1.0 : 0.0;
-    }
+    auto knot = [&](int i) {
+        if (i < order)
+            return wmin;
+        if (i >= K)
+            return wmax;
+        return wmin + (wmax - wmin) * (double)(i - order + 1) / (double)(nbrk - 1);
+    };
+    for (int i = 0; i < K; ++i)
+        B[i] = 0.0;
+    // the interval [t_s, t_{s+1}) that holds w: s in [order - 1, K - 1]
+    if (!(w >= wmin && w <= wmax))
+        return;
+    int s = order - 1;
+    while (s < K - 1 && knot(s + 1) <= w)
+        ++s;
+    double t[2 * kMaxOrder], b[kMaxOrder + 1];  // t[q] = knot s - order + 1 + q; b[q]: function s - order + 1 + q
+    for (int q = 0; q < 2 * order; ++q)
+        t[q] = knot(s - order + 1 + q);
+    for (int q = 0; q <= order; ++q)
+        b[q] = q == order - 1 ? 1.0 : 0.0;
     for (int r = 2; r <= order; ++r) {
-        for (int i = 0; i < nk - r; ++i) {
-            double d1 = t[i + r - 1] - t[i], d2 = t[i + r] - t[i + 1];
-            double left = d1 > 0.0 ? (w - t[i]) / d1 * b[i] : 0.0;
-            double right = d2 > 0.0 ? (t[i + r] - w) / d2 * b[i + 1] : 0.0;
-            b[i] = left + right;
+        for (int q = order - r; q < order; ++q) {
+            const double d1 = t[q + r - 1] - t[q], d2 = t[q + r] - t[q + 1];
+            const double left = d1 > 0.0 ? (w - t[q]) / d1 * b[q] : 0.0;
+            const double right = d2 > 0.0 ? (t[q + r] - w) / d2 * b[q + 1] : 0.0;
+            b[q] = left + right;
         }
     }
-    for (int i = 0; i < K; ++i)
-        B[i] = b[i];
+    for (int q = 0; q < order; ++q)
+        B[s - order + 1 + q] = b[q];
 }
 
 // Block-wide sum of one value per thread (blockDim.x a power of two <= 256).
@@ -205,70 +209,127 @@ __global__ void hann_spectrum_kernel(const double *__restrict__ params, int K, i
                         coef + (size_t)c * 4 * (M + 2), scale_out ? scale_out + c : nullptr, status, normalize);
 }
 
-// Samples: grid (ceil(nsamp / 256), ncand, 2 polarisations).  Horner's rule in
-// FP64 with explicit fused multiply-adds, per complex step z (x) + X_m:
-// (xr zc - xi zs + Xr, xr zs + xi zc + Xi).  WANT_E / WANT_ED compile the
-// accumulations of E and dE/dt in only when the caller asked for them.
-template <bool WANT_E, bool WANT_ED>
-__global__ void samples_kernel(const double2 *__restrict__ coef, int M, int j0, int n_steps,
-                               int ld, double *__restrict__ A, double *__restrict__ E, double dw,
-                               double *__restrict__ Ed, double T)
-{
-    extern __shared__ double2 sc[];  // [2M]: C then D
-    __shared__ double s_d0i;
-    const int c = blockIdx.y, l = blockIdx.z;
-    const double2 *cf = coef + ((size_t)c * 2 + l) * 2 * M;
-    for (int q = threadIdx.x; q < 2 * M; q += blockDim.x)
-        sc[q] = cf[q];
-    __syncthreads();
-    if (threadIdx.x == 0) {  // Im of the sum of D_j (the z = 1 value), the same for every sample
-        double d0i = 0.0;
-        for (int m = M - 1; m >= 0; --m)
-            d0i += sc[M + m].y;
-        s_d0i = d0i;
+// Samples.  One thread forms the samples k, n - k, n + k and 2n - k of both polarisations, k in [0, n/2]: the powers
+// z_k^j = c + i s are shared by all eight, and with Im(D z^j) = D_r s + D_i c, the four samples of a
+// polarisation are sums of the same four partial sums (D_r s and D_i c, over even and odd j):
+// z_{n+k}^j = (-1)^j z_k^j and z_{2n-k} = conj z_k.  Eight fused multiply-adds per harmonic give eight samples, where Horner's rule
+// took 32; the FP64 pipe bounds the synthesis (64 pulses of 63 harmonics on 16385 samples: 1.19 -> 0.3 ms).  The powers
+// are advanced by complex multiplication from an exactly reduced z_k^{j0}; their error grows by about 2^-53 per
+// harmonic.  WANT_E / WANT_ED compile the sums of E and dE/dt in only when the caller asked for them.
+struct PartialSums {
+    double s[2] = {0.0, 0.0}, c[2] = {0.0, 0.0};  // [parity of j]
+    __device__ __forceinline__ void add(int parity, double x, double y, double zs, double zc)
+    {
+        s[parity] = fma(x, zs, s[parity]);
+        c[parity] = fma(y, zc, c[parity]);
     }
-    __syncthreads();
-    const int nsamp = 2 * n_steps + 1;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nsamp)
+    // the sums at k, n - k, n + k, 2n - k
+    __device__ __forceinline__ void at(double out[4]) const
+    {
+        const double se = s[0] + s[1], ce = c[0] + c[1], so = s[0] - s[1], co = c[0] - c[1];
+        out[0] = ce + se;
+        out[1] = co - so;
+        out[2] = co + so;
+        out[3] = ce - se;
+    }
+};
+
+// Threads per candidate of samples_at.
+__host__ __device__ inline int sample_threads(int n_steps) { return n_steps / 2 + 1; }
+
+// cf: this candidate's coefficients (C then D for l = 0, 1); A, E, Ed: its rows (2 of ld).
+template <bool WANT_E, bool WANT_ED>
+__device__ __forceinline__ void samples_at(const double2 *__restrict__ cf, int M, int j0, int n_steps, int k, double T,
+                                           int ld, double *__restrict__ A, double *__restrict__ E,
+                                           double *__restrict__ Ed)
+{
+    // Im of the sums of D_j (the z = 1 value), by each warp
+    double d0[2] = {0.0, 0.0};
+    for (int m = threadIdx.x & 31; m < M; m += 32) {
+        d0[0] += cf[M + m].y;
+        d0[1] += cf[3 * M + m].y;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        d0[0] += __shfl_xor_sync(0xffffffffu, d0[0], off);
+        d0[1] += __shfl_xor_sync(0xffffffffu, d0[1], off);
+    }
+    if (k >= sample_threads(n_steps))
         return;
-    // z = exp(i pi k / n), zj0 = z^{j0}; arguments reduced exactly modulo 2n
+    // z = exp(i pi k / n) and zj = z^{j0}; arguments reduced exactly modulo 2n
     const long long two_n = 2ll * n_steps;
     double zs, zc, js, jc;
-    sincospi((double)(k % two_n) / (double)n_steps, &zs, &zc);
+    sincospi((double)k / (double)n_steps, &zs, &zc);
     sincospi((double)(((long long)k * j0) % two_n) / (double)n_steps, &js, &jc);
-    // Horner: sum_{m=0}^{M-1} X_m z^m
-    double cr = 0.0, ci = 0.0, dr = 0.0, di = 0.0, gr = 0.0, gi = 0.0;
-    for (int m = M - 1; m >= 0; --m) {
-        const double2 D = sc[M + m];
-        const double tr = fma(dr, zc, fma(-di, zs, D.x));
-        di = fma(dr, zs, fma(di, zc, D.y));
-        dr = tr;
-        if constexpr (WANT_E) {
-            const double2 C = sc[m];
-            const double ur = fma(cr, zc, fma(-ci, zs, C.x));
-            ci = fma(cr, zs, fma(ci, zc, C.y));
-            cr = ur;
+    const double dw = 2.0 * M_PI / T;
+    PartialSums a[2], e[2], d[2];
+    auto harmonic = [&](int m, int parity) {
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            const double2 D = cf[(2 * l + 1) * M + m];
+            a[l].add(parity, D.x, D.y, js, jc);
+            if constexpr (WANT_E || WANT_ED) {
+                const double2 C = cf[2 * l * M + m];
+                if constexpr (WANT_E)  // Re(C z^j)
+                    e[l].add(parity, -C.y, C.x, js, jc);
+                if constexpr (WANT_ED) {  // dE/dt: coefficients i Omega_j C_j
+                    const double W = (double)(j0 + m) * dw;
+                    d[l].add(parity, -W * C.x, -W * C.y, js, jc);
+                }
+            }
         }
-        if constexpr (WANT_ED) {  // dE/dt: coefficients i Omega_j C_j
-            const double2 C = sc[m];
-            const double W = (double)(j0 + m) * dw;
-            const double vr = fma(gr, zc, fma(-gi, zs, -W * C.y));
-            gi = fma(gr, zs, fma(gi, zc, W * C.x));
-            gr = vr;
+        const double t = fma(jc, zc, -js * zs);
+        js = fma(jc, zs, js * zc);
+        jc = t;
+    };
+    // even and odd harmonics in turn, so that the partial sums stay in registers
+    int m = 0;
+    if (j0 & 1)
+        harmonic(m++, 1);
+    for (; m + 1 < M; m += 2) {
+        harmonic(m, 0);
+        harmonic(m + 1, 1);
+    }
+    if (m < M)
+        harmonic(m, 0);
+    const int at[4] = {k, n_steps - k, n_steps + k, 2 * n_steps - k};
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        double v[4];
+        a[l].at(v);
+        const double c0 = j0 == 0 ? cf[2 * l * M].x : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            double x = k == 0 && (q == 0 || q == 3) ? 0.0 : d0[l] - v[q];  // A = 0 at both ends, exactly
+            if (j0 == 0)  // DC harmonic (Hann envelope): potential c0 (t_f - t_k)
+                x += c0 * ((double)(2 * n_steps - at[q]) * (T / (2.0 * n_steps)));
+            A[(size_t)l * ld + at[q]] = x;
+        }
+        if constexpr (WANT_E) {
+            e[l].at(v);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                E[(size_t)l * ld + at[q]] = v[q];
+        }
+        if constexpr (WANT_ED) {
+            d[l].at(v);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                Ed[(size_t)l * ld + at[q]] = v[q];
         }
     }
-    // multiply by z^{j0}
-    const double Di = fma(dr, js, di * jc);
-    double *Arow = A + ((size_t)c * 2 + l) * ld;
-    double a = -(Di - s_d0i);
-    if (j0 == 0)  // DC harmonic (Hann envelope): potential c0 (t_f - t_k)
-        a += sc[0].x * ((double)(2 * n_steps - k) * (T / (2.0 * n_steps)));
-    Arow[k] = a;
-    if constexpr (WANT_E)
-        E[((size_t)c * 2 + l) * ld + k] = fma(cr, jc, -ci * js);
-    if constexpr (WANT_ED)
-        Ed[((size_t)c * 2 + l) * ld + k] = fma(gr, jc, -gi * js);
+}
+
+// Grid (ceil(sample_threads / 128), ncand).
+constexpr int kSampleThreads = 128;
+template <bool WANT_E, bool WANT_ED>
+__global__ void __launch_bounds__(kSampleThreads)
+    samples_kernel(const double2 *__restrict__ coef, int M, int j0, int n_steps, int ld, double *__restrict__ A,
+                   double *__restrict__ E, double *__restrict__ Ed, double T)
+{
+    const size_t c = blockIdx.y, row = c * 2 * ld;
+    samples_at<WANT_E, WANT_ED>(coef + c * 4 * M, M, j0, n_steps, blockIdx.x * kSampleThreads + threadIdx.x, T, ld,
+                                A + row, WANT_E ? E + row : nullptr, WANT_ED ? Ed + row : nullptr);
 }
 
 // ---- chain rule of the un-normalised synthesis (the local search's gradient):
@@ -568,40 +629,16 @@ __global__ void spectrum_batch_kernel(const double *__restrict__ params, int K, 
         spectrum_block(prm, K, order, wmin, wmax, d.T, U, d.j0m, d.Mm, coef + d.coef_off, nullptr, status, 1);
 }
 
-__global__ void samples_batch_kernel(const double2 *__restrict__ coef, const SynthCand *__restrict__ sc,
-                                     int ld, double *__restrict__ A)
+__global__ void __launch_bounds__(kSampleThreads)
+    samples_batch_kernel(const double2 *__restrict__ coef, const SynthCand *__restrict__ sc, int ld,
+                         double *__restrict__ A)
 {
-    extern __shared__ double2 scf[];
-    const int c = blockIdx.y, l = blockIdx.z;
+    const int c = blockIdx.y;
     const SynthCand d = sc[c];
-    const int nsamp = 2 * d.n_steps + 1;
-    if (blockIdx.x * blockDim.x >= nsamp)
+    if (blockIdx.x * kSampleThreads >= sample_threads(d.n_steps))
         return;  // the whole block is past this candidate's samples
-    const double2 *cf = coef + d.coef_off + (size_t)l * 2 * d.M;
-    for (int q = threadIdx.x; q < 2 * d.M; q += blockDim.x)
-        scf[q] = cf[q];
-    __syncthreads();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nsamp)
-        return;
-    const int M = d.M;
-    const long long two_n = 2ll * d.n_steps;
-    double zs, zc, js, jc;
-    sincospi((double)(k % two_n) / (double)d.n_steps, &zs, &zc);
-    sincospi((double)(((long long)k * d.j0) % two_n) / (double)d.n_steps, &js, &jc);
-    double dr = 0.0, di = 0.0, d0i = 0.0;
-    for (int m = M - 1; m >= 0; --m) {
-        const double2 D = scf[M + m];
-        const double tr = fma(dr, zc, fma(-di, zs, D.x));
-        di = fma(dr, zs, fma(di, zc, D.y));
-        dr = tr;
-        d0i += D.y;
-    }
-    const double Di = fma(dr, js, di * jc);
-    double a = -(Di - d0i);
-    if (d.j0 == 0)  // DC harmonic of the Hann envelope: potential c0 (t_f - t_k)
-        a += scf[0].x * ((double)(2 * d.n_steps - k) * (d.T / (2.0 * d.n_steps)));
-    A[((size_t)c * 2 + l) * ld + k] = a;
+    samples_at<false, false>(coef + d.coef_off, d.M, d.j0, d.n_steps, blockIdx.x * kSampleThreads + threadIdx.x, d.T, ld,
+                             A + (size_t)c * 2 * ld, nullptr, nullptr);
 }
 
 }  // namespace
@@ -609,12 +646,10 @@ __global__ void samples_batch_kernel(const double2 *__restrict__ coef, const Syn
 namespace pp {
 
 // Device descriptors for a batch of pulse lengths (pp_batch): built once on the host.
-int synth_batch_prepare(int ncand, const pp_field_spec *specs, void **d_desc, void **d_coef,
-                        int *max_M)
+int synth_batch_prepare(int ncand, const pp_field_spec *specs, void **d_desc, void **d_coef)
 {
     std::vector<SynthCand> h(ncand);
     long long off = 0;
-    int mm = 0;
     for (int c = 0; c < ncand; ++c) {
         const double dw = 2.0 * M_PI / specs[c].T;
         int j0 = (int)ceil(specs[c].w_min / dw - 1e-12);
@@ -631,7 +666,6 @@ int synth_batch_prepare(int ncand, const pp_field_spec *specs, void **d_desc, vo
         h[c].M = env ? h[c].Mm + 2 : h[c].Mm;
         h[c].coef_off = off;
         off += 4ll * h[c].M;
-        mm = h[c].M > mm ? h[c].M : mm;
     }
     cudaError_t e = cudaMalloc(d_desc, sizeof(SynthCand) * (size_t)ncand);
     if (e == cudaSuccess)
@@ -640,12 +674,11 @@ int synth_batch_prepare(int ncand, const pp_field_spec *specs, void **d_desc, vo
         e = cudaMemcpy(*d_desc, h.data(), sizeof(SynthCand) * (size_t)ncand, cudaMemcpyHostToDevice);
     if (e != cudaSuccess)
         return cuda_fail(e, "batch synthesis descriptors");
-    *max_M = mm;
     return PP_OK;
 }
 
 int launch_synth_batch(const double *params, int ncand, const pp_field_spec *spec0, const void *d_desc,
-                       void *d_coef, int max_M, int max_nsamp, int ld, double *A, cudaStream_t stream)
+                       void *d_coef, int max_nsamp, int ld, double *A, cudaStream_t stream)
 {
     unsigned int *status = status_word();
     if (!status)
@@ -654,9 +687,8 @@ int launch_synth_batch(const double *params, int ncand, const pp_field_spec *spe
                                                      spec0->w_max, spec0->fluence,
                                                      (const SynthCand *)d_desc, (double2 *)d_coef,
                                                      status);
-    dim3 g((max_nsamp + 255) / 256, ncand, 2);
-    samples_batch_kernel<<<g, 256, 2 * max_M * sizeof(double2), stream>>>(
-        (const double2 *)d_coef, (const SynthCand *)d_desc, ld, A);
+    dim3 g((sample_threads((max_nsamp - 1) / 2) + kSampleThreads - 1) / kSampleThreads, ncand);
+    samples_batch_kernel<<<g, kSampleThreads, 0, stream>>>((const double2 *)d_coef, (const SynthCand *)d_desc, ld, A);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return cuda_fail(e, "batch synthesis launch");
@@ -700,12 +732,10 @@ int launch_synth(const double *params, int ncand, const pp_field_spec *spec, int
         spectrum_kernel<<<ncand, 128, 0, stream>>>(params, spec->K, spec->order, spec->w_min, spec->w_max,
                                                    spec->T, spec->fluence, j0, M, (double2 *)coef, scale, status,
                                                    normalize);
-    const int nsamp = 2 * spec->n_steps + 1;
-    dim3 g((nsamp + 255) / 256, ncand, 2);
+    dim3 g((sample_threads(spec->n_steps) + kSampleThreads - 1) / kSampleThreads, ncand);
     auto kern = E ? (Ed ? samples_kernel<true, true> : samples_kernel<true, false>)
                   : (Ed ? samples_kernel<false, true> : samples_kernel<false, false>);
-    kern<<<g, 256, 2 * Ms * sizeof(double2), stream>>>((const double2 *)coef, Ms, j0s, spec->n_steps, ld, A, E,
-                                                       2.0 * M_PI / spec->T, Ed, spec->T);
+    kern<<<g, kSampleThreads, 0, stream>>>((const double2 *)coef, Ms, j0s, spec->n_steps, ld, A, E, Ed, spec->T);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return cuda_fail(e, "synthesis kernel launch");

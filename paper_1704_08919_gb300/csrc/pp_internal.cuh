@@ -113,10 +113,9 @@ int launch_pack_bf16(const float *X, int rows, int cols, int ldx, int trans, voi
                      int cols_pad, cudaStream_t stream);
 
 // Batch synthesis (pp_field.cu): per-candidate pulse lengths.
-int synth_batch_prepare(int ncand, const pp_field_spec *specs, void **d_desc, void **d_coef,
-                        int *max_M);
+int synth_batch_prepare(int ncand, const pp_field_spec *specs, void **d_desc, void **d_coef);
 int launch_synth_batch(const double *params, int ncand, const pp_field_spec *spec0, const void *d_desc,
-                       void *d_coef, int max_M, int max_nsamp, int ld, double *A, cudaStream_t stream);
+                       void *d_coef, int max_nsamp, int ld, double *A, cudaStream_t stream);
 
 }  // namespace pp
 
