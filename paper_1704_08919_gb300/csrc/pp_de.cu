@@ -29,7 +29,8 @@ __device__ __forceinline__ int below(uint64_t x, int n)
     return (int)(((x >> 32) * (uint64_t)n) >> 32);
 }
 
-// One block per individual: thread 0 draws the donors and R, all threads build
+// One block per individual (blockIdx.x) and proposal (blockIdx.y, of generation gen + blockIdx.y, into
+// consecutive NP x D arrays): thread 0 draws the donors and R, all threads build
 // the trial coordinates.  Floating-point steps use explicit round-to-nearest
 // intrinsics so that no multiply-add is contracted.
 __global__ void de_propose_kernel(const double *__restrict__ pop, int NP, int D,
@@ -42,6 +43,8 @@ __global__ void de_propose_kernel(const double *__restrict__ pop, int NP, int D,
     const int i = blockIdx.x;
     if (gen_dev)
         gen = *gen_dev;
+    gen += blockIdx.y;
+    trial += (size_t)blockIdx.y * NP * D;
     const uint64_t key = sm64_at(sm64_at(seed, gen), (uint64_t)i);
     if (threadIdx.x == 0) {
         int r[3] = {-1, -1, -1};
@@ -135,9 +138,9 @@ namespace pp {
 
 int launch_de_propose(const double *pop, int NP, int D, const double *lo, const double *hi,
                       const uint8_t *periodic, double F, double CR, uint64_t seed, uint64_t gen,
-                      double *trial, cudaStream_t stream)
+                      double *trial, cudaStream_t stream, int R)
 {
-    de_propose_kernel<<<NP, 64, 0, stream>>>(pop, NP, D, lo, hi, periodic, F, CR, seed, gen, trial,
+    de_propose_kernel<<<dim3(NP, R), 64, 0, stream>>>(pop, NP, D, lo, hi, periodic, F, CR, seed, gen, trial,
                                              nullptr);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PP_OK : cuda_fail(e, "DE propose launch");

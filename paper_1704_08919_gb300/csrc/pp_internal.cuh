@@ -93,10 +93,10 @@ int launch_qke_pair_number(const double *A, const double *E, const double *Ed, i
 int launch_qke_gradient(const double *A, const double *E, const double *Ed, int ncand, int ld, int n_steps,
                         double dt, const pp_grid *g, int precision, double *J, double *gs, int ldg, cudaStream_t st);
 
-// DE launches (pp_de.cu).
+// DE launches (pp_de.cu).  R proposals: those of the generations gen .. gen + R - 1, one after the other in trial.
 int launch_de_propose(const double *pop, int NP, int D, const double *lo, const double *hi,
                       const uint8_t *periodic, double F, double CR, uint64_t seed, uint64_t gen,
-                      double *trial, cudaStream_t stream);
+                      double *trial, cudaStream_t stream, int R = 1);
 int launch_de_select(double *pop, double *fit, const double *trial, const double *trial_fit,
                      int NP, int D, cudaStream_t stream);
 // DE with a device-resident generation counter (captured loops, pp_batch).

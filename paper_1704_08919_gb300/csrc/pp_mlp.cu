@@ -795,10 +795,8 @@ int pp_de_screened_step(double *pop, double *fit, int32_t NP, const pp_field_spe
     int32_t *kp = kept_out ? kept_out : (int32_t *)kept;
     double *tr = trial_out ? trial_out : (double *)trial;
     double *tf = trial_fit_out ? trial_fit_out : (double *)tfit;
-    // R proposals per individual, each from its own counter-RNG stream (generation R g + r)
-    for (int r = 0; r < R && !rc; ++r)
-        rc = launch_de_propose(pop, NP, D, lo, hi, periodic, F, CR, seed, generation * (uint64_t)R + r,
-                               (double *)props + (size_t)r * NP * D, st);
+    // R proposals per individual, each from its own counter-RNG stream (generation R g + r), in one launch
+    rc = launch_de_propose(pop, NP, D, lo, hi, periodic, F, CR, seed, generation * (uint64_t)R, (double *)props, st, R);
     if (rc)
         return rc;
     features_kernel<<<nb((long long)R * NP * D), 256, 0, st>>>((const double *)props, R * NP, D, lo, hi, D,
