@@ -57,7 +57,7 @@ __global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(kPlanThreads
 // ROLE selects the slots this launch takes (see takes_candidate); items of the
 // other kinds are drawn from the queue and skipped.
 template <class P, int THREADS, int TILE_BYTES, Role ROLE>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, kResidentThreads<RolePolicy<P, ROLE>> / THREADS)
     propagate_batch_kernel(const double *__restrict__ A, int ld, const BatchCand *__restrict__ cands,
                            const int2 *__restrict__ work, int nwork, int *__restrict__ counter,
                            const typename P::Entry *__restrict__ table, double dt,

@@ -75,6 +75,15 @@ int scratch(int slot, size_t bytes, void **ptr)
     return PP_OK;
 }
 
+bool scratch_holds(int slot, size_t bytes)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
+        return false;
+    std::lock_guard<std::mutex> lk(g_mu);
+    return g_cap[dev][slot] >= bytes;
+}
+
 int release_scratch()
 {
     int dev = 0;

@@ -30,10 +30,11 @@ void clear_error();
 enum ScratchSlot {
     SCR_TABLE = 0, SCR_PARTIAL, SCR_A, SCR_TRIAL, SCR_TFIT, SCR_COEF,
     SCR_SCREEN_PROPS, SCR_SCREEN_X, SCR_SCREEN_Y, SCR_SCREEN_KEPT,
-    SCR_VJP, SCR_QKE_TABLE, SCR_QKE_CKPT, SCR_QKE_PART, SCR_QKE_G, SCR_QKE_FIELD, SCR_QKE_X, SCR_GRIDS, SCR_RATE,
+    SCR_VJP, SCR_QKE_TABLE, SCR_QKE_CKPT, SCR_QKE_PART, SCR_QKE_G, SCR_QKE_FIELD, SCR_QKE_X, SCR_GRIDS, SCR_RATE, SCR_SEGMENTS,
     SCR_NSLOTS
 };
 int scratch(int slot, size_t bytes, void **ptr);
+bool scratch_holds(int slot, size_t bytes);  // whether scratch() would return without allocating
 int release_scratch();  // frees every slot of the current device (after a device synchronisation)
 
 // Argument checks shared by the entry points (pp_capi.cu); they record the message.

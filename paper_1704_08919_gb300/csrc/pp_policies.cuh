@@ -725,6 +725,13 @@ __device__ __forceinline__ void rescale_state(State &st)
     }
 }
 
+// Sets the counts of finished segments to 0 (thread `at` of `all`).
+__device__ __forceinline__ void clear_counts(int *__restrict__ done, int ndone, int at, int all)
+{
+    for (int i = at; i < ndone; i += all)
+        done[i] = 0;
+}
+
 // Step tables of the policies without a plan, and of FP64 Magnus (grid (blocks, candidates), 256 threads).  For the
 // latter, plans[c] (zeroed before the launch) becomes kKindWide when any step of the candidate leaves the
 // polynomials' range.
@@ -754,9 +761,11 @@ template <class P>
 __global__ void build_table_kernel(const double *__restrict__ A, int ld, int ns_uniform,
                                    const int *__restrict__ ns_array, int padded, double dt,
                                    pp_grid g, typename P::Entry *__restrict__ table,
-                                   int *__restrict__ plans)
+                                   int *__restrict__ plans, int *__restrict__ done, int ndone)
 {
     const int c = blockIdx.y;
+    clear_counts(done, ndone, (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x,
+                 gridDim.x * gridDim.y * blockDim.x);
     const double *Ax = A + (size_t)c * 2 * ld;
     table_row<P>(Ax, Ax + ld, blockIdx.x * blockDim.x + threadIdx.x, ns_array ? ns_array[c] : ns_uniform, padded, dt, g,
                  table + (size_t)c * padded, plans + c);
@@ -845,9 +854,10 @@ template <bool COMP>
 __global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(kPlanThreads)
     plan_kernel(const double *__restrict__ A, int ld, int ns_uniform, const int *__restrict__ ns_array, int padded,
                 double dt, pp_grid g, typename MagnusPolicy<float, COMP>::Entry *__restrict__ table,
-                int *__restrict__ plans, bool densities)
+                int *__restrict__ plans, bool densities, int *__restrict__ done, int ndone)
 {
     const int c = blockIdx.x / kPlanCtas;
+    clear_counts(done, ndone, blockIdx.x * kPlanThreads + threadIdx.x, gridDim.x * kPlanThreads);
     const double *Ax = A + (size_t)c * 2 * ld;
     plan_and_table<COMP>(Ax, Ax + ld, ns_array ? ns_array[c] : ns_uniform, dt, g, table + (size_t)c * padded, plans + c,
                          densities);
@@ -869,6 +879,154 @@ __device__ __forceinline__ bool takes_candidate(const int *__restrict__ plans, i
 template <class P, Role ROLE>
 using RolePolicy = typename std::conditional<ROLE == MAIN, typename MainPolicy<P>::type, P>::type;
 
+// ---------------------------------------------------------------- segments of the time axis
+// A grid of few modes leaves SMs idle, or too few warps on each, while every thread walks its whole chain of steps.  Where the
+// policy builds up a propagator, the table's entries are cut into segments and the propagator of each is formed apart, from
+// the identity; the product of all, in order, is the propagator of the pulse.  The number of segments depends on the
+// grid and the number of steps alone, and the product is formed in the same order whether one CTA walks all segments or
+// CTAs of their own do (process_item), so results do not depend on which.
+// kSegTarget modes times segments are 16 CTAs of 128 threads per SM, so that the last wave weighs little.  A segment
+// repeats the FP64 head of a mode and the product (about 200 FP64 instructions) and stays long against that: 256
+// steps in FP64 (16000 instructions), 512 in FP32 RK4 and 1024 in blocks of steps.  One pulse of 8000 steps on 189 modes: FP64
+// 16.9 -> 0.77 ms, compensated RK4 566 -> 126 us, blocks 125 -> 65 us; 4000 FP64 steps on 32 x 32 x 16 modes 8.47 -> 7.38 ms; 2
+// pulses on 64 x 64 x 32 modes in FP64 241 -> 233 ms.
+constexpr int kSegTarget = 152 * 2048;
+constexpr int kMaxSegs = 24;
+template <class P>
+struct Segments {
+    static constexpr bool kCuts = !CarriesState<P>::value;
+    static constexpr int kLeast =
+        IsBlock<P>::value ? 1024
+                          : (sizeof(typename std::remove_reference<decltype(P::State::hi[0][0])>::type) == 8 ? 256 : 512);
+    // most segments of ns steps on a grid
+    __host__ __device__ static int most(int nmodes, int ns)
+    {
+        if (!kCuts)
+            return 1;
+        int k = kSegTarget / nmodes;
+        k = k < ns / kLeast ? k : ns / kLeast;
+        k = k < kMaxSegs ? k : kMaxSegs;
+        return k < 1 ? 1 : k;
+    }
+};
+
+// tot <- cur tot for the two channels' propagators (first columns; COMP: hi, then lo), not inlined: it runs once per
+// segment.
+template <typename T, bool COMP>
+__device__ __noinline__ void fold_segment(const T *cur, T *tot)
+{
+#pragma unroll 1
+    for (int s = 0; s < 2; ++s) {
+        const T *z = cur + 4 * s;
+        T *t = tot + 4 * s;
+        if constexpr (COMP) {
+            double a[4], b[4];
+            for (int q = 0; q < 4; ++q) {
+                a[q] = (double)z[q] + (double)z[q + 8];
+                b[q] = (double)t[q] + (double)t[q + 8];
+            }
+            const double r[4] = {fma(a[0], b[0], fma(-a[1], b[1], fma(-a[2], b[2], -a[3] * b[3]))),
+                                 fma(a[0], b[1], fma(a[1], b[0], fma(-a[2], b[3], a[3] * b[2]))),
+                                 fma(a[2], b[0], fma(-a[3], b[1], fma(a[0], b[2], a[1] * b[3]))),
+                                 fma(a[2], b[1], fma(a[3], b[0], fma(a[0], b[3], -a[1] * b[2])))};
+            for (int q = 0; q < 4; ++q) {
+                t[q] = (T)r[q];
+                t[q + 8] = (T)(r[q] - (double)t[q]);
+            }
+        } else {
+            const T r[4] = {fma(z[0], t[0], fma(-z[1], t[1], fma(-z[2], t[2], -z[3] * t[3]))),
+                            fma(z[0], t[1], fma(z[1], t[0], fma(-z[2], t[3], z[3] * t[2]))),
+                            fma(z[2], t[0], fma(-z[3], t[1], fma(z[0], t[2], z[1] * t[3]))),
+                            fma(z[2], t[1], fma(z[3], t[0], fma(z[0], t[3], -z[1] * t[2])))};
+            for (int q = 0; q < 4; ++q)
+                t[q] = r[q];
+        }
+    }
+}
+
+// A state's components in the order of fold_segment.
+template <class P, typename T>
+__device__ __forceinline__ void get_state(const typename P::State &st, T *v)
+{
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[4 * s + q] = st.hi[s][q];
+            if constexpr (P::kComp)
+                v[8 + 4 * s + q] = st.lo[s][q];
+        }
+}
+template <class P, typename T>
+__device__ __forceinline__ void set_state(typename P::State &st, const T *v)
+{
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            st.hi[s][q] = v[4 * s + q];
+            if constexpr (P::kComp)
+                st.lo[s][q] = v[8 + 4 * s + q];
+        }
+}
+
+// A finished segment's propagator joins the product (the first begins it); the state is the product so far.
+template <class P, typename T>
+__device__ __forceinline__ void join_segment(typename P::State &st, T *total, bool first)
+{
+    T cur[P::kComp ? 16 : 8];
+    get_state<P>(st, cur);
+    if (first) {
+#pragma unroll
+        for (int q = 0; q < (P::kComp ? 16 : 8); ++q)
+            total[q] = cur[q];
+        return;
+    }
+    fold_segment<T, P::kComp>(cur, total);
+    set_state<P>(st, total);
+    if constexpr (TracksNorm<P>::value) {
+        rescale_state<P::kComp>(st);
+        get_state<P>(st, total);
+    }
+}
+
+// Threads per SM that the registers must allow, timed from 640 to 1280 (and without a limit) for each policy: the loops need 45 to
+// 70 registers, and what the compiler makes of a limit moves them by up to 8% either way (64 pulses in blocks of steps: 19.0 ms
+// at 1280, 19.3 at 1024, 19.7 at 768).
+template <class P>
+struct Residency {
+    static constexpr int threads = sizeof(typename std::remove_reference<decltype(P::State::hi[0][0])>::type) == 8 ? 640 : 768;
+};
+template <>
+struct Residency<MagnusBlockPolicy<false>> {
+    static constexpr int threads = 1280;
+};
+template <>
+struct Residency<Rk4Policy<float, false>> {
+    static constexpr int threads = 1280;
+};
+template <bool C>
+struct Residency<MagnusPolicy<float, C>> {
+    static constexpr int threads = 1024;
+};
+template <class P>
+constexpr int kResidentThreads = Residency<P>::threads;
+
+// Table entries of a candidate.
+template <class P>
+__device__ __forceinline__ int item_entries(int ns, int plan)
+{
+    return IsBlock<P>::value ? (ns + plan_steps(plan) - 1) / plan_steps(plan) : ns;
+}
+
+// What a CTA of one segment needs: its segment (-1: it walks all), the buffer of this (candidate, block of modes)'s segment
+// propagators ([segment][component][thread]) and its count of finished segments (0 before the launch).
+struct SegmentWork {
+    int seg;
+    void *out;
+    int *done;
+};
+
 template <class P, int THREADS, int TILE_BYTES>
 struct ItemSmem {
     using V = typename P::Entry;
@@ -877,6 +1035,8 @@ struct ItemSmem {
     __align__(8) uint64_t bar[2];
     double red[THREADS / 32];
     double weight[3];  // of the grid's interior nodes, per axis
+    int last;          // whether this CTA's segment was the last to finish
+    double mode[3][THREADS];  // p_x, p_y, eps of each thread's mode: kept here while the steps need the registers
     typename Expands<P>::Coef coef[Expands<P>::value ? kExpandSpan : 1];
 };
 
@@ -890,6 +1050,8 @@ constexpr int kRescaleSpan = 32;
 // state in FP64 at the end.  The caller owns the shared-memory buffers and the two mbarriers; tile_base
 // is the number of tiles this CTA has consumed before (the barrier phases run
 // on across items) and is moved on.  Returns false if a bounded wait gave up.
+// work.seg < 0: all segments.  Otherwise one segment: its propagator goes to work.out, and the CTA that finishes the item's
+// last segment multiplies them and does the rest.
 template <class P, int THREADS, int TILE_BYTES, Role ROLE>
 __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &sm, int blk,
                                              const pp_grid &g, int ns, int plan,
@@ -899,9 +1061,11 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
                                              double *__restrict__ n_out,
                                              double *__restrict__ part_out, long long wait_limit,
                                              int skip_copies, unsigned int *__restrict__ status,
-                                             int &tile_base)
+                                             int &tile_base, SegmentWork work = SegmentWork{-1, nullptr, nullptr})
 {
     using V = typename P::Entry;
+    using Real = typename std::remove_reference<decltype(P::State::hi[0][0])>::type;
+    constexpr int kParts = P::kComp ? 16 : 8;  // components of a state
     constexpr int TILE = TILE_BYTES / (int)sizeof(V);
     static_assert(THREADS % kGroup == 0, "CTA size must be a multiple of the partial-sum group");
     const int tid = threadIdx.x;
@@ -909,21 +1073,28 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
     const int m = blk * THREADS + tid;
     const bool active = m < nmodes;
     const int per = IsBlock<P>::value ? plan_steps(plan) : 1;  // steps per table entry
-    const int nent = IsBlock<P>::value ? (ns + per - 1) / per : ns;
-    const int ntiles = (nent + TILE - 1) / TILE;
-    const int base = tile_base;
-    tile_base += ntiles;
-
-    int issued = 0;  // meaningful in thread 0 only
-    if (tid == 0 && !skip_copies) {
-        for (int t = 0; t < 2 && t < ntiles; ++t) {
-            const int k = base + t;
-            mbar_arrive_expect_tx(&sm.bar[k & 1], TILE * (uint32_t)sizeof(V));
-            bulk_copy_g2s(sm.buf[k & 1], trow + (size_t)t * TILE, TILE * (uint32_t)sizeof(V),
-                          &sm.bar[k & 1]);
-            ++issued;
-        }
-    }
+    const int nent = item_entries<P>(ns, plan);
+    constexpr bool kCuts = Segments<P>::kCuts;
+    const int seg_len = kCuts ? (nent + Segments<P>::most(nmodes, ns) - 1) / Segments<P>::most(nmodes, ns) : nent;
+    const int nseg = kCuts ? (nent + seg_len - 1) / seg_len : 1;
+    const int seg0 = kCuts && work.seg >= 0 ? work.seg : 0;
+    // tile t of the segment's `count` entries from `first`, as the CTA's tile number `base` + t (by thread 0)
+    auto fetch = [&](int first, int count, int base, int t) {
+        const int k = base + t;
+        const uint32_t bytes = min(TILE, count - t * TILE) * (uint32_t)sizeof(V);
+        mbar_arrive_expect_tx(&sm.bar[k & 1], bytes);
+        bulk_copy_g2s(sm.buf[k & 1], trow + first + (size_t)t * TILE, bytes, &sm.bar[k & 1]);
+    };
+    auto fetch_first = [&](int seg) {  // a segment's first two tiles; how many there are
+        const int first = seg * seg_len, count = min(seg_len, nent - first);
+        int t = 0;
+        for (; t < 2 && t * TILE < count; ++t)
+            fetch(first, count, tile_base, t);
+        return t;
+    };
+    int issued = 0;  // tiles of the current segment; meaningful in thread 0 only
+    if (tid == 0 && !skip_copies)
+        issued = fetch_first(seg0);  // they arrive while the FP64 head of the modes is computed
 
     if (tid < 3)  // read after the barriers of the tile loop
         sm.weight[tid] = tid == 0   ? axis_weight(g.nx, g.x0, g.x1, 0)
@@ -931,141 +1102,196 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
                                     : axis_weight(g.nz, g.z0, g.z1, g.mirror_z);
 
     // ---- this thread's momentum mode
-    int ix = 0, iy = 0, iz = 0;
-    if (active) {
-        ix = m % g.nx;
-        iy = (m / g.nx) % g.ny;
-        iz = m / (g.nx * g.ny);
-    }
-    const double px = axis_node(ix, g.nx, g.x0, g.x1);
-    const double py = axis_node(iy, g.ny, g.y0, g.y1);
-    const double pz = axis_node(iz, g.nz, g.z0, g.z1);
-    const double eperp = sqrt(1.0 + pz * pz);
-
     typename P::State st;
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            st.hi[s][q] = q == 0 ? 1 : 0;
-            st.lo[s][q] = 0;
+    {
+        int ix = 0, iy = 0, iz = 0;
+        if (active) {
+            ix = m % g.nx;
+            iy = (m / g.nx) % g.ny;
+            iz = m / (g.nx * g.ny);
         }
-    if constexpr (CarriesState<P>::value) {
-        const double hx = px - Ax[0], hy = py - Ay[0];
-        const Eigen e = eigen(hx, hy, eperp);
-        double v[2][4];
-        eig_neg(e, 0, v[0]);
-        eig_neg(e, 1, v[1]);
-        if constexpr (IsSplit<P>::value) {
-            const auto h = P::half_step(px, py, eperp, dt);
-            P::apply_half(h, 1.0, px, py, eperp, v[0]);
-            P::apply_half(h, 1.0, px, -py, eperp, v[1]);
-        }
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                st.hi[s][q] = v[s][q];
-                st.lo[s][q] = v[s][q] - (double)st.hi[s][q];
+        const double px = axis_node(ix, g.nx, g.x0, g.x1);
+        const double py = axis_node(iy, g.ny, g.y0, g.y1);
+        const double pz = axis_node(iz, g.nz, g.z0, g.z1);
+        const double eperp = sqrt(1.0 + pz * pz);
+        sm.mode[0][tid] = px;
+        sm.mode[1][tid] = py;
+        sm.mode[2][tid] = eperp;
+        if constexpr (CarriesState<P>::value) {
+            const double hx = px - Ax[0], hy = py - Ay[0];
+            const Eigen e = eigen(hx, hy, eperp);
+            double v[2][4];
+            eig_neg(e, 0, v[0]);
+            eig_neg(e, 1, v[1]);
+            if constexpr (IsSplit<P>::value) {
+                const auto h = P::half_step(px, py, eperp, dt);
+                P::apply_half(h, 1.0, px, py, eperp, v[0]);
+                P::apply_half(h, 1.0, px, -py, eperp, v[1]);
             }
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    st.hi[s][q] = v[s][q];
+                    st.lo[s][q] = v[s][q] - (double)st.hi[s][q];
+                }
+        }
+        P::scale(st, px, py, eperp, per * dt);
     }
-    P::scale(st, px, py, eperp, per * dt);
 
     bool timed_out = false;
-    int t_fail = 0;
-    for (int t = 0; t < ntiles; ++t) {
-        const int k = base + t;
-        const int b = k & 1;
-        const uint32_t par = (k >> 1) & 1;
-        bool ok = mbar_wait_bounded(&sm.bar[b], par, wait_limit);
-        ok = __syncthreads_and(ok);
-        if (!ok) {
-            timed_out = true;
-            t_fail = t;
-            break;
+    Real total[kParts];  // the product of the finished segments
+#pragma unroll 1
+    for (int seg = seg0; seg < (work.seg >= 0 ? seg0 + 1 : nseg); ++seg) {
+        const int first = seg * seg_len, count = min(seg_len, nent - first);
+        const int ntiles = (count + TILE - 1) / TILE;
+        if (seg > seg0 && tid == 0 && !skip_copies)
+            issued = fetch_first(seg);
+        const int base = tile_base;
+        tile_base += ntiles;
+        if constexpr (!CarriesState<P>::value) {
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    st.hi[s][q] = q == 0 ? 1 : 0;
+                    st.lo[s][q] = 0;
+                }
         }
-        const int nst = min(TILE, nent - t * TILE);
-        const V *tb = sm.buf[b];
-        if constexpr (Expands<P>::value) {
-            for (int k0 = 0; k0 < nst; k0 += kExpandSpan) {
-                const int m1 = min(kExpandSpan, nst - k0);
-                if (tid < m1) {
-                    // the step's start is the end of the step before it
-                    const int n = t * TILE + k0 + tid;
-                    const double a0x = n ? (k0 + tid ? tb[k0 + tid - 1].z : trow[n - 1].z) : dt * Ax[0];
-                    const double a0y = n ? (k0 + tid ? tb[k0 + tid - 1].w : trow[n - 1].w) : dt * Ay[0];
-                    const V e = tb[k0 + tid];
-                    sm.coef[tid] = P::coef(a0x, a0y, e.x, e.y, e.z, e.w);
-                }
-                __syncthreads();
-                if (active) {
-#pragma unroll 2
-                    for (int kk = 0; kk < m1; ++kk)
-                        P::step(st, sm.coef[kk]);
-                }
-                __syncthreads();  // every thread is done with coef
+
+        int t_fail = 0;
+        for (int t = 0; t < ntiles; ++t) {
+            const int k = base + t;
+            const int b = k & 1;
+            const uint32_t par = (k >> 1) & 1;
+            bool ok = mbar_wait_bounded(&sm.bar[b], par, wait_limit);
+            ok = __syncthreads_and(ok);
+            if (!ok) {
+                timed_out = true;
+                t_fail = t;
+                break;
             }
-        } else if (active) {
-            if constexpr (IsBlock<P>::value) {
-                // the last entry holds the remaining ns % per steps, if any
-                const bool ragged = t == ntiles - 1 && ns % per != 0;
-                const int full = nst - (ragged ? 1 : 0);
-                for (int k0 = 0; k0 < full; k0 += kRescaleSpan) {
-                    const int k1 = min(k0 + kRescaleSpan, full);
+            const int nst = min(TILE, count - t * TILE);
+            const V *tb = sm.buf[b];
+            if constexpr (Expands<P>::value) {
+                for (int k0 = 0; k0 < nst; k0 += kExpandSpan) {
+                    const int m1 = min(kExpandSpan, nst - k0);
+                    if (tid < m1) {
+                        // the step's start is the end of the step before it
+                        const int n = first + t * TILE + k0 + tid;
+                        const double a0x = n ? (k0 + tid ? tb[k0 + tid - 1].z : trow[n - 1].z) : dt * Ax[0];
+                        const double a0y = n ? (k0 + tid ? tb[k0 + tid - 1].w : trow[n - 1].w) : dt * Ay[0];
+                        const V e = tb[k0 + tid];
+                        sm.coef[tid] = P::coef(a0x, a0y, e.x, e.y, e.z, e.w);
+                    }
+                    __syncthreads();
+                    if (active) {
 #pragma unroll 2
-                    for (int kk = k0; kk < k1; ++kk)
-                        P::step(st, tb[kk]);
-                    rescale_state<P::kComp>(st);
+                        for (int kk = 0; kk < m1; ++kk)
+                            P::step(st, sm.coef[kk]);
+                    }
+                    __syncthreads();  // every thread is done with coef
                 }
-                if (ragged) {
-                    P::scale(st, px, py, eperp, (ns % per) * dt);
-                    P::step(st, tb[full]);
-                }
-            } else {
-                bool wide = false;
-                if constexpr (ROLE == REST) {
-                    wide = plan_kind(plan) == kKindWide;
-                    if (wide)
-                        for (int kk = 0; kk < nst; ++kk)
-                            P::step_wide(st, tb[kk]);
-                }
-                // (FP64 Magnus has no series candidates outside its main kernel)
-                if constexpr (ROLE != REST || TracksNorm<P>::value) {
-                    if (!wide) {
+            } else if (active) {
+                if constexpr (IsBlock<P>::value) {
+                    // the last entry holds the remaining ns % per steps, if any
+                    const bool ragged = first + t * TILE + nst == nent && ns % per != 0;
+                    const int full = nst - (ragged ? 1 : 0);
+                    for (int k0 = 0; k0 < full; k0 += kRescaleSpan) {
+                        const int k1 = min(k0 + kRescaleSpan, full);
 #pragma unroll 2
-                        for (int kk = 0; kk < nst; ++kk)
+                        for (int kk = k0; kk < k1; ++kk)
                             P::step(st, tb[kk]);
-                        if constexpr (TracksNorm<P>::value)
-                            rescale_state<P::kComp>(st);
+                        rescale_state<P::kComp>(st);
+                    }
+                    if (ragged) {
+                        P::scale(st, sm.mode[0][tid], sm.mode[1][tid], sm.mode[2][tid], (ns % per) * dt);
+                        P::step(st, tb[full]);
+                    }
+                } else {
+                    bool wide = false;
+                    if constexpr (ROLE == REST) {
+                        wide = plan_kind(plan) == kKindWide;
+                        if (wide)
+                            for (int kk = 0; kk < nst; ++kk)
+                                P::step_wide(st, tb[kk]);
+                    }
+                    // (FP64 Magnus has no series candidates outside its main kernel)
+                    if constexpr (ROLE != REST || TracksNorm<P>::value) {
+                        if (!wide) {
+#pragma unroll 2
+                            for (int kk = 0; kk < nst; ++kk)
+                                P::step(st, tb[kk]);
+                            if constexpr (TracksNorm<P>::value)
+                                rescale_state<P::kComp>(st);
+                        }
                     }
                 }
             }
+            __syncthreads();  // every thread is done with buf[b]
+            if (tid == 0 && !skip_copies && t + 2 < ntiles) {
+                fetch(first, count, base, t + 2);
+                ++issued;
+            }
         }
-        __syncthreads();  // every thread is done with buf[b]
-        if (tid == 0 && !skip_copies && t + 2 < ntiles) {
-            mbar_arrive_expect_tx(&sm.bar[b], TILE * (uint32_t)sizeof(V));
-            bulk_copy_g2s(sm.buf[b], trow + (size_t)(t + 2) * TILE, TILE * (uint32_t)sizeof(V),
-                          &sm.bar[b]);
-            ++issued;
+
+        if (timed_out) {
+            // Drain every copy this CTA issued (bounded) before shared memory is reused or released.
+            if (tid == 0) {
+                pp_flag(status, PP_FLAG_TIMEOUT);
+                // copies t_fail <= t < issued were never consumed: wait for each in order
+                for (int t = t_fail; t < issued; ++t) {
+                    const int k = base + t;
+                    mbar_wait_bounded(&sm.bar[k & 1], (k >> 1) & 1, 1ll << 24);
+                }
+            }
+            __syncthreads();
+            break;
+        }
+        if constexpr (kCuts) {
+            if (work.seg < 0 && nseg > 1)
+                join_segment<P, Real>(st, total, seg == 0);
         }
     }
 
-    if (timed_out) {
-        // Drain every copy this CTA issued (bounded) before shared memory is reused or released.
-        if (tid == 0) {
-            pp_flag(status, PP_FLAG_TIMEOUT);
-            // copies t_fail <= t < issued were never consumed: wait for each in order
-            for (int t = t_fail; t < issued; ++t) {
-                const int k = base + t;
-                mbar_wait_bounded(&sm.bar[k & 1], (k >> 1) & 1, 1ll << 24);
+    if constexpr (kCuts) {
+        if (work.seg >= 0 && nseg > 1) {
+            // this segment's propagator; the last CTA of the item goes on with all of them
+            Real *out = (Real *)work.out + tid;
+            Real cur[kParts];
+            get_state<P>(st, cur);
+            if (timed_out)
+                cur[0] = cur[4] = __longlong_as_double(0x7ff8000000000000ll);
+            if (active)
+#pragma unroll
+                for (int q = 0; q < kParts; ++q)
+                    out[((size_t)work.seg * kParts + q) * THREADS] = cur[q];
+            __threadfence();
+            __syncthreads();
+            if (tid == 0)
+                sm.last = atomicAdd(work.done, 1) == nseg - 1;
+            __syncthreads();
+            const bool last = sm.last;
+            __syncthreads();  // sm.last is read before the next item writes it
+            if (!last)
+                return !timed_out;
+            __threadfence();
+            if (active) {
+                for (int seg = 0; seg < nseg; ++seg) {
+#pragma unroll
+                    for (int q = 0; q < kParts; ++q)
+                        cur[q] = __ldcg(out + ((size_t)seg * kParts + q) * THREADS);
+                    set_state<P>(st, cur);
+                    join_segment<P, Real>(st, total, seg == 0);
+                }
             }
         }
-        __syncthreads();
     }
 
     // ---- FP64 projection of the final states onto the positive-energy states at t_end
     double f = 0.0;
     if (active) {
+        const double px = sm.mode[0][tid], py = sm.mode[1][tid], eperp = sm.mode[2][tid];
         const double Poutx = px - Ax[2 * ns], Pouty = py - Ay[2 * ns];
         double psi[2][4];
 #pragma unroll
@@ -1105,6 +1331,7 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
     }
     double wf = 0.0;
     if (active) {
+        const int ix = m % g.nx, iy = (m / g.nx) % g.ny, iz = m / (g.nx * g.ny);
         const double w = __dmul_rn(__dmul_rn(node_weight(ix, g.nx, sm.weight[0]), node_weight(iy, g.ny, sm.weight[1])),
                                    node_weight(iz, g.nz, sm.weight[2]));
         wf = w * f;

@@ -29,15 +29,17 @@
 
 namespace {
 
-// One CTA per block of modes and candidate (grid (blocks, candidates)); a CTA of a candidate that another launch takes returns at
+// One CTA per block of modes and candidate (grid (blocks, candidates)), and per segment where seg_out is given
+// (grid (blocks, candidates, layers)): room for seg_rows segments per block and candidate, seg_done a count for each.  A CTA of a candidate that another launch takes returns at
 // once.  ROLE: MAIN or SERIES.
 template <class P, int THREADS, int TILE_BYTES, Role ROLE>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, kResidentThreads<RolePolicy<P, ROLE>> / THREADS)
     propagate_kernel(const double *__restrict__ A, int ld, int ns_uniform,
                      const int *__restrict__ ns_array, const typename P::Entry *__restrict__ table,
                      int padded, double dt, pp_grid g, double *__restrict__ n_p,
                      double *__restrict__ partial, long long wait_limit, int skip_copies,
-                     unsigned int *__restrict__ status, const int *__restrict__ plans)
+                     unsigned int *__restrict__ status, const int *__restrict__ plans, void *__restrict__ seg_out,
+                     int *__restrict__ seg_done, int seg_rows)
 {
     using Q = RolePolicy<P, ROLE>;
     __shared__ ItemSmem<Q, THREADS, TILE_BYTES> sm;
@@ -55,10 +57,25 @@ __global__ void __launch_bounds__(THREADS)
     }
     __syncthreads();
     int tiles = 0;
-    process_item<Q, THREADS, TILE_BYTES, ROLE>(
-        sm, blockIdx.x, g, ns, HasPlan<P>::value ? plans[c] : 0,
-        reinterpret_cast<const typename Q::Entry *>(table + (size_t)c * padded), Ax, Ax + ld, dt,
-        n_p ? n_p + (size_t)c * nmodes : nullptr, partial + (size_t)c * ngroups, wait_limit, skip_copies, status, tiles);
+    const int plan = HasPlan<P>::value ? plans[c] : 0;
+    const auto *row = reinterpret_cast<const typename Q::Entry *>(table + (size_t)c * padded);
+    double *n_out = n_p ? n_p + (size_t)c * nmodes : nullptr, *part = partial + (size_t)c * ngroups;
+    SegmentWork work{-1, nullptr, nullptr};
+    if constexpr (Segments<Q>::kCuts) {
+        // one CTA per segment (blockIdx.z)
+        if (seg_out) {
+            const int nent = item_entries<Q>(ns, plan), most = Segments<Q>::most(nmodes, ns);
+            const int len = (nent + most - 1) / most;
+            const size_t item = (size_t)c * gridDim.x + blockIdx.x;
+            using Real = typename std::remove_reference<decltype(Q::State::hi[0][0])>::type;
+            work = SegmentWork{(int)blockIdx.z, (Real *)seg_out + item * seg_rows * (Q::kComp ? 16 : 8) * THREADS,
+                               seg_done + item};
+            if (work.seg * len >= nent)
+                return;
+        }
+    }
+    process_item<Q, THREADS, TILE_BYTES, ROLE>(sm, blockIdx.x, g, ns, plan, row, Ax, Ax + ld, dt, n_out, part, wait_limit,
+                                               skip_copies, status, tiles, work);
 }
 
 // The candidates that the other launches leave: a grid that fills the GPU at most once walks over all items, so that it costs
@@ -133,6 +150,7 @@ struct CallBuffers {
     double *partial;
     int *plans;
     int *ns;
+    bool segments;  // whether segments of the time axis may have CTAs of their own, with scratch for their propagators
 };
 
 // Step counts of a call: the largest, and whether all are equal.
@@ -162,6 +180,33 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
     const int nblk = (nmodes + THREADS - 1) / THREADS;
     const int ngroups = (nmodes + kGroup - 1) / kGroup;
     V *table = (V *)buf.table;
+    using Q = typename MainPolicy<P>::type;
+    // Segments get CTAs of their own while the launch has less than 16 CTAs per SM without them.
+    int layers = buf.segments && (long long)nblk * ncand < 152 * 16 ? Segments<Q>::most(nmodes, sc.max) : 1;
+    void *seg_out = nullptr;
+    int *seg_done = nullptr;
+    int seg_rows = 0, ndone = 0;
+    if (layers > 1) {
+        using Real = typename std::remove_reference<decltype(Q::State::hi[0][0])>::type;
+        seg_rows = layers;
+        ndone = nblk * ncand;
+        const size_t bytes = (size_t)ndone * seg_rows * (Q::kComp ? 16 : 8) * THREADS * sizeof(Real);
+        // without the memory, or with a stream in capture that must not allocate it, each CTA walks all segments, to the
+        // same result
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaStreamIsCapturing(stream, &cap);
+        const size_t need = bytes + ndone * sizeof(int);
+        if ((cap == cudaStreamCaptureStatusNone || pp::scratch_holds(pp::SCR_SEGMENTS, need)) &&
+            pp::scratch(pp::SCR_SEGMENTS, need, &seg_out) == PP_OK) {
+            seg_done = (int *)((char *)seg_out + bytes);
+        } else {
+            cudaGetLastError();
+            pp::clear_error();
+            seg_out = nullptr;
+            layers = 1;
+            ndone = 0;
+        }
+    }
     const int *ns_array = nullptr;
     if (!sc.uniform) {
         cudaError_t e = cudaMemcpyAsync(buf.ns, ns_host, sizeof(int) * ncand, cudaMemcpyHostToDevice, stream);
@@ -171,7 +216,7 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
     }
     if constexpr (IsBlock<typename MainPolicy<P>::type>::value) {
         plan_kernel<P::kComp><<<ncand * kPlanCtas, kPlanThreads, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table,
-                                                                  buf.plans, n_p != nullptr);
+                                                                  buf.plans, n_p != nullptr, seg_done, ndone);
     } else {
         if constexpr (HasPlan<P>::value) {
             cudaError_t e = cudaMemsetAsync(buf.plans, 0, sizeof(int) * ncand, stream);
@@ -179,21 +224,23 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
                 return pp::cuda_fail(e, "plan reset");
         }
         dim3 tg((padded + 255) / 256, ncand);
-        build_table_kernel<P><<<tg, 256, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table, buf.plans);
+        build_table_kernel<P><<<tg, 256, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table, buf.plans, seg_done,
+                                                     ndone);
     }
     dim3 pg(nblk, ncand);
     pp::profile_mark_start(stream);
-    propagate_kernel<P, THREADS, TILE_BYTES, MAIN><<<pg, THREADS, 0, stream>>>(
+    propagate_kernel<P, THREADS, TILE_BYTES, MAIN><<<dim3(nblk, ncand, layers), THREADS, 0, stream>>>(
         A, ld, sc.first, ns_array, table, padded, dt, *grid, n_p, buf.partial, (long long)pp::wait_limit(),
-        pp::skip_copies(), status, buf.plans);
+        pp::skip_copies(), status, buf.plans, seg_out, seg_done, seg_rows);
     if constexpr (HasPlan<P>::value) {
         // single steps are rare (rough potentials) except for the densities of long runs, which get a kernel of their own
         int first_rest = kKindSeries;
         if constexpr (IsBlock<typename MainPolicy<P>::type>::value && !P::kComp) {
             if (n_p && single_steps(sc.max, dt)) {
-                propagate_kernel<P, THREADS, TILE_BYTES, SERIES><<<pg, THREADS, 0, stream>>>(
+                // (CTAs of 256 threads: 131 ms where 128-thread CTAs take 140, 4 pulses on 128 x 128 x 64 modes, 20000 steps)
+                propagate_kernel<P, 256, 8192, SERIES><<<dim3((nmodes + 255) / 256, ncand), 256, 0, stream>>>(
                     A, ld, sc.first, ns_array, table, padded, dt, *grid, n_p, buf.partial,
-                    (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans);
+                    (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans, nullptr, nullptr, 0);
                 first_rest = kKindWide;
             }
         }
@@ -234,6 +281,7 @@ int run(const double *A, int ncand, int ld, const int32_t *ns_host, double dt, c
     buf.partial = (double *)partial;
     buf.plans = (int *)(((uintptr_t)(buf.partial + (size_t)ncand * ngroups) + 255) & ~(uintptr_t)255);
     buf.ns = (int *)(((uintptr_t)(buf.plans + ncand) + 255) & ~(uintptr_t)255);
+    buf.segments = true;
     return launch<P, THREADS, TILE_BYTES>(buf, sc, padded, A, ncand, ld, ns_host, dt, grid, N, n_p, stream);
 }
 
@@ -292,7 +340,7 @@ int run_static(const double *A, int ncand, int ld, const int32_t *ns_host, doubl
     if (!base)
         return pp::fail(PP_ERR_CUDA, "cudaGetSymbolAddress of the static scratch failed");
     const CallBuffers buf{base, (double *)(base + table_bytes), (int *)(base + table_bytes + part_bytes),
-                          (int *)(base + table_bytes + part_bytes + plan_bytes)};
+                          (int *)(base + table_bytes + part_bytes + plan_bytes), false};
     return launch<P, THREADS, TILE_BYTES>(buf, sc, padded, A, ncand, ld, ns_host, dt, grid, N, n_p, stream);
 }
 
@@ -361,7 +409,7 @@ const PolicySlot &policy_slot(int precision, int scheme)
     static const PolicySlot slots[3][3] = {
         {{d_rk4.run_fn, d_rk4.static_fn, true, 1}, {d_mag.run_fn, d_mag.static_fn, false, 0},
          {d_spl.run_fn, d_spl.static_fn, false, 0}},
-        {{f_rk4.run_fn, f_rk4.static_fn, true, 4}, {f_mag.run_fn, f_mag.static_fn, true, 1},
+        {{f_rk4.run_fn, f_rk4.static_fn, true, 1}, {f_mag.run_fn, f_mag.static_fn, true, 1},
          {f_spl.run_fn, f_spl.static_fn, true, 0}},
         {{x_rk4.run_fn, x_rk4.static_fn, true, 1}, {x_mag.run_fn, x_mag.static_fn, true, 1},
          {x_spl.run_fn, x_spl.static_fn, true, 0}},
@@ -401,7 +449,13 @@ int chosen_config(int precision, int scheme, int ncand, int ld, const int32_t *n
         return 0;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tuned.find(make_key(precision, scheme, ncand, ld, ns, g));
-    return it == g_tuned.end() ? slot.default_cfg : it->second;
+    if (it != g_tuned.end())
+        return it->second;
+    // FP32 RK4 on few modes is bound by each warp's chain, which a tile's end holds up: tiles of 1024 steps
+    // instead of 256 (8 pulses on 600 modes, 800 steps: 80 us instead of 92), where CTAs would not share an SM's memory
+    if (precision != PP_FP64 && scheme == PP_RK4 && (long long)ncand * g->nx * g->ny * g->nz <= 152 * 3 * 128)
+        return 4;
+    return slot.default_cfg;
 }
 
 }  // namespace
