@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(THREADS, kResidentThreads<RolePolicy<P, ROLE>>
         }
         const BatchCand d = cands[w.x];
         const double *Ax = A + (size_t)w.x * 2 * ld;
-        if (!process_item<Q, THREADS, TILE_BYTES, ROLE>(
+        if (!process_item<Q, THREADS, TILE_BYTES, ROLE, std::is_same<Q, MagnusBlockPolicy<false>>::value>(
                 sm, w.y, d.g, d.ns, HasPlan<P>::value ? plans[w.x] : 0,
                 reinterpret_cast<const typename Q::Entry *>(table + d.table_off), Ax, Ax + ld, dt,
                 n_p ? n_p + d.n_off : nullptr, partial + d.part_off, wait_limit, skip_copies, status, tiles))

@@ -45,6 +45,27 @@ __device__ __forceinline__ double axis_node(int i, int n, double a, double b)
     return __dadd_rn(a, __ddiv_rn(__dmul_rn(__dsub_rn(b, a), (double)i), (double)(n - 1)));
 }
 
+// The nodes of a grid's axes: p_x [nx], p_y [ny], eps_perp [nz], written once per call by the table's kernel (thread
+// `at` of `all`).  The three FP64 divisions and the root per mode were a third of the FP64 work around the steps.
+__host__ __device__ inline int node_count(const pp_grid &g) { return g.nx + g.ny + g.nz; }
+__device__ __forceinline__ void fill_nodes(double *__restrict__ nodes, const pp_grid &g, int at, int all)
+{
+    if (!nodes)
+        return;
+    for (int i = at; i < g.nx + g.ny + g.nz; i += all) {
+        double v;
+        if (i < g.nx) {
+            v = axis_node(i, g.nx, g.x0, g.x1);
+        } else if (i < g.nx + g.ny) {
+            v = axis_node(i - g.nx, g.ny, g.y0, g.y1);
+        } else {
+            const double pz = axis_node(i - g.nx - g.ny, g.nz, g.z0, g.z1);
+            v = sqrt(1.0 + pz * pz);
+        }
+        nodes[i] = v;
+    }
+}
+
 // Trapezoid weight of an interior node.
 __device__ __forceinline__ double axis_weight(int n, double a, double b, int mirror)
 {
@@ -118,7 +139,7 @@ __device__ __forceinline__ void apply_su2(const double z[4], const Eigen &e, int
 //     g = (1 - M/6) u + (1/6 - M/12) c + (1/6 - M/24) d x u - (M/48) (d x c)_z z.
 // The first two terms of g keep their form under the reflection y -> -y that takes spin channel s = +1 to
 // s = -1 and the last two change sign, so everything but g's last additions is formed once for both channels.
-// 30 multiply-adds to form the step and 16 per channel to apply it, 62 in all, where the four stages applied to
+// 29 operations to form the step and 16 per channel to apply it, 61 in all, where the four stages applied to
 // the state took 148 (FP64) and 184 (compensated FP32).  The path is bound by the FP64 / FP32 lanes, so the time
 // follows: 2 pulses on 64 x 64 x 32 modes, 8192 steps in FP64 576.6 -> 241.1 ms; 32 x 32 x 16 modes, 4000 steps
 // 40.3 -> 16.9 ms; in compensated FP32, 8 pulses on 600 modes, 800 steps 208 -> 132 us (whole calls).
@@ -131,7 +152,7 @@ template <typename T, bool COMP>
 struct Rk4Policy {
     static constexpr bool kComp = COMP;
     struct alignas(sizeof(T) * 8) Coef {
-        T ax, ay, cx, cy, dx, dy, q, p;  // p = (d x c)_z / 48
+        T ax, ay, cx, cy, dx, dy, q, p;  // q: here q / 24 - 1/2; p = (d x c)_z / 48
     };
     static constexpr bool kExpands = sizeof(T) == 8;
     using Entry = typename std::conditional<kExpands, dbl4, Coef>::type;
@@ -148,7 +169,7 @@ struct Rk4Policy {
         e.cy = (T)cy;
         e.dx = (T)dx;
         e.dy = (T)dy;
-        e.q = (T)(0.25 * (fma(cx, cx, cy * cy) - fma(dx, dx, dy * dy)));
+        e.q = (T)(0.25 / 24.0 * (fma(cx, cx, cy * cy) - fma(dx, dx, dy * dy)) - 0.5);
         e.p = (T)((dx * cy - dy * cx) / 48.0);
         return e;
     }
@@ -192,8 +213,8 @@ struct Rk4Policy {
         const T Ez = fma(st.uz, e1, st.lz);
         const T kz = k * st.uz;
         const T Oz = fma(k, fma(e.dx, uy, -e.dy * ux), -M * e.p);
-        const T am1 = fma(M, fma((M + Y) + e.q, (T)(1.0 / 24.0), (T)-0.5), Y * (T)(-1.0 / 6.0));
-        const T al = (T)1 + am1;
+        const T r = fma(M + Y, (T)(1.0 / 24.0), e.q);
+        const T am1 = fma(M, r, Y * (T)(-1.0 / 6.0)), al = fma(M, r, fma(Y, (T)(-1.0 / 6.0), (T)1));  // one of the two is used
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const T gx = s ? fma(-e.dy, kz, Ex) : fma(e.dy, kz, Ex);
@@ -761,11 +782,14 @@ template <class P>
 __global__ void build_table_kernel(const double *__restrict__ A, int ld, int ns_uniform,
                                    const int *__restrict__ ns_array, int padded, double dt,
                                    pp_grid g, typename P::Entry *__restrict__ table,
-                                   int *__restrict__ plans, int *__restrict__ done, int ndone)
+                                   int *__restrict__ plans, int *__restrict__ done, int ndone,
+                                   double *__restrict__ nodes)
 {
     const int c = blockIdx.y;
-    clear_counts(done, ndone, (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x,
-                 gridDim.x * gridDim.y * blockDim.x);
+    const int at = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x,
+              all = gridDim.x * gridDim.y * blockDim.x;
+    clear_counts(done, ndone, at, all);
+    fill_nodes(nodes, g, at, all);
     const double *Ax = A + (size_t)c * 2 * ld;
     table_row<P>(Ax, Ax + ld, blockIdx.x * blockDim.x + threadIdx.x, ns_array ? ns_array[c] : ns_uniform, padded, dt, g,
                  table + (size_t)c * padded, plans + c);
@@ -854,10 +878,13 @@ template <bool COMP>
 __global__ void __cluster_dims__(kPlanCtas, 1, 1) __launch_bounds__(kPlanThreads)
     plan_kernel(const double *__restrict__ A, int ld, int ns_uniform, const int *__restrict__ ns_array, int padded,
                 double dt, pp_grid g, typename MagnusPolicy<float, COMP>::Entry *__restrict__ table,
-                int *__restrict__ plans, bool densities, int *__restrict__ done, int ndone)
+                int *__restrict__ plans, bool densities, int *__restrict__ done, int ndone,
+                double *__restrict__ nodes)
 {
     const int c = blockIdx.x / kPlanCtas;
-    clear_counts(done, ndone, blockIdx.x * kPlanThreads + threadIdx.x, gridDim.x * kPlanThreads);
+    const int at = blockIdx.x * kPlanThreads + threadIdx.x, all = gridDim.x * kPlanThreads;
+    clear_counts(done, ndone, at, all);
+    fill_nodes(nodes, g, at, all);
     const double *Ax = A + (size_t)c * 2 * ld;
     plan_and_table<COMP>(Ax, Ax + ld, ns_array ? ns_array[c] : ns_uniform, dt, g, table + (size_t)c * padded, plans + c,
                          densities);
@@ -886,18 +913,18 @@ using RolePolicy = typename std::conditional<ROLE == MAIN, typename MainPolicy<P
 // grid and the number of steps alone, and the product is formed in the same order whether one CTA walks all segments or
 // CTAs of their own do (process_item), so results do not depend on which.
 // kSegTarget modes times segments are 16 CTAs of 128 threads per SM, so that the last wave weighs little.  A segment
-// repeats the FP64 head of a mode and the product (about 200 FP64 instructions) and stays long against that: 256
-// steps in FP64 (16000 instructions), 512 in FP32 RK4 and 1024 in blocks of steps.  One pulse of 8000 steps on 189 modes: FP64
-// 16.9 -> 0.77 ms, compensated RK4 566 -> 126 us, blocks 125 -> 65 us; 4000 FP64 steps on 32 x 32 x 16 modes 8.47 -> 7.38 ms; 2
-// pulses on 64 x 64 x 32 modes in FP64 241 -> 233 ms.
+// repeats the head of a mode and the product on the last CTA, so it stays long against those: 64 steps in FP64 (4000
+// FP64 instructions against 200; a CTA's warps share one FP64 pipe, so CTAs are what counts), 256 in FP32 RK4 and
+// 1024 in blocks of steps (256 and 512 took 0 to 10% longer on grids of 4000 modes and up).  One pulse of 8000 steps on 189
+// modes: FP64 16.9 -> 0.37 ms, compensated RK4 566 -> 70 us, blocks 125 -> 65 us; 4000 FP64 steps on 32 x 32 x 16 modes 8.47
+// -> 7.16 ms; 2 pulses on 64 x 64 x 32 modes in FP64 241 -> 233 ms.  (Both at 62 operations a step; 6.90 and 224 ms at 61.)
 constexpr int kSegTarget = 152 * 2048;
-constexpr int kMaxSegs = 24;
 template <class P>
 struct Segments {
     static constexpr bool kCuts = !CarriesState<P>::value;
-    static constexpr int kLeast =
-        IsBlock<P>::value ? 1024
-                          : (sizeof(typename std::remove_reference<decltype(P::State::hi[0][0])>::type) == 8 ? 256 : 512);
+    static constexpr bool kFp64 = sizeof(typename std::remove_reference<decltype(P::State::hi[0][0])>::type) == 8;
+    static constexpr int kLeast = kFp64 ? 64 : (IsBlock<P>::value ? 1024 : 256);
+    static constexpr int kMost = kFp64 ? 76 : 32;
     // most segments of ns steps on a grid
     __host__ __device__ static int most(int nmodes, int ns)
     {
@@ -905,13 +932,28 @@ struct Segments {
             return 1;
         int k = kSegTarget / nmodes;
         k = k < ns / kLeast ? k : ns / kLeast;
-        k = k < kMaxSegs ? k : kMaxSegs;
+        k = k < kMost ? k : kMost;
         return k < 1 ? 1 : k;
     }
 };
 
+// Two-float sums and products (Dekker 1971, Knuth; the product's low part by a fused multiply-add).
+struct Pair {
+    float h, l;
+};
+__device__ __forceinline__ Pair pair_fma(Pair a, Pair b, Pair c)  // a b + c
+{
+    const float p = a.h * b.h;
+    const float e = fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)));
+    const float s = p + c.h, v = s - p;
+    const float t = ((p - (s - v)) + (c.h - v)) + (e + c.l);
+    const float h = s + t;
+    return Pair{h, t - (h - s)};
+}
+__device__ __forceinline__ Pair operator-(Pair a) { return Pair{-a.h, -a.l}; }
+
 // tot <- cur tot for the two channels' propagators (first columns; COMP: hi, then lo), not inlined: it runs once per
-// segment.
+// segment.  Compensated states are multiplied as two-floats: in FP64 the products of 15 segments on the last CTA's SM took 37 us.
 template <typename T, bool COMP>
 __device__ __noinline__ void fold_segment(const T *cur, T *tot)
 {
@@ -920,18 +962,20 @@ __device__ __noinline__ void fold_segment(const T *cur, T *tot)
         const T *z = cur + 4 * s;
         T *t = tot + 4 * s;
         if constexpr (COMP) {
-            double a[4], b[4];
+            Pair a[4], b[4];
             for (int q = 0; q < 4; ++q) {
-                a[q] = (double)z[q] + (double)z[q + 8];
-                b[q] = (double)t[q] + (double)t[q + 8];
+                a[q] = Pair{z[q], z[q + 8]};
+                b[q] = Pair{t[q], t[q + 8]};
             }
-            const double r[4] = {fma(a[0], b[0], fma(-a[1], b[1], fma(-a[2], b[2], -a[3] * b[3]))),
-                                 fma(a[0], b[1], fma(a[1], b[0], fma(-a[2], b[3], a[3] * b[2]))),
-                                 fma(a[2], b[0], fma(-a[3], b[1], fma(a[0], b[2], a[1] * b[3]))),
-                                 fma(a[2], b[1], fma(a[3], b[0], fma(a[0], b[3], -a[1] * b[2])))};
+            const Pair o{0.0f, 0.0f};
+            const Pair r[4] = {
+                pair_fma(a[0], b[0], pair_fma(-a[1], b[1], pair_fma(-a[2], b[2], pair_fma(-a[3], b[3], o)))),
+                pair_fma(a[0], b[1], pair_fma(a[1], b[0], pair_fma(-a[2], b[3], pair_fma(a[3], b[2], o)))),
+                pair_fma(a[2], b[0], pair_fma(-a[3], b[1], pair_fma(a[0], b[2], pair_fma(a[1], b[3], o)))),
+                pair_fma(a[2], b[1], pair_fma(a[3], b[0], pair_fma(a[0], b[3], pair_fma(-a[1], b[2], o))))};
             for (int q = 0; q < 4; ++q) {
-                t[q] = (T)r[q];
-                t[q + 8] = (T)(r[q] - (double)t[q]);
+                t[q] = r[q].h;
+                t[q + 8] = r[q].l;
             }
         } else {
             const T r[4] = {fma(z[0], t[0], fma(-z[1], t[1], fma(-z[2], t[2], -z[3] * t[3]))),
@@ -1044,15 +1088,66 @@ struct ItemSmem {
 // norm stays below 1e38.
 constexpr int kRescaleSpan = 32;
 
+// f(p) of one mode from its final state or propagator v (two channels of four components), in FP64.
+template <class P>
+__device__ __forceinline__ double finish_mode(const double *v, double px, double py, double eperp, const double *__restrict__ Ax,
+                                           const double *__restrict__ Ay, int ns, double dt)
+{
+    // (first: with this difference at its use the split operator's loop is allocated 10% slower)
+    const double outx = px - Ax[2 * ns], outy = py - Ay[2 * ns];
+    double psi[2][4];
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            psi[s][q] = v[4 * s + q];
+    if constexpr (!CarriesState<P>::value) {
+        const double hx = px - Ax[0], hy = py - Ay[0];
+        const Eigen e = eigen(hx, hy, eperp);
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const double z[4] = {psi[s][0], psi[s][1], psi[s][2], psi[s][3]};
+            apply_su2(z, e, s, psi[s]);
+        }
+    }
+    if constexpr (IsSplit<P>::value) {
+        const auto h = P::half_step(px, py, eperp, dt);
+        P::apply_half(h, -1.0, px, py, eperp, psi[0]);
+        P::apply_half(h, -1.0, px, -py, eperp, psi[1]);
+    }
+    const Eigen e = eigen(outx, outy, eperp);
+    const double f0 = proj_pos2(e, 0, psi[0]), f1 = proj_pos2(e, 1, psi[1]);
+    if constexpr (TracksNorm<P>::value) {  // the states' norms grew
+        double n[2];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+            n[s] = fma(psi[s][0], psi[s][0], fma(psi[s][1], psi[s][1], fma(psi[s][2], psi[s][2], psi[s][3] * psi[s][3])));
+        return fma(f0, n[1], f1 * n[0]) / (n[0] * n[1]);
+    } else {
+        return f0 + f1;
+    }
+}
+
+// ... as a call.  In the persistent kernel of uncompensated blocks the compiler's allocation for the loop over the steps is better with
+// the projection out of sight (66.9 instead of 70.3 ms for 128 uneven pulses); elsewhere it is worse (2 to 5%).
+template <class P>
+__device__ __noinline__ double finish_mode_call(const double *v, double px, double py, double eperp,
+                                                const double *__restrict__ Ax, const double *__restrict__ Ay, int ns,
+                                                double dt)
+{
+    return finish_mode<P>(v, px, py, eperp, Ax, Ay, ns, dt);
+}
+
 // One work item: the modes [blk * THREADS, (blk + 1) * THREADS) of one candidate with ns steps (P: the policy
 // that runs, plan: the candidate's where it has one).  Each spin channel carries its state, or the first column of
 // its propagator (an SU(2) element or a multiple of one), which is applied to the initial
 // state in FP64 at the end.  The caller owns the shared-memory buffers and the two mbarriers; tile_base
 // is the number of tiles this CTA has consumed before (the barrier phases run
 // on across items) and is moved on.  Returns false if a bounded wait gave up.
-// work.seg < 0: all segments.  Otherwise one segment: its propagator goes to work.out, and the CTA that finishes the item's
+// nodes: see fill_nodes (nullptr: they are computed here).  work.seg < 0: all segments.  Otherwise one segment: its propagator goes to work.out, and the CTA that finishes the item's
 // last segment multiplies them and does the rest.
-template <class P, int THREADS, int TILE_BYTES, Role ROLE>
+// CALL: see finish_mode_call.
+template <class P, int THREADS, int TILE_BYTES, Role ROLE, bool CALL = false>
 __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &sm, int blk,
                                              const pp_grid &g, int ns, int plan,
                                              const typename P::Entry *__restrict__ trow,
@@ -1061,7 +1156,8 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
                                              double *__restrict__ n_out,
                                              double *__restrict__ part_out, long long wait_limit,
                                              int skip_copies, unsigned int *__restrict__ status,
-                                             int &tile_base, SegmentWork work = SegmentWork{-1, nullptr, nullptr})
+                                             int &tile_base, const double *__restrict__ nodes = nullptr,
+                                             SegmentWork work = SegmentWork{-1, nullptr, nullptr})
 {
     using V = typename P::Entry;
     using Real = typename std::remove_reference<decltype(P::State::hi[0][0])>::type;
@@ -1110,10 +1206,17 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
             iy = (m / g.nx) % g.ny;
             iz = m / (g.nx * g.ny);
         }
-        const double px = axis_node(ix, g.nx, g.x0, g.x1);
-        const double py = axis_node(iy, g.ny, g.y0, g.y1);
-        const double pz = axis_node(iz, g.nz, g.z0, g.z1);
-        const double eperp = sqrt(1.0 + pz * pz);
+        double px, py, eperp;
+        if (nodes) {
+            px = nodes[ix];
+            py = nodes[g.nx + iy];
+            eperp = nodes[g.nx + g.ny + iz];
+        } else {
+            px = axis_node(ix, g.nx, g.x0, g.x1);
+            py = axis_node(iy, g.ny, g.y0, g.y1);
+            const double pz = axis_node(iz, g.nz, g.z0, g.z1);
+            eperp = sqrt(1.0 + pz * pz);
+        }
         sm.mode[0][tid] = px;
         sm.mode[1][tid] = py;
         sm.mode[2][tid] = eperp;
@@ -1291,39 +1394,16 @@ __device__ __forceinline__ bool process_item(ItemSmem<P, THREADS, TILE_BYTES> &s
     // ---- FP64 projection of the final states onto the positive-energy states at t_end
     double f = 0.0;
     if (active) {
-        const double px = sm.mode[0][tid], py = sm.mode[1][tid], eperp = sm.mode[2][tid];
-        const double Poutx = px - Ax[2 * ns], Pouty = py - Ay[2 * ns];
-        double psi[2][4];
+        double v[8];
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                psi[s][q] = P::kComp ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
-        if constexpr (!CarriesState<P>::value) {
-            const double hx = px - Ax[0], hy = py - Ay[0];
-            const Eigen e = eigen(hx, hy, eperp);
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const double z[4] = {psi[s][0], psi[s][1], psi[s][2], psi[s][3]};
-                apply_su2(z, e, s, psi[s]);
-            }
-        }
-        if constexpr (IsSplit<P>::value) {
-            const auto h = P::half_step(px, py, eperp, dt);
-            P::apply_half(h, -1.0, px, py, eperp, psi[0]);
-            P::apply_half(h, -1.0, px, -py, eperp, psi[1]);
-        }
-        const Eigen e = eigen(Poutx, Pouty, eperp);
-        const double f0 = proj_pos2(e, 0, psi[0]), f1 = proj_pos2(e, 1, psi[1]);
-        if constexpr (TracksNorm<P>::value) {  // the states' norms grew
-            double n[2];
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-                n[s] = fma(psi[s][0], psi[s][0], fma(psi[s][1], psi[s][1], fma(psi[s][2], psi[s][2], psi[s][3] * psi[s][3])));
-            f = fma(f0, n[1], f1 * n[0]) / (n[0] * n[1]);
-        } else {
-            f = f0 + f1;
-        }
+                v[4 * s + q] = P::kComp ? (double)st.hi[s][q] + (double)st.lo[s][q] : (double)st.hi[s][q];
+        if constexpr (CALL)
+            f = finish_mode_call<P>(v, sm.mode[0][tid], sm.mode[1][tid], sm.mode[2][tid], Ax, Ay, ns, dt);
+        else
+            f = finish_mode<P>(v, sm.mode[0][tid], sm.mode[1][tid], sm.mode[2][tid], Ax, Ay, ns, dt);
         if (timed_out)
             f = __longlong_as_double(0x7ff8000000000000ll);
         if (n_out)

@@ -38,8 +38,9 @@ __global__ void __launch_bounds__(THREADS, kResidentThreads<RolePolicy<P, ROLE>>
                      const int *__restrict__ ns_array, const typename P::Entry *__restrict__ table,
                      int padded, double dt, pp_grid g, double *__restrict__ n_p,
                      double *__restrict__ partial, long long wait_limit, int skip_copies,
-                     unsigned int *__restrict__ status, const int *__restrict__ plans, void *__restrict__ seg_out,
-                     int *__restrict__ seg_done, int seg_rows)
+                     unsigned int *__restrict__ status, const int *__restrict__ plans,
+                     const double *__restrict__ nodes, void *__restrict__ seg_out, int *__restrict__ seg_done,
+                     int seg_rows)
 {
     using Q = RolePolicy<P, ROLE>;
     __shared__ ItemSmem<Q, THREADS, TILE_BYTES> sm;
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(THREADS, kResidentThreads<RolePolicy<P, ROLE>>
         }
     }
     process_item<Q, THREADS, TILE_BYTES, ROLE>(sm, blockIdx.x, g, ns, plan, row, Ax, Ax + ld, dt, n_out, part, wait_limit,
-                                               skip_copies, status, tiles, work);
+                                               skip_copies, status, tiles, nodes, work);
 }
 
 // The candidates that the other launches leave: a grid that fills the GPU at most once walks over all items, so that it costs
@@ -86,7 +87,8 @@ __global__ void __launch_bounds__(THREADS)
                           const int *__restrict__ ns_array, const typename P::Entry *__restrict__ table,
                           int padded, double dt, pp_grid g, int ncand, double *__restrict__ n_p,
                           double *__restrict__ partial, long long wait_limit, int skip_copies,
-                          unsigned int *__restrict__ status, const int *__restrict__ plans, int first_rest)
+                          unsigned int *__restrict__ status, const int *__restrict__ plans,
+                          const double *__restrict__ nodes, int first_rest)
 {
     __shared__ ItemSmem<P, THREADS, TILE_BYTES> sm;
     const int nmodes = g.nx * g.ny * g.nz;
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(THREADS)
             if (!process_item<P, THREADS, TILE_BYTES, REST>(
                     sm, blk, g, ns, plans[c], table + (size_t)c * padded, Ax, Ax + ld, dt,
                     n_p ? n_p + (size_t)c * nmodes : nullptr, partial + (size_t)c * ngroups, wait_limit, skip_copies,
-                    status, tiles))
+                    status, tiles, nodes))
                 return;  // barrier phases are unknown after a wait gave up: this CTA stops
     }
 }
@@ -143,13 +145,15 @@ __global__ void finalize_kernel(const double *__restrict__ partial, int nblk, do
     }
 }
 
-// A call's device buffers: the step table, the partial sums, the plans (one int per candidate) and, for uneven step
-// counts, room for a copy of n_steps.
+// A call's device buffers: the step table, the partial sums, the plans (one int per candidate), for uneven step
+// counts room for a copy of n_steps, and the nodes of the grid up to kMaxNodes of them.
+constexpr int kMaxNodes = 8192;
 struct CallBuffers {
     void *table;
     double *partial;
     int *plans;
     int *ns;
+    double *nodes;  // room for the grid's nodes (fill_nodes), or nullptr
     bool segments;  // whether segments of the time axis may have CTAs of their own, with scratch for their propagators
 };
 
@@ -216,7 +220,7 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
     }
     if constexpr (IsBlock<typename MainPolicy<P>::type>::value) {
         plan_kernel<P::kComp><<<ncand * kPlanCtas, kPlanThreads, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table,
-                                                                  buf.plans, n_p != nullptr, seg_done, ndone);
+                                                                  buf.plans, n_p != nullptr, seg_done, ndone, buf.nodes);
     } else {
         if constexpr (HasPlan<P>::value) {
             cudaError_t e = cudaMemsetAsync(buf.plans, 0, sizeof(int) * ncand, stream);
@@ -225,13 +229,13 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
         }
         dim3 tg((padded + 255) / 256, ncand);
         build_table_kernel<P><<<tg, 256, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table, buf.plans, seg_done,
-                                                     ndone);
+                                                     ndone, buf.nodes);
     }
     dim3 pg(nblk, ncand);
     pp::profile_mark_start(stream);
     propagate_kernel<P, THREADS, TILE_BYTES, MAIN><<<dim3(nblk, ncand, layers), THREADS, 0, stream>>>(
         A, ld, sc.first, ns_array, table, padded, dt, *grid, n_p, buf.partial, (long long)pp::wait_limit(),
-        pp::skip_copies(), status, buf.plans, seg_out, seg_done, seg_rows);
+        pp::skip_copies(), status, buf.plans, buf.nodes, seg_out, seg_done, seg_rows);
     if constexpr (HasPlan<P>::value) {
         // single steps are rare (rough potentials) except for the densities of long runs, which get a kernel of their own
         int first_rest = kKindSeries;
@@ -240,7 +244,8 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
                 // (CTAs of 256 threads: 131 ms where 128-thread CTAs take 140, 4 pulses on 128 x 128 x 64 modes, 20000 steps)
                 propagate_kernel<P, 256, 8192, SERIES><<<dim3((nmodes + 255) / 256, ncand), 256, 0, stream>>>(
                     A, ld, sc.first, ns_array, table, padded, dt, *grid, n_p, buf.partial,
-                    (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans, nullptr, nullptr, 0);
+                    (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans, buf.nodes, nullptr, nullptr,
+                    0);
                 first_rest = kKindWide;
             }
         }
@@ -249,7 +254,7 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
         propagate_rest_kernel<P, THREADS, TILE_BYTES>
             <<<(int)(items < kRestCtas ? items : kRestCtas), THREADS, 0, stream>>>(
                 A, ld, sc.first, ns_array, table, padded, dt, *grid, ncand, n_p, buf.partial,
-                (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans, first_rest);
+                (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans, buf.nodes, first_rest);
     }
     pp::profile_mark_stop(stream);
     finalize_kernel<<<ncand, 256, 0, stream>>>(buf.partial, ngroups, N, status);
@@ -273,14 +278,17 @@ int run(const double *A, int ncand, int ld, const int32_t *ns_host, double dt, c
     int rc = pp::scratch(pp::SCR_TABLE, (size_t)ncand * padded * sizeof(V), &buf.table);
     if (rc)
         return rc;
-    rc = pp::scratch(pp::SCR_PARTIAL, (size_t)ncand * ngroups * sizeof(double) + 512 * sizeof(int) +
-                                          2 * (size_t)ncand * sizeof(int),
+    rc = pp::scratch(pp::SCR_PARTIAL, (size_t)ncand * ngroups * sizeof(double) + 1024 * sizeof(int) +
+                                          2 * (size_t)ncand * sizeof(int) + kMaxNodes * sizeof(double),
                      &partial);
     if (rc)
         return rc;
     buf.partial = (double *)partial;
     buf.plans = (int *)(((uintptr_t)(buf.partial + (size_t)ncand * ngroups) + 255) & ~(uintptr_t)255);
     buf.ns = (int *)(((uintptr_t)(buf.plans + ncand) + 255) & ~(uintptr_t)255);
+    buf.nodes = node_count(*grid) <= kMaxNodes
+                    ? (double *)(((uintptr_t)(buf.ns + ncand) + 255) & ~(uintptr_t)255)
+                    : nullptr;
     buf.segments = true;
     return launch<P, THREADS, TILE_BYTES>(buf, sc, padded, A, ncand, ld, ns_host, dt, grid, N, n_p, stream);
 }
@@ -289,8 +297,8 @@ int run(const double *A, int ncand, int ld, const int32_t *ns_host, double dt, c
 // Scratch of pp_pair_number_static: a fixed device array in this file, held by
 // every GPU that loads the library until the process exits.  It holds, in
 // order, the step table, the per-block partial sums, the per-candidate
-// plans and (for uneven step
-// counts) a copy of n_steps; each call writes every byte it later reads, and
+// plans, (for uneven step
+// counts) a copy of n_steps and the grid's nodes; each call writes every byte it later reads, and
 // calls that overlap on the GPU race on it.
 constexpr size_t kStaticScratchBytes = (size_t)16 << 20;
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
@@ -339,8 +347,11 @@ int run_static(const double *A, int ncand, int ld, const int32_t *ns_host, doubl
     unsigned char *base = static_scratch_address();
     if (!base)
         return pp::fail(PP_ERR_CUDA, "cudaGetSymbolAddress of the static scratch failed");
+    // the nodes where there is room for them: without, they are computed by each mode, to the same values
+    const bool room = node_count(*grid) <= kMaxNodes && need + node_count(*grid) * sizeof(double) <= kStaticScratchBytes;
     const CallBuffers buf{base, (double *)(base + table_bytes), (int *)(base + table_bytes + part_bytes),
-                          (int *)(base + table_bytes + part_bytes + plan_bytes), false};
+                          (int *)(base + table_bytes + part_bytes + plan_bytes), room ? (double *)(base + need) : nullptr,
+                          false};
     return launch<P, THREADS, TILE_BYTES>(buf, sc, padded, A, ncand, ld, ns_host, dt, grid, N, n_p, stream);
 }
 
