@@ -41,122 +41,190 @@ __device__ __forceinline__ size_t packed_off(int r, int c, int cols_pad)
            (r % 8) * 8 + (c % 8);
 }
 
-// Z (B x H) += bias; A = gelu(Z); Ap = packed BF16 of A.  Rows >= nvalid are zeroed.
-__global__ void bias_gelu_pack_kernel(float *__restrict__ Z, const float *__restrict__ bias, int B, int H,
-                                      int nvalid, float *__restrict__ A, uint16_t *__restrict__ Ap)
+// The passes between the products work on 32 x 32 tiles: a CTA reads a tile once, a row per warp,
+// and from shared memory writes it both packed and packed transposed (a product wants its operands
+// along the index that is summed, and the weight gradients sum over rows), and sums its columns.
+// Packed, eight elements of a row are 16 bytes and eight such rows 128 bytes, so every store is a
+// full line.  At 256 rows these passes and the products are launches of 3 to 8 us that hardly fill
+// the chip: what counts is their number, and that no thread walks down all rows.  Loss and gradient
+// of 256 rows, 32 -> 256 -> 256 -> 256 -> 1: 209 us in 34 launches, of which 79 us of column sums by
+// one thread per column -> 119 us in 19 launches.  (256 threads of 4 elements: the same.)
+constexpr int kSide = 32;
+constexpr int kTileThreads = kSide * kSide;
+using Tile = float[kSide][kSide + 1];
+
+// Rows r0 .., columns c0 .. of a matrix: P packed with cols_pad columns, PT its transpose packed
+// with rows_pad columns; either may be NULL.  Warps 0 .. 3 write the one, 4 .. 7 the other.
+__device__ __forceinline__ void store_packed(const Tile &s, int r0, int c0, int rows_pad, int cols_pad, uint16_t *P,
+                                             uint16_t *PT)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)B * H)
+    constexpr int kRuns = kSide * kSide / 8;
+    const bool trans = threadIdx.x >= kRuns;
+    uint16_t *out = trans ? PT : P;
+    if (!out || threadIdx.x >= 2 * kRuns)
         return;
-    const int r = (int)(i / H), c = (int)(i % H);
-    float z = Z[i] + bias[c];
-    float a = gelu(z);
-    if (r >= nvalid) {
-        z = 0.0f;
-        a = 0.0f;
+    const int i = threadIdx.x % kRuns, line = i / 4, run = i % 4 * 8;
+    uint32_t w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float a = trans ? s[run + 2 * j][line] : s[line][run + 2 * j];
+        const float b = trans ? s[run + 2 * j + 1][line] : s[line][run + 2 * j + 1];
+        w[j] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
+               (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16;
     }
-    Z[i] = z;
-    A[i] = a;
-    Ap[packed_off(r, c, H)] = __bfloat16_as_ushort(__float2bfloat16_rn(a));
+    const size_t at = trans ? packed_off(c0 + line, r0 + run, rows_pad) : packed_off(r0 + line, c0 + run, cols_pad);
+    *(uint4 *)(out + at) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// y[r] = A3[r] . w4 + b4, one warp per row.
-__global__ void output_kernel(const float *__restrict__ A, const float *__restrict__ w4, const float *__restrict__ b4,
-                              int B, int H, float *__restrict__ y)
+// X (B x C) -> packed, and packed transposed.
+__global__ void __launch_bounds__(kTileThreads)
+    pack_input_kernel(const float *__restrict__ X, int B, int C, uint16_t *__restrict__ P, uint16_t *__restrict__ PT)
+{
+    __shared__ Tile s;
+    const int r0 = blockIdx.y * kSide, c0 = blockIdx.x * kSide, r = threadIdx.x / kSide, c = threadIdx.x % kSide;
+    s[r][c] = X[(size_t)(r0 + r) * C + c0 + c];
+    __syncthreads();
+    store_packed(s, r0, c0, B, C, P, PT);
+}
+
+// Z (B x H) += bias; Ap = packed gelu(Z).  Rows >= nvalid are zeroed.  For a gradient (AT not
+// NULL) Z is kept and gelu(Z) is packed transposed too.
+__global__ void __launch_bounds__(kTileThreads)
+    bias_gelu_pack_kernel(float *__restrict__ Z, const float *__restrict__ bias, int B, int H, int nvalid,
+                          uint16_t *__restrict__ Ap, uint16_t *__restrict__ AT)
+{
+    __shared__ Tile s;
+    const int r0 = blockIdx.y * kSide, c0 = blockIdx.x * kSide, r = threadIdx.x / kSide, c = threadIdx.x % kSide;
+    const size_t at = (size_t)(r0 + r) * H + c0 + c;
+    const float z = r0 + r < nvalid ? Z[at] + bias[c0 + c] : 0.0f;
+    s[r][c] = gelu(z);
+    if (AT)
+        Z[at] = z;
+    __syncthreads();
+    store_packed(s, r0, c0, B, H, Ap, AT);
+}
+
+// Last layer: Z (B x H) += bias (zero in rows >= nvalid, kept for a gradient), y[r] = gelu(Z[r]) . w4 + b4;
+// one warp per row.
+__global__ void output_kernel(float *__restrict__ Z, const float *__restrict__ bias, const float *__restrict__ w4,
+                              const float *__restrict__ b4, int B, int H, int nvalid, bool keep,
+                              float *__restrict__ y)
 {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= B)
         return;
     float acc = 0.0f;
-    for (int c = lane; c < H; c += 32)
-        acc = fmaf(A[(size_t)warp * H + c], w4[c], acc);
+    for (int c = lane; c < H; c += 32) {
+        const float z = warp < nvalid ? Z[(size_t)warp * H + c] + bias[c] : 0.0f;
+        if (keep)
+            Z[(size_t)warp * H + c] = z;
+        acc = fmaf(gelu(z), w4[c], acc);
+    }
     for (int off = 16; off > 0; off >>= 1)
         acc += __shfl_down_sync(0xffffffffu, acc, off);
     if (lane == 0)
         y[warp] = acc + b4[0];
 }
 
-// loss = mean (y - t)^2 over the valid rows (fixed-order single-block sum);
-// dy = 2 (y - t) / nvalid (0 on padded rows).
+// loss = mean (y - t)^2 over the valid rows, dy = 2 (y - t) / nvalid (0 on padded rows) and
+// db4 = sum dy (fixed-order single-block sums).
 __global__ void loss_kernel(const float *__restrict__ y, const float *__restrict__ t, int B, int nvalid,
-                            float *__restrict__ dy, float *__restrict__ loss)
+                            float *__restrict__ dy, float *__restrict__ loss, float *__restrict__ db4)
 {
-    __shared__ float red[256];
-    float acc = 0.0f;
+    __shared__ float red[2][256];
+    float acc = 0.0f, sum = 0.0f;
     for (int r = threadIdx.x; r < B; r += blockDim.x) {
         const float e = r < nvalid ? y[r] - t[r] : 0.0f;
-        dy[r] = 2.0f * e / (float)nvalid;
+        const float d = 2.0f * e / (float)nvalid;
+        dy[r] = d;
         acc += e * e;
+        sum += d;
     }
-    red[threadIdx.x] = acc;
+    red[0][threadIdx.x] = acc;
+    red[1][threadIdx.x] = sum;
     __syncthreads();
     for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            red[threadIdx.x] += red[threadIdx.x + s];
+        if (threadIdx.x < s) {
+            red[0][threadIdx.x] += red[0][threadIdx.x + s];
+            red[1][threadIdx.x] += red[1][threadIdx.x + s];
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0 && loss)
-        *loss = red[0] / (float)nvalid;
+    if (threadIdx.x == 0) {
+        if (loss)
+            *loss = red[0][0] / (float)nvalid;
+        *db4 = red[1][0];
+    }
 }
 
-// dA3 = dy w4^T; dZ3 = dA3 gelu'(Z3)  (B x H)
-__global__ void output_backward_kernel(const float *__restrict__ dy, const float *__restrict__ w4,
-                                       const float *__restrict__ Z, int B, int H, float *__restrict__ dZ)
+// dZ = dA gelu'(Z), packed and packed transposed, and its column sums per tile row of 32 into
+// part[blockIdx.y][c].  dA is the product of the layer above or, in the last layer (OUT), dy w4^T;
+// there part4 takes the sums of dy gelu(Z).
+template <bool OUT>
+__global__ void __launch_bounds__(kTileThreads)
+    delta_kernel(const float *__restrict__ dA, const float *__restrict__ w4, const float *__restrict__ Z, int B, int H,
+                 uint16_t *__restrict__ P, uint16_t *__restrict__ PT, float *__restrict__ part,
+                 float *__restrict__ part4)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)B * H)
+    __shared__ Tile s, s4;
+    const int r0 = blockIdx.y * kSide, c0 = blockIdx.x * kSide, r = threadIdx.x / kSide, c = threadIdx.x % kSide;
+    const size_t at = (size_t)(r0 + r) * H + c0 + c;
+    const float z = Z[at];
+    if constexpr (OUT) {
+        const float dy = dA[r0 + r];
+        s[r][c] = dy * w4[c0 + c] * gelu_grad(z);
+        s4[r][c] = dy * gelu(z);
+    } else {
+        s[r][c] = dA[at] * gelu_grad(z);
+    }
+    __syncthreads();
+    store_packed(s, r0, c0, B, H, P, PT);
+    // columns: by warps that store nothing
+    if (r == kSide - 1 || (OUT && r == kSide - 2)) {
+        const Tile &x = r == kSide - 1 ? s : s4;
+        float acc = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kSide; ++k)
+            acc += x[k][c];
+        (r == kSide - 1 ? part : part4)[(size_t)blockIdx.y * H + c0 + c] = acc;
+    }
+}
+
+// The rest of the gradient: blocks [0, 4 H / 32) sum the tile rows' column sums of the four vectors
+// (32 columns each, 32 threads a column, fixed order); the others copy W1's block from the
+// product, whose rows are padded to ldd.
+struct GradientEnd {
+    const float *part;      // [4][tiles][H]
+    float *sums[4];
+    const float *D;         // rows x ldd, NULL: in place already
+    float *W1;
+    int tiles, H, din, ldd;
+};
+
+__global__ void __launch_bounds__(kTileThreads) gradient_end_kernel(GradientEnd q)
+{
+    const int groups = q.H / kSide;
+    if ((int)blockIdx.x >= 4 * groups) {
+        const long long i = (long long)(blockIdx.x - 4 * groups) * kTileThreads + threadIdx.x;
+        if (i < (long long)q.H * q.din)
+            q.W1[i] = q.D[(size_t)(i / q.din) * q.ldd + i % q.din];
         return;
-    const int r = (int)(i / H), c = (int)(i % H);
-    dZ[i] = dy[r] * w4[c] * gelu_grad(Z[i]);
-}
-
-// dZ = dA gelu'(Z) in place on dA
-__global__ void gelu_backward_kernel(float *__restrict__ dA, const float *__restrict__ Z, long long n)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n)
-        dA[i] *= gelu_grad(Z[i]);
-}
-
-// out[c] = sum_r X[r][c] (column sums over B rows, fixed order per column)
-__global__ void colsum_kernel(const float *__restrict__ X, int B, int H, float *__restrict__ out)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= H)
-        return;
+    }
+    constexpr int kWays = kTileThreads / kSide;
+    __shared__ Tile red;
+    const int v = blockIdx.x / groups, c = blockIdx.x % groups * kSide + threadIdx.x % kSide, w = threadIdx.x / kSide;
+    const float *part = q.part + (size_t)v * q.tiles * q.H + c;
     float acc = 0.0f;
-    for (int r = 0; r < B; ++r)
-        acc += X[(size_t)r * H + c];
-    out[c] = acc;
-}
-
-// dw4[c] = sum_r dy[r] A3[r][c]; db4 = sum_r dy[r]
-__global__ void output_grad_kernel(const float *__restrict__ dy, const float *__restrict__ A, int B, int H,
-                                   float *__restrict__ dw4, float *__restrict__ db4)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < H) {
-        float acc = 0.0f;
-        for (int r = 0; r < B; ++r)
-            acc = fmaf(dy[r], A[(size_t)r * H + c], acc);
-        dw4[c] = acc;
+    for (int i = w; i < q.tiles; i += kWays)
+        acc += part[(size_t)i * q.H];
+    red[w][threadIdx.x % kSide] = acc;
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+        for (int k = 1; k < kWays; ++k)
+            acc += red[k][threadIdx.x];
+        q.sums[v][c] = acc;
     }
-    if (c == 0) {
-        float acc = 0.0f;
-        for (int r = 0; r < B; ++r)
-            acc += dy[r];
-        db4[0] = acc;
-    }
-}
-
-// copies an FP32 D (rows x ldd) block into a flat gradient slice (rows x cols)
-__global__ void copy_block_kernel(const float *__restrict__ D, int rows, int cols, int ldd,
-                                  float *__restrict__ out)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)rows * cols)
-        return;
-    out[i] = D[(size_t)(i / cols) * ldd + i % cols];
 }
 
 // Adam (Kingma, Ba 2015) with bias correction; step is the 1-based step number.
@@ -377,9 +445,10 @@ struct pp_mlp {
     // packed weights
     void *W1p = nullptr, *W2p = nullptr, *W3p = nullptr, *W2Tp = nullptr, *W3Tp = nullptr;
     // activations (bmax rows)
-    float *X = nullptr, *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *A1 = nullptr, *A2 = nullptr,
-          *A3 = nullptr, *y = nullptr, *dy = nullptr, *dZ = nullptr, *dA = nullptr, *D = nullptr;
-    void *Xp = nullptr, *A1p = nullptr, *A2p = nullptr, *Tp1 = nullptr, *Tp2 = nullptr;
+    float *X = nullptr, *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *y = nullptr, *dy = nullptr, *dA = nullptr,
+          *D = nullptr, *part = nullptr;
+    void *Xp = nullptr, *A1p = nullptr, *A2p = nullptr, *dZp = nullptr;
+    void *XTp = nullptr, *A1Tp = nullptr, *A2Tp = nullptr, *dZTp = nullptr;  // transposed, for the gradients
     // shuffled mini-batches of pp_mlp_fit (bmax rows)
     float *Xs = nullptr, *ts = nullptr;
 };
@@ -393,8 +462,8 @@ void mlp_free(pp_mlp *h)
     if (!h)
         return;
     void *ptrs[] = {h->p, h->m, h->v, h->g, h->W1p, h->W2p, h->W3p, h->W2Tp, h->W3Tp, h->X, h->Z1, h->Z2,
-                    h->Z3, h->A1, h->A2, h->A3, h->y, h->dy, h->dZ, h->dA, h->D, h->Xp, h->A1p, h->A2p,
-                    h->Tp1, h->Tp2, h->Xs, h->ts};
+                    h->Z3, h->y, h->dy, h->dA, h->D, h->part, h->Xp, h->A1p, h->A2p, h->dZp, h->XTp, h->A1Tp,
+                    h->A2Tp, h->dZTp, h->Xs, h->ts};
     for (void *q : ptrs)
         if (q)
             cudaFree(q);
@@ -416,83 +485,73 @@ int repack_weights(pp_mlp *h, cudaStream_t st)
     return rc;
 }
 
-// Forward on X (rows x din, already in h->X, rows padded to Bp); y into h->y.
-int forward(pp_mlp *h, int Bp, int nvalid, cudaStream_t st)
+// CTAs of the tiled passes over a (rows x cols) matrix
+dim3 tiles(int rows, int cols) { return dim3(cols / kSide, rows / kSide); }
+
+// Forward on X (rows x din, already in h->X, rows padded to Bp); y into h->y.  grad: what the
+// backward pass reads is kept (the sums of each layer, the activations transposed).
+int forward(pp_mlp *h, int Bp, int nvalid, bool grad, cudaStream_t st)
 {
     const int H = h->H;
-    const long long BH = (long long)Bp * H;
-    int rc = pp::launch_pack_bf16(h->X, Bp, h->dinp, h->dinp, 0, h->Xp, Bp, h->dinp, st);
-    if (!rc)
-        rc = pp::launch_gemm_bf16(h->Xp, h->W1p, h->Z1, Bp, H, h->dinp, H, st);
+    pack_input_kernel<<<tiles(Bp, h->dinp), kTileThreads, 0, st>>>(h->X, Bp, h->dinp, (uint16_t *)h->Xp,
+                                                                  grad ? (uint16_t *)h->XTp : nullptr);
+    int rc = pp::launch_gemm_bf16(h->Xp, h->W1p, h->Z1, Bp, H, h->dinp, H, st);
     if (rc)
         return rc;
-    bias_gelu_pack_kernel<<<nb(BH), 256, 0, st>>>(h->Z1, h->p + h->off_b1, Bp, H, nvalid, h->A1,
-                                                  (uint16_t *)h->A1p);
+    bias_gelu_pack_kernel<<<tiles(Bp, H), kTileThreads, 0, st>>>(h->Z1, h->p + h->off_b1, Bp, H, nvalid,
+                                                                (uint16_t *)h->A1p,
+                                                                grad ? (uint16_t *)h->A1Tp : nullptr);
     rc = pp::launch_gemm_bf16(h->A1p, h->W2p, h->Z2, Bp, H, H, H, st);
     if (rc)
         return rc;
-    bias_gelu_pack_kernel<<<nb(BH), 256, 0, st>>>(h->Z2, h->p + h->off_b2, Bp, H, nvalid, h->A2,
-                                                  (uint16_t *)h->A2p);
+    bias_gelu_pack_kernel<<<tiles(Bp, H), kTileThreads, 0, st>>>(h->Z2, h->p + h->off_b2, Bp, H, nvalid,
+                                                                (uint16_t *)h->A2p,
+                                                                grad ? (uint16_t *)h->A2Tp : nullptr);
     rc = pp::launch_gemm_bf16(h->A2p, h->W3p, h->Z3, Bp, H, H, H, st);
     if (rc)
         return rc;
-    bias_gelu_pack_kernel<<<nb(BH), 256, 0, st>>>(h->Z3, h->p + h->off_b3, Bp, H, nvalid, h->A3,
-                                                  (uint16_t *)h->A2p /* scratch: A3 is not re-packed */);
-    output_kernel<<<nb((long long)Bp * 32), 256, 0, st>>>(h->A3, h->p + h->off_w4, h->p + h->off_b4, Bp, H, h->y);
+    output_kernel<<<nb((long long)Bp * 32), 256, 0, st>>>(h->Z3, h->p + h->off_b3, h->p + h->off_w4, h->p + h->off_b4,
+                                                           Bp, H, nvalid, grad, h->y);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PP_OK : pp::cuda_fail(e, "surrogate forward");
 }
 
-// Backward after forward; gradient into h->g.
+// Backward after forward with grad; gradient into h->g.  The weight gradients of the hidden layers
+// are products straight into their blocks of it.
 int backward(pp_mlp *h, const float *t, int Bp, int nvalid, float *loss, cudaStream_t st)
 {
-    const int H = h->H;
-    const long long BH = (long long)Bp * H;
-    loss_kernel<<<1, 256, 0, st>>>(h->y, t, Bp, nvalid, h->dy, loss);
-    output_grad_kernel<<<nb(H, 128), 128, 0, st>>>(h->dy, h->A3, Bp, H, h->g + h->off_w4, h->g + h->off_b4);
-    output_backward_kernel<<<nb(BH), 256, 0, st>>>(h->dy, h->p + h->off_w4, h->Z3, Bp, H, h->dZ);  // dZ3
-    // layer 3: dW3 = dZ3^T A2, db3, dA2 = dZ3 W3
-    int rc = pp::launch_pack_bf16(h->dZ, H, Bp, H, 1, h->Tp1, H, Bp, st);   // dZ3^T (H x Bp)
+    const int H = h->H, ntile = Bp / kSide;
+    float *g = h->g, *part = h->part;
+    uint16_t *dZp = (uint16_t *)h->dZp, *dZTp = (uint16_t *)h->dZTp;
+    const size_t np = (size_t)ntile * H;
+    loss_kernel<<<1, 256, 0, st>>>(h->y, t, Bp, nvalid, h->dy, loss, g + h->off_b4);
+    // layer 3: dZ3, dW3 = dZ3^T A2, dA2 = dZ3 W3
+    delta_kernel<true><<<tiles(Bp, H), kTileThreads, 0, st>>>(h->dy, h->p + h->off_w4, h->Z3, Bp, H, dZp, dZTp, part,
+                                                             part + 3 * np);
+    int rc = pp::launch_gemm_bf16(dZTp, h->A2Tp, g + h->off_W3, H, H, Bp, H, st);
     if (!rc)
-        rc = pp::launch_pack_bf16(h->A2, H, Bp, H, 1, h->Tp2, H, Bp, st);   // A2^T (H x Bp)
-    if (!rc)
-        rc = pp::launch_gemm_bf16(h->Tp1, h->Tp2, h->D, H, H, Bp, H, st);
+        rc = pp::launch_gemm_bf16(dZp, h->W3Tp, h->dA, Bp, H, H, H, st);
     if (rc)
         return rc;
-    copy_block_kernel<<<nb((long long)H * H), 256, 0, st>>>(h->D, H, H, H, h->g + h->off_W3);
-    colsum_kernel<<<nb(H, 128), 128, 0, st>>>(h->dZ, Bp, H, h->g + h->off_b3);
-    rc = pp::launch_pack_bf16(h->dZ, Bp, H, H, 0, h->Tp1, Bp, H, st);       // dZ3 (Bp x H)
+    // layer 2
+    delta_kernel<false><<<tiles(Bp, H), kTileThreads, 0, st>>>(h->dA, nullptr, h->Z2, Bp, H, dZp, dZTp, part + np,
+                                                              nullptr);
+    rc = pp::launch_gemm_bf16(dZTp, h->A1Tp, g + h->off_W2, H, H, Bp, H, st);
     if (!rc)
-        rc = pp::launch_gemm_bf16(h->Tp1, h->W3Tp, h->dA, Bp, H, H, H, st);  // dA2
+        rc = pp::launch_gemm_bf16(dZp, h->W2Tp, h->dA, Bp, H, H, H, st);
     if (rc)
         return rc;
-    gelu_backward_kernel<<<nb(BH), 256, 0, st>>>(h->dA, h->Z2, BH);          // dZ2 in dA
-    // layer 2: dW2 = dZ2^T A1, db2, dA1 = dZ2 W2
-    rc = pp::launch_pack_bf16(h->dA, H, Bp, H, 1, h->Tp1, H, Bp, st);
-    if (!rc)
-        rc = pp::launch_pack_bf16(h->A1, H, Bp, H, 1, h->Tp2, H, Bp, st);
-    if (!rc)
-        rc = pp::launch_gemm_bf16(h->Tp1, h->Tp2, h->D, H, H, Bp, H, st);
+    // layer 1: dW1 = dZ1^T X, its columns padded unless d_in is a multiple of 64
+    delta_kernel<false><<<tiles(Bp, H), kTileThreads, 0, st>>>(h->dA, nullptr, h->Z1, Bp, H, nullptr, dZTp,
+                                                              part + 2 * np, nullptr);
+    const bool padded = h->din != h->dinp;
+    rc = pp::launch_gemm_bf16(dZTp, h->XTp, padded ? h->D : g + h->off_W1, H, h->dinp, Bp, h->dinp, st);
     if (rc)
         return rc;
-    copy_block_kernel<<<nb((long long)H * H), 256, 0, st>>>(h->D, H, H, H, h->g + h->off_W2);
-    colsum_kernel<<<nb(H, 128), 128, 0, st>>>(h->dA, Bp, H, h->g + h->off_b2);
-    rc = pp::launch_pack_bf16(h->dA, Bp, H, H, 0, h->Tp1, Bp, H, st);
-    if (!rc)
-        rc = pp::launch_gemm_bf16(h->Tp1, h->W2Tp, h->dZ, Bp, H, H, H, st);  // dA1 in dZ
-    if (rc)
-        return rc;
-    gelu_backward_kernel<<<nb(BH), 256, 0, st>>>(h->dZ, h->Z1, BH);          // dZ1
-    // layer 1: dW1 = dZ1^T X, db1
-    rc = pp::launch_pack_bf16(h->dZ, H, Bp, H, 1, h->Tp1, H, Bp, st);
-    if (!rc)
-        rc = pp::launch_pack_bf16(h->X, h->dinp, Bp, h->dinp, 1, h->Tp2, h->dinp, Bp, st);  // X^T
-    if (!rc)
-        rc = pp::launch_gemm_bf16(h->Tp1, h->Tp2, h->D, H, h->dinp, Bp, h->dinp, st);
-    if (rc)
-        return rc;
-    copy_block_kernel<<<nb((long long)H * h->din), 256, 0, st>>>(h->D, H, h->din, h->dinp, h->g + h->off_W1);
-    colsum_kernel<<<nb(H, 128), 128, 0, st>>>(h->dZ, Bp, H, h->g + h->off_b1);
+    GradientEnd q = {part, {g + h->off_b3, g + h->off_b2, g + h->off_b1, g + h->off_w4}, h->D, g + h->off_W1, ntile, H,
+                     h->din, h->dinp};
+    const unsigned copies = padded ? nb((long long)H * h->din, kTileThreads) : 0;
+    gradient_end_kernel<<<4 * (H / kSide) + copies, kTileThreads, 0, st>>>(q);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PP_OK : pp::cuda_fail(e, "surrogate backward");
 }
@@ -561,18 +620,20 @@ int pp_mlp_create(int32_t d_in, int32_t hidden, int32_t max_batch, pp_mlp **out)
     alloc(&h->W2Tp, packed_bytes(hidden, hidden));
     alloc(&h->W3Tp, packed_bytes(hidden, hidden));
     alloc((void **)&h->X, sizeof(float) * (size_t)h->bmax * h->dinp);
-    float **acts[] = {&h->Z1, &h->Z2, &h->Z3, &h->A1, &h->A2, &h->A3, &h->dZ, &h->dA};
+    float **acts[] = {&h->Z1, &h->Z2, &h->Z3, &h->dA};
     for (float **a : acts)
         alloc((void **)a, sizeof(float) * BH);
-    alloc((void **)&h->D, sizeof(float) * (size_t)std::max(BH, (size_t)hidden * hidden));
+    alloc((void **)&h->D, sizeof(float) * (size_t)hidden * h->dinp);
+    alloc((void **)&h->part, sizeof(float) * 4 * BH / kSide);
     alloc((void **)&h->y, sizeof(float) * h->bmax);
     alloc((void **)&h->dy, sizeof(float) * h->bmax);
     alloc(&h->Xp, packed_bytes(h->bmax, h->dinp));
-    alloc(&h->A1p, packed_bytes(h->bmax, hidden));
-    alloc(&h->A2p, packed_bytes(h->bmax, hidden));
-    const size_t tp = std::max(packed_bytes(h->bmax, hidden), packed_bytes(hidden, h->bmax));
-    alloc(&h->Tp1, tp);
-    alloc(&h->Tp2, std::max(tp, packed_bytes(h->dinp, h->bmax)));
+    alloc(&h->XTp, packed_bytes(h->dinp, h->bmax));
+    void **hidden_packed[] = {&h->A1p, &h->A2p, &h->dZp}, **hidden_trans[] = {&h->A1Tp, &h->A2Tp, &h->dZTp};
+    for (int i = 0; i < 3; ++i) {
+        alloc(hidden_packed[i], packed_bytes(h->bmax, hidden));
+        alloc(hidden_trans[i], packed_bytes(hidden, h->bmax));
+    }
     alloc((void **)&h->Xs, sizeof(float) * (size_t)h->bmax * h->din);
     alloc((void **)&h->ts, sizeof(float) * h->bmax);
     if (e != cudaSuccess) {
@@ -643,7 +704,7 @@ int pp_mlp_forward(pp_mlp *h, const float *X, int32_t B, float *y, void *stream)
     const int Bp = (B + kRows - 1) / kRows * kRows;
     int rc = stage_inputs(h, X, B, st);
     if (!rc)
-        rc = forward(h, Bp, B, st);
+        rc = forward(h, Bp, B, false, st);
     if (rc)
         return rc;
     cudaError_t e = cudaMemcpyAsync(y, h->y, sizeof(float) * B, cudaMemcpyDeviceToDevice, st);
@@ -660,7 +721,7 @@ int pp_mlp_loss_grad(pp_mlp *h, const float *X, const float *t, int32_t B, float
     const int Bp = (B + kRows - 1) / kRows * kRows;
     int rc = stage_inputs(h, X, B, st);
     if (!rc)
-        rc = forward(h, Bp, B, st);
+        rc = forward(h, Bp, B, true, st);
     if (!rc) {
         // targets on padded rows are never read (dy = 0 there)
         rc = backward(h, t, Bp, B, loss, st);
