@@ -110,6 +110,9 @@ int launch_de_set_generation(unsigned long long *gen_dev, uint64_t v, cudaStream
 // BF16 tensor-core GEMM and operand packing (pp_gemm.cu).
 int launch_gemm_bf16(const void *A, const void *B, float *D, int M, int N, int K, int ldd,
                      cudaStream_t stream);
+// Two products (ldd = N each), neither reading what the other writes, in one launch where that is possible.
+int launch_gemm_pair_bf16(const void *A0, const void *B0, float *D0, int M0, int N0, int K0, const void *A1,
+                          const void *B1, float *D1, int M1, int N1, int K1, cudaStream_t stream);
 int launch_pack_bf16(const float *X, int rows, int cols, int ldx, int trans, void *P, int rows_pad,
                      int cols_pad, cudaStream_t stream);
 

@@ -528,17 +528,13 @@ int backward(pp_mlp *h, const float *t, int Bp, int nvalid, float *loss, cudaStr
     // layer 3: dZ3, dW3 = dZ3^T A2, dA2 = dZ3 W3
     delta_kernel<true><<<tiles(Bp, H), kTileThreads, 0, st>>>(h->dy, h->p + h->off_w4, h->Z3, Bp, H, dZp, dZTp, part,
                                                              part + 3 * np);
-    int rc = pp::launch_gemm_bf16(dZTp, h->A2Tp, g + h->off_W3, H, H, Bp, H, st);
-    if (!rc)
-        rc = pp::launch_gemm_bf16(dZp, h->W3Tp, h->dA, Bp, H, H, H, st);
+    int rc = pp::launch_gemm_pair_bf16(dZTp, h->A2Tp, g + h->off_W3, H, H, Bp, dZp, h->W3Tp, h->dA, Bp, H, H, st);
     if (rc)
         return rc;
     // layer 2
     delta_kernel<false><<<tiles(Bp, H), kTileThreads, 0, st>>>(h->dA, nullptr, h->Z2, Bp, H, dZp, dZTp, part + np,
                                                               nullptr);
-    rc = pp::launch_gemm_bf16(dZTp, h->A1Tp, g + h->off_W2, H, H, Bp, H, st);
-    if (!rc)
-        rc = pp::launch_gemm_bf16(dZp, h->W2Tp, h->dA, Bp, H, H, H, st);
+    rc = pp::launch_gemm_pair_bf16(dZTp, h->A1Tp, g + h->off_W2, H, H, Bp, dZp, h->W2Tp, h->dA, Bp, H, H, st);
     if (rc)
         return rc;
     // layer 1: dW1 = dZ1^T X, its columns padded unless d_in is a multiple of 64

@@ -53,3 +53,19 @@ def test_gradient_at_the_edges_of_tiles(pp, d_in, H, B):
         n = int(np.prod(s))
         assert np.linalg.norm(g[o:o + n] - ref[o:o + n]) < 1e-2 * np.linalg.norm(ref[o:o + n]), k
     net.close()
+
+
+@pytest.mark.parametrize("M,N,K", [(128, 64, 64), (128, 96, 128), (256, 192, 128), (256, 256, 512), (128, 128, 576),
+                                   (128 * 20, 256, 192), (128 * 152, 256, 64)])
+def test_products_split_by_columns(pp, M, N, K):
+    # 2 CTAs of 32 columns; none (48 would straddle, 192 / 2 too); 8 of 32 with B resident; streamed; 4 of 64; none.
+    # FP32 sums of K products of BF16 numbers: relative 2e-5 of the largest as for any product of these sizes.
+    gen = torch.Generator(device="cpu").manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=gen)
+    B = torch.randn(N, K, generator=gen)
+    Ap, _, _ = pp.pack_bf16(A.cuda())
+    Bp, _, _ = pp.pack_bf16(B.cuda())
+    D = pp.gemm_bf16(Ap, Bp, M, N, K)
+    assert pp.sync_status() == pp.PP_OK
+    ref = A.to(torch.bfloat16).double() @ B.to(torch.bfloat16).double().T
+    assert (D.cpu().double() - ref).abs().max().item() < 2e-5 * ref.abs().max().item() + 1e-5 * K ** 0.5
