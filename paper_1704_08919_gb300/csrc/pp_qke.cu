@@ -17,18 +17,19 @@
 //
 // The gradient is the exact adjoint of the discrete forward map: the adjoint
 // state (final value -w(p) e_1, i.e. lambda_1(t_f) = -1 of Eq. (adj) times the
-// quadrature weight) runs backwards through the transposed RK4 stages, and each
-// stage k = N y contributes kb (x) y to the adjoint of N, whose projections on
-// S_Q, S_R, S_W are the adjoints of Q, R, omega -- the inner product
-// <chi, grad N lambda> of Eq. (grad) taken stage by stage.  The forward states
-// are kept at every S-th step (checkpoints in HBM) and recomputed a segment at a
-// time into per-thread shared-memory slots for the backward sweep.  Each sample's six sensitivities
-// are summed over the CTA's modes (warp shuffles, then warps in fixed order) into
-// a per-CTA row; a second kernel sums the rows in fixed order.
+// quadrature weight) runs backwards through the transposed RK4 steps, and each
+// step's derivatives with respect to the coefficients at its three samples are the
+// adjoints of Q, R, omega there -- the inner product <chi, grad N lambda> of Eq. (grad)
+// taken step by step.  The forward states are kept at every S-th step (checkpoints in
+// HBM) and recomputed a segment at a time into per-thread shared-memory slots for the
+// backward sweep.  Seven terms per sample are summed over the CTA's modes (warps through
+// shared memory, then the warps in fixed order) into a per-CTA row; a second kernel sums
+// the rows in fixed order and forms the sample's six sensitivities.
 #include <math.h>
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 #include <vector>
 
 #include "pp_policies.cuh"
@@ -44,39 +45,69 @@ struct alignas(sizeof(T) * 8) QkeS {
     T ax, ay, ex, ey, edx, edy, ee, cr;
 };
 
+// The six components fall into two independent channels: p = (chi_0 + chi_5, chi_1 + chi_4, chi_2 + chi_3)
+// and m, the differences, each turned by a generator of the same form,
+//   x' = -Q y,  y' = Q x - V z,  z' = V y,   V = 2 omega - R for p and 2 omega + R for m,
+// so that N costs 4 products per channel instead of 12, and RK4, being linear in chi, is the same iterates.
+// Both channels start at x = 1, y = z = 0, and f = -(delta x_p + delta x_m) / 2 (two terms of one sign).
+// A channel's three components are u = (x, z) and y: with a = dt (-Q, V), u' dt = a y and y' dt = -a.u.
+// The channels run as the two halves of packed FP32 operations (one instruction for both; FP64: one after
+// the other).  The adjoint kernel issues 692 instructions per mode-step with six components and halving
+// exchanges, about 460 with two channels and WarpSum; it is bound by issue at 4 warps per scheduler.  16 starts on
+// 32 x 32 x 16 modes, 16384 steps, whole evaluation: 101.2 -> 84.5 ms; the warps' sums as two-floats, the six
+// sensitivities after the sum over CTAs, running pointers: 79.2 ms; two backward steps per pass of the loop (no
+// copies of what one step hands to the next): 76.0 ms.
+template <typename T>
+using Two = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+
+__device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ double2 mul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ double2 add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c)
+{
+    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+template <typename T>
+__device__ __forceinline__ Two<T> both(T v)
+{
+    Two<T> r;
+    r.x = v;
+    r.y = v;
+    return r;
+}
+
+// a = dt (-Q, V) of both channels
 template <typename T>
 struct Coef {
-    T Q, R, W2;  // W2 = 2 omega
+    Two<T> x, z;
+};
+
+// delta = chi - e_1 of both channels
+template <typename T>
+struct State {
+    Two<T> x, y, z;
+};
+
+// One mode: momentum, p_z^2, eps_perp, and the step in the forms the coefficients want.
+template <typename T>
+struct Mode {
+    T px, py, pz2, eperp, ep_dt, dt2, ndt;
 };
 
 // Reciprocal square root.  FP32: the special-function unit's approximation
 // (rsqrtf, at most 2 ulp), one instruction instead of a square root and a
 // division; its error is far below the FP32 RK4 rounding of the state.  The
-// forward, recomputed and adjoint sweeps all call this one function, so the
-// recomputed trajectory is the forward one bit for bit.
+// forward, recomputed and adjoint sweeps all call the same functions, and these leave
+// the compiler no choice of what to contract, so every kernel's trajectory is the
+// same bit for bit.
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
 
-template <typename T>
-__device__ __forceinline__ Coef<T> coef_at(const QkeS<T> &s, T px, T py, T pz2, T eperp)
-{
-    const T Px = px - s.ax, Py = py - s.ay;
-    const T w2 = ((Px * Px + Py * Py) + pz2) + T(1);
-    const T iw = rsq(w2);
-    const T EP = s.ex * Px + s.ey * Py;
-    const T X = w2 * s.ee - EP * EP;
-    Coef<T> c;
-    c.W2 = T(2) * (w2 * iw);
-    if (X > T(0)) {
-        const T rX = rsq(X);
-        c.Q = (X * rX) * (iw * iw);
-        c.R = eperp * (w2 * iw) * s.cr * (rX * rX);
-    } else {
-        c.Q = T(0);
-        c.R = T(0);
-    }
-    return c;
-}
+// A product that is not contracted with a following addition
+__device__ __forceinline__ float product(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double product(double a, double b) { return __dmul_rn(a, b); }
 
 // The mode-dependent quantities of one sample that both the coefficients and
 // their derivatives need.
@@ -86,141 +117,131 @@ struct Basics {
 };
 
 template <typename T>
-__device__ __forceinline__ Basics<T> basics(const QkeS<T> &s, T px, T py, T pz2)
+__device__ __forceinline__ Basics<T> basics(const QkeS<T> &s, const Mode<T> &k)
 {
     Basics<T> b;
-    b.Px = px - s.ax;
-    b.Py = py - s.ay;
-    b.w2 = ((b.Px * b.Px + b.Py * b.Py) + pz2) + T(1);
+    b.Px = k.px - s.ax;
+    b.Py = k.py - s.ay;
+    b.w2 = fma(b.Px, b.Px, fma(b.Py, b.Py, k.pz2)) + T(1);
     b.iw = rsq(b.w2);
-    b.EP = s.ex * b.Px + s.ey * b.Py;
-    b.X = b.w2 * s.ee - b.EP * b.EP;
+    b.EP = fma(s.ex, b.Px, product(s.ey, b.Py));
+    b.X = fma(b.w2, s.ee, -product(b.EP, b.EP));
     b.rX = b.X > T(0) ? rsq(b.X) : T(0);
     return b;
 }
 
-// the same values as coef_at, from precomputed basics
 template <typename T>
-__device__ __forceinline__ Coef<T> coef_from(const Basics<T> &b, const QkeS<T> &s, T eperp)
+__device__ __forceinline__ Coef<T> coef_from(const Basics<T> &b, const QkeS<T> &s, const Mode<T> &k)
 {
+    const T w = b.w2 * b.iw, W = product(k.dt2, w);
+    const bool field = b.X > T(0);
+    const T q = field ? (b.X * b.rX) * (b.iw * (k.ndt * b.iw)) : T(0);
+    const T R = field ? product(k.ep_dt * w * s.cr, b.rX * b.rX) : T(0);
     Coef<T> c;
-    c.W2 = T(2) * (b.w2 * b.iw);
-    if (b.X > T(0)) {
-        c.Q = (b.X * b.rX) * (b.iw * b.iw);
-        c.R = eperp * (b.w2 * b.iw) * s.cr * (b.rX * b.rX);
-    } else {
-        c.Q = T(0);
-        c.R = T(0);
-    }
+    c.x = both(q);
+    c.z.x = W - R;
+    c.z.y = W + R;
     return c;
 }
 
-// out = N (e_1 + v) (ONE) or N v; Q (1 + v_0) is formed as Q + Q v_0 in one FMA,
-// which also keeps the low bits of the small v_0.
-template <bool ONE, typename T>
-__device__ __forceinline__ void nmul(const Coef<T> &c, const T v[6], T out[6])
+template <typename T>
+__device__ __forceinline__ Coef<T> coef_at(const QkeS<T> &s, const Mode<T> &k)
 {
-    out[0] = -c.Q * v[1];
-    const T q1 = ONE ? fma(c.Q, v[0], c.Q) : c.Q * v[0];
-    out[1] = fma(c.R, v[3], fma(-c.W2, v[2], q1));
-    out[2] = fma(c.W2, v[1], -c.R * v[4]);
-    out[3] = fma(c.W2, v[4], -c.R * v[1]);
-    out[4] = fma(c.Q, v[5], fma(-c.W2, v[3], c.R * v[2]));
-    out[5] = -c.Q * v[4];
+    return coef_from(basics(s, k), s, k);
 }
 
-// out = base - N v, each component one chain of FMAs (N as in nmul).
+// dt k of a stage at delta y, its y component negated: -(dt k)_y = a.(e_1 + u), formed as a_x + a_x u_x + a_z u_z,
+// which also keeps the low bits of a small u_x.
 template <typename T>
-__device__ __forceinline__ void nmul_sub(const Coef<T> &c, const T v[6], const T base[6], T out[6])
+__device__ __forceinline__ State<T> stage(const Coef<T> &c, const State<T> &y)
 {
-    out[0] = fma(c.Q, v[1], base[0]);
-    out[1] = fma(-c.R, v[3], fma(c.W2, v[2], fma(-c.Q, v[0], base[1])));
-    out[2] = fma(c.R, v[4], fma(-c.W2, v[1], base[2]));
-    out[3] = fma(-c.W2, v[4], fma(c.R, v[1], base[3]));
-    out[4] = fma(-c.Q, v[5], fma(c.W2, v[3], fma(-c.R, v[2], base[4])));
-    out[5] = fma(c.Q, v[4], base[5]);
+    State<T> k;
+    k.x = mul(c.x, y.y);
+    k.z = mul(c.z, y.y);
+    k.y = fma2(c.z, y.z, fma2(c.x, y.x, c.x));
+    return k;
 }
 
-// One RK4 step of delta: chi = e_1 + delta.
+// d + f k (k as from stage)
 template <typename T>
-__device__ __forceinline__ void rk4_step(T d[6], const Coef<T> &c0, const Coef<T> &ch, const Coef<T> &c1, T dt)
+__device__ __forceinline__ State<T> along(const State<T> &d, T f, const State<T> &k)
 {
-    const T hd = T(0.5) * dt, sx = dt / T(6);
-    T k1[6], k2[6], k3[6], k4[6], y[6];
-    nmul<true>(c0, d, k1);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        y[i] = d[i] + hd * k1[i];
-    nmul<true>(ch, y, k2);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        y[i] = d[i] + hd * k2[i];
-    nmul<true>(ch, y, k3);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        y[i] = d[i] + dt * k3[i];
-    nmul<true>(c1, y, k4);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        d[i] = d[i] + sx * (((k1[i] + T(2) * k2[i]) + T(2) * k3[i]) + k4[i]);
+    State<T> y;
+    y.x = fma2(k.x, both(f), d.x);
+    y.y = fma2(k.y, both(-f), d.y);
+    y.z = fma2(k.z, both(f), d.z);
+    return y;
 }
 
-// Adjoints of (Q, R, omega) from one stage k = N (e_1 + y) with stage adjoint kb,
-// accumulated term by term: acc[0] += Qb, acc[1] += Rb, acc[2] += wb / 2 (the
-// factor 2 of N's omega entries is applied once per sample, in sens_from).
+// One RK4 step of delta.
 template <typename T>
-__device__ __forceinline__ void coef_adj(const T kb[6], const T y[6], T acc[3])
+__device__ __forceinline__ void rk4_step(State<T> &d, const Coef<T> &c0, const Coef<T> &ch, const Coef<T> &c1)
 {
-    T a = fma(kb[1], y[0], acc[0] + kb[1]);
-    a = fma(-kb[0], y[1], a);
-    a = fma(kb[4], y[5], a);
-    acc[0] = fma(-kb[5], y[4], a);
-    a = fma(kb[1], y[3], acc[1]);
-    a = fma(-kb[2], y[4], a);
-    a = fma(kb[4], y[2], a);
-    acc[1] = fma(-kb[3], y[1], a);
-    a = fma(kb[2], y[1], acc[2]);
-    a = fma(-kb[1], y[2], a);
-    a = fma(kb[3], y[4], a);
-    acc[2] = fma(-kb[4], y[3], a);
+    const State<T> k1 = stage(c0, d);
+    const State<T> k2 = stage(ch, along(d, T(0.5), k1));
+    const State<T> k3 = stage(ch, along(d, T(0.5), k2));
+    const State<T> k4 = stage(c1, along(d, T(1), k3));
+    State<T> k;
+    k.x = fma2(add(k2.x, k3.x), both(T(2)), add(k1.x, k4.x));
+    k.y = fma2(add(k2.y, k3.y), both(T(2)), add(k1.y, k4.y));
+    k.z = fma2(add(k2.z, k3.z), both(T(2)), add(k1.z, k4.z));
+    d = along(d, T(1) / T(6), k);
 }
 
-// Sensitivities (A_x, A_y, E_x, E_y, Ed_x, Ed_y) of one sample from the
-// adjoints (Qb, Rb, wb / 2) of its coefficients, as coef_adj accumulates them.
+// The adjoint of one step in closed form.  With a, b, c the coefficients at the step's three samples and
+// (mu, t) the adjoint state along u and y, the step's map is, in the products ab = a.b, bb, cb, au = a.u, bu, cu,
+// ma = mu.a, mb, mc,
+//   L = mu.u + t y - t y (ab + bb + cb) / 6 + t y ab cb / 24 - t (au + 4 bu + cu) / 6 + t (bb au + cb bu) / 12
+//       + y (ma + 4 mb + mc) / 6 - y (ab mb + bb mc) / 12 - (mb (au + bu) + mc bu) / 6 + mc bb au / 24,
+// the four stages multiplied out; the adjoints of a, b, c and the new (mu, t) are its derivatives, which share
+// their factors.  86 operations per channel, half as many packed instructions, where the stages, their adjoints
+// and the adjoints of Q, R, omega took 108 scalar ones.  acc: the adjoint of c so far, to which c's part is added; h and next: those of b and a.
 template <typename T>
-__device__ __forceinline__ void sample_sens(const QkeS<T> &s, T px, T py, T pz2, T eperp, const T ab[3], T out[6])
+__device__ __forceinline__ void step_adjoint(const State<T> &d, const Coef<T> &a, const Coef<T> &b, const Coef<T> &c,
+                                             State<T> &bar, Coef<T> &acc, Coef<T> &h, Coef<T> &next)
 {
-    const T Px = px - s.ax, Py = py - s.ay;
-    const T w2 = ((Px * Px + Py * Py) + pz2) + T(1);
-    const T iw = rsq(w2), w = w2 * iw, iw2 = iw * iw;
-    const T EP = s.ex * Px + s.ey * Py;
-    const T X = w2 * s.ee - EP * EP;
-    const T P[2] = {Px, Py}, E[2] = {s.ex, s.ey};
-    const T dcr_dE[2] = {s.edy, -s.edx}, dcr_dEd[2] = {-s.ey, s.ex};
-    const T Qb = ab[0], Rb = ab[1], wb = ab[2] + ab[2];
-    const bool pos = X > T(0);
-    const T rX = pos ? rsq(X) : T(0);
-    const T sX = X * rX, iX = rX * rX;
-    const T hq = T(0.5) * rX * iw2;  // dQ/dX = 1 / (2 sqrt(X) omega^2)
-    const T cx = s.cr * iX;
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        const T dw_dP = P[a] * iw;
-        T dQ_dP = 0, dQ_dE = 0, dR_dP = 0, dR_dE = 0, dR_dEd = 0;
-        if (pos) {
-            const T dX_dP = T(2) * P[a] * s.ee - T(2) * EP * E[a];
-            const T dX_dE = T(2) * w2 * E[a] - T(2) * EP * P[a];
-            dQ_dP = dX_dP * hq - sX * T(2) * P[a] * (iw2 * iw2);
-            dQ_dE = dX_dE * hq;
-            // grouped so that no 1/X^2 is formed on its own (FP32 range)
-            dR_dP = eperp * cx * (dw_dP - w * (dX_dP * iX));
-            dR_dE = eperp * w * iX * (dcr_dE[a] - s.cr * (dX_dE * iX));
-            dR_dEd = eperp * w * dcr_dEd[a] * iX;
-        }
-        out[a] = -((Qb * dQ_dP + Rb * dR_dP) + wb * dw_dP);
-        out[2 + a] = Qb * dQ_dE + Rb * dR_dE;
-        out[4 + a] = Rb * dR_dEd;
-    }
+    using V = Two<T>;
+    const V sixth = both(T(-1) / T(6)), neg = both(T(-1)), two = both(T(2)), half = both(T(0.5));
+    const V x = add(d.x, both(T(1))), y = d.y, z = d.z, m0 = bar.x, t = bar.y, m2 = bar.z;
+    // the factors -1/6 of u, y, mu and t
+    const V nx = mul(x, sixth), nz = mul(z, sixth), ny = mul(y, sixth);
+    const V n0 = mul(m0, sixth), n2 = mul(m2, sixth), nt = mul(t, sixth);
+    const V ab = fma2(a.z, b.z, mul(a.x, b.x)), bb = fma2(b.z, b.z, mul(b.x, b.x)),
+            cb = fma2(c.z, b.z, mul(c.x, b.x));
+    const V au = fma2(nz, a.z, mul(nx, a.x)), bu = fma2(nz, b.z, mul(nx, b.x));
+    const V ma = fma2(n2, a.z, mul(n0, a.x)), mb = fma2(n2, b.z, mul(n0, b.x)), mc = fma2(n2, c.z, mul(n0, c.x));
+    const V nbb = mul(bb, both(T(-0.25)));
+    const V e = fma2(nt, two, mc), g = fma2(ny, both(T(-2)), au);
+    const V c2 = fma2(cb, both(T(-0.5)), two), a2 = fma2(ab, half, both(T(-2)));
+    const V f = fma2(nt, c2, mb);
+    const V da = fma2(nbb, e, add(nt, mb));                    // dL/d(au)
+    const V db = fma2(nt, c2, add(e, mb));                     // dL/d(bu)
+    const V dmb = fma2(ny, a2, add(g, bu));                    // dL/d(mb)
+    const V dmc = fma2(nbb, g, fma2(ny, neg, bu));             // dL/d(mc)
+    const V dab = mul(mul(ny, both(T(-3))), f);                // dL/d(ab)
+    const V dcb = mul(mul(nt, both(T(3))), fma2(ny, a2, bu));  // dL/d(cb)
+    const V dbb = mul(mul(e, both(T(3))), g);                  // 2 dL/d(bb)
+    const V s6 = mul(ny, neg);
+    acc.x = fma2(x, nt, fma2(m0, dmc, fma2(b.x, dcb, acc.x)));
+    acc.z = fma2(z, nt, fma2(m2, dmc, fma2(b.z, dcb, acc.z)));
+    h.x = fma2(x, db, fma2(m0, dmb, fma2(a.x, dab, fma2(b.x, dbb, mul(c.x, dcb)))));
+    h.z = fma2(z, db, fma2(m2, dmb, fma2(a.z, dab, fma2(b.z, dbb, mul(c.z, dcb)))));
+    bar.x = add(m0, fma2(a.x, da, fma2(b.x, db, mul(c.x, nt))));
+    bar.z = add(m2, fma2(a.z, da, fma2(b.z, db, mul(c.z, nt))));
+    const V r = fma2(ab, mb, mul(bb, mc)), sum = fma2(mb, both(T(4)), add(ma, mc));
+    const V w = fma2(mul(cb, a2), both(T(-0.5)), add(ab, bb));
+    bar.y = add(t, fma2(nt, w, fma2(r, half, mul(sum, neg))));
+    next.x = fma2(x, da, fma2(m0, s6, mul(b.x, dab)));
+    next.z = fma2(z, da, fma2(m2, s6, mul(b.z, dab)));
+}
+
+// Adjoints (Q, R, 2 omega), in this order, of a sample from those of its coefficients
+template <typename T>
+__device__ __forceinline__ void coef_adjoint(const Coef<T> &c, T out[3])
+{
+    out[0] = -(c.x.x + c.x.y);
+    out[1] = c.z.y - c.z.x;
+    out[2] = c.z.y + c.z.x;
 }
 
 // f = 1 - chi_1 = -delta_1, or NaN where RK4 let |chi|^2 = 1 + 2 delta_1 + |delta|^2
@@ -229,13 +250,11 @@ __device__ __forceinline__ void sample_sens(const QkeS<T> &s, T px, T py, T pz2,
 constexpr double kGrowthTol = 1e-3;
 
 template <typename T>
-__device__ __forceinline__ double density(const T d[6])
+__device__ __forceinline__ double density(const State<T> &d)
 {
-    T g = T(2) * d[0];
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        g += d[i] * d[i];
-    return (double)g <= kGrowthTol ? -(double)d[0] : __longlong_as_double(0x7ff8000000000000ll);
+    const Two<T> sq = fma2(d.z, d.z, fma2(d.y, d.y, fma2(d.x, d.x, add(d.x, d.x))));
+    const T g = T(0.5) * (sq.x + sq.y);  // |chi|^2 is the mean of the channels'
+    return (double)g <= kGrowthTol ? -0.5 * ((double)d.x.x + (double)d.x.y) : __longlong_as_double(0x7ff8000000000000ll);
 }
 
 // Per-mode terms of one sample's sensitivities, from precomputed basics and the
@@ -252,7 +271,7 @@ __device__ __forceinline__ double density(const T d[6])
 //   out = (mu P_x, mu P_y, nu, 2 kappa omega^2, nu P_x, nu P_y, gam),
 // and sample_sens_from_sums applies the sample's constants once.  R is divided by
 // X before it meets dX (FP32 range near zeros of E).  Where X <= 0, rX = 0 makes
-// every Q and R term vanish, as in sample_sens.
+// every Q and R term vanish.
 constexpr int kSensTerms = 7;
 
 template <typename T>
@@ -290,24 +309,63 @@ __device__ __forceinline__ double sample_sens_from_sums(int i, double ex, double
     }
 }
 
-// Sums v[0..15] over the warp by halving exchanges (16 shuffles instead of 80):
-// afterwards lanes L and L^1 hold the total of value (L >> 1) & 15.
+// Sums over the warp of 16 values per lane, through a warp's 32 x 16 block of shared memory: the lanes write their
+// rows 16 bytes at a time, read columns and finish with three (FP64: two) exchanges; about 36 instructions in FP32, where
+// halving exchanges of the 16 values take 75.  Chunks of 16 bytes are stored at chunk ^ swizzle(row), so that neither
+// side has bank conflicts.  Afterwards lane L holds the total of value warp_value(L) (several lanes hold the same).
 template <typename T>
-__device__ __forceinline__ T warp_sum16(T v[16], int lane)
-{
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int o = 16 >> r, w = 8 >> r;
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < w; ++i) {
-            const T send = up ? v[i] : v[i + w];
-            const T keep = up ? v[i + w] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
+struct WarpSum {
+    static constexpr int kPer = 16 / (int)sizeof(T), kChunks = 16 / kPer, kGroups = 32 / kChunks;
+    using Chunk = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    __device__ static __forceinline__ int place(int row, int chunk)
+    {
+        return row * kChunks + (chunk ^ (sizeof(T) == 4 ? (row >> 1) & 3 : row & 7));
     }
-    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
+    __device__ static __forceinline__ T run(Chunk *buf, const T *v, int lane)
+    {
+#pragma unroll
+        for (int k = 0; k < kChunks; ++k) {
+            Chunk c;
+            T *t = reinterpret_cast<T *>(&c);
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+                t[i] = v[k * kPer + i];
+            buf[place(lane, k)] = c;
+        }
+        __syncwarp();
+        const int chunk = lane % kChunks, row = lane / kChunks;
+        T acc[kPer];
+#pragma unroll
+        for (int r = 0; r < kChunks; ++r) {
+            const Chunk c = buf[place(row + r * kGroups, chunk)];
+            const T *t = reinterpret_cast<const T *>(&c);
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+                acc[i] = r ? acc[i] + t[i] : t[i];
+        }
+        __syncwarp();
+        int o = 16;
+#pragma unroll
+        for (int w = kPer / 2; w > 0; w /= 2, o /= 2) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < w; ++i) {
+                const T send = up ? acc[i] : acc[i + w], keep = up ? acc[i + w] : acc[i];
+                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+#pragma unroll
+        for (; o >= kChunks; o /= 2)
+            acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+        return acc[0];
+    }
+    // of lane: its value, and whether it is the one lane that reports it
+    __device__ static __forceinline__ int value(int lane)
+    {
+        return lane % kChunks * kPer + (sizeof(T) == 4 ? (lane >> 4 & 1) * 2 + (lane >> 3 & 1) : lane >> 4 & 1);
+    }
+    __device__ static __forceinline__ bool reports(int lane) { return sizeof(T) == 4 ? !(lane & 4) : !(lane & 8); }
+};
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v)
@@ -316,6 +374,29 @@ __device__ __forceinline__ T warp_sum(T v)
     for (int off = 16; off > 0; off >>= 1)
         v += __shfl_xor_sync(0xffffffffu, v, off);
     return v;
+}
+
+// Sum of the warps' values v[w stride] in fixed order.  FP32 values are added as a two-float (TwoSum, Knuth): their
+// sum is as good as in FP64 (the values are FP32 sums themselves) and FP64 conversions and additions go at a 64th of
+// the rate; with the seven terms' FP64 sums and the six sensitivities per CTA they held the FP64 pipe 9.5% of the time,
+// between barriers.
+__device__ __forceinline__ double sum_warps(const double *v, int stride)
+{
+    double acc = v[0];
+    for (int w = 1; w < kQWarps; ++w)
+        acc += v[w * stride];
+    return acc;
+}
+__device__ __forceinline__ double sum_warps(const float *v, int stride)
+{
+    float hi = v[0], lo = 0.0f;
+#pragma unroll
+    for (int w = 1; w < kQWarps; ++w) {
+        const float b = v[w * stride], s = hi + b, z = s - hi;
+        lo += (hi - (s - z)) + (b - z);
+        hi = s;
+    }
+    return isinf(hi) ? (double)hi : (double)hi + (double)lo;  // (an infinite sum's low part is NaN)
 }
 
 struct ModeGeom {
@@ -342,6 +423,13 @@ __device__ __forceinline__ ModeGeom mode_geom(const pp_grid &g, int m)
                                node_weight(iz, g.nz, axis_weight(g.nz, g.z0, g.z1, g.mirror_z)))
                    : 0.0;
     return r;
+}
+
+template <typename T>
+__device__ __forceinline__ Mode<T> mode_of(const ModeGeom &mg, double dt)
+{
+    const double eperp = sqrt(1.0 + mg.pz * mg.pz);
+    return {(T)mg.px, (T)mg.py, (T)(mg.pz * mg.pz), (T)eperp, (T)(eperp * dt), (T)(2.0 * dt), (T)-dt};
 }
 
 // fixed-order CTA sum of one double per thread; the result is valid in thread 0
@@ -395,10 +483,10 @@ __global__ void __launch_bounds__(kQThreads) qke_forward_kernel(const QkeS<T> *_
     const int nmodes = g.nx * g.ny * g.nz;
     const int m = blk * kQThreads + threadIdx.x;
     const ModeGeom mg = mode_geom(g, m);
-    const T px = (T)mg.px, py = (T)mg.py, pz2 = (T)(mg.pz * mg.pz), eperp = (T)sqrt(1.0 + mg.pz * mg.pz);
+    const Mode<T> k = mode_of<T>(mg, dt);
     const QkeS<T> *tr = tab + (size_t)c * ldt;
-    T d[6] = {0, 0, 0, 0, 0, 0};
-    Coef<T> c0 = coef_at(tr[0], px, py, pz2, eperp);
+    State<T> d = {};
+    Coef<T> c0 = coef_at(tr[0], k);
     for (int n0 = 0; n0 < n_steps; n0 += kTile) {
         const int cnt = min(kTile, n_steps - n0);
         __syncthreads();
@@ -406,9 +494,9 @@ __global__ void __launch_bounds__(kQThreads) qke_forward_kernel(const QkeS<T> *_
             seg[threadIdx.x] = tr[2 * n0 + threadIdx.x];
         __syncthreads();
         for (int q = 0; q < cnt; ++q) {
-            const Coef<T> ch = coef_at(seg[2 * q + 1], px, py, pz2, eperp);
-            const Coef<T> c1 = coef_at(seg[2 * q + 2], px, py, pz2, eperp);
-            rk4_step(d, c0, ch, c1, (T)dt);
+            const Coef<T> ch = coef_at(seg[2 * q + 1], k);
+            const Coef<T> c1 = coef_at(seg[2 * q + 2], k);
+            rk4_step(d, c0, ch, c1);
             c0 = c1;
         }
     }
@@ -420,13 +508,13 @@ __global__ void __launch_bounds__(kQThreads) qke_forward_kernel(const QkeS<T> *_
         part[(size_t)c * gridDim.x + blk] = s;
 }
 
-// Per-thread asynchronous copies of one 4- or 8-byte value global -> shared
+// Per-thread asynchronous copies of one 8- or 16-byte value global -> shared
 // (cp.async), one commit group per step, so that a thread can wait for its own
 // copies without a barrier.
 template <typename T>
 __device__ __forceinline__ void cp_async_value(T *smem, const T *gmem)
 {
-    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "cp.async copies 4, 8 or 16 bytes");
+    static_assert(sizeof(T) == 8 || sizeof(T) == 16, "cp.async copies 4, 8 or 16 bytes");
     const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"((int)sizeof(T))
                  : "memory");
@@ -436,7 +524,7 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // Forward with checkpoints, then the backward sweep segment by segment.
-// ckpt[c][seg][6][nmp] (T), part[c][blk][6][ldg] (FP64), partJ[c][blk].
+// ckpt[c][seg][3][nmp] (pairs of T: x, y, z of both channels), part[c][blk][7][ldg] (FP64: the sums of sens_from), partJ[c][blk].
 // S = 1: every step's state is kept, and the backward sweep reads it back through
 // a per-thread ring of kQRing shared-memory slots filled kQRing - 1 steps ahead by
 // cp.async (no recomputation).  S > 1: one state per S steps, and each segment is
@@ -453,7 +541,7 @@ constexpr int q_group_steps() { return sizeof(T) == 4 ? 64 : 32; }
 constexpr int kQRing = 4;
 template <typename T, int S>
 __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint_kernel(const QkeS<T> *__restrict__ tab, int ldt, int n_steps,
-                                                                double dt_d, pp_grid g, T *__restrict__ ckpt, int nmp,
+                                                                double dt, pp_grid g, Two<T> *__restrict__ ckpt, int nmp,
                                                                 double *__restrict__ part, int ldg,
                                                                 double *__restrict__ partJ)
 {
@@ -462,47 +550,50 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
     constexpr int kQGroup = GS / S;  // segments per group
     __shared__ double red[kQWarps];
     __shared__ T sb[kQWarps][2 * GS][kSensTerms];       // per-warp sums of the terms
-    __shared__ double usum[2 * GS][kSensTerms];         // their sums over the warps
     __shared__ QkeS<T> seg[2 * GS + 1];  // the samples of the current group (broadcast reads)
-    // per-thread state slots, sst[(q * 6 + i) * kQThreads + tid]: the segment's
-    // recomputed states (S > 1) or the prefetch ring (S = 1, slot q = step % kQRing)
+    // a warp's block for WarpSum, then per-thread state slots, sst[(q * 3 + i) * kQThreads + tid]: the
+    // segment's recomputed states (S > 1) or the prefetch ring (S = 1, slot q = step % kQRing)
     extern __shared__ __align__(16) unsigned char qke_dyn[];
-    T *sst = reinterpret_cast<T *>(qke_dyn);
+    typename WarpSum<T>::Chunk *wbuf =
+        reinterpret_cast<typename WarpSum<T>::Chunk *>(qke_dyn) + (threadIdx.x >> 5) * (32 * WarpSum<T>::kChunks);
+    Two<T> *sst = reinterpret_cast<Two<T> *>(qke_dyn + kQThreads * 16 * sizeof(T));
     const int c = blockIdx.y, blk = blockIdx.x, nblk = gridDim.x;
     const int m = blk * kQThreads + threadIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const ModeGeom mg = mode_geom(g, m);
-    const T px = (T)mg.px, py = (T)mg.py, pz2 = (T)(mg.pz * mg.pz), eperp = (T)sqrt(1.0 + mg.pz * mg.pz);
-    const T dt = (T)dt_d, hd = T(0.5) * dt, sx = dt / T(6);
+    const Mode<T> k = mode_of<T>(mg, dt);
     const QkeS<T> *tr = tab + (size_t)c * ldt;
     const int nseg = (n_steps + S - 1) / S;
     const int mm = min(m, nmp - 1);  // inactive threads store into a valid slot they own alone
-    T *ck = ckpt + (size_t)c * nseg * 6 * nmp;
-    auto stage = [&](int n0, int cnt) {  // samples 2 n0 .. 2 (n0 + cnt) into shared memory
+    Two<T> *ck = ckpt + (size_t)c * nseg * 3 * nmp;
+    auto fetch = [&](int n0, int cnt) {  // samples 2 n0 .. 2 (n0 + cnt) into shared memory
         __syncthreads();
-        for (int k = threadIdx.x; k < 2 * cnt + 1; k += kQThreads)
-            seg[k] = tr[2 * n0 + k];
+        for (int i = threadIdx.x; i < 2 * cnt + 1; i += kQThreads)
+            seg[i] = tr[2 * n0 + i];
         __syncthreads();
     };
     const int ngrp = (nseg + kQGroup - 1) / kQGroup;
 
     // ---- phase A: forward, keeping the state at the start of every segment
-    T d[6] = {0, 0, 0, 0, 0, 0};
+    State<T> d = {};
     {
-        Coef<T> c0 = coef_at(tr[0], px, py, pz2, eperp);
+        Coef<T> c0 = coef_at(tr[0], k);
+        Two<T> *dst = ck + mm;
         for (int gr = 0; gr < ngrp; ++gr) {
             const int g0 = gr * kQGroup, n0g = g0 * S;
-            stage(n0g, min(GS, n_steps - n0g));
+            fetch(n0g, min(GS, n_steps - n0g));
             for (int s = g0; s < min(g0 + kQGroup, nseg); ++s) {
-                if (mg.active)
-#pragma unroll
-                    for (int i = 0; i < 6; ++i)
-                        ck[((size_t)s * 6 + i) * nmp + mm] = d[i];
+                if (mg.active) {
+                    dst[0] = d.x;
+                    dst[nmp] = d.y;
+                    dst[2 * (size_t)nmp] = d.z;
+                }
+                dst += 3 * (size_t)nmp;
                 const int so = (s - g0) * S, cnt = min(S, n_steps - s * S);
                 for (int q = 0; q < cnt; ++q) {
-                    const Coef<T> ch = coef_at(seg[2 * (so + q) + 1], px, py, pz2, eperp);
-                    const Coef<T> c1 = coef_at(seg[2 * (so + q) + 2], px, py, pz2, eperp);
-                    rk4_step(d, c0, ch, c1, dt);
+                    const Coef<T> ch = coef_at(seg[2 * (so + q) + 1], k);
+                    const Coef<T> c1 = coef_at(seg[2 * (so + q) + 2], k);
+                    rk4_step(d, c0, ch, c1);
                     c0 = c1;
                 }
             }
@@ -515,171 +606,140 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
     }
 
     // ---- phase B: backward
-    double *prow = part + ((size_t)c * nblk + blk) * 6 * ldg;
-    T bar[6] = {(T)(-mg.w), 0, 0, 0, 0, 0};
-    T pend[3] = {0, 0, 0};  // coefficient adjoints of the sample at the top of the next step
-    Coef<T> c1 = coef_at(tr[2 * n_steps], px, py, pz2, eperp);
-    Basics<T> b1 = basics(tr[2 * n_steps], px, py, pz2);  // of the sample at the top of the step
+    double *prow = part + ((size_t)c * nblk + blk) * kSensTerms * ldg;
+    // dJ/d delta: J = sum -w (x_p + x_m) / 2; times dt, the factor of every coefficient
+    State<T> bar = {};
+    bar.x = both((T)(-0.5 * mg.w * dt));
+    Coef<T> pend = {};  // adjoints of the coefficients of the sample at the top of the next step
+    Basics<T> b1 = basics(tr[2 * n_steps], k);  // of the sample at the top of the step
+    Coef<T> c1 = coef_from(b1, tr[2 * n_steps], k);
     // S = 1: this thread's stored state at the start of step n into ring slot n % kQRing
+    const Two<T> *src = ck + (size_t)(nseg - 1) * 3 * nmp + mm;  // of the next one
     auto prefetch = [&](int n) {
         if (n >= 0) {
-            T *dst = sst + (size_t)(n % kQRing) * 6 * kQThreads + threadIdx.x;
-            const T *src = ck + (size_t)n * 6 * nmp + mm;
+            Two<T> *dst = sst + (unsigned)n % kQRing * 3 * kQThreads + threadIdx.x;
 #pragma unroll
-            for (int i = 0; i < 6; ++i)
+            for (int i = 0; i < 3; ++i)
                 cp_async_value(dst + i * kQThreads, src + (size_t)i * nmp);
+            src -= 3 * (size_t)nmp;
         }
         cp_async_commit();  // one group per step, empty below step 0
     };
+    // where this lane's total goes: term vi of sample 2n + 2 (slot 2q + 1) or vi - 7 of 2n + 1 (slot 2q)
+    const int vi = WarpSum<T>::value(lane);
+    const bool reports = WarpSum<T>::reports(lane) && vi < 2 * kSensTerms;
+    T *slot = vi < kSensTerms ? &sb[warp][1][vi] : &sb[warp][0][(vi - kSensTerms) % kSensTerms];
     if constexpr (S == 1)
         for (int n = n_steps - 1; n > n_steps - kQRing; --n)
             prefetch(n);
     for (int gr = ngrp - 1; gr >= 0; --gr) {
         const int g0 = gr * kQGroup, n0g = g0 * S, cntg = min(GS, n_steps - n0g);
-        stage(n0g, cntg);
+        fetch(n0g, cntg);
+#pragma unroll(S == 1 ? 2 : 1)
         for (int s = min(g0 + kQGroup, nseg) - 1; s >= g0; --s) {
             const int so = (s - g0) * S, cnt = min(S, n_steps - s * S);
-            const T *xs = sst;  // the states x_q of this segment: xs[(q * 6 + i) * kQThreads + tid]
+            const Two<T> *xs = sst + threadIdx.x;  // the states x_q of this segment: xs[(q * 3 + i) * kQThreads]
             if constexpr (S == 1) {
                 prefetch(s - (kQRing - 1));
                 cp_async_wait<kQRing - 1>();  // this thread's copy of step s has landed
-                xs = sst + (size_t)(s % kQRing) * 6 * kQThreads;
+                xs += (unsigned)s % kQRing * 3 * kQThreads;
             } else {
-#pragma unroll
-                for (int i = 0; i < 6; ++i)
-                    d[i] = mg.active ? ck[((size_t)s * 6 + i) * nmp + mm] : T(0);
+                d = State<T>{};
+                if (mg.active) {
+                    const Two<T> *src = ck + (size_t)s * 3 * nmp + mm;
+                    d.x = src[0];
+                    d.y = src[nmp];
+                    d.z = src[2 * (size_t)nmp];
+                }
                 // the segment's states x_0 .. x_{cnt-1}; x_cnt (the next checkpoint) is not needed
-                Coef<T> c0 = coef_at(seg[2 * so], px, py, pz2, eperp);
+                Coef<T> c0 = coef_at(seg[2 * so], k);
 #pragma unroll 1
                 for (int q = 0;; ++q) {
-#pragma unroll
-                    for (int i = 0; i < 6; ++i)
-                        sst[(q * 6 + i) * kQThreads + threadIdx.x] = d[i];
+                    Two<T> *dst = sst + (size_t)q * 3 * kQThreads + threadIdx.x;
+                    dst[0] = d.x;
+                    dst[kQThreads] = d.y;
+                    dst[2 * kQThreads] = d.z;
                     if (q + 1 >= cnt)
                         break;
-                    const Coef<T> ch = coef_at(seg[2 * (so + q) + 1], px, py, pz2, eperp);
-                    const Coef<T> cn = coef_at(seg[2 * (so + q) + 2], px, py, pz2, eperp);
-                    rk4_step(d, c0, ch, cn, dt);
+                    const Coef<T> ch = coef_at(seg[2 * (so + q) + 1], k);
+                    const Coef<T> cn = coef_at(seg[2 * (so + q) + 2], k);
+                    rk4_step(d, c0, ch, cn);
                     c0 = cn;
                 }
             }
 #pragma unroll 1
-            for (int q = cnt - 1; q >= 0; --q) {
-                {
-                    const QkeS<T> e0 = seg[2 * (so + q)], eh = seg[2 * (so + q) + 1], e1 = seg[2 * (so + q) + 2];
-                    const Basics<T> bh = basics(eh, px, py, pz2);
-                    const Basics<T> b0 = basics(e0, px, py, pz2);
-                    const Coef<T> c0 = coef_from(b0, e0, eperp);
-                    const Coef<T> ch = coef_from(bh, eh, eperp);
-                    T x[6];
+            for (int q = S == 1 ? 0 : cnt - 1; q >= 0; --q) {
+                const QkeS<T> e0 = seg[2 * (so + q)], eh = seg[2 * (so + q) + 1], e1 = seg[2 * (so + q) + 2];
+                const Basics<T> bh = basics(eh, k);
+                const Basics<T> b0 = basics(e0, k);
+                const Coef<T> c0 = coef_from(b0, e0, k);
+                const Coef<T> ch = coef_from(bh, eh, k);
+                const Two<T> *xq = xs + (size_t)q * 3 * kQThreads;
+                const State<T> x = {xq[0], xq[kQThreads], xq[2 * kQThreads]};
+                Coef<T> half, next;
+                step_adjoint(x, c0, ch, c1, bar, pend, half, next);
+                // samples 2n+2 (terms 0..6) and 2n+1 (terms 7..13)
+                T o[16], adj[3];
+                coef_adjoint(pend, adj);
+                sens_from(b1, e1, k.eperp, adj, o);
+                coef_adjoint(half, adj);
+                sens_from(bh, eh, k.eperp, adj, o + kSensTerms);
 #pragma unroll
-                    for (int i = 0; i < 6; ++i)
-                        x[i] = xs[(q * 6 + i) * kQThreads + threadIdx.x];
-                    T k1[6], k2[6], k3[6], y2[6], y3[6], y4[6];
-                    nmul<true>(c0, x, k1);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i)
-                        y2[i] = x[i] + hd * k1[i];
-                    nmul<true>(ch, y2, k2);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i)
-                        y3[i] = x[i] + hd * k2[i];
-                    nmul<true>(ch, y3, k3);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i)
-                        y4[i] = x[i] + dt * k3[i];
-                    T kb1[6], kb2[6], kb3[6], kb4[6], xb[6], yb[6];
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) {
-                        kb1[i] = sx * bar[i];
-                        kb2[i] = T(2) * sx * bar[i];
-                        kb3[i] = kb2[i];
-                        kb4[i] = kb1[i];
-                        xb[i] = bar[i];
-                    }
-                    // k4 = N1 (e1 + y4): completes the sample 2n+2
-                    coef_adj(kb4, y4, pend);
-                    nmul<false>(c1, kb4, yb);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) {
-                        xb[i] -= yb[i];
-                        kb3[i] -= dt * yb[i];
-                    }
-                    T hacc[3] = {0, 0, 0};
-                    coef_adj(kb3, y3, hacc);  // k3 = Nh (e1 + y3)
-                    nmul<false>(ch, kb3, yb);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) {
-                        xb[i] -= yb[i];
-                        kb2[i] -= hd * yb[i];
-                    }
-                    coef_adj(kb2, y2, hacc);  // k2 = Nh (e1 + y2)
-                    nmul<false>(ch, kb2, yb);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) {
-                        xb[i] -= yb[i];
-                        kb1[i] -= hd * yb[i];
-                    }
-                    T nacc[3] = {0, 0, 0};
-                    coef_adj(kb1, x, nacc);  // k1 = N0 (e1 + x)
-                    nmul_sub(c0, kb1, xb, bar);
-                    // emit samples 2n+2 (terms 0..6, slot 2q+1) and 2n+1 (terms 7..13, slot 2q)
-                    T o[16];
-                    sens_from(b1, e1, eperp, pend, o);
-                    sens_from(bh, eh, eperp, hacc, o + kSensTerms);
-#pragma unroll
-                    for (int i = 2 * kSensTerms; i < 16; ++i)
-                        o[i] = T(0);
-                    const T tot = warp_sum16(o, lane);
-                    const int vi = (lane >> 1) & 15;
-                    if ((lane & 1) == 0 && vi < 2 * kSensTerms)
-                        sb[warp][vi < kSensTerms ? 2 * (so + q) + 1 : 2 * (so + q)]
-                          [vi < kSensTerms ? vi : vi - kSensTerms] = tot;
-#pragma unroll
-                    for (int i = 0; i < 3; ++i)
-                        pend[i] = nacc[i];
-                    c1 = c0;
-                    b1 = b0;
-                }
+                for (int i = 2 * kSensTerms; i < 16; ++i)
+                    o[i] = T(0);
+                const T tot = WarpSum<T>::run(wbuf, o, lane);
+                if (reports)
+                    slot[2 * (so + q) * kSensTerms] = tot;
+                pend = next;
+                c1 = c0;
+                b1 = b0;
             }
         }
         __syncthreads();
-        // sample 2 n0g + 1 + kk: each of its seven terms summed over the warps in
-        // fixed order (FP64), then its six sensitivities from the sample's E and Ed
+        // sample 2 n0g + 1 + kk: each of its seven terms summed over the warps in fixed order
         for (int t = threadIdx.x; t < 2 * cntg * kSensTerms; t += kQThreads) {
             const int j = t / (2 * cntg), kk = t % (2 * cntg);
-            double acc = (double)sb[0][kk][j];
-            for (int w = 1; w < kQWarps; ++w)
-                acc += (double)sb[w][kk][j];
-            usum[kk][j] = acc;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < 2 * cntg * 6; t += kQThreads) {
-            const int i = t / (2 * cntg), kk = t % (2 * cntg);
-            const QkeS<T> &e = seg[kk + 1];
-            prow[(size_t)i * ldg + 2 * n0g + 1 + kk] =
-                sample_sens_from_sums(i, (double)e.ex, (double)e.ey, (double)e.edx, (double)e.edy, usum[kk]);
+            prow[(size_t)j * ldg + 2 * n0g + 1 + kk] = sum_warps(&sb[0][kk][j], 2 * GS * kSensTerms);
         }
         __syncthreads();
     }
     // sample 0 (t_i): only the first step's k1 stage reaches it
     {
-        T o[6];
-        sample_sens(tr[0], px, py, pz2, eperp, pend, o);
+        T o[kSensTerms], adj[3];
+        coef_adjoint(pend, adj);
+        sens_from(b1, tr[0], k.eperp, adj, o);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
+        for (int i = 0; i < kSensTerms; ++i) {
             const T v = warp_sum(o[i]);
             if (lane == 0)
                 sb[warp][0][i] = v;
         }
         __syncthreads();
-        if (threadIdx.x < 6) {
-            double acc = 0.0;
-            for (int w = 0; w < kQWarps; ++w)
-                acc += (double)sb[w][0][threadIdx.x];
-            prow[(size_t)threadIdx.x * ldg] = acc;
-        }
+        if (threadIdx.x < kSensTerms)
+            prow[(size_t)threadIdx.x * ldg] = sum_warps(&sb[0][0][threadIdx.x], 2 * GS * kSensTerms);
     }
+}
+
+// The six sensitivities of every sample: the sums over blocks (fixed order) of its seven terms, then its E and Ed.
+template <typename T>
+__global__ void sample_sens_kernel(const double *__restrict__ part, int nblk, int ldg, int nsamp,
+                                   const QkeS<T> *__restrict__ tab, int ldt, double *__restrict__ gs)
+{
+    const int c = blockIdx.y, k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= ldg)
+        return;
+    double u[kSensTerms] = {};
+    const double *p = part + (size_t)c * nblk * kSensTerms * ldg + k;
+    if (k < nsamp)
+        for (int b = 0; b < nblk; ++b, p += (size_t)kSensTerms * ldg)
+#pragma unroll
+            for (int j = 0; j < kSensTerms; ++j)
+                u[j] += p[(size_t)j * ldg];
+    const QkeS<T> e = tab[(size_t)c * ldt + min(k, nsamp - 1)];
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+        gs[((size_t)c * 6 + i) * ldg + k] =
+            sample_sens_from_sums(i, (double)e.ex, (double)e.ey, (double)e.edx, (double)e.edy, u);
 }
 
 // out[c][...] = sum over blocks of part[c][blk][...] (fixed order); n per candidate.
@@ -740,7 +800,7 @@ size_t adjoint_bytes(int S, int n_steps, int nmodes, int ldg)
 {
     const int nblk = (nmodes + kQThreads - 1) / kQThreads;
     const size_t ck = sizeof(T) * 6 * (size_t)((n_steps + S - 1) / S) * nmodes;
-    const size_t pr = sizeof(double) * 6 * (size_t)nblk * ldg;
+    const size_t pr = sizeof(double) * kSensTerms * (size_t)nblk * ldg;
     return ck + pr;
 }
 
@@ -755,8 +815,8 @@ int sm_count()
 // Relative duration of a launch of n equal CTAs, ctas_per_sm at a time on each of
 // sms SMs: every full wave costs 1; a last partial wave costs 1 if some SM runs
 // more than one CTA of it, else kLoneWave (a CTA alone on its SM runs faster:
-// measured 0.61 for the FP32 adjoint at 2 CTAs per SM).
-constexpr double kLoneWave = 0.61;
+// measured 0.63, whole evaluations, for the FP32 adjoint at 2 CTAs per SM).
+constexpr double kLoneWave = 0.63;
 double launch_cost(long long n, int ctas_per_sm, int sms)
 {
     const long long slots = (long long)ctas_per_sm * sms;
@@ -795,7 +855,7 @@ int adjoint_scratch(int n_steps, int nmodes, int ldg, int chunk, AdjointScratch 
     const int nseg = (n_steps + S - 1) / S;
     int rc = pp::scratch(pp::SCR_QKE_CKPT, sizeof(T) * 6 * (size_t)nseg * nmodes * chunk, &a->ck);
     if (!rc)
-        rc = pp::scratch(pp::SCR_QKE_PART, sizeof(double) * 6 * (size_t)nblk * ldg * chunk, &a->part);
+        rc = pp::scratch(pp::SCR_QKE_PART, sizeof(double) * kSensTerms * (size_t)nblk * ldg * chunk, &a->part);
     if (!rc)
         rc = pp::scratch(pp::SCR_QKE_X, sizeof(double) * (size_t)nblk * chunk, &a->pj);
     return rc;
@@ -808,7 +868,7 @@ int run_adjoint(const void *tab, int ldt, int ncand, int n_steps, double dt, con
     void *ck = a.ck, *part = a.part, *pj = a.pj;
     const int nmodes = g->nx * g->ny * g->nz;
     const int nblk = (nmodes + kQThreads - 1) / kQThreads;
-    const size_t dyn = sizeof(T) * (S == 1 ? kQRing : S) * 6 * kQThreads;
+    const size_t dyn = sizeof(T) * (16 + (S == 1 ? kQRing : S) * 6) * kQThreads;
     cudaError_t ea = cudaFuncSetAttribute(qke_adjoint_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)dyn);
     if (ea != cudaSuccess)
@@ -816,10 +876,11 @@ int run_adjoint(const void *tab, int ldt, int ncand, int n_steps, double dt, con
     for (int c0 = 0; c0 < ncand; c0 += chunk) {
         const int nc = std::min(chunk, ncand - c0);
         qke_adjoint_kernel<T, S><<<dim3(nblk, nc), kQThreads, dyn, st>>>(
-            (const QkeS<T> *)tab + (size_t)c0 * ldt, ldt, n_steps, dt, *g, (T *)ck, nmodes, (double *)part, ldg,
+            (const QkeS<T> *)tab + (size_t)c0 * ldt, ldt, n_steps, dt, *g, (Two<T> *)ck, nmodes, (double *)part, ldg,
             (double *)pj);
-        sum_blocks_kernel<<<dim3(nbk(6ll * ldg), nc), 256, 0, st>>>((const double *)part, nblk, 6ll * ldg,
-                                                                    gs + (size_t)c0 * 6 * ldg);
+        sample_sens_kernel<T><<<dim3(nbk(ldg, 128), nc), 128, 0, st>>>(
+            (const double *)part, nblk, ldg, 2 * n_steps + 1, (const QkeS<T> *)tab + (size_t)c0 * ldt, ldt,
+            gs + (size_t)c0 * 6 * ldg);
         sum_blocks_kernel<<<dim3(1, nc), 32, 0, st>>>((const double *)pj, nblk, 1, J + c0);
     }
     cudaError_t e = cudaGetLastError();

@@ -142,3 +142,33 @@ def test_rough_and_long_candidates_keep_single_steps(pp):
     assert pp.sync_status() == pp.PP_OK
     No = float(np.sum(w * no))
     assert abs(N.item() / No - 1) < 1e-4 and abs(Nb.item() / No - 1) < 1e-4
+
+
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 129])
+def test_qke_adjoint_at_the_edges_of_its_groups(pp, n):
+    # groups of 64 (FP32) and 32 (FP64) steps, recomputed segments of 8 and 4, 2 CTAs of modes with a ragged warp.
+    # FP64 to 1e-9 of the largest component; FP32 sums ~200 products of rounded factors: 1e-3 of the norm.  The forward
+    # and the adjoint kernel take the same steps: J bit for bit.
+    dt = 0.02
+    A, E, Ed = oracle.gaussian_rotating_field(0.3, 0.9, 3.0, -0.5 * n * dt, dt / 2, 2 * n + 1)
+    grid = inputs.small_grid(7, 9, 5, ext=1.3)
+    p, w = oracle.grid_modes(grid)
+    Jo, _, gA, gE, gEd = oracle.qke6_grad(A, E, Ed, n, dt, p, w)
+    ref = np.concatenate([gA, gE, gEd])
+    fields = [torch.tensor(x[None], device=DEV) for x in (A, E, Ed)]
+    for precision, j_tol in (("fp64", 1e-9), ("fp32", 1e-4)):
+        J, g = pp.qke_sample_gradient(*fields, dt, grid, precision)
+        old = pp.set_qke_state_budget(0)
+        try:
+            J2, g2 = pp.qke_sample_gradient(*fields, dt, grid, precision)
+        finally:
+            pp.set_qke_state_budget(old)
+        Jf, _ = pp.qke_pair_number(*fields, dt, grid, precision)
+        assert pp.sync_status() == pp.PP_OK
+        assert torch.equal(J, J2) and torch.equal(g, g2) and torch.equal(J, Jf)
+        assert abs(J.item() / Jo - 1) < j_tol
+        g = g[0].cpu().numpy()
+        if precision == "fp64":
+            assert np.abs(g - ref).max() < 1e-9 * np.abs(ref).max()
+        else:
+            assert np.linalg.norm(g - ref) < 1e-3 * np.linalg.norm(ref)
