@@ -161,14 +161,16 @@ struct Product {
     int M, N, K, ldd;
 };
 
-template <bool RB>
+// FEW: few row tiles, with the columns split over blockIdx.y or a second product in blockIdx.z.  Large products keep
+// a kernel without these choices (with them 131072 x 256 x 256 took 0.046 instead of 0.039 ms).
+template <bool RB, bool FEW>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_bf16_kernel(Product p0, Product p1, long long wait_limit, unsigned int *__restrict__ status, int skip_copies)
 {
     using Plan = GemmPlan<RB>;
     constexpr int kStages = Plan::stages;
-    const Product &p = blockIdx.z ? p1 : p0;
-    const int K = p.K, ldd = p.ldd, N = p.N / (int)gridDim.y, col0 = (int)blockIdx.y * N;  // this CTA's columns
+    const Product &p = FEW && blockIdx.z ? p1 : p0;
+    const int K = p.K, ldd = p.ldd, N = FEW ? p.N / (int)gridDim.y : p.N, col0 = FEW ? (int)blockIdx.y * N : 0;  // this CTA's columns
     const uint8_t *__restrict__ A = p.A;
     // rows col0 .. of B: its 128-row tiles are K / 64 tiles long, 8 rows of a chunk 1 KiB
     const uint8_t *__restrict__ B =
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ntiles = p.M / kBM, nchunks = K / kKC;
     const int nb = N > kBM ? 2 : 1;  // packed B row tiles per chunk
-    const uint32_t b_bytes = nb > 1 ? kTileBytes : (uint32_t)N / 8 * 1024;
+    const uint32_t b_bytes = !FEW || nb > 1 ? kTileBytes : (uint32_t)N / 8 * 1024;
     const uint32_t stage_tx = kTileBytes + (RB ? 0 : nb * b_bytes);
 
     if (warp == 1)
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
         const int quad = warp & 3;                     // TMEM lanes 32 quad .. 32 quad + 31
         // this warp's column half: of the accumulator, or of N when that is whole 16s
-        const int half = N > kBM || N % 32 ? kBN / 2 : N / 2;
+        const int half = !FEW || N > kBM || N % 32 ? kBN / 2 : N / 2;
         const int cbeg = ((warp - 2) >> 2) * half, cend = min(N, cbeg + half);
         float *stg = stage_all + (warp - 2) * 32 * kEpiPitch;
         const bool vec = ((uintptr_t)D % 16 == 0) && (ldd % 4 == 0);
@@ -412,11 +414,16 @@ static int launch_products(const Product *p, int count, cudaStream_t stream)
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             GemmPlan<false>::smem_bytes);
+        const auto allow = [](auto kernel, int bytes) {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        };
+        cudaError_t e = allow(gemm_bf16_kernel<false, false>, GemmPlan<false>::smem_bytes);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(gemm_bf16_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     GemmPlan<true>::smem_bytes);
+            e = allow(gemm_bf16_kernel<true, false>, GemmPlan<true>::smem_bytes);
+        if (e == cudaSuccess)
+            e = allow(gemm_bf16_kernel<false, true>, GemmPlan<false>::smem_bytes);
+        if (e == cudaSuccess)
+            e = allow(gemm_bf16_kernel<true, true>, GemmPlan<true>::smem_bytes);
         if (e != cudaSuccess)
             return cuda_fail(e, "GEMM shared-memory attribute");
         int n = 0;
@@ -446,12 +453,11 @@ static int launch_products(const Product *p, int count, cudaStream_t stream)
     }
     const dim3 grid(have > 0 && have < most ? have : most, split, count);
     const Product &q = p[count - 1];
-    if (resident)
-        gemm_bf16_kernel<true><<<grid, kThreads, GemmPlan<true>::smem_bytes, stream>>>(
-            p[0], q, (long long)wait_limit(), status, skip_copies());
-    else
-        gemm_bf16_kernel<false><<<grid, kThreads, GemmPlan<false>::smem_bytes, stream>>>(
-            p[0], q, (long long)wait_limit(), status, skip_copies());
+    const bool few = split > 1 || count > 1;
+    auto *kernel = resident ? (few ? gemm_bf16_kernel<true, true> : gemm_bf16_kernel<true, false>)
+                            : (few ? gemm_bf16_kernel<false, true> : gemm_bf16_kernel<false, false>);
+    kernel<<<grid, kThreads, resident ? GemmPlan<true>::smem_bytes : GemmPlan<false>::smem_bytes, stream>>>(
+        p[0], q, (long long)wait_limit(), status, skip_copies());
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PP_OK : cuda_fail(e, "GEMM launch");
 }
