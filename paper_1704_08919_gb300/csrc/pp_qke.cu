@@ -99,9 +99,9 @@ struct Mode {
 // Reciprocal square root.  FP32: the special-function unit's approximation
 // (rsqrtf, at most 2 ulp), one instruction instead of a square root and a
 // division; its error is far below the FP32 RK4 rounding of the state.  The
-// forward, recomputed and adjoint sweeps all call the same functions, and these leave
-// the compiler no choice of what to contract, so every kernel's trajectory is the
-// same bit for bit.
+// forward, recomputed and adjoint sweeps all call the same functions, and every
+// multiply-add of this file is written as one (it is compiled without contraction), so
+// every kernel's trajectory and sensitivities are the same bit for bit.
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
 
@@ -283,8 +283,8 @@ __device__ __forceinline__ void sens_from(const Basics<T> &b, const QkeS<T> &s, 
     const T ewX = eperp * w * iX;     // R / cr
     const T RbR = Rb * (ewX * s.cr);  // Rb R
     const T gam = Rb * ewX;
-    const T beta = (wb * b.iw + RbR * iw2) - T(2) * Qb * sX * (iw2 * iw2);
-    const T k2 = Qb * (b.rX * iw2) - T(2) * (RbR * iX);  // 2 kappa
+    const T beta = fma(T(-2) * (Qb * sX), iw2 * iw2, fma(RbR, iw2, wb * b.iw));
+    const T k2 = fma(T(-2), RbR * iX, Qb * (b.rX * iw2));  // 2 kappa
     const T mu = fma(k2, s.ee, beta), nu = k2 * b.EP;
     out[0] = mu * b.Px;
     out[1] = mu * b.Py;
@@ -300,10 +300,10 @@ __device__ __forceinline__ double sample_sens_from_sums(int i, double ex, double
                                                         const double u[7])
 {
     switch (i) {
-    case 0: return -u[0] + ex * u[2];
-    case 1: return -u[1] + ey * u[2];
-    case 2: return (ex * u[3] - u[4]) + edy * u[6];
-    case 3: return (ey * u[3] - u[5]) - edx * u[6];
+    case 0: return fma(ex, u[2], -u[0]);
+    case 1: return fma(ey, u[2], -u[1]);
+    case 2: return fma(edy, u[6], fma(ex, u[3], -u[4]));
+    case 3: return fma(-edx, u[6], fma(ey, u[3], -u[5]));
     case 4: return -ey * u[6];
     default: return ex * u[6];
     }
