@@ -56,7 +56,7 @@ struct alignas(sizeof(T) * 8) QkeS {
 // exchanges, about 460 with two channels and WarpSum; it is bound by issue at 4 warps per scheduler.  16 starts on
 // 32 x 32 x 16 modes, 16384 steps, whole evaluation: 101.2 -> 84.5 ms; the warps' sums as two-floats, the six
 // sensitivities after the sum over CTAs, running pointers: 79.2 ms; two backward steps per pass of the loop (no
-// copies of what one step hands to the next): 76.0 ms.
+// copies of what one step hands to the next): 75.9 ms; coefficients of two neighbouring samples at once: 73.8 ms.
 template <typename T>
 using Two = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
 
@@ -69,6 +69,13 @@ __device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c)
 {
     return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
 }
+// ... and of one number, to the same roundings (products not contracted with what follows)
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float fma2(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double fma2(double a, double b, double c) { return fma(a, b, c); }
 template <typename T>
 __device__ __forceinline__ Two<T> both(T v)
 {
@@ -105,49 +112,136 @@ struct Mode {
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
 
-// A product that is not contracted with a following addition
-__device__ __forceinline__ float product(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double product(double a, double b) { return __dmul_rn(a, b); }
-
-// The mode-dependent quantities of one sample that both the coefficients and
-// their derivatives need.
-template <typename T>
-struct Basics {
-    T Px, Py, w2, iw, EP, X, rX;  // rX = 1/sqrt(X) where X > 0, else 0
+// What the coefficients read of a sample (some of it negated), for one sample (V = T) or for two neighbours as a pair.
+template <typename V>
+struct alignas(16) Sample {
+    V nax, nay, ex, ey, nee, cr;
 };
+template <typename T>
+__device__ __forceinline__ Sample<T> sample_of(const QkeS<T> &s)
+{
+    return {-s.ax, -s.ay, s.ex, s.ey, -s.ee, s.cr};
+}
+template <typename T>
+__device__ __forceinline__ Sample<T> half_of(const Sample<Two<T>> &s, int h)
+{
+    return h ? Sample<T>{s.nax.y, s.nay.y, s.ex.y, s.ey.y, s.nee.y, s.cr.y}
+             : Sample<T>{s.nax.x, s.nay.x, s.ex.x, s.ey.x, s.nee.x, s.cr.x};
+}
+
+// The mode-dependent quantities of a sample that both the coefficients and
+// their derivatives need.
+template <typename V>
+struct Basics {
+    V Px, Py, w2, iw, EP, nX, rX;  // nX = -X; rX = 1/sqrt(X) where X > 0, else 0
+};
+template <typename T>
+__device__ __forceinline__ Basics<T> half_of(const Basics<Two<T>> &b, int h)
+{
+    return h ? Basics<T>{b.Px.y, b.Py.y, b.w2.y, b.iw.y, b.EP.y, b.nX.y, b.rX.y}
+             : Basics<T>{b.Px.x, b.Py.x, b.w2.x, b.iw.x, b.EP.x, b.nX.x, b.rX.x};
+}
 
 template <typename T>
-__device__ __forceinline__ Basics<T> basics(const QkeS<T> &s, const Mode<T> &k)
+__device__ __forceinline__ T like(T v, T)
 {
-    Basics<T> b;
-    b.Px = k.px - s.ax;
-    b.Py = k.py - s.ay;
-    b.w2 = fma(b.Px, b.Px, fma(b.Py, b.Py, k.pz2)) + T(1);
-    b.iw = rsq(b.w2);
-    b.EP = fma(s.ex, b.Px, product(s.ey, b.Py));
-    b.X = fma(b.w2, s.ee, -product(b.EP, b.EP));
-    b.rX = b.X > T(0) ? rsq(b.X) : T(0);
+    return v;
+}
+__device__ __forceinline__ float2 like(float v, float2) { return both(v); }
+__device__ __forceinline__ double2 like(double v, double2) { return both(v); }
+__device__ __forceinline__ float rsq_each(float x) { return rsq(x); }
+__device__ __forceinline__ double rsq_each(double x) { return rsq(x); }
+__device__ __forceinline__ float2 rsq_each(float2 x) { return make_float2(rsq(x.x), rsq(x.y)); }
+__device__ __forceinline__ double2 rsq_each(double2 x) { return make_double2(rsq(x.x), rsq(x.y)); }
+__device__ __forceinline__ float rsq_minus(float x) { return x < 0.0f ? rsq(-x) : 0.0f; }
+__device__ __forceinline__ double rsq_minus(double x) { return x < 0.0 ? rsq(-x) : 0.0; }
+__device__ __forceinline__ float2 rsq_minus(float2 x) { return make_float2(rsq_minus(x.x), rsq_minus(x.y)); }
+__device__ __forceinline__ double2 rsq_minus(double2 x) { return make_double2(rsq_minus(x.x), rsq_minus(x.y)); }
+
+template <typename V, typename T>
+__device__ __forceinline__ Basics<V> basics(const Sample<V> &s, const Mode<T> &k)
+{
+    Basics<V> b;
+    b.Px = add(like(k.px, V()), s.nax);
+    b.Py = add(like(k.py, V()), s.nay);
+    b.w2 = add(fma2(b.Px, b.Px, fma2(b.Py, b.Py, like(k.pz2, V()))), like(T(1), V()));
+    b.iw = rsq_each(b.w2);
+    b.EP = fma2(s.ex, b.Px, mul(s.ey, b.Py));
+    b.nX = fma2(b.EP, b.EP, mul(b.w2, s.nee));
+    b.rX = rsq_minus(b.nX);
     return b;
 }
 
-template <typename T>
-__device__ __forceinline__ Coef<T> coef_from(const Basics<T> &b, const QkeS<T> &s, const Mode<T> &k)
+// dt (-Q, R, 2 omega) of one sample or of two
+template <typename V>
+struct Rates {
+    V q, R, W;
+};
+template <typename V, typename T>
+__device__ __forceinline__ Rates<V> rates_from(const Basics<V> &b, const Sample<V> &s, const Mode<T> &k)
 {
-    const T w = b.w2 * b.iw, W = product(k.dt2, w);
-    const bool field = b.X > T(0);
-    const T q = field ? (b.X * b.rX) * (b.iw * (k.ndt * b.iw)) : T(0);
-    const T R = field ? product(k.ep_dt * w * s.cr, b.rX * b.rX) : T(0);
-    Coef<T> c;
-    c.x = both(q);
-    c.z.x = W - R;
-    c.z.y = W + R;
-    return c;
+    const V w = mul(b.w2, b.iw);
+    Rates<V> r;
+    r.W = mul(like(k.dt2, V()), w);
+    r.q = mul(mul(b.nX, b.rX), mul(b.iw, mul(like(-k.ndt, V()), b.iw)));
+    r.R = mul(mul(mul(like(k.ep_dt, V()), w), s.cr), mul(b.rX, b.rX));
+    return r;
 }
 
 template <typename T>
-__device__ __forceinline__ Coef<T> coef_at(const QkeS<T> &s, const Mode<T> &k)
+__device__ __forceinline__ Coef<T> coef_of(T nX, T q, T R, T W)
 {
-    return coef_from(basics(s, k), s, k);
+    const bool field = nX < T(0);  // (X or R not finite: no field either)
+    Coef<T> c;
+    c.x = both(field ? q : T(0));
+    const T r = field ? R : T(0);
+    c.z.x = W - r;
+    c.z.y = W + r;
+    return c;
+}
+template <typename T>
+__device__ __forceinline__ Coef<T> coef_from(const Basics<T> &b, const Rates<T> &r)
+{
+    return coef_of(b.nX, r.q, r.R, r.W);
+}
+template <typename T>
+__device__ __forceinline__ void coef_from(const Basics<Two<T>> &b, const Rates<Two<T>> &r, Coef<T> &first, Coef<T> &second)
+{
+    first = coef_of<T>(b.nX.x, r.q.x, r.R.x, r.W.x);
+    second = coef_of<T>(b.nX.y, r.q.y, r.R.y, r.W.y);
+}
+
+template <typename T>
+__device__ __forceinline__ Coef<T> coef_at(const Sample<T> &s, const Mode<T> &k)
+{
+    const Basics<T> b = basics(s, k);
+    return coef_from(b, rates_from(b, s, k));
+}
+// of both samples of a pair
+template <typename T>
+__device__ __forceinline__ void coef_at(const Sample<Two<T>> &s, const Mode<T> &k, Coef<T> &first, Coef<T> &second)
+{
+    const Basics<Two<T>> b = basics(s, k);
+    coef_from<T>(b, rates_from(b, s, k), first, second);
+}
+
+// cnt pairs of neighbouring samples, tr[0 .. 2 cnt), into shared memory: pair j holds samples 2j and 2j + 1, so the
+// steps' coefficients are formed for two samples at once in packed operations.
+template <typename T>
+__device__ __forceinline__ void fetch_pairs(Sample<Two<T>> *seg, const QkeS<T> *__restrict__ tr, int cnt)
+{
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * cnt; i += kQThreads) {
+        const QkeS<T> e = tr[i];
+        T *dst = reinterpret_cast<T *>(seg + i / 2) + i % 2;
+        dst[0] = -e.ax;
+        dst[2] = -e.ay;
+        dst[4] = e.ex;
+        dst[6] = e.ey;
+        dst[8] = -e.ee;
+        dst[10] = e.cr;
+    }
+    __syncthreads();
 }
 
 // dt k of a stage at delta y, its y component negated: -(dt k)_y = a.(e_1 + u), formed as a_x + a_x u_x + a_z u_z,
@@ -275,17 +369,17 @@ __device__ __forceinline__ double density(const State<T> &d)
 constexpr int kSensTerms = 7;
 
 template <typename T>
-__device__ __forceinline__ void sens_from(const Basics<T> &b, const QkeS<T> &s, T eperp, const T ab[3], T out[7])
+__device__ __forceinline__ void sens_from(const Basics<T> &b, T nee, T cr, T eperp, const T ab[3], T out[7])
 {
     const T w = b.w2 * b.iw, iw2 = b.iw * b.iw;
-    const T sX = b.X * b.rX, iX = b.rX * b.rX;
+    const T sX = -b.nX * b.rX, iX = b.rX * b.rX;
     const T Qb = ab[0], Rb = ab[1], wb = ab[2] + ab[2];
     const T ewX = eperp * w * iX;     // R / cr
-    const T RbR = Rb * (ewX * s.cr);  // Rb R
+    const T RbR = Rb * (ewX * cr);  // Rb R
     const T gam = Rb * ewX;
     const T beta = fma(T(-2) * (Qb * sX), iw2 * iw2, fma(RbR, iw2, wb * b.iw));
     const T k2 = fma(T(-2), RbR * iX, Qb * (b.rX * iw2));  // 2 kappa
-    const T mu = fma(k2, s.ee, beta), nu = k2 * b.EP;
+    const T mu = fma(-k2, nee, beta), nu = k2 * b.EP;
     out[0] = mu * b.Px;
     out[1] = mu * b.Py;
     out[2] = nu;
@@ -478,7 +572,7 @@ __global__ void __launch_bounds__(kQThreads) qke_forward_kernel(const QkeS<T> *_
 {
     constexpr int kTile = 32;  // steps per staged tile
     __shared__ double red[kQWarps];
-    __shared__ QkeS<T> seg[2 * kTile + 1];
+    __shared__ Sample<Two<T>> seg[kTile];
     const int c = blockIdx.y, blk = blockIdx.x;
     const int nmodes = g.nx * g.ny * g.nz;
     const int m = blk * kQThreads + threadIdx.x;
@@ -486,16 +580,13 @@ __global__ void __launch_bounds__(kQThreads) qke_forward_kernel(const QkeS<T> *_
     const Mode<T> k = mode_of<T>(mg, dt);
     const QkeS<T> *tr = tab + (size_t)c * ldt;
     State<T> d = {};
-    Coef<T> c0 = coef_at(tr[0], k);
+    Coef<T> c0 = coef_at(sample_of(tr[0]), k);
     for (int n0 = 0; n0 < n_steps; n0 += kTile) {
         const int cnt = min(kTile, n_steps - n0);
-        __syncthreads();
-        if (threadIdx.x < 2 * cnt + 1)
-            seg[threadIdx.x] = tr[2 * n0 + threadIdx.x];
-        __syncthreads();
+        fetch_pairs(seg, tr + 2 * n0 + 1, cnt);
         for (int q = 0; q < cnt; ++q) {
-            const Coef<T> ch = coef_at(seg[2 * q + 1], k);
-            const Coef<T> c1 = coef_at(seg[2 * q + 2], k);
+            Coef<T> ch, c1;
+            coef_at(seg[q], k, ch, c1);
             rk4_step(d, c0, ch, c1);
             c0 = c1;
         }
@@ -550,7 +641,7 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
     constexpr int kQGroup = GS / S;  // segments per group
     __shared__ double red[kQWarps];
     __shared__ T sb[kQWarps][2 * GS][kSensTerms];       // per-warp sums of the terms
-    __shared__ QkeS<T> seg[2 * GS + 1];  // the samples of the current group (broadcast reads)
+    __shared__ Sample<Two<T>> seg[GS];  // the samples of the current group in pairs (broadcast reads)
     // a warp's block for WarpSum, then per-thread state slots, sst[(q * 3 + i) * kQThreads + tid]: the
     // segment's recomputed states (S > 1) or the prefetch ring (S = 1, slot q = step % kQRing)
     extern __shared__ __align__(16) unsigned char qke_dyn[];
@@ -566,22 +657,16 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
     const int nseg = (n_steps + S - 1) / S;
     const int mm = min(m, nmp - 1);  // inactive threads store into a valid slot they own alone
     Two<T> *ck = ckpt + (size_t)c * nseg * 3 * nmp;
-    auto fetch = [&](int n0, int cnt) {  // samples 2 n0 .. 2 (n0 + cnt) into shared memory
-        __syncthreads();
-        for (int i = threadIdx.x; i < 2 * cnt + 1; i += kQThreads)
-            seg[i] = tr[2 * n0 + i];
-        __syncthreads();
-    };
     const int ngrp = (nseg + kQGroup - 1) / kQGroup;
 
     // ---- phase A: forward, keeping the state at the start of every segment
     State<T> d = {};
     {
-        Coef<T> c0 = coef_at(tr[0], k);
+        Coef<T> c0 = coef_at(sample_of(tr[0]), k);
         Two<T> *dst = ck + mm;
         for (int gr = 0; gr < ngrp; ++gr) {
             const int g0 = gr * kQGroup, n0g = g0 * S;
-            fetch(n0g, min(GS, n_steps - n0g));
+            fetch_pairs(seg, tr + 2 * n0g + 1, min(GS, n_steps - n0g));
             for (int s = g0; s < min(g0 + kQGroup, nseg); ++s) {
                 if (mg.active) {
                     dst[0] = d.x;
@@ -591,8 +676,8 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
                 dst += 3 * (size_t)nmp;
                 const int so = (s - g0) * S, cnt = min(S, n_steps - s * S);
                 for (int q = 0; q < cnt; ++q) {
-                    const Coef<T> ch = coef_at(seg[2 * (so + q) + 1], k);
-                    const Coef<T> c1 = coef_at(seg[2 * (so + q) + 2], k);
+                    Coef<T> ch, c1;
+                    coef_at(seg[so + q], k, ch, c1);
                     rk4_step(d, c0, ch, c1);
                     c0 = c1;
                 }
@@ -611,8 +696,10 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
     State<T> bar = {};
     bar.x = both((T)(-0.5 * mg.w * dt));
     Coef<T> pend = {};  // adjoints of the coefficients of the sample at the top of the next step
-    Basics<T> b1 = basics(tr[2 * n_steps], k);  // of the sample at the top of the step
-    Coef<T> c1 = coef_from(b1, tr[2 * n_steps], k);
+    const Sample<T> e1 = sample_of(tr[2 * n_steps]);  // the sample at the top of the step
+    Basics<T> b1 = basics(e1, k);
+    Coef<T> c1 = coef_from(b1, rates_from(b1, e1, k));
+    T nee1 = e1.nee, cr1 = e1.cr;
     // S = 1: this thread's stored state at the start of step n into ring slot n % kQRing
     const Two<T> *src = ck + (size_t)(nseg - 1) * 3 * nmp + mm;  // of the next one
     auto prefetch = [&](int n) {
@@ -634,7 +721,7 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
             prefetch(n);
     for (int gr = ngrp - 1; gr >= 0; --gr) {
         const int g0 = gr * kQGroup, n0g = g0 * S, cntg = min(GS, n_steps - n0g);
-        fetch(n0g, cntg);
+        fetch_pairs(seg, tr + 2 * n0g, cntg);
 #pragma unroll(S == 1 ? 2 : 1)
         for (int s = min(g0 + kQGroup, nseg) - 1; s >= g0; --s) {
             const int so = (s - g0) * S, cnt = min(S, n_steps - s * S);
@@ -652,7 +739,7 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
                     d.z = src[2 * (size_t)nmp];
                 }
                 // the segment's states x_0 .. x_{cnt-1}; x_cnt (the next checkpoint) is not needed
-                Coef<T> c0 = coef_at(seg[2 * so], k);
+                Coef<T> c0 = coef_at(half_of<T>(seg[so], 0), k);
 #pragma unroll 1
                 for (int q = 0;; ++q) {
                     Two<T> *dst = sst + (size_t)q * 3 * kQThreads + threadIdx.x;
@@ -661,19 +748,18 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
                     dst[2 * kQThreads] = d.z;
                     if (q + 1 >= cnt)
                         break;
-                    const Coef<T> ch = coef_at(seg[2 * (so + q) + 1], k);
-                    const Coef<T> cn = coef_at(seg[2 * (so + q) + 2], k);
+                    const Coef<T> ch = coef_at(half_of<T>(seg[so + q], 1), k);
+                    const Coef<T> cn = coef_at(half_of<T>(seg[so + q + 1], 0), k);
                     rk4_step(d, c0, ch, cn);
                     c0 = cn;
                 }
             }
 #pragma unroll 1
             for (int q = S == 1 ? 0 : cnt - 1; q >= 0; --q) {
-                const QkeS<T> e0 = seg[2 * (so + q)], eh = seg[2 * (so + q) + 1], e1 = seg[2 * (so + q) + 2];
-                const Basics<T> bh = basics(eh, k);
-                const Basics<T> b0 = basics(e0, k);
-                const Coef<T> c0 = coef_from(b0, e0, k);
-                const Coef<T> ch = coef_from(bh, eh, k);
+                const Sample<Two<T>> e = seg[so + q];  // samples 2n and 2n + 1
+                const Basics<Two<T>> b = basics(e, k);
+                Coef<T> c0, ch;
+                coef_from<T>(b, rates_from(b, e, k), c0, ch);
                 const Two<T> *xq = xs + (size_t)q * 3 * kQThreads;
                 const State<T> x = {xq[0], xq[kQThreads], xq[2 * kQThreads]};
                 Coef<T> half, next;
@@ -681,9 +767,9 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
                 // samples 2n+2 (terms 0..6) and 2n+1 (terms 7..13)
                 T o[16], adj[3];
                 coef_adjoint(pend, adj);
-                sens_from(b1, e1, k.eperp, adj, o);
+                sens_from(b1, nee1, cr1, k.eperp, adj, o);
                 coef_adjoint(half, adj);
-                sens_from(bh, eh, k.eperp, adj, o + kSensTerms);
+                sens_from(half_of<T>(b, 1), e.nee.y, e.cr.y, k.eperp, adj, o + kSensTerms);
 #pragma unroll
                 for (int i = 2 * kSensTerms; i < 16; ++i)
                     o[i] = T(0);
@@ -692,7 +778,9 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
                     slot[2 * (so + q) * kSensTerms] = tot;
                 pend = next;
                 c1 = c0;
-                b1 = b0;
+                b1 = half_of<T>(b, 0);
+                nee1 = e.nee.x;
+                cr1 = e.cr.x;
             }
         }
         __syncthreads();
@@ -707,7 +795,7 @@ __global__ void __launch_bounds__(kQThreads, sizeof(T) == 4 ? 2 : 1) qke_adjoint
     {
         T o[kSensTerms], adj[3];
         coef_adjoint(pend, adj);
-        sens_from(b1, tr[0], k.eperp, adj, o);
+        sens_from(b1, nee1, cr1, k.eperp, adj, o);
 #pragma unroll
         for (int i = 0; i < kSensTerms; ++i) {
             const T v = warp_sum(o[i]);
