@@ -34,17 +34,19 @@ CFG = inputs.DE_BATCH
 # Arithmetic of one mode-step (one momentum mode, both spin channels, one
 # step) of the propagation kernel, counted from its source: (flop with
 # FMA = 2, FP32/FP64 instructions).  FP32 paths use compensated accumulation.
-#  rk4:     4 matrix applications, 3 stage updates, increment sum, Fast2Sum
-#  magnus4: dt h_eff, |.|^2, tan(th)/th polynomial (FP32, tracked norm; FP64: cos-1 and
-#           sinc polynomials), scaled vector, increment, Fast2Sum
+#  rk4:     the step's matrix, its application, Fast2Sum
+#  magnus4, FP32: a block of steps as one matrix, 130 flop in 73 instructions (compensated:
+#           164 in 113), divided by the longest block, 10 (4) steps; where the field asks
+#           for shorter blocks a step costs more, so the fractions are lower bounds
+#  magnus4, FP64: dt h_eff, |.|^2, cos-1 and sinc polynomials, scaled vector
 #  split2:  coupling factor, stage, free factor, Fast2Sum
-WORK = {("fp32", "rk4"): (268, 184), ("fp32", "magnus4"): (116, 84), ("fp32", "split2"): (144, 96),
-        ("fp32fast", "rk4"): (244, 160), ("fp32fast", "magnus4"): (92, 52),
+WORK = {("fp32", "rk4"): (137, 94), ("fp32", "magnus4"): (164 / 4, 113 / 4), ("fp32", "split2"): (144, 96),
+        ("fp32fast", "rk4"): (105, 61), ("fp32fast", "magnus4"): (130 / 10, 73 / 10),
         ("fp32fast", "split2"): (112, 64),
-        ("fp64", "rk4"): (244, 148), ("fp64", "magnus4"): (114, 64), ("fp64", "split2"): (112, 64)}
+        ("fp64", "rk4"): (105, 61), ("fp64", "magnus4"): (114, 64), ("fp64", "split2"): (112, 64)}
 # DRAM bytes per candidate per launch of the propagation kernel, from ncu captures
-# (profiles/): the FP32-fast Magnus kernel (256 threads, 8 KiB tiles) read 1.090816 MB for 4 candidates.
-TRAFFIC_PER_CAND = {("fp32fast", "magnus4"): 1.090816e6 / 4}
+# (profiles/): the FP32-fast Magnus kernel (128 threads, 8 KiB tiles) read 0.277 MB and wrote 0.015 MB for 4 candidates.
+TRAFFIC_PER_CAND = {("fp32fast", "magnus4"): 0.29184e6 / 4}
 FP32_LANES_PER_SM = 128
 # GB300 FP64 rate from the part's datasheet figure (no measured FP64 peak exists
 # for this pool); FP32 is derived from the device's SM count and maximum clock.
@@ -496,11 +498,11 @@ def gemm_measure(pp, torch, reps=20):
 
 # FP32 work per mode-step of the QKE adjoint kernel with every forward state kept
 # (forward step and backward step; the variant the default state budget selects at
-# the local-search size), from the kernel's executed instruction counts (ncu,
-# 7 starts x 16384 modes x 1024 steps): 223.0 FFMA + 153.1 FMUL + 67.0 FADD
-# thread-instructions, i.e. 666 flop (FMA = 2) in 443 FP32 instructions.
-QKE_ADJ_FLOP = 666
-QKE_ADJ_FP32_INSTR = 443
+# the local-search size), counted from its source; a packed operation counts for both
+# of its channels.  Coefficients 2 x 42, RK4 step 74, its adjoint 172, sensitivities 60,
+# sums 21 operations.
+QKE_ADJ_FLOP = 571
+QKE_ADJ_FP32_INSTR = 411
 
 
 def localsearch_main(args):
@@ -582,7 +584,7 @@ def localsearch_main(args):
                      / pk["fp32_lanes_per_s"],
                      "peak_source": pk["fp32_source"],
                      **measured_peak(pk, True, achieved),
-                     "note": "%d FP32 flop (%d instructions) per mode-step from ncu SASS counts of the "
+                     "note": "%d FP32 flop (%d operations) per mode-step of the "
                              "kept-state adjoint; whole evaluation (synthesis, adjoint, chain rule) timed"
                              % (QKE_ADJ_FLOP, QKE_ADJ_FP32_INSTR)},
         "search": None if r is None else {
@@ -1109,7 +1111,7 @@ def main():
         "traffic": (TRAFFIC_PER_CAND[(args.precision, args.scheme)] * NP
                     if (args.precision, args.scheme) in TRAFFIC_PER_CAND else None),
         "traffic_source": ("dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of this kernel "
-                           "at 4 candidates (1.091 MB, nothing written), scaled by candidates: the "
+                           "at 4 candidates (0.292 MB), scaled by candidates: the "
                            "per-candidate step table is read from DRAM once, every other access hits L2"
                            if (args.precision, args.scheme) in TRAFFIC_PER_CAND else None)}
 
