@@ -55,8 +55,9 @@ typedef enum {
     PP_FP64 = 0,     /* FP64 throughout (the parity path) */
     PP_FP32 = 1,     /* FP32 propagation with compensated (two-float) state accumulation;
                         FP64 initial state, projection and momentum sum */
-    PP_FP32_FAST = 2 /* as PP_FP32 but with plain FP32 accumulation of the state: about 27%
-                        faster; N stays within ~2e-6 of FP64 on the DE-batch workload while
+    PP_FP32_FAST = 2 /* as PP_FP32 but with plain FP32 accumulation of the state: three
+                        times as fast with PP_MAGNUS4 (PP_RK4 with densities
+                        runs as PP_FP32); N stays within ~2e-6 of FP64 on the DE-batch workload while
                         single n(p) values lose accuracy (a rounding walk of ~1e-6 in the
                         transition amplitude): n_p is written in this mode but is not accurate
                         mode by mode, and no flag marks it; use PP_FP32 or PP_FP64 where n(p)
@@ -90,6 +91,11 @@ typedef enum {
  *             back), which is exact for th up to 0.2 * 2^60 and costs about 2k more
  *             instructions per step.  The workloads here stay near th = 0.11-0.14
  *             (dt ~ 0.02, |p| <= 2.5), where only the polynomials run.
+ *             In FP32, where a candidate's potential is smooth over them, up to 10
+ *             steps (compensated: 4) are applied as one matrix, the product of
+ *             their exponentials up to 6e-7; the length is chosen per candidate
+ *             on the device from its samples.  Densities of uncompensated runs
+ *             with n_steps * T > 1.7e6 keep single steps.
  *  PP_SPLIT2  second-order Strang split operator, the paper's own integrator
  *             (Sec. II.A): free part alpha.p + beta (two half steps), coupling
  *             -alpha.A(t_n + dt/2) (one full step), each factor an exact
