@@ -41,7 +41,7 @@ CFG = inputs.DE_BATCH
 #  magnus4, FP64: dt h_eff, |.|^2, cos-1 and sinc polynomials, scaled vector
 #  split2:  coupling factor, stage, free factor, Fast2Sum
 WORK = {("fp32", "rk4"): (137, 94), ("fp32", "magnus4"): (164 / 4, 113 / 4), ("fp32", "split2"): (144, 96),
-        ("fp32fast", "rk4"): (105, 61), ("fp32fast", "magnus4"): (130 / 10, 73 / 10),
+        ("fp32fast", "rk4"): (137, 94), ("fp32fast", "magnus4"): (130 / 10, 73 / 10),
         ("fp32fast", "split2"): (112, 64),
         ("fp64", "rk4"): (105, 61), ("fp64", "magnus4"): (114, 64), ("fp64", "split2"): (112, 64)}
 # DRAM bytes per candidate per launch of the propagation kernel, from ncu captures

@@ -56,8 +56,9 @@ typedef enum {
     PP_FP32 = 1,     /* FP32 propagation with compensated (two-float) state accumulation;
                         FP64 initial state, projection and momentum sum */
     PP_FP32_FAST = 2 /* as PP_FP32 but with plain FP32 accumulation of the state: three
-                        times as fast with PP_MAGNUS4 (PP_RK4 with densities
-                        runs as PP_FP32); N stays within ~2e-6 of FP64 on the DE-batch workload while
+                        times as fast with PP_MAGNUS4, 1.5 times with PP_SPLIT2; PP_RK4 is
+                        the same compensated path in either FP32 precision.  N stays within
+                        ~2e-6 of FP64 on the DE-batch workload while
                         single n(p) values lose accuracy (a rounding walk of ~1e-6 in the
                         transition amplitude): n_p is written in this mode but is not accurate
                         mode by mode, and no flag marks it; use PP_FP32 or PP_FP64 where n(p)

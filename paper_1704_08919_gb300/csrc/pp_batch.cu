@@ -248,7 +248,7 @@ const BatchTable &batch_table(int precision, int scheme)
          make_batch_table<SplitPolicy<double, false>>(false, 0)},
         {make_batch_table<Rk4Policy<float, true>>(true, 0), make_batch_table<MagnusPolicy<float, true>>(true, 2),
          make_batch_table<SplitPolicy<float, true>>(true, 0)},
-        {make_batch_table<Rk4Policy<float, false>>(true, 0),
+        {make_batch_table<Rk4Policy<float, true>>(true, 0),  // compensated in either precision, as in the uniform path
          make_batch_table<MagnusPolicy<float, false>>(true, 0),
          make_batch_table<SplitPolicy<float, false>>(true, 0)},
     };
@@ -339,7 +339,7 @@ BatchLaunch launch_args(const pp_batch *b, const double *A, double *N, double *n
 int batch_pair_number(const pp_batch *b, const double *A, double *N, double *n_p, int cfg,
                       cudaStream_t stream)
 {
-    return batch_table(pp::precision_of(b->precision, b->scheme, n_p), b->scheme)
+    return batch_table(b->precision, b->scheme)
         .run[cfg](launch_args(b, A, N, n_p, cfg), stream);
 }
 
@@ -788,5 +788,5 @@ int pp_pair_number_grids(const double *A, int32_t ncand, int32_t ld, const int32
     L.partial = (double *)(b + o_part);
     L.N = N;
     L.grid_ctas = std::max(1, std::min((int)work.size(), sms * std::max(blocks, 1)));
-    return batch_table(precision_of(precision, scheme, n_p), scheme).run[cfg](L, st);
+    return tab.run[cfg](L, st);
 }

@@ -51,9 +51,6 @@ void profile_mark_stop(cudaStream_t stream);
 int64_t wait_limit();
 int skip_copies();
 
-// The precision that a call's state is held in (pp_propagate.cu).
-int precision_of(int precision, int scheme, const double *n_p);
-
 // Launch the propagation for one precision (pp_propagate.cu).
 int launch_pair_number(const double *A, int ncand, int ld, const int32_t *n_steps_host, double dt,
                        const pp_grid *grid, int precision, int scheme, double *N, double *n_p,

@@ -1045,10 +1045,6 @@ template <>
 struct Residency<MagnusBlockPolicy<false>> {
     static constexpr int threads = 1280;
 };
-template <>
-struct Residency<Rk4Policy<float, false>> {
-    static constexpr int threads = 1280;
-};
 template <bool C>
 struct Residency<MagnusPolicy<float, C>> {
     static constexpr int threads = 1024;
