@@ -172,6 +172,14 @@ struct StepCounts {
     }
 };
 
+// Scratch of the segments' propagators.  Segments get CTAs of their own while a launch has less than kSegmentCtas CTAs without them
+// (16 per SM).  The scratch has one size, whatever the call's, so that it never moves while a captured graph holds its address:
+// room for the propagators of kSegmentBytes and a count per CTA.  A candidate needs at most 64 bytes for each of kSegTarget
+// modes times segments and a partly filled block per segment, 23 MB; calls of more candidates than fit take several launches of
+// thousands of CTAs each, so that the size costs nothing.
+constexpr int kSegmentCtas = 152 * 16;
+constexpr size_t kSegmentBytes = (size_t)64 << 20, kSegmentScratch = kSegmentBytes + kSegmentCtas * sizeof(int);
+
 template <class P, int THREADS, int TILE_BYTES>
 int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const double *A, int ncand, int ld,
            const int32_t *ns_host, double dt, const pp_grid *grid, double *N, double *n_p, cudaStream_t stream)
@@ -185,30 +193,29 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
     const int ngroups = (nmodes + kGroup - 1) / kGroup;
     V *table = (V *)buf.table;
     using Q = typename MainPolicy<P>::type;
-    // Segments get CTAs of their own while the launch has less than 16 CTAs per SM without them.
-    int layers = buf.segments && (long long)nblk * ncand < 152 * 16 ? Segments<Q>::most(nmodes, sc.max) : 1;
+    int layers = buf.segments && (long long)nblk * ncand < kSegmentCtas ? Segments<Q>::most(nmodes, sc.max) : 1;
     void *seg_out = nullptr;
     int *seg_done = nullptr;
-    int seg_rows = 0, ndone = 0;
+    int seg_rows = 0, ndone = 0, per_launch = ncand;
     if (layers > 1) {
         using Real = typename std::remove_reference<decltype(Q::State::hi[0][0])>::type;
-        seg_rows = layers;
-        ndone = nblk * ncand;
-        const size_t bytes = (size_t)ndone * seg_rows * (Q::kComp ? 16 : 8) * THREADS * sizeof(Real);
+        const size_t per = (size_t)nblk * layers * (Q::kComp ? 16 : 8) * THREADS * sizeof(Real);  // of one candidate
         // without the memory, or with a stream in capture that must not allocate it, each CTA walks all segments, to the
         // same result
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         cudaStreamIsCapturing(stream, &cap);
-        const size_t need = bytes + ndone * sizeof(int);
-        if ((cap == cudaStreamCaptureStatusNone || pp::scratch_holds(pp::SCR_SEGMENTS, need)) &&
-            pp::scratch(pp::SCR_SEGMENTS, need, &seg_out) == PP_OK) {
-            seg_done = (int *)((char *)seg_out + bytes);
+        if (per <= kSegmentBytes &&
+            (cap == cudaStreamCaptureStatusNone || pp::scratch_holds(pp::SCR_SEGMENTS, kSegmentScratch)) &&
+            pp::scratch(pp::SCR_SEGMENTS, kSegmentScratch, &seg_out) == PP_OK) {
+            seg_rows = layers;
+            ndone = nblk * ncand;
+            per_launch = (int)(kSegmentBytes / per < (size_t)ncand ? kSegmentBytes / per : (size_t)ncand);
+            seg_done = (int *)((char *)seg_out + kSegmentBytes);
         } else {
             cudaGetLastError();
             pp::clear_error();
             seg_out = nullptr;
             layers = 1;
-            ndone = 0;
         }
     }
     const int *ns_array = nullptr;
@@ -231,11 +238,16 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
         build_table_kernel<P><<<tg, 256, 0, stream>>>(A, ld, sc.first, ns_array, padded, dt, *grid, table, buf.plans, seg_done,
                                                      ndone, buf.nodes);
     }
-    dim3 pg(nblk, ncand);
     pp::profile_mark_start(stream);
-    propagate_kernel<P, THREADS, TILE_BYTES, MAIN><<<dim3(nblk, ncand, layers), THREADS, 0, stream>>>(
-        A, ld, sc.first, ns_array, table, padded, dt, *grid, n_p, buf.partial, (long long)pp::wait_limit(),
-        pp::skip_copies(), status, buf.plans, buf.nodes, seg_out, seg_done, seg_rows);
+    // as many candidates at a time as the segments' scratch holds (one launch without segments)
+    for (int c0 = 0; c0 < ncand; c0 += per_launch) {
+        const int nc = ncand - c0 < per_launch ? ncand - c0 : per_launch;
+        propagate_kernel<P, THREADS, TILE_BYTES, MAIN><<<dim3(nblk, nc, layers), THREADS, 0, stream>>>(
+            A + (size_t)c0 * 2 * ld, ld, sc.first, ns_array ? ns_array + c0 : nullptr, table + (size_t)c0 * padded, padded,
+            dt, *grid, n_p ? n_p + (size_t)c0 * nmodes : nullptr, buf.partial + (size_t)c0 * ngroups,
+            (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans + c0, buf.nodes, seg_out,
+            seg_done ? seg_done + (size_t)c0 * nblk : nullptr, seg_rows);
+    }
     if constexpr (HasPlan<P>::value) {
         // single steps are rare (rough potentials) except for the densities of long runs, which get a kernel of their own
         int first_rest = kKindSeries;
