@@ -36,11 +36,11 @@ CFG = inputs.DE_BATCH
 # FMA = 2, FP32/FP64 instructions).  FP32 paths use compensated accumulation.
 #  rk4:     the step's matrix, its application, Fast2Sum
 #  magnus4, FP32: a block of steps as one matrix, 130 flop in 73 instructions (compensated:
-#           164 in 113), divided by the longest block, 10 (4) steps; where the field asks
+#           166 in 115), divided by the longest block, 10 (4) steps; where the field asks
 #           for shorter blocks a step costs more, so the fractions are lower bounds
 #  magnus4, FP64: dt h_eff, |.|^2, cos-1 and sinc polynomials, scaled vector
 #  split2:  coupling factor, stage, free factor, Fast2Sum
-WORK = {("fp32", "rk4"): (137, 94), ("fp32", "magnus4"): (164 / 4, 113 / 4), ("fp32", "split2"): (144, 96),
+WORK = {("fp32", "rk4"): (137, 94), ("fp32", "magnus4"): (166 / 4, 115 / 4), ("fp32", "split2"): (144, 96),
         ("fp32fast", "rk4"): (137, 94), ("fp32fast", "magnus4"): (130 / 10, 73 / 10),
         ("fp32fast", "split2"): (112, 64),
         ("fp64", "rk4"): (105, 61), ("fp64", "magnus4"): (114, 64), ("fp64", "split2"): (112, 64)}

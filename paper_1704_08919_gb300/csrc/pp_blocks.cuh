@@ -6,7 +6,7 @@
 // forming a step's generator and applying it to both spin channels, with the pipe 80% busy.  A time grid that
 // resolves the pulse makes the generators of neighbouring steps nearly equal, so the product of m of them is
 // exp(-i Omega.sigma) with an Omega that a short expansion gives to far below FP32 rounding: 73
-// instructions per m <= 10 steps (compensated state, m = 4: 112 per 4 steps instead of 84 per step).
+// instructions per m <= 10 steps (compensated state, m = 4: 115 per 4 steps instead of 84 per step).
 // Fewer roundings also make the result more accurate: n(p) 2.6 times nearer to the FP64 step's (relative 2-norm 4.6e-6
 // instead of 1.2e-5 at 8192 steps), N 3 times.  One generation of 64 pulses on 64 x 64 x 32 modes, 8192 steps:
 // 112.8 -> 27.0 ms; 8 uneven pulses on 47 x 45 x 23 modes, up to 9001 steps, compensated: 7.4 -> 2.9 ms.
@@ -46,10 +46,21 @@ __host__ __device__ __forceinline__ T low_part(double dt, double p, T hi)
         return (T)(dt * p - (double)hi);
 }
 
+// v to a multiple of 2^-24: the difference of two such numbers that is below 1 has no rounding.
+__host__ __device__ __forceinline__ float on_grid(double v)
+{
+    return rintf(16777216.0f * (float)v) * (1.0f / 16777216.0f);
+}
+
 constexpr int kMaxBlock = 10;       // steps per block, uncompensated FP32
 constexpr int kMaxBlockComp = 4;    // compensated: a block's own rounding grows with its angle
 constexpr float kBlockAngle = 1.3f;      // most |Omega| per block: the tangent's quotient, and the growth of the state
-constexpr float kBlockAngleComp = 0.6f;  // the tangent's polynomial
+// The tangent's polynomial holds to 0.6; the roundings at the block's angle, which add up over a long run, ask for less.  With the
+// roundings of S out of the sum (on_grid, the low parts in the rest) n(p) of 120 pulses of 600 to 18000 steps is off by 1.06e-6
+// (root mean square; single steps 1.09e-6, blocks without 1.19e-6), and none of them 1.5 times as far as by single steps and
+// visibly (9 without), for 2 instructions of 113: 8 uneven pulses on 47 x 45 x 23 modes 2.24 instead of 2.16 ms.  (The state's
+// increment formed from S and the rest apart: 0.9 times as far off, but 133 instructions and 3.1 ms.)
+constexpr float kBlockAngleComp = 0.5f;
 // Most estimated error of an amplitude per sqrt(step).  At this line (m = 10 at steps of 0.0244) the expansion is off by
 // 2e-7 in n(p) (2-norm) and 1e-7 in N, FP32 rounding by 2e-6 to 1e-5 and 2e-7; m = 8 (1.6e-7) left 5e-8 and
 // 2e-8, m = 12 (1.5e-6) 7e-7 and 4e-7, more than rounding leaves in N.
@@ -91,7 +102,7 @@ struct MagnusBlockPolicy {
         float ax, ay, c0, c1;  // m dt mean Abar; 1 - l|W|^2 (COMP: without the 1) and its slope in x
         float qx, qy, dx, dy;  // Q; sqrt(l) W
         float wx, wy, vx, vy;  // W, W_1
-        float cz, cz1, pad0, pad1;
+        float cz, cz1, lx, ly;  // COMP: low parts of (ax, ay)
     };
 
     struct State {
@@ -102,8 +113,8 @@ struct MagnusBlockPolicy {
     // Sets the scale h = m dt of the blocks that follow.
     __host__ __device__ static void scale(State &st, double px, double py, double eperp, double h)
     {
-        st.px = (float)(h * px);
-        st.py = (float)(h * py);
+        st.px = COMP ? on_grid(h * px) : (float)(h * px);
+        st.py = COMP ? on_grid(h * py) : (float)(h * py);
         st.sz = (float)(h * eperp);
         st.sz2 = (float)((h * eperp) * (h * eperp));
         st.lx = low_part(h, px, st.px);
@@ -132,10 +143,11 @@ struct MagnusBlockPolicy {
         const float f = fmaf(q * 0.144f, q, fmaf(x, e.c1, e.c0));
         float Ex, Ey, Ez;
         if constexpr (COMP) {
-            // formed as S plus a small rest, so that the rest's roundings stay below S's
+            // formed as S plus a small rest, so that the rest's roundings stay below S's; S itself has none (on_grid), and
+            // the low parts of dt p and of the potential are in the rest
             const float g = fmaf(f, t, yr + tm1);
-            Ex = fmaf(g, Sx, fmaf(qy, e.dx, fmaf(-xy, e.qx, st.lx)));
-            Ey = fmaf(g, Sy, fmaf(qy, e.dy, fmaf(-xy, e.qy, st.ly)));
+            Ex = fmaf(g, Sx, fmaf(qy, e.dx, fmaf(-xy, e.qx, st.lx - e.lx)));
+            Ey = fmaf(g, Sy, fmaf(qy, e.dy, fmaf(-xy, e.qy, st.ly - e.ly)));
             Ez = fmaf(g, st.sz, st.lz);
         } else {
             const float g = fmaf(f, t, yr);
@@ -330,8 +342,11 @@ __host__ __device__ __forceinline__ typename MagnusBlockPolicy<COMP>::Entry bloc
     const float W2 = w0x * w0x + w0y * w0y;
     // third order in the change: -1/840 |D|^2 of the unit-interval slope D = -6 W
     const float third = 1.0f - 0.257f * (1.0f - i4) * W2;
-    e.ax = (float)(dt * (m * x0 + sx));
-    e.ay = (float)(dt * (m * y0 + sy));
+    const double ax = dt * (m * x0 + sx), ay = dt * (m * y0 + sy);
+    e.ax = COMP ? on_grid(ax) : (float)ax;
+    e.ay = COMP ? on_grid(ay) : (float)ay;
+    e.lx = COMP ? (float)(ax - (double)e.ax) : 0.0f;
+    e.ly = COMP ? (float)(ay - (double)e.ay) : 0.0f;
     e.c0 = COMP ? -l * W2 : 1.0f - l * W2;
     e.c1 = -0.241f * l * W2;
     e.qx = 2.0f * m2x - 2.0f * ux * im;
@@ -344,7 +359,6 @@ __host__ __device__ __forceinline__ typename MagnusBlockPolicy<COMP>::Entry bloc
     e.vy = (m1y - 4.0f * m3y) * (-1.0f / 3.0f);
     e.cz = cz;
     e.cz1 = m > 1 ? 3.283f * (w0x * e.qy - w0y * e.qx) : 0.0f;
-    e.pad0 = e.pad1 = 0.0f;
     return e;
 }
 
