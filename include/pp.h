@@ -95,8 +95,10 @@ typedef enum {
  *             (dt ~ 0.02, |p| <= 2.5), where only the polynomials run.
  *             In FP32, where a candidate's potential is smooth over them, up to 10
  *             steps (compensated: 4) are applied as one matrix, the product of
- *             their exponentials up to 6e-7; the length is chosen per candidate
- *             on the device from its samples.  Densities of uncompensated runs
+ *             their exponentials up to terms whose sum over the pulse stays below
+ *             the rounding of the single steps; the length is chosen per candidate
+ *             on the device from its samples (rough, fast or strong fields keep
+ *             shorter matrices or single steps).  Densities of uncompensated runs
  *             with n_steps * T > 1.7e6 keep single steps.
  *  PP_SPLIT2  second-order Strang split operator, the paper's own integrator
  *             (Sec. II.A): free part alpha.p + beta (two half steps), coupling

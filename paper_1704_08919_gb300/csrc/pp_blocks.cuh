@@ -29,7 +29,7 @@
 // channels: in tracked form (MagnusPolicy) a channel costs 3 additions for its vector and 12 multiply-adds.
 //
 // When.  The expansion is left off where a next term of it could be seen; m is chosen per candidate from the
-// potential itself, before any mode is propagated (plan_block).  With m = 1 the block is the step itself.
+// potential itself, before any mode is propagated (longest_block, plan_block).
 #pragma once
 
 #include <math.h>
@@ -61,14 +61,19 @@ constexpr float kBlockAngle = 1.3f;      // most |Omega| per block: the tangent'
 // visibly (9 without), for 2 instructions of 113: 8 uneven pulses on 47 x 45 x 23 modes 2.24 instead of 2.16 ms.  (The state's
 // increment formed from S and the rest apart: 0.9 times as far off, but 133 instructions and 3.1 ms.)
 constexpr float kBlockAngleComp = 0.5f;
-// Most estimated error of an amplitude per sqrt(step).  At this line (m = 10 at steps of 0.0244) the expansion is off by
-// 2e-7 in n(p) (2-norm) and 1e-7 in N, FP32 rounding by 2e-6 to 1e-5 and 2e-7; m = 8 (1.6e-7) left 5e-8 and
-// 2e-8, m = 12 (1.5e-6) 7e-7 and 4e-7, more than rounding leaves in N.
-constexpr float kBlockTol = 6e-7f;
+// The largest estimated error of an amplitude over the whole pulse (plan_block) and the largest angles that the pulse's own frequency
+// and its potential turn by over a block (longest_block).  Set so that what the blocks leave out stays below the rounding of the
+// single steps that they replace: over 10200 random pulses (bands to 60, bursts and flat tops of frequency 0.5 to 12 and fields to
+// 20, steps of 0.005 to 0.08, momenta to 8) it is at most 0.98 times as large in n(p) (2-norm) but for two strong bursts (1.5 and
+// 1.7), and above half of it in 0.13%; compensated at most 0.52 times but for one burst of A = 10 (1.2).  On pulses of band 2 and
+// fluence 2 it is 1e-8 to 7e-8 of N at m = 10 and steps of 0.0244.
+constexpr float kBlockTol = 2e-6f, kBlockTolComp = 1e-7f;
+constexpr float kBlockPhase = 0.5f, kBlockPhaseComp = 0.35f;
+constexpr float kBlockDepth = 0.65f;
 
 // tan(th)/th on x = th^2 <= kBlockAngle^2 as a quotient, least squares at the Chebyshev nodes with the coefficients
 // rounded to FP32 one after the other (relative error 3e-10 with the rounded ones; 6 instructions and a reciprocal
-// where a sine and a cosine take 10), and (tan(th)/th - 1)/x on x <= kBlockAngleComp^2 by interpolation there (3e-10 before
+// where a sine and a cosine take 10), and (tan(th)/th - 1)/x on x <= 0.36 by interpolation there (3e-10 before
 // rounding), for the compensated step, whose small rest must not carry the quotient's rounding.
 struct BlockSeries {
     __host__ __device__ static __forceinline__ float tanc(float x)
@@ -218,27 +223,43 @@ __host__ __device__ constexpr int plan_steps(int plan) { return plan >> 8; }
 constexpr double kDensityLine = 1.7e6;
 __host__ __device__ inline bool single_steps(int n, double dt) { return (double)n * ((double)n * dt) > kDensityLine; }
 
-// What plan_block reads of one step: the bound on its angle (squared) and the size of the expansion's terms.
+// What the plan reads of one step: the bound on its angle and the potential's part of it (squared; their maxima count), the sizes
+// of the expansion's terms (dq and rough squared) and of the potential's second and third differences (squared; sums over the steps).
 struct StepSize {
-    float th2, dq, rough, cube;
+    float th2, depth2, dq, rough, cube, d2, d3;
 };
+
+// The longest block that the pulse's variation allows: w dt = (sum |third differences|^2 / sum |second|^2)^(1/2), a mean
+// frequency that leans to the fast parts (the first differences in place of the second would let a strong slow pulse
+// hide a fast one that makes the pairs) and that quiet stretches do not change.  The expansion is one in m w dt: at 1 its error is
+// 1e-6 of N for bands of 8 and 15, at 3 1e-5 for a band of 40, however weak the field.  The depth, m dt |A|, bounds the terms
+// of higher order in a strong field, which the sums of plan_block do not see (A = 18, w = 0.5: 1.5e-5 of N at a depth of 0.8).
+__host__ __device__ inline int longest_block(float depth, float d2, float d3, int most, float phase)
+{
+    const float w = d3 > 0.0f ? sqrtf(d3 / d2) : (d3 == 0.0f && d2 >= 0.0f ? 0.0f : NAN);
+    int m = most;
+    while (m > 1 && !(m * w <= phase && m * depth <= kBlockDepth))
+        --m;
+    return m;
+}
 
 // The block size from the largest angle of a step, th, and the sums of StepSize over the n steps.  The first neglected
 // terms are of second order in the pulse's change over the block, S^2 W Q with W = m^2 d / 6 and
 // Q = m^3 q / 180 (d = dt^2 A', q = dt^3 A''), and of third, S W^3; what the moments leave out
-// where the samples are not smooth goes with their own differences (rough).  The weights were fitted to the exact product
-// over random pulses (dt 0.02 to 0.05, fluence 0.3 to 13, momenta to 2.5).
-__host__ __device__ inline int plan_block(float th, float dq, float rough, float cube, int n, int most, float angle)
+// where the samples are not smooth goes with their own differences (rough).  A block's terms of the first two kinds turn with the
+// mode's phase and add up by their squares; the third, which has one sign, adds up as it is.  Neither sum grows when a pulse is
+// padded with quiet steps.  The weights were fitted to the exact product over random pulses.
+__host__ __device__ inline int plan_block(float th, float dq, float rough, float cube, int n, int most, float angle,
+                                          float tol = kBlockTol)
 {
-    const float per = 1.0f / sqrtf((float)n);
     for (int m = most; m >= 2; --m) {
         if (m > n || !(m * th <= angle))
             continue;
         const float s = m * th, m2 = (float)(m * m);
-        const float e1 = s * s * m2 * m2 * (1.0f / 320.0f) * dq;  // 3.4 / 1080, m^5 per block, 1/m blocks per step
-        const float e2 = s * s * s * (float)m * (0.03f / 180.0f) * rough;
-        const float e3 = s * m2 * m2 * (float)m * (0.05f / 216.0f) * cube;
-        if ((e1 + e2 + e3) * per <= kBlockTol)
+        const float e1 = s * s * m2 * m2 * (1.0f / 320.0f);  // 3.4 / 1080, m^5 per block, 1/m blocks per step
+        const float e2 = s * s * s * (float)m * (0.1f / 180.0f);
+        const float e3 = s * m2 * m2 * (float)m * (0.3f / 216.0f) * cube;
+        if (e1 * e1 * dq + e2 * e2 * rough + e3 * e3 <= tol * tol)
             return m;
     }
     return 1;
@@ -261,25 +282,32 @@ __host__ __device__ __forceinline__ StepSize step_size(const double *Ax, const d
     const float bx = h * Px + ax + E * uy, by = h * Py + ay + E * ux;
     const float bz = h * E + uy * Px + ux * Py + d6 * fabsf(x0 * dy - y0 * dx);
     r.th2 = 1.000002f * (bx * bx + by * by + bz * bz);
+    r.depth2 = ax * ax + ay * ay;
     const float d = h * sqrtf(dx * dx + dy * dy);
     // second differences, inside the step and across its end; third and fourth across the steps
     const float ix = dx - 2.0f * hx, iy = dy - 2.0f * hy;
     float q = 4.0f * sqrtf(ix * ix + iy * iy);
     float v3 = 0.0f, f4 = 0.0f;
+    r.d2 = r.d3 = 0.0f;
     if (n + 2 <= ns) {
         const float sx = rx(4) - 2.0f * dx, sy = ry(4) - 2.0f * dy;
         q = fmaxf(q, sqrtf(sx * sx + sy * sy));
         if (n >= 1) {
             const float ox = rx(-2) + dx, oy = ry(-2) + dy;
-            v3 = fabsf(sx - ox) + fabsf(sy - oy);
+            const float tx = sx - ox, ty = sy - oy;
+            v3 = fabsf(tx) + fabsf(ty);
             // the middles' own second difference against the ends' fourth-order one
             const float mx = rx(3) + rx(-1) - 2.0f * hx, my = ry(3) + ry(-1) - 2.0f * hy;
-            f4 = fabsf(mx - 0.5f * (sx + ox)) + fabsf(my - 0.5f * (sy + oy));
+            const float fx = mx - 0.5f * (sx + ox), fy = my - 0.5f * (sy + oy);
+            f4 = fabsf(fx) + fabsf(fy);
+            r.d2 = sx * sx + sy * sy;
+            r.d3 = (tx * tx + ty * ty) + (fx * fx + fy * fy);
         }
     }
     q *= h;
-    r.dq = d * q;
+    r.dq = d * q * (d * q);
     r.rough = h * (v3 * (1.0f / 6.0f) + 2.0f * f4);
+    r.rough *= r.rough;
     r.cube = d * d * d;
     return r;
 }

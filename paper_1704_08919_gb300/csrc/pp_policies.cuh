@@ -811,53 +811,59 @@ __device__ __forceinline__ void plan_and_table(const double *__restrict__ Ax, co
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
-    __shared__ float s_warp[4][kPlanThreads / 32], s_cta[4];
+    constexpr int kMaxima = 2, kValues = 7;  // the maxima first, then the sums
+    __shared__ float s_warp[kValues][kPlanThreads / 32], s_cta[kValues];
     __shared__ int s_plan;
     const int tid = threadIdx.x, rank = (int)cluster.block_rank();
     const int at = rank * kPlanThreads + tid;
     constexpr int kStride = kPlanCtas * kPlanThreads;
     const float Px = (float)fmax(fabs(g.x0), fabs(g.x1)), Py = (float)fmax(fabs(g.y0), fabs(g.y1));
     const float Pz = (float)fmax(fabs(g.z0), fabs(g.z1)), E = sqrtf(1.0f + Pz * Pz);
-    float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // th2's maximum, then the sums
+    float sum[kValues] = {};
     for (int n = at; n < ns; n += kStride) {
         const StepSize r = step_size(Ax, Ay, n, ns, (float)dt, Px, Py, E);
         sum[0] = fmaxf(sum[0], r.th2);
-        sum[1] += r.dq;
-        sum[2] += r.rough;
-        sum[3] += r.cube;
+        sum[1] = fmaxf(sum[1], r.depth2);
+        sum[2] += r.dq;
+        sum[3] += r.rough;
+        sum[4] += r.cube;
+        sum[5] += r.d2;
+        sum[6] += r.d3;
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kValues; ++k) {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             const float o = __shfl_xor_sync(0xffffffffu, sum[k], off);
-            sum[k] = k == 0 ? fmaxf(sum[k], o) : sum[k] + o;
+            sum[k] = k < kMaxima ? fmaxf(sum[k], o) : sum[k] + o;
         }
         if ((tid & 31) == 0)
             s_warp[k][tid >> 5] = sum[k];
     }
     __syncthreads();
-    if (tid < 4) {
+    if (tid < kValues) {
         float v = s_warp[tid][0];
         for (int w = 1; w < kPlanThreads / 32; ++w)
-            v = tid == 0 ? fmaxf(v, s_warp[tid][w]) : v + s_warp[tid][w];
+            v = tid < kMaxima ? fmaxf(v, s_warp[tid][w]) : v + s_warp[tid][w];
         s_cta[tid] = v;
     }
     cluster.sync();
     if (tid == 0) {  // every CTA forms the same plan
-        float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float v[kValues] = {};
         for (int r = 0; r < kPlanCtas; ++r) {
             const float *o = cluster.map_shared_rank(s_cta, r);
-            v[0] = fmaxf(v[0], o[0]);
-            for (int k = 1; k < 4; ++k)
-                v[k] += o[k];
+            for (int k = 0; k < kValues; ++k)
+                v[k] = k < kMaxima ? fmaxf(v[k], o[k]) : v[k] + o[k];
         }
         const float th = sqrtf(v[0]);
         // a NaN in the potential fails every comparison: single steps, which carry it to the result
-        const int m = !COMP && densities && single_steps(ns, dt)
-                          ? 1
-                          : plan_block(th, v[1], v[2], v[3], ns, COMP ? kMaxBlockComp : kMaxBlock,
-                                       COMP ? kBlockAngleComp : kBlockAngle);
+        int m = 1;
+        if (COMP || !densities || !single_steps(ns, dt)) {
+            m = longest_block(sqrtf(v[1]), v[5], v[6], COMP ? kMaxBlockComp : kMaxBlock,
+                              COMP ? kBlockPhaseComp : kBlockPhase);
+            m = plan_block(th, v[2], v[3], v[4], ns, m, COMP ? kBlockAngleComp : kBlockAngle,
+                           COMP ? kBlockTolComp : kBlockTol);
+        }
         s_plan = m > 1 ? plan_pack(kKindMain, m) : plan_pack(th > (float)kSeriesLimit ? kKindWide : kKindSeries, 1);
         if (rank == 0)
             *plan_out = s_plan;

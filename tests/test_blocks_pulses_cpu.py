@@ -1,14 +1,22 @@
-"""Whole pulses in blocks of Magnus steps (csrc/pp_blocks.cuh) on the CPU: the header's own tables and step, compiled for the
+"""Whole pulses in blocks of Magnus steps (csrc/pp_blocks.cuh) on the CPU: the header's own plan, tables and step, compiled for the
 host, against the exact product of the pulse's steps, beside the single steps that the blocks replace.
+
+The pulses go beyond those that the plan's weights were fitted to: bands of 2 to 40, bursts in short and long windows, flat tops,
+strong slow fields, a fast burst under a strong slow pulse, jumps, kinks and noise; momenta to 8; both FP32 precisions.  What
+the blocks leave out (the header with its FP32 numbers in FP64) may take at most the single steps' own error on the same pulse
+and modes, in n(p) (2-norm), for every pulse; the error of N with all roundings twice theirs, in the root mean square over the
+pulses (a single pulse's N may be right by chance).
 """
 import math
 import os
+import re
 import shutil
 import subprocess
 
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1704_08919_gb300", "csrc")
 NVCC = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "bin", "nvcc")
 NVCC = NVCC if os.path.exists(NVCC) else shutil.which("nvcc")
 pytestmark = pytest.mark.skipif(NVCC is None, reason="needs nvcc")
@@ -23,6 +31,7 @@ SRC = r"""
 #include <string>
 #include <vector>
 #include "pp_blocks.cuh"
+#include "blocks_double.cuh"
 typedef std::vector<double> V;
 struct Pulse { std::string name; int n; double dt, P; V X, Y; };
 struct Mode { double px, py, eps; };
@@ -84,12 +93,13 @@ static double exact(const Pulse &p, const Mode &m)
     }
     return project(p, m, z);
 }
-static void rescale(float hi[4], float lo[4])
+template <typename T>
+static void rescale(T hi[4], T lo[4])
 {
     double n2 = 0;
     for (int q = 0; q < 4; ++q)
         n2 += (double)hi[q] * hi[q];
-    const float f = ldexpf(1, -(ilogb(n2) >> 1));
+    const T f = (T)ldexp(1, -(ilogb(n2) >> 1));
     for (int q = 0; q < 4; ++q) {
         hi[q] *= f;
         lo[q] *= f;
@@ -138,10 +148,10 @@ static double single(const Pulse &p, const Mode &m)
             z[s][q] = (double)hi[s][q] + lo[s][q];
     return project(p, m, z);
 }
-template <bool COMP>
-static double blocks(const Pulse &p, const Mode &md, int m)
+// P: the policy in FP32, or in FP64, which leaves what the blocks leave out
+template <class P, class ENTRY>
+static double blocks(const Pulse &p, const Mode &md, int m, ENTRY entry)
 {
-    typedef MagnusBlockPolicy<COMP> P;
     typename P::State st;
     memset(&st, 0, sizeof st);
     st.hi[0][0] = st.hi[1][0] = 1;
@@ -150,7 +160,7 @@ static double blocks(const Pulse &p, const Mode &md, int m)
         const int k = std::min(m, p.n - n0);
         if (k < m)
             P::scale(st, md.px, md.py, md.eps, k * p.dt);
-        P::step(st, block_entry<COMP>(p.X.data(), p.Y.data(), n0, k, p.dt));
+        P::step(st, entry(p.X.data(), p.Y.data(), n0, k, p.dt));
         if (b % 32 == 31)
             for (int s = 0; s < 2; ++s)
                 rescale(st.hi[s], st.lo[s]);
@@ -158,21 +168,24 @@ static double blocks(const Pulse &p, const Mode &md, int m)
     double z[2][4];
     for (int s = 0; s < 2; ++s)
         for (int q = 0; q < 4; ++q)
-            z[s][q] = (double)st.hi[s][q] + (COMP ? (double)st.lo[s][q] : 0.0);
+            z[s][q] = (double)st.hi[s][q] + (P::kComp ? (double)st.lo[s][q] : 0.0);
     return project(p, md, z);
 }
+// the kernel's plan: maxima and sums over the steps, in FP32
 template <bool COMP>
 static int plan(const Pulse &p)
 {
-    float th2 = 0, s[3] = {0, 0, 0};
+    float v[7] = {};
     for (int j = 0; j < p.n; ++j) {
         const StepSize r = step_size(p.X.data(), p.Y.data(), j, p.n, (float)p.dt, (float)p.P, (float)p.P, sqrtf(1 + (float)(p.P * p.P)));
-        th2 = fmaxf(th2, r.th2);
-        s[0] += r.dq;
-        s[1] += r.rough;
-        s[2] += r.cube;
+        v[0] = fmaxf(v[0], r.th2);
+        v[1] = fmaxf(v[1], r.depth2);
+        const float s[5] = {r.dq, r.rough, r.cube, r.d2, r.d3};
+        for (int k = 0; k < 5; ++k)
+            v[2 + k] += s[k];
     }
-    return plan_block(sqrtf(th2), s[0], s[1], s[2], p.n, COMP ? kMaxBlockComp : kMaxBlock, COMP ? kBlockAngleComp : kBlockAngle);
+    const int most = longest_block(sqrtf(v[1]), v[5], v[6], COMP ? kMaxBlockComp : kMaxBlock, COMP ? kBlockPhaseComp : kBlockPhase);
+    return plan_block(sqrtf(v[0]), v[2], v[3], v[4], p.n, most, COMP ? kBlockAngleComp : kBlockAngle, COMP ? kBlockTolComp : kBlockTol);
 }
 static Pulse empty(std::string name, int n, double dt, double P) { return Pulse{name, n, dt, P, V(2 * n + 1, 0.0), V(2 * n + 1, 0.0)}; }
 // modes on [w0, w1], amplitudes and phases interpolated from 8 random control points each, int E^2 dt = fluence: a pulse in the
@@ -212,21 +225,45 @@ static Pulse band(std::string name, int n, double dt, double P, double w0, doubl
         }
     return p;
 }
-template <bool COMP>
-static void line(const Pulse &p, const std::vector<Mode> &md, const V &fe, int m)
+// rotating field of peak E, frequency w and Gaussian width tau in the middle of the window
+static Pulse burst(std::string name, int n, double dt, double P, double E, double w, double tau)
 {
-    double N = 0, n2 = 0, e[2] = {0, 0}, e2[2] = {0, 0};
+    Pulse p = empty(name, n, dt, P);
+    for (int k = 0; k <= 2 * n; ++k) {
+        const double t = (0.5 * k - 0.5 * n) * dt, a = E / w * exp(-t * t / (tau * tau));
+        p.X[k] = -a * sin(w * t);
+        p.Y[k] = a * cos(w * t);
+    }
+    return p;
+}
+static Pulse plus(Pulse a, const Pulse &b)
+{
+    for (size_t k = 0; k < a.X.size(); ++k) {
+        a.X[k] += b.X[k];
+        a.Y[k] += b.Y[k];
+    }
+    return a;
+}
+template <bool COMP>
+static void line(const Pulse &p, const std::vector<Mode> &md, const V &fe)
+{
+    const int m = plan<COMP>(p);
+    double N = 0, n2 = 0, e[3] = {}, e2[3] = {};
     for (size_t i = 0; i < md.size(); ++i) {
-        const double d[2] = {single<COMP>(p, md[i]) - fe[i], m > 1 ? blocks<COMP>(p, md[i], m) - fe[i] : 0.0};
+        const double d[3] = {single<COMP>(p, md[i]) - fe[i],
+                             m > 1 ? blocks<MagnusBlockPolicy<COMP>>(p, md[i], m, block_entry<COMP>) - fe[i] : 0.0,
+                             m > 1 ? blocks<dbl::MagnusBlockPolicy<false>>(p, md[i], m, dbl::block_entry<false>) - fe[i] : 0.0};
         N += fe[i];
         n2 += fe[i] * fe[i];
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < 3; ++k) {
             e[k] += d[k];
             e2[k] += d[k] * d[k];
         }
     }
-    printf("%s %d %d %d %.3e %.3e %.3e %.3e\n", p.name.c_str(), COMP, p.n, m, fabs(e[0]) / N, sqrt(e2[0] / n2), fabs(e[1]) / N,
-           sqrt(e2[1] / n2));
+    printf("%s %d %d %d", p.name.c_str(), COMP, p.n, m);
+    for (int k = 0; k < 3; ++k)
+        printf(" %.3e %.3e", fabs(e[k]) / N, sqrt(e2[k] / n2));
+    printf("\n");
 }
 int main(int, char **argv)
 {
@@ -236,8 +273,43 @@ int main(int, char **argv)
     const double dts[4] = {0.02, 0.02, 200.0 / 8192, 0.05};
     for (int i = 0; i < 64; ++i)
         all.push_back(band("work", (int)(600 * pow(30.0, i / 63.0)), dts[i % 4], 1.5 + 0.5 * (i / 4 % 3), 0, 2, 2, 100 + i));
-    std::mt19937_64 g(4);
+    for (double P : {2.0, 2.5})
+        for (int n : {900, 4100}) {
+            all.push_back(band("step.02", n, 0.02, P, 0, 2, 2, 5 + n));
+            all.push_back(band("step.024", n, 200.0 / 8192, P, 0, 2, 2, 6 + n));
+        }
+    all.push_back(band("step.05", 1500, 0.05, 2, 0, 2, 2, 7));
+    all.push_back(band("strong", 4100, 200.0 / 8192, 2, 0, 2, 13, 8));
+    all.push_back(band("weak", 4100, 200.0 / 8192, 2, 0, 2, 0.3, 9));
+    for (double w : {5.0, 15.0, 40.0})
+        for (double P : {2.0, 8.0})
+            for (double dt : {0.01, 0.019})
+                all.push_back(band("band" + std::to_string((int)w), 2000, dt, P, 0, w, 2, 10 + (int)w));
+    all.push_back(band("band.4-8", 2000, 0.02, 2, 4, 8, 2, 11));
+    all.push_back(band("band.4-8.weak", 2000, 0.02, 2, 4, 8, 0.01, 12));
+    for (int n : {1000, 12000})
+        all.push_back(burst("burst.w4", n, 0.05, 2, 0.5, 4, 5));
+    all.push_back(burst("burst.w6.A10", 2000, 0.01, 2, 60, 6, 0.6));
+    all.push_back(burst("burst.w4.A3", 2000, 0.02, 2, 12, 4, 1));
+    all.push_back(burst("slow.A18", 3495, 0.0089, 3.8, 9.5, 0.52, 4.8));
+    all.push_back(burst("slow.A6", 1951, 0.0081, 2, 6.4, 1, 2.2));
+    all.push_back(burst("flat", 8000, 0.05, 2, 0.5, 1.8, 130));
+    all.push_back(plus(band("slow+burst", 4096, 0.02, 2, 0, 2, 2, 13), burst("", 4096, 0.02, 2, 0.2, 5, 5)));
+    all.push_back(plus(band("slow+carrier", 4096, 0.02, 2, 0, 2, 2, 14), band("", 4096, 0.02, 2, 6, 6.3, 0.02, 15)));
+    Pulse jump = empty("jump", 2000, 0.02, 2), kink = empty("kink", 2000, 0.02, 2), noise = band("noise", 2000, 0.02, 2, 0, 2, 2, 16);
+    for (int k = 0; k <= 4000; ++k) {
+        jump.X[k] = k > 1503 ? 0.03 : 0;
+        jump.Y[k] = k > 2200 ? -0.01 : 0;
+        kink.X[k] = -0.003 * std::min(std::max(k - 1001, 0), 1507);
+        kink.Y[k] = 0.001 * std::min(std::max(k - 2013, 0), 600);
+    }
+    std::mt19937_64 g(4), r(5);
     std::uniform_real_distribution<double> U(-1, 1);
+    for (double &v : noise.X)
+        v += 5e-4 * U(r);
+    all.push_back(jump);
+    all.push_back(kink);
+    all.push_back(noise);
     for (const Pulse &p : all) {
         std::vector<Mode> md;
         V fe;
@@ -246,7 +318,8 @@ int main(int, char **argv)
             md.push_back({x, y, sqrt(1 + z * z)});
             fe.push_back(exact(p, md.back()));
         }
-        line<true>(p, md, fe, plan<true>(p));
+        line<false>(p, md, fe);
+        line<true>(p, md, fe);
     }
 }
 """
@@ -258,15 +331,43 @@ def rows(tmp_path_factory):
     src, exe = str(d / "pulses.cu"), str(d / "pulses")
     with open(src, "w") as f:
         f.write(SRC)
-    subprocess.run([NVCC, "-std=c++17", "-O2", "-Xcompiler", "-ffp-contract=off", "-w", "-I",
-                    os.path.join(ROOT, "paper_1704_08919_gb300", "csrc"), "-o", exe, src], check=True)
+    with open(os.path.join(CSRC, "pp_blocks.cuh")) as f:
+        text = f.read().replace("#pragma once", "").replace("namespace {", "namespace dbl {")
+    text = re.sub(r"\bfloat\b", "double", re.sub(r"\b(fma|sqrt|fabs|fmax|rint)f\b", r"\1", text))
+    with open(str(d / "blocks_double.cuh"), "w") as f:
+        f.write(text)
+    subprocess.run([NVCC, "-std=c++17", "-O2", "-Xcompiler", "-ffp-contract=off", "-w", "-I", CSRC, "-I", str(d), "-o", exe, src],
+                   check=True)
     out = subprocess.run([exe, str(MODES)], check=True, capture_output=True, text=True).stdout.splitlines()
     return [(x[0], x[1] == "1", int(x[2]), int(x[3])) + tuple(float(v) for v in x[4:]) for x in map(str.split, out)]
 
 
 def test_compensated_blocks_round_no_more_than_single_steps(rows):
     # n(p) (2-norm): not more in the geometric mean over the pulses, and in few pulses visibly (1.5 times, and more than 1e-6)
-    of = [(x[5], x[7]) for x in rows if x[0] == "work" and x[3] > 1]
+    of = [(x[5], x[7]) for x in rows if x[0] == "work" and x[1] and x[3] > 1]
     assert len(of) >= 48
     assert sum(math.log(block / single) for single, block in of) <= 0.0, of
     assert sum(block > max(1e-6, 1.5 * single) for single, block in of) <= len(of) // 10, of
+
+
+def test_blocks_leave_out_less_than_single_steps_round(rows):
+    for name, comp, n, m, _, single, _, _, _, left in rows:
+        assert left <= single, (name, comp, n, m, single, left)
+    for comp in (False, True):
+        of = [(x[4], x[6]) for x in rows if x[1] == comp and x[3] > 1]
+        single, block = (sum(v[k] ** 2 for v in of) ** 0.5 for k in (0, 1))
+        assert block <= 2 * single, (comp, of)
+
+
+def test_the_plan_of_the_workloads_and_of_what_it_must_refuse(rows):
+    got = {}
+    for name, comp, n, m, *_ in rows:
+        got.setdefault((name, comp), []).append(m)
+    assert set(got["step.02", False]) == {10} and min(got["step.02", True]) >= 3
+    assert min(got["step.024", False]) >= 8 and min(got["step.024", True]) >= 3
+    for name, comp, most in (("jump", False, 1), ("jump", True, 1), ("burst.w6.A10", True, 2), ("burst.w4.A3", True, 2)):
+        assert max(got[name, comp]) <= most, (name, comp, got[name, comp])
+    # padding a pulse with quiet steps does not lengthen its blocks
+    for comp in (False, True):
+        a, b = got["burst.w4", comp]
+        assert a == b
