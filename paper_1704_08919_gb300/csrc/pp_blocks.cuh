@@ -55,12 +55,13 @@ __host__ __device__ __forceinline__ float on_grid(double v)
 constexpr int kMaxBlock = 10;       // steps per block, uncompensated FP32
 constexpr int kMaxBlockComp = 4;    // compensated: a block's own rounding grows with its angle
 constexpr float kBlockAngle = 1.3f;      // most |Omega| per block: the tangent's quotient, and the growth of the state
-// The tangent's polynomial holds to 0.6; the roundings at the block's angle, which add up over a long run, ask for less.  With the
-// roundings of S out of the sum (on_grid, the low parts in the rest) n(p) of 120 pulses of 600 to 18000 steps is off by 1.06e-6
-// (root mean square; single steps 1.09e-6, blocks without 1.19e-6), and none of them 1.5 times as far as by single steps and
-// visibly (9 without), for 2 instructions of 113: 8 uneven pulses on 47 x 45 x 23 modes 2.24 instead of 2.16 ms.  (The state's
-// increment formed from S and the rest apart: 0.9 times as far off, but 133 instructions and 3.1 ms.)
-constexpr float kBlockAngleComp = 0.5f;
+// The tangent's polynomial.  The roundings at the block's angle add up over a long run: with those of S out of the sum (on_grid, the low
+// parts in the rest) n(p) of 120 pulses of 600 to 18000 steps is off by 1.05e-6 (root mean square; single steps 1.09e-6, blocks
+// without 1.19e-6) and in 1 of them 1.5 times as far as by single steps and visibly (9 without; 5 the other way), for 2 instructions
+// of 113: 8 pulses of 5000 steps on 47 x 45 x 23 modes 1.98 instead of 1.92 ms.  (An angle of 0.5 is no more exact, 1.06e-6, and takes 2.73
+// instead of 2.07 ms for 2 pulses on 64 x 64 x 32 modes at steps of 0.0244; the state's increment formed from S and the rest apart: 0.9
+// times as far off, but 133 instructions and 3.1 ms.)
+constexpr float kBlockAngleComp = 0.6f;
 // The largest estimated error of an amplitude over the whole pulse (plan_block) and the largest angles that the pulse's own frequency
 // and its potential turn by over a block (longest_block).  Set so that what the blocks leave out stays below the rounding of the
 // single steps that they replace: over 10200 random pulses (bands to 60, bursts and flat tops of frequency 0.5 to 12 and fields to
