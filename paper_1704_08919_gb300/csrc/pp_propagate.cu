@@ -172,6 +172,17 @@ struct StepCounts {
     }
 };
 
+// The least that a step's angle can be bounded by, whatever the potential (step_size, MagnusPolicy::make_entry6), and the angle of a step
+// from which on the main kernel takes none.
+double least_angle(const pp_grid &g, double dt)
+{
+    const double px = fmax(fabs(g.x0), fabs(g.x1)), py = fmax(fabs(g.y0), fabs(g.y1)), pz = fmax(fabs(g.z0), fabs(g.z1));
+    return dt * sqrt(px * px + py * py + 1.0 + pz * pz);
+}
+template <class P>
+constexpr double kMainAngle = 1.00001 * (IsBlock<typename MainPolicy<P>::type>::value ? (P::kComp ? kBlockAngleComp : kBlockAngle) / 2
+                                                                                        : kSeriesLimit);
+
 // Scratch of the segments' propagators.  Segments get CTAs of their own while a launch has less than kSegmentCtas CTAs without them
 // (16 per SM).  The scratch has one size, whatever the call's, so that it never moves while a captured graph holds its address:
 // room for the propagators of kSegmentBytes and a count per CTA.  A candidate needs at most 64 bytes for each of kSegTarget
@@ -239,8 +250,10 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
                                                      ndone, buf.nodes);
     }
     pp::profile_mark_start(stream);
+    // Steps that leave the main kernel's range by the grid's momenta alone leave it nothing to do.
+    const bool main_empty = HasPlan<P>::value && least_angle(*grid, dt) > kMainAngle<P>;
     // as many candidates at a time as the segments' scratch holds (one launch without segments)
-    for (int c0 = 0; c0 < ncand; c0 += per_launch) {
+    for (int c0 = 0; c0 < ncand && !main_empty; c0 += per_launch) {
         const int nc = ncand - c0 < per_launch ? ncand - c0 : per_launch;
         propagate_kernel<P, THREADS, TILE_BYTES, MAIN><<<dim3(nblk, nc, layers), THREADS, 0, stream>>>(
             A + (size_t)c0 * 2 * ld, ld, sc.first, ns_array ? ns_array + c0 : nullptr, table + (size_t)c0 * padded, padded,
@@ -261,10 +274,13 @@ int launch(const CallBuffers &buf, const StepCounts &sc, int padded, const doubl
                 first_rest = kKindWide;
             }
         }
-        constexpr int kRestCtas = 152 * (1024 / THREADS);
+        // Where the kernel finds nothing to do it should cost little, so it fills the GPU once; where it has everything to do, CTAs that
+        // come and go overlap one item's FP64 ends with another's steps (16 pulses on 64 x 64 x 32 modes, 400 steps of 0.3: 3.26 ms
+        // with the empty main kernel and 8 CTAs per SM, 2.99 with 64 and without it; one launch for each kind of step took 3.05).
+        const int most = 152 * ((main_empty ? 8192 : 1024) / THREADS);
         const long long items = (long long)nblk * ncand;
         propagate_rest_kernel<P, THREADS, TILE_BYTES>
-            <<<(int)(items < kRestCtas ? items : kRestCtas), THREADS, 0, stream>>>(
+            <<<(int)(items < most ? items : most), THREADS, 0, stream>>>(
                 A, ld, sc.first, ns_array, table, padded, dt, *grid, ncand, n_p, buf.partial,
                 (long long)pp::wait_limit(), pp::skip_copies(), status, buf.plans, buf.nodes, first_rest);
     }
