@@ -99,7 +99,11 @@ typedef enum {
  *             the rounding of the single steps; the length is chosen per candidate
  *             on the device from its samples (rough, fast or strong fields keep
  *             shorter matrices or single steps).  Densities of uncompensated runs
- *             with n_steps * T > 1.7e6 keep single steps.
+ *             with n_steps * T > 1.7e6 keep single steps, so that they compare mode
+ *             by mode (2e-5) with densities kept from earlier runs; N of such a call
+ *             is their sum, and the same pulses without densities give another N
+ *             within the rounding of either (about 1e-6).  In every other case N
+ *             does not depend on whether n_p is asked for.
  *  PP_SPLIT2  second-order Strang split operator, the paper's own integrator
  *             (Sec. II.A): free part alpha.p + beta (two half steps), coupling
  *             -alpha.A(t_n + dt/2) (one full step), each factor an exact

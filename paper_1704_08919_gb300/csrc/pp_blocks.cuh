@@ -214,13 +214,12 @@ __host__ __device__ constexpr int plan_pack(int kind, int m) { return kind + 256
 __host__ __device__ constexpr int plan_kind(int plan) { return plan & 255; }
 __host__ __device__ constexpr int plan_steps(int plan) { return plan >> 8; }
 
-// Uncompensated FP32 densities n(p) of a long run keep single steps.  Both ways are right to FP32's own rounding walk, which for
-// single steps is the larger (relative 2-norm 1.1e-5 against 4.8e-6 at 8192 steps, T = 200), but densities
-// kept from single steps and new ones are compared mode by mode, and should agree to 2e-5.  The walk of an amplitude grows
-// as sqrt(n), and the amplitudes themselves fall as 1 / sqrt(T) for a given fluence, so the line is one
-// in n T: over 70 runs below it (1000 to 9300 steps of 0.02 to 0.05, fluence 2) the two differ by at most 1.74e-5, from
-// 2e6 on by up to 2.3e-5.  N, in which the modes' walks average out, is not concerned (at most 1.5e-6 apart,
-// the single steps' error).
+// Uncompensated FP32 densities n(p) of a long run keep single steps.  Blocks are nearer to the FP64 steps (relative 2-norm 4.8e-6
+// against 1.1e-5 at 8192 steps, T = 200), but densities kept from earlier runs are single steps' and are compared mode by mode, to
+// 2e-5.  The rounding walk of an amplitude grows as sqrt(n), and the amplitudes themselves fall as 1 / sqrt(T) for a given
+// fluence, so the line is one in n T: over 70 runs below it (1000 to 9300 steps of 0.02 to 0.05, fluence 2) the two differ by at
+// most 1.74e-5, from 2e6 on by up to 2.3e-5.  N, in which the modes' walks average out, takes blocks when it is asked for alone: it then
+// differs from the densities' sum by the single steps' error (1.4e-6 in the root mean square over 120 pulses; blocks 0.6e-6).
 constexpr double kDensityLine = 1.7e6;
 __host__ __device__ inline bool single_steps(int n, double dt) { return (double)n * ((double)n * dt) > kDensityLine; }
 
