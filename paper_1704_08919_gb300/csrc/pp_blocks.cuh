@@ -9,7 +9,7 @@
 // instructions per m <= 10 steps (compensated state, m = 4: 115 per 4 steps instead of 84 per step).
 // Fewer roundings also make the result more accurate: n(p) 2.6 times nearer to the FP64 step's (relative 2-norm 4.6e-6
 // instead of 1.2e-5 at 8192 steps), N 3 times.  One generation of 64 pulses on 64 x 64 x 32 modes, 8192 steps:
-// 112.8 -> 27.0 ms; 8 uneven pulses on 47 x 45 x 23 modes, up to 9001 steps, compensated: 7.4 -> 2.9 ms.
+// 112.9 -> 19.3 ms; 8 uneven pulses on 47 x 45 x 23 modes, up to 9001 steps, compensated: 6.33 -> 2.25 ms.
 //
 // What.  Step j is exp(-i (E_j + s O_j).sigma) up to the reflection y -> -y that maps spin channel s = +1 to
 // s = -1, with E_j = dt (p - Abar_j) (z part dt eps) and O_j = -(dt^2/6) h_0 x h_1 = E_j x V_j + z cz_j,
