@@ -64,13 +64,14 @@ constexpr float kBlockAngle = 1.3f;      // most |Omega| per block: the tangent'
 constexpr float kBlockAngleComp = 0.6f;
 // The largest estimated error of an amplitude over the whole pulse (plan_block) and the largest angles that the pulse's own frequency
 // and its potential turn by over a block (longest_block).  Set so that what the blocks leave out stays below the rounding of the
-// single steps that they replace: over 10200 random pulses (bands to 60, bursts and flat tops of frequency 0.5 to 12 and fields to
-// 20, steps of 0.005 to 0.08, momenta to 8) it is at most 0.98 times as large in n(p) (2-norm) but for two strong bursts (1.5 and
-// 1.7), and above half of it in 0.13%; compensated at most 0.52 times but for one burst of A = 10 (1.2).  On pulses of band 2 and
-// fluence 2 it is 1e-8 to 7e-8 of N at m = 10 and steps of 0.0244.
+// single steps that they replace: over 20400 random pulses (bands to 60, bursts and flat tops of frequency 0.5 to 12 and fields to
+// 20, noise and jumps to 0.3, steps of 0.005 to 0.08, momenta to 8) it is smaller in n(p) (2-norm) in all but 7 strong fields
+// (1.05 to 1.6 times, 3.0 in one burst of A = 8), and above half of it in 0.2%; compensated at most 0.84 times.  On pulses of
+// band 2 and fluence 2 it is 1e-8 to 7e-8 of N at m = 10 and steps of 0.0244.
 constexpr float kBlockTol = 2e-6f, kBlockTolComp = 1e-7f;
 constexpr float kBlockPhase = 0.5f, kBlockPhaseComp = 0.35f;
 constexpr float kBlockDepth = 0.65f;
+constexpr float kBlockPair = 0.35f, kBlockPairComp = 0.0f;
 
 // tan(th)/th on x = th^2 <= kBlockAngle^2 as a quotient, least squares at the Chebyshev nodes with the coefficients
 // rounded to FP32 one after the other (relative error 3e-10 with the rounded ones; 6 instructions and a reciprocal
@@ -234,11 +235,13 @@ struct StepSize {
 // hide a fast one that makes the pairs) and that quiet stretches do not change.  The expansion is one in m w dt: at 1 its error is
 // 1e-6 of N for bands of 8 and 15, at 3 1e-5 for a band of 40, however weak the field.  The depth, m dt |A|, bounds the terms
 // of higher order in a strong field, which the sums of plan_block do not see (A = 18, w = 0.5: 1.5e-5 of N at a depth of 0.8).
-__host__ __device__ inline int longest_block(float depth, float d2, float d3, int most, float phase)
+// Two steps leave one moment to know, so a pair is exact to first order whatever its samples: up to an angle of `pair` the frequency
+// does not count for it (rough potentials; 16 pulses with noise of 0.05 on 64 x 64 x 32 modes: 5.63 ms, in single steps 7.47).
+__host__ __device__ inline int longest_block(float th, float depth, float d2, float d3, int most, float phase, float pair)
 {
     const float w = d3 > 0.0f ? sqrtf(d3 / d2) : (d3 == 0.0f && d2 >= 0.0f ? 0.0f : NAN);
     int m = most;
-    while (m > 1 && !(m * w <= phase && m * depth <= kBlockDepth))
+    while (m > 1 && !((m * w <= phase || (m == 2 && 2.0f * th <= pair)) && m * depth <= kBlockDepth))
         --m;
     return m;
 }

@@ -859,8 +859,8 @@ __device__ __forceinline__ void plan_and_table(const double *__restrict__ Ax, co
         // a NaN in the potential fails every comparison: single steps, which carry it to the result
         int m = 1;
         if (COMP || !densities || !single_steps(ns, dt)) {
-            m = longest_block(sqrtf(v[1]), v[5], v[6], COMP ? kMaxBlockComp : kMaxBlock,
-                              COMP ? kBlockPhaseComp : kBlockPhase);
+            m = longest_block(th, sqrtf(v[1]), v[5], v[6], COMP ? kMaxBlockComp : kMaxBlock,
+                              COMP ? kBlockPhaseComp : kBlockPhase, COMP ? kBlockPairComp : kBlockPair);
             m = plan_block(th, v[2], v[3], v[4], ns, m, COMP ? kBlockAngleComp : kBlockAngle,
                            COMP ? kBlockTolComp : kBlockTol);
         }

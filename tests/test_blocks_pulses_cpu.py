@@ -184,7 +184,8 @@ static int plan(const Pulse &p)
         for (int k = 0; k < 5; ++k)
             v[2 + k] += s[k];
     }
-    const int most = longest_block(sqrtf(v[1]), v[5], v[6], COMP ? kMaxBlockComp : kMaxBlock, COMP ? kBlockPhaseComp : kBlockPhase);
+    const int most = longest_block(sqrtf(v[0]), sqrtf(v[1]), v[5], v[6], COMP ? kMaxBlockComp : kMaxBlock,
+                                   COMP ? kBlockPhaseComp : kBlockPhase, COMP ? kBlockPairComp : kBlockPair);
     return plan_block(sqrtf(v[0]), v[2], v[3], v[4], p.n, most, COMP ? kBlockAngleComp : kBlockAngle, COMP ? kBlockTolComp : kBlockTol);
 }
 static Pulse empty(std::string name, int n, double dt, double P) { return Pulse{name, n, dt, P, V(2 * n + 1, 0.0), V(2 * n + 1, 0.0)}; }
@@ -365,7 +366,7 @@ def test_the_plan_of_the_workloads_and_of_what_it_must_refuse(rows):
         got.setdefault((name, comp), []).append(m)
     assert set(got["step.02", False]) == {10} and min(got["step.02", True]) >= 3
     assert min(got["step.024", False]) >= 8 and min(got["step.024", True]) >= 3
-    for name, comp, most in (("jump", False, 1), ("jump", True, 1), ("burst.w6.A10", True, 2), ("burst.w4.A3", True, 2)):
+    for name, comp, most in (("jump", False, 2), ("jump", True, 1), ("noise", False, 2), ("noise", True, 1), ("burst.w6.A10", True, 2), ("burst.w4.A3", True, 2)):
         assert max(got[name, comp]) <= most, (name, comp, got[name, comp])
     # padding a pulse with quiet steps does not lengthen its blocks
     for comp in (False, True):
